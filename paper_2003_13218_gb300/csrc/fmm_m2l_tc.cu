@@ -45,10 +45,20 @@
 // drain it and add it to the row held in FP32 registers (round to nearest)
 // while the tensor core works on the next run.
 //
-// Roles (6 warps): warp 0 lane 0 issues TMA loads into a 2..6-stage ring, warp 1
-// lane 0 issues tcgen05.mma, warps 2..5 drain TMEM (warp w reads TMEM lanes
-// 32 (w mod 4) .. +31, one target row per thread) and write the FP32 level
-// array.  Every mbarrier wait is bounded (globaltimer); on a timeout the
+// Roles (6 warps): warp 0 issues TMA loads into a 2..6-stage ring, warp 1
+// issues tcgen05.mma (both run with all lanes, one elected lane issues), warps
+// 2..5 drain TMEM (warp w reads TMEM lanes 32 (w mod 4) .. +31, one target row
+// per thread) and write the FP32 level array.
+//
+// The issuer's instruction stream bounds the launch, not the tensor pipe or the
+// copies: halving the copied bytes or the MMAs per stage moved the level-6
+// launch (N = 1M, p = 12) by 1-6 %, taking a quarter of the ring away by 2 %,
+// while its per-stage code took ~900 cycles against 350-700 of MMA time.
+// Issued from a single-lane branch every TMA / MMA operand is moved to uniform
+// registers first; run by the whole warp, with the chunk structure fixed at
+// compile time (NCH) and the grading unpacked once per tile, the launch went
+// 3.69 -> 2.69 ms (N = 1M, p = 12), 24.9 -> 16.1 ms (N = 10M, p = 10) and
+// 2.00 -> 1.51 ms (N = 100k, ws = 2, p = 8).  Every mbarrier wait is bounded (globaltimer); on a timeout the
 // kernel records FMM_ERR_TIMEOUT, waits (bounded) for its copies and MMAs in
 // flight, frees TMEM and returns.
 #include <cuda.h>
@@ -168,10 +178,6 @@ __device__ __forceinline__ int chunk_products(uint32_t g, int kc)
     return c == 0 ? 3 : c;
 }
 
-// First K16 step of chunk kc (a 3-product chunk) whose lowest input degree reaches D2: from there on the
-// chunk drops x1 y0 (0: no such step).
-__device__ __forceinline__ int step_split(uint32_t gs, int kc) { return (int)((gs >> (3 * kc)) & 7u); }
-
 // A graded offset's stages: two consecutive chunks of one product each (x0 y0 only) share one stage, their
 // A0 / B0 boxes in the places of the two terms; returns how many chunks the stage starting at kc covers.
 __device__ __forceinline__ int stage_chunks(uint32_t g, int kc, int kchunks)
@@ -201,6 +207,21 @@ __device__ __forceinline__ uint64_t global_ns()
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
+
+// 1 in one lane of a converged warp (the same lane every time a warp asks), 0 in the others
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t e;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(e));
+    return e;
+}
+
+// a value that every lane of the warp holds alike, made visibly so (uniform registers)
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
@@ -244,6 +265,46 @@ __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_fla
     }
 }
 
+__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// The bounded wait of a whole converged warp: every lane gets the same answer (lanes that read the clock at
+// different times must not leave a loop with warp-wide instructions in it one by one).  CLUSTER: with
+// cluster-scope acquire.  The clock is read out of line: the usual wait is one poll and one vote.
+template <bool CLUSTER>
+__device__ __forceinline__ bool mbar_poll_warp(uint32_t bar, uint32_t parity)
+{
+    return __all_sync(0xffffffffu, CLUSTER ? mbar_try_cluster(bar, parity) : mbar_try(bar, parity)) != 0;
+}
+
+template <bool CLUSTER>
+__device__ __noinline__ bool mbar_wait_warp_slow(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                 uint64_t limit_ns)
+{
+    uint64_t t0 = global_ns();
+    for (uint32_t i = 0;; ++i) {
+        if (mbar_poll_warp<CLUSTER>(bar, parity)) return true;
+        if ((i & 63) == 63 && __any_sync(0xffffffffu, *abort_flag != 0 || global_ns() - t0 > limit_ns)) return false;
+    }
+}
+
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                               uint64_t limit_ns)
+{
+    return mbar_poll_warp<CLUSTER>(bar, parity) || mbar_wait_warp_slow<CLUSTER>(bar, parity, abort_flag, limit_ns);
+}
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2,
                                             int c3)
 {
@@ -265,27 +326,38 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
 
 // tcgen05 shared-memory matrix descriptor: K-major, SW-byte swizzle (layout
 // code 4 for 64 bytes, 2 for 128 bytes), 8-row groups 8 SW bytes apart
-// (stride byte offset), version field 1.
+// (stride byte offset), version field 1.  The high word is a constant; the low
+// word holds the address in 16-byte units (14 bits: shared-memory addresses
+// stay below 2^18) and the leading byte offset (unused for swizzled K-major),
+// so an operand o bytes further on has the low word + o / 16.
 template <int SW>
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr)
+constexpr uint32_t sdesc_hi()
 {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;                              // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(((8u * SW) >> 4) & 0x3FFFu) << 32;   // stride byte offset
-    d |= (uint64_t)1 << 46;                              // descriptor version
-    d |= (uint64_t)(SW == 128 ? 2 : 4) << 61;            // swizzle mode
-    return d;
+    return ((8u * SW) >> 4) | (1u << 14) | ((SW == 128 ? 2u : 4u) << 29);
 }
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFFu) | (1u << 16); }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc)
+// D += A . B (acc = 0: D = A . B), both descriptors with the high word `hi`
+template <bool PAIR>
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                        uint32_t acc)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-        : "memory");
+    if (PAIR)  // 2-SM: 128 rows of A and N / 2 rows of B per CTA, 128 lanes of D in each CTA's TMEM
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+            "setp.ne.b32 p, %5, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(tmem_d),
+            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+            "setp.ne.b32 p, %5, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(tmem_d),
+            "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc)
+            : "memory");
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar)
@@ -411,26 +483,10 @@ __device__ __forceinline__ void cluster_sync_all()
 __device__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                   uint64_t limit_ns = WAIT_LIMIT_NS)
 {
-    uint32_t ok0;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok0)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok0) return true;  // the usual case: no clock read
+    if (mbar_try_cluster(bar, parity)) return true;  // the usual case: no clock read
     uint64_t t0 = global_ns();
     for (uint32_t i = 0;; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
+        if (mbar_try_cluster(bar, parity)) return true;
         if ((i & 63) == 63) {
             if (*abort_flag) return false;
             if (global_ns() - t0 > limit_ns) return false;
@@ -438,10 +494,12 @@ __device__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int *a
     }
 }
 
-// arrive on an mbarrier of the peer CTA (shared::cluster address)
+// arrive on an mbarrier of the peer CTA (shared::cluster address).  No cluster-scope release: what it orders
+// are the epilogue's TMEM loads, which tcgen05.wait::ld has completed, and a release there is a memory barrier
+// of ~2,400 cycles per drain while the copies stream in.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 
 // TMA loads into this CTA's shared memory whose completion is counted on the
@@ -463,18 +521,6 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
         "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
         "%4}], [%5];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
-        : "memory");
-}
-
-// 2-SM MMA: D (128 lanes in each CTA's TMEM) += A (128 rows per CTA) . B (N/2 rows per CTA)
-__device__ __forceinline__ void mma_f16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                             uint32_t acc)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
         : "memory");
 }
 
@@ -513,67 +559,57 @@ struct Products<2, 3> {
     __device__ static constexpr int b(int k) { return k == 1 ? 1 : k == 3 ? 2 : 0; }
 };
 
-// The MMAs of one K chunk: the first NP products over the chunk's nk valid K16 steps (the third, x1 y0, only
-// on steps below S2), straight-line code (operand addresses are compile-time offsets from the stage bases);
-// `first` starts a new accumulator.
-template <int NP, typename PR, int K16, int SW, bool PAIR, int S2 = K16>
-__device__ __forceinline__ void issue_chunk(uint32_t tmem_d, uint32_t a0, uint32_t b0, uint32_t stageA, uint32_t stageB,
-                                            int nk, uint32_t idesc, bool first)
-{
-    // descriptors of the stage bases once; an operand at byte offset o from a base is the base's descriptor
-    // plus o / 16 in the address field (14 bits of 16-byte units: shared-memory addresses stay below 2^18,
-    // so the sum never carries out of the field)
-    const uint64_t ad0 = sdesc<SW>(a0), bd0 = sdesc<SW>(b0);
-    const uint64_t sa = stageA >> 4, sb = stageB >> 4;
+// What a pipeline stage holds, per K chunk of an offset: kind 1 one chunk with np products (of the third,
+// x1 y0, the K16 steps below s2), kind 2 this chunk and the next with the product x0 y0 each, kind 0 nothing
+// (the chunk went into the stage before).  Worked out once per tile; NCH fixes the number of chunks and of
+// valid K16 steps, so the issuer's per-stage code is straight.
+template <int KC>
+struct ChunkPlan {
+    int kind[KC], np[KC], s2[KC];
+    __device__ __forceinline__ ChunkPlan(uint32_t gchunks, uint32_t gsteps, int nprod, int k16)
+    {
+        bool taken = false;
 #pragma unroll
-    for (int pr = 0; pr < NP; ++pr) {
-#pragma unroll
-        for (int k16 = 0; k16 < K16; ++k16) {
-            if (k16 >= nk) continue;         // zero fill beyond K
-            if (pr == 2 && k16 >= S2) continue;  // steps of degree >= D2: x0 y0 + x0 y1 only
-            const uint64_t ad = ad0 + (uint64_t)PR::a(pr) * sa + (uint64_t)(k16 * 2);
-            const uint64_t bd = bd0 + (uint64_t)PR::b(pr) * sb + (uint64_t)(k16 * 2);
-            const uint32_t acc = (first && pr == 0 && k16 == 0) ? 0u : 1u;
-            if (PAIR) mma_f16_pair(tmem_d, ad, bd, idesc, acc);
-            else mma_bf16(tmem_d, ad, bd, idesc, acc);
+        for (int kc = 0; kc < KC; ++kc) {
+            const int c = (int)((gchunks >> (2 * kc)) & 3u), st = (int)((gsteps >> (3 * kc)) & 7u);
+            np[kc] = c == 0 ? nprod : c;
+            s2[kc] = st == 0 ? k16 : st;
+            const bool two = !taken && c == 1 && kc + 1 < KC && ((gchunks >> (2 * (kc + 1))) & 3u) == 1u;
+            kind[kc] = taken ? 0 : two ? 2 : 1;
+            taken = two;
         }
     }
-}
+};
 
-// The MMAs of a merged stage: chunk kc0 + t in term place t (t = 0, 1), product x0 y0 only; nk1 valid
-// K16 steps in the second chunk.
-template <int K16, int SW, bool PAIR>
-__device__ __forceinline__ void issue_merged(uint32_t tmem_d, uint32_t a0, uint32_t b0, uint32_t stageA,
-                                             uint32_t stageB, int nk1, uint32_t idesc, bool first)
-{
-    const uint64_t ad0 = sdesc<SW>(a0), bd0 = sdesc<SW>(b0);  // stepped as in issue_chunk
-    const uint64_t sa = stageA >> 4, sb = stageB >> 4;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-#pragma unroll
-        for (int k16 = 0; k16 < K16; ++k16) {
-            if (t == 1 && k16 >= nk1) continue;
-            const uint64_t ad = ad0 + (uint64_t)t * sa + (uint64_t)(k16 * 2);
-            const uint64_t bd = bd0 + (uint64_t)t * sb + (uint64_t)(k16 * 2);
-            const uint32_t acc = (first && t == 0 && k16 == 0) ? 0u : 1u;
-            if (PAIR) mma_f16_pair(tmem_d, ad, bd, idesc, acc);
-            else mma_bf16(tmem_d, ad, bd, idesc, acc);
-        }
-    }
-}
-
-// A chunk with all of the split's products, x1 y0 dropped from step s2 on (s2 = 0: on no step): one
-// compile-time variant per split point
+// The MMAs of one stage (operand addresses are compile-time steps from the stage's descriptor words): nk valid
+// K16 steps in the chunk, nk1 in the second one of a kind-2 stage; acc0 = 0 starts a new accumulator.  Products
+// outer, K16 steps inner.
 template <typename PR, int K16, int SW, bool PAIR>
-__device__ __forceinline__ void issue_full_chunk(int s2, uint32_t tmem_d, uint32_t a0, uint32_t b0, uint32_t stageA,
-                                                 uint32_t stageB, int nk, uint32_t idesc, bool first)
+__device__ __forceinline__ void issue_stage(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t sa, uint32_t sb,
+                                            int nk, int nk1, int kind, int np, int s2, uint32_t idesc, uint32_t acc0)
 {
-    if constexpr (PR::n == 3 && K16 == 4) {
-        if (s2 == 1) return issue_chunk<3, PR, K16, SW, PAIR, 1>(tmem_d, a0, b0, stageA, stageB, nk, idesc, first);
-        if (s2 == 2) return issue_chunk<3, PR, K16, SW, PAIR, 2>(tmem_d, a0, b0, stageA, stageB, nk, idesc, first);
-        if (s2 == 3) return issue_chunk<3, PR, K16, SW, PAIR, 3>(tmem_d, a0, b0, stageA, stageB, nk, idesc, first);
+    constexpr uint32_t hi = sdesc_hi<SW>();
+    if (PR::n == 3 && kind == 2) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int k16 = 0; k16 < K16; ++k16) {
+                if (k16 >= (t == 0 ? nk : nk1)) continue;
+                mma_f16<PAIR>(tmem_d, a_lo + (uint32_t)t * sa + 2 * k16, b_lo + (uint32_t)t * sb + 2 * k16, hi, idesc,
+                              (t == 0 && k16 == 0) ? acc0 : 1u);
+            }
+        return;
     }
-    issue_chunk<PR::n, PR, K16, SW, PAIR>(tmem_d, a0, b0, stageA, stageB, nk, idesc, first);
+#pragma unroll
+    for (int pr = 0; pr < PR::n; ++pr) {
+        if (PR::n == 3 && pr >= np) continue;
+#pragma unroll
+        for (int k16 = 0; k16 < K16; ++k16) {
+            if (k16 >= nk || (PR::n == 3 && pr == 2 && k16 >= s2)) continue;
+            mma_f16<PAIR>(tmem_d, a_lo + (uint32_t)PR::a(pr) * sa + 2 * k16, b_lo + (uint32_t)PR::b(pr) * sb + 2 * k16, hi,
+                          idesc, (pr == 0 && k16 == 0) ? acc0 : 1u);
+        }
+    }
 }
 
 // One CTA sums, for 128 target rows, the products of a list of offsets:
@@ -607,12 +643,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __shared__ int produced_sh, consumed_sh;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t smem0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    const uint32_t smem0 = warp_uniform((smem_u32(smem_dyn) + 1023u) & ~1023u);
     constexpr int KCH = kchunk_of(SW);  // K elements per stage
     constexpr int K16 = SW / 32;        // MMAs (K = 16) per stage and product
-    const uint32_t stageA = TC_ROWS * SW;
-    const uint32_t stageB = (uint32_t)a.npad * SW;
-    const uint32_t stage_bytes = PA * stageA + PB * stageB;
+    constexpr uint32_t stageA = TC_ROWS * SW;
+    constexpr uint32_t stageB = NCH * 16u * SW;
+    constexpr uint32_t stage_bytes = PA * stageA + PB * stageB;
     constexpr bool kGradable = PA == 2 && PB == 2;  // the degree grading applies to the 2 x 2-term products
 
     // M2L: the 8 parity classes of one brick run side by side, so CTAs resident
@@ -656,11 +692,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tmem_sh;
+    const uint32_t tmem = warp_uniform(tmem_sh);
     volatile int *abort_flag = &abort_sh;
 
+    // The producer and issuer warps run their loops with all lanes (waits and ring arithmetic are the same in
+    // every lane) and one elected lane issues: operands of a TMA copy or an MMA then come from uniform
+    // registers, where a single-lane branch has to move each of them there per instruction.
+    const uint32_t el = elect_one();
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // ---------------- producer: TMA loads of the A brick and the B operator
             const CUtensorMap *mA[3] = {&mA0, &mA1, &mA2};
             const CUtensorMap *mL[3] = {&mL0, &mL1, &mL1};
@@ -673,35 +713,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             auto load_offset = [&](const CUtensorMap *const *src, int c1, int c2, int c3, int oslot, bool graded) {
                 for (int kc = 0; kc < a.kchunks && ok;) {
                     if (it >= a.stages &&
-                        !mbar_wait(smem_u32(&bar_empty[s]), (round & 1u) ^ 1u, abort_flag, a.wait_ns)) {
+                        !mbar_wait_warp(smem_u32(&bar_empty[s]), (round & 1u) ^ 1u, abort_flag, a.wait_ns)) {
                         ok = false;
                         break;
                     }
                     const uint32_t full = smem_u32(&bar_full[s]);
                     const uint32_t base = smem0 + (uint32_t)s * stage_bytes;
                     const int nkc = (kGradable && graded) ? stage_chunks(a.gchunks, kc, a.kchunks) : 1;
-                    if (nkc == 2) {  // two x0 y0 chunks: A0 and B0 of chunk kc + t in term place t
-                        mbar_expect_tx(full, 2u * ((uint32_t)(a.rows * SW) + stageB));
+                    if (el) {
+                        if (nkc == 2) {  // two x0 y0 chunks: A0 and B0 of chunk kc + t in term place t
+                            mbar_expect_tx(full, 2u * ((uint32_t)(a.rows * SW) + stageB));
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {
-                            tma_load_4d(base + t * stageA, src[0], full, (kc + t) * KCH, c1, c2, c3);
-                            tma_load_3d(base + PA * stageA + t * stageB, mB[0], full, (kc + t) * KCH, 0, oslot);
+                            for (int t = 0; t < 2; ++t) {
+                                tma_load_4d(base + t * stageA, src[0], full, (kc + t) * KCH, c1, c2, c3);
+                                tma_load_3d(base + PA * stageA + t * stageB, mB[0], full, (kc + t) * KCH, 0, oslot);
+                            }
+                        } else {
+                            int na = PA, nb = PB;
+                            if (kGradable && graded) {
+                                const int np = chunk_products(a.gchunks, kc);
+                                na = np == 3 ? 2 : 1;
+                                nb = np >= 2 ? 2 : 1;
+                            }
+                            mbar_expect_tx(full, (uint32_t)(na * a.rows * SW) + (uint32_t)nb * stageB);
+#pragma unroll
+                            for (int i = 0; i < PA; ++i)
+                                if (i < na) tma_load_4d(base + i * stageA, src[i], full, kc * KCH, c1, c2, c3);
+#pragma unroll
+                            for (int j = 0; j < PB; ++j)
+                                if (j < nb) tma_load_3d(base + PA * stageA + j * stageB, mB[j], full, kc * KCH, 0, oslot);
                         }
-                    } else {
-                        int na = PA, nb = PB;
-                        if (kGradable && graded) {
-                            const int np = chunk_products(a.gchunks, kc);
-                            na = np == 3 ? 2 : 1;
-                            nb = np >= 2 ? 2 : 1;
-                        }
-                        mbar_expect_tx(full, (uint32_t)(na * a.rows * SW) + (uint32_t)nb * stageB);
-#pragma unroll
-                        for (int i = 0; i < PA; ++i)
-                            if (i < na) tma_load_4d(base + i * stageA, src[i], full, kc * KCH, c1, c2, c3);
-#pragma unroll
-                        for (int j = 0; j < PB; ++j)
-                            if (j < nb) tma_load_3d(base + PA * stageA + j * stageB, mB[j], full, kc * KCH, 0, oslot);
                     }
+                    __syncwarp();
                     kc += nkc;
                     ++it;
                     if (++s == a.stages) {
@@ -733,81 +776,78 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 for (int o = o_begin; o < o_end && ok; ++o)
                     load_offset(mA, x0 + a.ws, y0 + a.ws, o * a.src_np2 + z0 + a.ws, a.noff + o, false);
             }
-            produced_sh = it;
-            if (!ok) {
-                abort_sh = 1;
-                atomicOr(a.err, ERRF_TIMEOUT);
+            if (el) {
+                produced_sh = it;
+                if (!ok) {
+                    abort_sh = 1;
+                    atomicOr(a.err, ERRF_TIMEOUT);
+                }
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             // ---------------- MMA issuer: one fresh accumulator per group of offsets
             using PR = Products<PA, PB>;
+            constexpr int KC = (NCH + K16 - 1) / K16;
+            const ChunkPlan<KC> graded_plan(kGradable && a.mode == 0 ? a.gchunks : 0u,
+                                            kGradable && a.mode == 0 ? a.gsteps : 0u, PR::n, K16);
+            const uint32_t a_lo0 = sdesc_lo(smem0), b_lo0 = sdesc_lo(smem0 + PA * stageA);
+            const uint32_t full0 = smem_u32(&bar_full[0]), empty0 = smem_u32(&bar_empty[0]);
             int it = 0, s = 0;
-            uint32_t round = 0;
+            uint32_t phase = 0;
             // the test hook makes this thread's first wait run out (its budget), as a lost copy would
-            bool ok = !(a.inject_stall && !mbar_wait(smem_u32(&bar_never), 0, abort_flag, a.wait_ns));
+            bool ok = !(a.inject_stall && !mbar_wait_warp(smem_u32(&bar_never), 0, abort_flag, a.wait_ns));
             for (int g = 0; g < groups.ng && ok; ++g) {
                 const int acc = g & 1;
                 const uint32_t use = (uint32_t)(g >> 1);
-                if (g >= 2 && !mbar_wait(smem_u32(&bar_tempty[acc]), (use - 1u) & 1u, abort_flag, a.wait_ns)) {
+                if (g >= 2 && !mbar_wait_warp(smem_u32(&bar_tempty[acc]), (use - 1u) & 1u, abort_flag, a.wait_ns)) {
                     ok = false;
                     break;
                 }
                 fence_after();
                 const uint32_t tmem_d = tmem + (uint32_t)(acc * 256);
-                bool first = true;  // the group's first MMA overwrites the accumulator
+                uint32_t acc0 = 0;  // the group's first MMA overwrites the accumulator
                 for (int o = groups.begin(g); o < groups.end(g) && ok; ++o) {
-                    const bool graded =
-                        kGradable && (a.gchunks | a.gsteps) != 0u && a.mode == 0 && o_begin + o < a.n_il;
-                    for (int kc = 0; kc < a.kchunks;) {
-                        if (!mbar_wait(smem_u32(&bar_full[s]), round & 1u, abort_flag, a.wait_ns)) {
+                    const bool graded = a.mode == 0 && o_begin + o < a.n_il;
+#pragma unroll
+                    for (int kc = 0; kc < KC; ++kc) {
+                        const int kind = graded ? graded_plan.kind[kc] : 1;
+                        if (kind == 0 || !ok) continue;
+                        if (!mbar_wait_warp(full0 + 8u * (uint32_t)s, phase, abort_flag, a.wait_ns)) {
                             ok = false;
-                            break;
+                            continue;
                         }
                         fence_after();
-                        const uint32_t base = smem0 + (uint32_t)s * stage_bytes;
-                        const int nk = a.ksteps - K16 * kc < K16 ? a.ksteps - K16 * kc : K16;
-                        const int np = graded ? chunk_products(a.gchunks, kc) : PR::n;
-                        const int nkc = graded ? stage_chunks(a.gchunks, kc, a.kchunks) : 1;
-                        if constexpr (kGradable) {
-                            if (nkc == 2) {
-                                const int nk1 = a.ksteps - K16 * (kc + 1) < K16 ? a.ksteps - K16 * (kc + 1) : K16;
-                                issue_merged<K16, SW, false>(tmem_d, base, base + PA * stageA, stageA, stageB, nk1,
-                                                             a.idesc, first);
-                            } else if (np == 1)
-                                issue_chunk<1, PR, K16, SW, false>(tmem_d, base, base + PA * stageA, stageA, stageB, nk,
-                                                                   a.idesc, first);
-                            else if (np == 2)
-                                issue_chunk<2, PR, K16, SW, false>(tmem_d, base, base + PA * stageA, stageA, stageB, nk,
-                                                                   a.idesc, first);
-                            else
-                                issue_full_chunk<PR, K16, SW, false>(graded ? step_split(a.gsteps, kc) : 0, tmem_d, base,
-                                                                     base + PA * stageA, stageA, stageB, nk, a.idesc,
-                                                                     first);
-                        } else {
-                            issue_chunk<PR::n, PR, K16, SW, false>(tmem_d, base, base + PA * stageA, stageA, stageB, nk,
-                                                                   a.idesc, first);
+                        if (el) {
+                            const uint32_t at = (uint32_t)s * (stage_bytes >> 4);
+                            const int nk = NCH - K16 * kc < K16 ? NCH - K16 * kc : K16;
+                            const int nk1 = NCH - K16 * (kc + 1) < K16 ? NCH - K16 * (kc + 1) : K16;
+                            issue_stage<PR, K16, SW, false>(tmem_d, a_lo0 + at, b_lo0 + at, stageA >> 4, stageB >> 4, nk, nk1,
+                                                            kind, graded ? graded_plan.np[kc] : PR::n,
+                                                            graded ? graded_plan.s2[kc] : K16, a.idesc, acc0);
+                            mma_commit(empty0 + 8u * (uint32_t)s);
                         }
-                        first = false;
-                        kc += nkc;
-                        mma_commit(smem_u32(&bar_empty[s]));
+                        __syncwarp();
+                        acc0 = 1;
                         ++it;
                         if (++s == a.stages) {
                             s = 0;
-                            ++round;
+                            phase ^= 1u;
                         }
                     }
                 }
-                if (ok) mma_commit(smem_u32(&bar_tfull[acc]));
+                if (ok && el) mma_commit(smem_u32(&bar_tfull[acc]));
+                __syncwarp();
             }
-            consumed_sh = it;
-            if (!ok) {
-                abort_sh = 1;
-                atomicOr(a.err, ERRF_TIMEOUT);
+            if (el) {
+                consumed_sh = it;
+                if (!ok) {
+                    abort_sh = 1;
+                    atomicOr(a.err, ERRF_TIMEOUT);
+                }
+                mma_commit(smem_u32(&bar_done));  // arrives once every issued MMA has completed
             }
-            mma_commit(smem_u32(&bar_done));  // arrives once every issued MMA has completed
         }
         __syncwarp();
     } else {
@@ -824,7 +864,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         for (int g = 0; g < groups.ng; ++g) {
             const int acc = g & 1;
             const uint32_t use = (uint32_t)(g >> 1);
-            if (!mbar_wait(smem_u32(&bar_tfull[acc]), use & 1u, abort_flag, a.wait_ns)) {
+            if (!mbar_wait_warp(smem_u32(&bar_tfull[acc]), use & 1u, abort_flag, a.wait_ns)) {
                 ok = false;
                 break;
             }
@@ -836,7 +876,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (lane == 0) mbar_arrive(smem_u32(&bar_tempty[acc]));
         }
         float mx = 0.f;  // largest |out_i sx(i)| of this thread's row (a.amax_out)
-        if (!__all_sync(0xffffffffu, ok)) {
+        if (!ok) {
             abort_sh = 1;
             if (lane == 0) atomicOr(a.err, ERRF_TIMEOUT);
         } else {
@@ -949,17 +989,17 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
                                           const CUtensorMap *mB1, const CUtensorMap *mL0, const CUtensorMap *mL1,
                                           const TcArgs &a, int pair, uint32_t rank, uint32_t smem0, float *stage,
                                           bool staged, PairBars &bars, uint32_t tmem, volatile int *abort_flag,
-                                          PairPipe &pp)
+                                          PairPipe &pp, uint32_t el)
 {
     constexpr int PA = 2, PB = 2, SW = 128;
     constexpr int KCH = kchunk_of(SW), K16 = SW / 32;
     using PR = Products<PA, PB>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool leader = rank == 0;
-    const uint32_t halfN = (uint32_t)a.npad / 2;
-    const uint32_t stageA = TC_ROWS * SW;
-    const uint32_t stageB = halfN * SW;
-    const uint32_t stage_bytes = PA * stageA + PB * stageB;
+    constexpr uint32_t halfN = NCH * 8u;  // rows of B per CTA
+    constexpr uint32_t stageA = TC_ROWS * SW;
+    constexpr uint32_t stageB = halfN * SW;
+    constexpr uint32_t stage_bytes = PA * stageA + PB * stageB;
 
     const int grp = pair % a.groups;
     const int cls = (pair / a.groups) & 7;
@@ -975,8 +1015,9 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
     const int cx = cls & 1, cy = (cls >> 1) & 1, cz = (cls >> 2) & 1;
     const int np2 = a.np + 2 * a.ws;
 
+    // as in k_m2l_tc, the producer and issuer warps run with all lanes and the elected lane `el` issues
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // ---------------- producer (both CTAs): own A brick, own half of B, completing on the leader's barrier
             const CUtensorMap *mA[2] = {mA0, mA1};
             const CUtensorMap *mL[2] = {mL0, mL1};
@@ -984,8 +1025,8 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
             bool ok = true;
             auto load_offset = [&](const CUtensorMap *const *src, int c1, int c2, int c3, int oslot, bool graded) {
                 for (int kc = 0; kc < a.kchunks && ok;) {
-                    if (pp.it >= a.stages && !mbar_wait_cluster(smem_u32(&bars.empty[pp.s]), (pp.round & 1u) ^ 1u,
-                                                                abort_flag, a.wait_ns)) {
+                    if (pp.it >= a.stages &&
+                        !mbar_wait_warp(smem_u32(&bars.empty[pp.s]), (pp.round & 1u) ^ 1u, abort_flag, a.wait_ns)) {
                         ok = false;
                         break;
                     }
@@ -993,33 +1034,36 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
                     const uint32_t full = map_shared(full_local, 0);
                     const uint32_t base = smem0 + (uint32_t)pp.s * stage_bytes;
                     const int nkc = graded ? stage_chunks(a.gchunks, kc, a.kchunks) : 1;
-                    if (nkc == 2) {  // two x0 y0 chunks: A0 and B0 of chunk kc + t in term place t
-                        // the leader's barrier counts both CTAs' copies (the same boxes in each)
-                        if (leader) mbar_expect_tx(full_local, 2u * 2u * ((uint32_t)(a.rows * SW) + stageB));
+                    if (el) {
+                        if (nkc == 2) {  // two x0 y0 chunks: A0 and B0 of chunk kc + t in term place t
+                            // the leader's barrier counts both CTAs' copies (the same boxes in each)
+                            if (leader) mbar_expect_tx(full_local, 2u * 2u * ((uint32_t)(a.rows * SW) + stageB));
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {
-                            tma_load_4d_pair(base + t * stageA, src[0], full, (kc + t) * KCH, c1, c2, c3);
-                            tma_load_3d_pair(base + PA * stageA + t * stageB, mB[0], full, (kc + t) * KCH,
-                                             (int)(rank * halfN), oslot);
-                        }
-                    } else {
-                        int na = PA, nb = PB;
-                        if (graded) {
-                            const int np = chunk_products(a.gchunks, kc);
-                            na = np == 3 ? 2 : 1;
-                            nb = np >= 2 ? 2 : 1;
-                        }
-                        if (leader)
-                            mbar_expect_tx(full_local, 2u * ((uint32_t)(na * a.rows * SW) + (uint32_t)nb * stageB));
-#pragma unroll
-                        for (int i = 0; i < PA; ++i)
-                            if (i < na) tma_load_4d_pair(base + i * stageA, src[i], full, kc * KCH, c1, c2, c3);
-#pragma unroll
-                        for (int j = 0; j < PB; ++j)
-                            if (j < nb)
-                                tma_load_3d_pair(base + PA * stageA + j * stageB, mB[j], full, kc * KCH,
+                            for (int t = 0; t < 2; ++t) {
+                                tma_load_4d_pair(base + t * stageA, src[0], full, (kc + t) * KCH, c1, c2, c3);
+                                tma_load_3d_pair(base + PA * stageA + t * stageB, mB[0], full, (kc + t) * KCH,
                                                  (int)(rank * halfN), oslot);
+                            }
+                        } else {
+                            int na = PA, nb = PB;
+                            if (graded) {
+                                const int np = chunk_products(a.gchunks, kc);
+                                na = np == 3 ? 2 : 1;
+                                nb = np >= 2 ? 2 : 1;
+                            }
+                            if (leader)
+                                mbar_expect_tx(full_local, 2u * ((uint32_t)(na * a.rows * SW) + (uint32_t)nb * stageB));
+#pragma unroll
+                            for (int i = 0; i < PA; ++i)
+                                if (i < na) tma_load_4d_pair(base + i * stageA, src[i], full, kc * KCH, c1, c2, c3);
+#pragma unroll
+                            for (int j = 0; j < PB; ++j)
+                                if (j < nb)
+                                    tma_load_3d_pair(base + PA * stageA + j * stageB, mB[j], full, kc * KCH,
+                                                     (int)(rank * halfN), oslot);
+                        }
                     }
+                    __syncwarp();
                     kc += nkc;
                     ++pp.it;
                     if (++pp.s == a.stages) {
@@ -1043,66 +1087,68 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
                     }
             if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
                 load_offset(mL, x0, y0, z0, a.noff + 8 + cls, false);
-            if (!ok) {
+            if (!ok && el) {
                 *abort_flag = 1;
                 atomicOr(a.err, ERRF_TIMEOUT);
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
             // ---------------- MMA issuer (even CTA): 256-row MMAs over both CTAs' operands
+            constexpr int KC = (NCH + K16 - 1) / K16;
+            const ChunkPlan<KC> graded_plan(a.gchunks, a.gsteps, PR::n, K16);
+            const uint32_t a_lo0 = sdesc_lo(smem0), b_lo0 = sdesc_lo(smem0 + PA * stageA);
+            const uint32_t full0 = smem_u32(&bars.full[0]), empty0 = smem_u32(&bars.empty[0]);
+            int s = pp.s;
+            uint32_t phase = pp.round & 1u;
             bool ok = true;
             for (int g = 0; g < groups.ng && ok; ++g) {
                 const uint32_t gg = pp.g + (uint32_t)g;
                 const int acc = (int)(gg & 1u);
                 const uint32_t use = gg >> 1;
-                if (gg >= 2 &&
-                    !mbar_wait_cluster(smem_u32(&bars.tempty[acc]), (use - 1u) & 1u, abort_flag, a.wait_ns)) {
+                if (gg >= 2 && !mbar_wait_warp(smem_u32(&bars.tempty[acc]), (use - 1u) & 1u, abort_flag, a.wait_ns)) {
                     ok = false;
                     break;
                 }
                 fence_after();
                 const uint32_t tmem_d = tmem + (uint32_t)(acc * 256);
-                bool first = true;  // the group's first MMA overwrites the accumulator
+                uint32_t acc0 = 0;  // the group's first MMA overwrites the accumulator
                 for (int o = groups.begin(g); o < groups.end(g) && ok; ++o) {
-                    const bool graded = (a.gchunks | a.gsteps) != 0u && o_begin + o < a.n_il;
-                    for (int kc = 0; kc < a.kchunks;) {
-                        if (!mbar_wait_cluster(smem_u32(&bars.full[pp.s]), pp.round & 1u, abort_flag, a.wait_ns)) {
+                    const bool graded = o_begin + o < a.n_il;
+#pragma unroll
+                    for (int kc = 0; kc < KC; ++kc) {
+                        const int kind = graded ? graded_plan.kind[kc] : 1;
+                        if (kind == 0 || !ok) continue;
+                        if (!mbar_wait_warp(full0 + 8u * (uint32_t)s, phase, abort_flag, a.wait_ns)) {
                             ok = false;
-                            break;
+                            continue;
                         }
                         fence_after();
-                        const uint32_t base = smem0 + (uint32_t)pp.s * stage_bytes;
-                        const int nk = a.ksteps - K16 * kc < K16 ? a.ksteps - K16 * kc : K16;
-                        const int np = graded ? chunk_products(a.gchunks, kc) : PR::n;
-                        const int nkc = graded ? stage_chunks(a.gchunks, kc, a.kchunks) : 1;
-                        if (nkc == 2) {
-                            const int nk1 = a.ksteps - K16 * (kc + 1) < K16 ? a.ksteps - K16 * (kc + 1) : K16;
-                            issue_merged<K16, SW, true>(tmem_d, base, base + PA * stageA, stageA, stageB, nk1, a.idesc,
-                                                        first);
-                        } else if (np == 1)
-                            issue_chunk<1, PR, K16, SW, true>(tmem_d, base, base + PA * stageA, stageA, stageB, nk,
-                                                              a.idesc, first);
-                        else if (np == 2)
-                            issue_chunk<2, PR, K16, SW, true>(tmem_d, base, base + PA * stageA, stageA, stageB, nk,
-                                                              a.idesc, first);
-                        else
-                            issue_full_chunk<PR, K16, SW, true>(graded ? step_split(a.gsteps, kc) : 0, tmem_d, base,
-                                                                base + PA * stageA, stageA, stageB, nk, a.idesc, first);
-                        first = false;
-                        kc += nkc;
-                        mma_commit_pair(smem_u32(&bars.empty[pp.s]));
-                        if (++pp.s == a.stages) {
-                            pp.s = 0;
-                            ++pp.round;
+                        if (el) {
+                            const uint32_t at = (uint32_t)s * (stage_bytes >> 4);
+                            const int nk = NCH - K16 * kc < K16 ? NCH - K16 * kc : K16;
+                            const int nk1 = NCH - K16 * (kc + 1) < K16 ? NCH - K16 * (kc + 1) : K16;
+                            issue_stage<PR, K16, SW, true>(tmem_d, a_lo0 + at, b_lo0 + at, stageA >> 4, stageB >> 4, nk, nk1,
+                                                           kind, graded ? graded_plan.np[kc] : PR::n,
+                                                           graded ? graded_plan.s2[kc] : K16, a.idesc, acc0);
+                            mma_commit_pair(empty0 + 8u * (uint32_t)s);
+                        }
+                        __syncwarp();
+                        acc0 = 1;
+                        if (++s == a.stages) {
+                            s = 0;
+                            phase ^= 1u;
                         }
                     }
                 }
-                if (ok) mma_commit_pair(smem_u32(&bars.tfull[acc]));
+                if (ok && el) mma_commit_pair(smem_u32(&bars.tfull[acc]));
+                __syncwarp();
             }
+            pp.s = s;
+            pp.round = phase;
             pp.g += (uint32_t)groups.ng;
-            if (!ok) {
+            if (!ok && el) {
                 *abort_flag = 1;
                 atomicOr(a.err, ERRF_TIMEOUT);
             }
@@ -1121,7 +1167,7 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
             const uint32_t gg = pp.g + (uint32_t)g;
             const int acc = (int)(gg & 1u);
             const uint32_t use = gg >> 1;
-            if (!mbar_wait_cluster(smem_u32(&bars.tfull[acc]), use & 1u, abort_flag, a.wait_ns)) {
+            if (!mbar_wait_warp(smem_u32(&bars.tfull[acc]), use & 1u, abort_flag, a.wait_ns)) {
                 ok = false;
                 break;
             }
@@ -1138,7 +1184,7 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
         }
         pp.g += (uint32_t)groups.ng;
         float mx = 0.f;  // largest |out_i sx(i)| of this thread's row (a.amax_out)
-        if (!__all_sync(0xffffffffu, ok)) {
+        if (!ok) {
             *abort_flag = 1;
             if (lane == 0) atomicOr(a.err, ERRF_TIMEOUT);
         } else if (!staged) {
@@ -1195,8 +1241,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     __shared__ int abort_sh;
 
     const int warp = threadIdx.x >> 5;
-    const uint32_t rank = cluster_rank();
-    const uint32_t smem0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    const uint32_t rank = warp_uniform(cluster_rank());
+    const uint32_t smem0 = warp_uniform((smem_u32(smem_dyn) + 1023u) & ~1023u);
     if (threadIdx.x == 0) {
         pair_bars_init(bars, a.stages);
         abort_sh = 0;
@@ -1211,12 +1257,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tmem_sh;
+    const uint32_t tmem = warp_uniform(tmem_sh);
+    const uint32_t el = elect_one();
     PairPipe pp;
     float *stage = reinterpret_cast<float *>(smem_dyn + (smem0 - smem_u32(smem_dyn)));
     pair_tile<NCH>(&mA0, &mA1, &mB0, &mB1, &mL0, &mL1, a, (int)(blockIdx.x >> 1), rank, smem0, stage, true, bars,
-                   tmem, &abort_sh, pp);
-    if (warp == 1 && (threadIdx.x & 31) == 0 && rank == 0)
+                   tmem, &abort_sh, pp, el);
+    if (warp == 1 && el && rank == 0)
         mma_commit_pair(smem_u32(&bars.done));  // arrives in both CTAs once every MMA has completed
 
     // ---------------- teardown: every MMA done (bounded wait), pair barrier, collective TMEM release
@@ -1569,9 +1616,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     __shared__ int item_sh;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_rank();
+    const uint32_t rank = warp_uniform(cluster_rank());
     const bool leader = rank == 0;
-    const uint32_t smem0 = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    const uint32_t smem0 = warp_uniform((smem_u32(smem_dyn) + 1023u) & ~1023u);
     if (threadIdx.x == 0) {
         pair_bars_init(bars, stages);
         abort_sh = 0;
@@ -1587,7 +1634,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     fence_before();
     __syncthreads();
     fence_after();
-    const uint32_t tmem = tmem_sh;
+    const uint32_t tmem = warp_uniform(tmem_sh);
+    const uint32_t el = elect_one();
     float *stage = reinterpret_cast<float *>(smem_dyn + (smem0 - smem_u32(smem_dyn)));
     PairPipe pp;
     int done_entry = -1, done_stage = 0;  // the item the pair finished last (leader thread 0)
@@ -1621,7 +1669,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
         if (it.x == 1) {
             // stage M: one tile pair; the maps live in global memory, and the planes it copies were written
             // by other pairs through the generic proxy
-            if (warp == 0 && lane == 0) {
+            if (warp == 0 && el) {
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
                     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&e.mA[m]) : "memory");
@@ -1636,7 +1684,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
             for (int g = 0; g < e.gpi; ++g) {
                 if (*(volatile int *)&abort_sh) break;  // a wait ran out: the remaining groups are skipped
                 pair_tile<NCH>(&e.mA[0], &e.mA[1], &e.mB[0], &e.mB[1], &e.mL[0], &e.mL[1], e.a, it.z * e.gpi + g,
-                               rank, smem0, stage, g == e.gpi - 1, bars, tmem, &abort_sh, pp);
+                               rank, smem0, stage, g == e.gpi - 1, bars, tmem, &abort_sh, pp, el);
             }
         } else if (it.x == 0) {
             // stage P: parent cells [SWEEP_P_CELLS it.z, ...) of level l - 1, one warp per cell over the pair
@@ -1669,7 +1717,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     }
 
     // ---------------- teardown: every MMA done (bounded wait), pair barrier, collective TMEM release
-    if (warp == 1 && lane == 0 && leader) mma_commit_pair(smem_u32(&bars.done));
+    if (warp == 1 && el && leader) mma_commit_pair(smem_u32(&bars.done));
     __syncthreads();
     if (threadIdx.x == 0) {
         volatile int no_abort = 0;
