@@ -93,6 +93,15 @@ constexpr size_t TC_SMEM_BUDGET = 224 * 1024;
 
 // operator slots of the B tables: the noff(ws) M2L offsets, then M2M and L2L per child octant
 
+// Tensor maps of one launch.  Operand rows are stored chunk by chunk, [term][chunk][cell or operator row][KCH],
+// so that a row of a copy box and the rows of neighbouring cells are contiguous; of A (halo'd planes), B
+// (operators) and L (parent-level local expansions, natural order):
+//   S  one box of one term and chunk (term and chunk folded into the slowest cell coordinate);
+//   P  both terms of a chunk in one copy;  C  term 0 of two consecutive chunks in one copy (fp16 split).
+struct TcMaps {
+    CUtensorMap aS, aP, aC, bS, bP, bC, lS, lP;
+};
+
 struct TcState {
     bool f16 = false;               // fp16x2 split with balanced scaling (and tensor-core translations)
     int pa = 0, pb = 0;             // terms of the plan's split
@@ -105,11 +114,9 @@ struct TcState {
     uint16_t *ops = nullptr;
     size_t ops_part_elems = 0;
     bool ops_borrowed = false;      // ops belongs to another plan's state (tc_share_operators)
-    CUtensorMap mapA[9][3];
-    CUtensorMap mapB[3];
-    CUtensorMap mapB2[2];           // fp16: operator tiles boxed N/2 rows (one half per CTA of a pair)
-    CUtensorMap mapL[9][2];         // fp16: parent-level local expansions for the fused L2L of level l
-    uint16_t *planesL = nullptr;    // natural order [part][z][y][x][kp], sized for level d - 1
+    TcMaps maps[9];                 // per level; the B maps box whole operator tiles
+    CUtensorMap mapB2[3];           // S, P, C of operator tiles boxed N/2 rows (one half per CTA of a pair)
+    uint16_t *planesL = nullptr;    // natural order [term][chunk][z][y][x][KCH], sized for level d - 1
     size_t partL_elems = 0;
     int bx[9], by[9], bz[9];
     int groups[9], per_group[9];    // offset groups per tile (small levels run more CTAs)
@@ -125,7 +132,8 @@ struct TcState {
 struct TcArgs {
     int mode;               // 0: M2L (+ fused L2L), 1: M2M
     int np, bx, by, bz, rows, tiles_x, tiles_y, tiles_per_class;
-    int nc, npad, kchunks, ksteps, stages;
+    int nc, npad, stages;
+    int nslots;             // operator slots of the B tables
     int groups, per_group;  // the offsets split over `groups` CTAs per tile (small levels)
     int n_off;              // offsets: 189 (+1 with the fused L2L) or 8 (M2M)
     int src_np2;            // M2M: halo'd side of the child level's planes
@@ -169,20 +177,6 @@ __device__ inline int gain_m_exp(unsigned bits)
     if (bits == 0u) return 0;
     const int e = GAIN_M_EXP - exp_of_bits(bits);
     return e < -100 ? -100 : (e > 100 ? 100 : e);
-}
-
-// Products of K chunk kc of a graded M2L offset: x0 y0 (+ x0 y1 (+ x1 y0)), 2 bits per chunk (0 = all 3).
-__device__ __forceinline__ int chunk_products(uint32_t g, int kc)
-{
-    const int c = (int)((g >> (2 * kc)) & 3u);
-    return c == 0 ? 3 : c;
-}
-
-// A graded offset's stages: two consecutive chunks of one product each (x0 y0 only) share one stage, their
-// A0 / B0 boxes in the places of the two terms; returns how many chunks the stage starting at kc covers.
-__device__ __forceinline__ int stage_chunks(uint32_t g, int kc, int kchunks)
-{
-    return (chunk_products(g, kc) == 1 && kc + 1 < kchunks && chunk_products(g, kc + 1) == 1) ? 2 : 1;
 }
 
 // Accumulation groups of one CTA's offsets: the M2L (or M2M) offsets, local indices 0 .. nm - 1, in runs
@@ -312,6 +306,16 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
         "[%6];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2,
+                                            int c3, int c4)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
+        "[%7];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
         : "memory");
 }
 
@@ -514,6 +518,16 @@ __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_5d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1,
+                                                 int c2, int c3, int c4)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+        "%4, %5, %6}], [%7];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1,
                                                  int c2)
 {
@@ -581,6 +595,67 @@ struct ChunkPlan {
     }
 };
 
+// Bytes that the copies of one stage bring to this CTA (copy_bytes), and the copies: A from the box at (c1, c2, c3) of the planes (zspan slowest cells per chunk; the L
+// planes when `l2l`), B rows n0 .. of operator slot `oslot`.  With at least 8 rows (`fused`) the two terms or
+// the two chunks of an operand are one copy and lie rows * SW bytes apart: with four copies a stage the
+// producer took ~550 cycles of its own code, as long as the MMAs of a stage at p <= 10.  Two copies a stage and
+// the epilogue's scale factors in shared memory: level-d launch 16.1 -> 12.4 ms (N = 10M, p = 10), 2.69 -> 2.50 ms
+// (N = 1M, p = 12), 1.51 -> 1.29 ms (N = 100k, ws = 2, p = 8), the upward pass 0.63 -> 0.56 ms at 1M.
+template <int KC, int PA, int PB, int SW, bool PAIR>
+__device__ __forceinline__ uint32_t copy_bytes(int kind, int np, uint32_t rows_bytes, uint32_t stageB)
+{
+    if (PA == 2 && PB == 2 && SW == 128) {
+        if (kind == 2) return 2u * (rows_bytes + stageB);
+        return (np == 3 ? 2u : 1u) * rows_bytes + (np >= 2 ? 2u : 1u) * stageB;
+    }
+    return (uint32_t)PA * rows_bytes + (uint32_t)PB * stageB;
+}
+
+template <int KC, int PA, int PB, int SW, bool PAIR>
+__device__ __forceinline__ void issue_copies(const TcMaps &m, bool l2l, uint32_t full, uint32_t base, uint32_t sa,
+                                             uint32_t stageA, uint32_t stageB, int kc, int kind, int np, bool fused,
+                                             int c1, int c2, int c3, int zspan, int n0, int oslot, int nslots)
+{
+    const uint32_t bB = base + PA * stageA;
+    auto a4 = [&](uint32_t dst, int term, int chunk) {
+        const CUtensorMap *map = l2l ? &m.lS : &m.aS;
+        if (PAIR) tma_load_4d_pair(dst, map, full, 0, c1, c2, (term * KC + chunk) * zspan + c3);
+        else tma_load_4d(dst, map, full, 0, c1, c2, (term * KC + chunk) * zspan + c3);
+    };
+    auto b3 = [&](uint32_t dst, int term, int chunk) {
+        if (PAIR) tma_load_3d_pair(dst, &m.bS, full, 0, n0, (term * KC + chunk) * nslots + oslot);
+        else tma_load_3d(dst, &m.bS, full, 0, n0, (term * KC + chunk) * nslots + oslot);
+    };
+    if (PA == 2 && PB == 2 && SW == 128) {
+        if (kind == 2) {
+            if (!fused) {
+                a4(base, 0, kc);
+                a4(base + sa, 0, kc + 1);
+            } else if (PAIR) tma_load_5d_pair(base, &m.aC, full, 0, c1, c2, c3, kc);
+            else tma_load_5d(base, &m.aC, full, 0, c1, c2, c3, kc);
+            if (PAIR) tma_load_4d_pair(bB, &m.bC, full, 0, n0, oslot, kc);
+            else tma_load_4d(bB, &m.bC, full, 0, n0, oslot, kc);
+            return;
+        }
+        if (np == 3 && fused) {
+            const CUtensorMap *map = l2l ? &m.lP : &m.aP;
+            if (PAIR) tma_load_5d_pair(base, map, full, 0, c1, c2, kc * zspan + c3, 0);
+            else tma_load_5d(base, map, full, 0, c1, c2, kc * zspan + c3, 0);
+        } else {
+            a4(base, 0, kc);
+            if (np == 3) a4(base + sa, 1, kc);
+        }
+        if (np == 1) b3(bB, 0, kc);
+        else if (PAIR) tma_load_4d_pair(bB, &m.bP, full, 0, n0, kc * nslots + oslot, 0);
+        else tma_load_4d(bB, &m.bP, full, 0, n0, kc * nslots + oslot, 0);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < PA; ++i) a4(base + i * stageA, i, kc);
+#pragma unroll
+    for (int j = 0; j < PB; ++j) b3(bB + j * stageB, j, kc);
+}
+
 // The MMAs of one stage (operand addresses are compile-time steps from the stage's descriptor words): nk valid
 // K16 steps in the chunk, nk1 in the second one of a kind-2 stage; acc0 = 0 starts a new accumulator.  Products
 // outer, K16 steps inner.
@@ -612,6 +687,20 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem_d, uint32_t a_lo, uint
     }
 }
 
+// Per output coefficient i: the factor that undoes the balancing and the gains, x^ = x~ post(i) / (gM gT), and
+// s(i) or 1 / s(i) for the level maximum, in shared memory for the epilogue warps (threads t = 0 .. 127, their
+// named barrier): read from global memory in the row loop, one dependent load after another, they took 31,000
+// of the 381,000 cycles of a tile at p = 12.
+__device__ __forceinline__ void load_scales(const TcArgs &a, float2 *sc, int n, int t)
+{
+    const float g = a.post ? pow2f(-gain_m_exp(__ldcg(a.amax)) - GAIN_T_EXP) : 1.f;
+    asm volatile("bar.sync 1, 128;" ::: "memory");  // the tile before is done with them
+    for (int i = t; i < n; i += 128)
+        sc[i] = i < a.nc ? make_float2(a.post ? __ldg(a.post + i) * g : 1.f, a.amax_out ? __ldg(a.sx + i) : 0.f)
+                         : make_float2(0.f, 0.f);
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+}
+
 // One CTA sums, for 128 target rows, the products of a list of offsets:
 //   mode 0 (M2L): the 189 interaction-list offsets of parity class `cls`, A
 //     from the halo'd source planes of the level; with fused L2L (fp16 split)
@@ -626,10 +715,7 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem_d, uint32_t a_lo, uint
 // accumulator width held in registers); SW: bytes per swizzled operand row.
 template <int PA, int PB, int NCH, int SW>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    k_m2l_tc(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
-             const __grid_constant__ CUtensorMap mA2, const __grid_constant__ CUtensorMap mB0,
-             const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mB2,
-             const __grid_constant__ CUtensorMap mL0, const __grid_constant__ CUtensorMap mL1, TcArgs a)
+    k_m2l_tc(const __grid_constant__ TcMaps maps, TcArgs a)
 {
     extern __shared__ uint8_t smem_dyn[];
     __shared__ __align__(8) uint64_t bar_full[TC_MAX_STAGES];
@@ -641,6 +727,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __shared__ uint32_t tmem_sh;
     __shared__ int abort_sh;
     __shared__ int produced_sh, consumed_sh;
+    __shared__ float2 scale_sh[NCH * 16];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem0 = warp_uniform((smem_u32(smem_dyn) + 1023u) & ~1023u);
@@ -666,6 +753,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int z0 = (tile / (a.tiles_x * a.tiles_y)) * a.bz;
     const int cx = cls & 1, cy = (cls >> 1) & 1, cz = (cls >> 2) & 1;
     const int np2 = a.np + 2 * a.ws;
+    // the second term (or chunk) of A lies right behind the tile's rows when it comes with the first in one copy
+    const bool fused = kGradable && SW == 128 && a.rows >= 8;
+    const uint32_t rows_bytes = (uint32_t)(a.rows * SW);
+    const uint32_t sa = fused ? rows_bytes : stageA;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < a.stages; ++s) {
@@ -702,54 +793,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (warp == 0) {
         {
             // ---------------- producer: TMA loads of the A brick and the B operator
-            const CUtensorMap *mA[3] = {&mA0, &mA1, &mA2};
-            const CUtensorMap *mL[3] = {&mL0, &mL1, &mL1};
-            const CUtensorMap *mB[3] = {&mB0, &mB1, &mB2};
+            constexpr int KC = (NCH + K16 - 1) / K16;
+            const ChunkPlan<KC> graded_plan(kGradable && a.mode == 0 ? a.gchunks : 0u,
+                                            kGradable && a.mode == 0 ? a.gsteps : 0u, PB == 2 ? 3 : PA + PB, K16);
+            const uint32_t full0 = smem_u32(&bar_full[0]), empty0 = smem_u32(&bar_empty[0]);
             int it = 0, s = 0;
-            uint32_t round = 0;
+            uint32_t phase = 1;
             bool ok = true;
-            // all K chunks of one offset: A from maps `src` at (c1, c2, c3), B at operator slot `oslot`; a
-            // graded (M2L) offset copies only the terms its chunk's products read
-            auto load_offset = [&](const CUtensorMap *const *src, int c1, int c2, int c3, int oslot, bool graded) {
-                for (int kc = 0; kc < a.kchunks && ok;) {
-                    if (it >= a.stages &&
-                        !mbar_wait_warp(smem_u32(&bar_empty[s]), (round & 1u) ^ 1u, abort_flag, a.wait_ns)) {
+            // all K chunks of one offset: A from the planes (or the L planes) at (c1, c2, c3), B at operator slot
+            // `oslot`; a graded (M2L) offset copies only the terms its chunk's products read
+            auto load_offset = [&](bool l2l, int c1, int c2, int c3, int zspan, int oslot, bool graded) {
+#pragma unroll
+                for (int kc = 0; kc < KC; ++kc) {
+                    const int kind = graded ? graded_plan.kind[kc] : 1;
+                    const int np = graded ? graded_plan.np[kc] : 3;
+                    if (kind == 0 || !ok) continue;
+                    if (it >= a.stages && !mbar_wait_warp(empty0 + 8u * (uint32_t)s, phase, abort_flag, a.wait_ns)) {
                         ok = false;
-                        break;
+                        continue;
                     }
-                    const uint32_t full = smem_u32(&bar_full[s]);
-                    const uint32_t base = smem0 + (uint32_t)s * stage_bytes;
-                    const int nkc = (kGradable && graded) ? stage_chunks(a.gchunks, kc, a.kchunks) : 1;
                     if (el) {
-                        if (nkc == 2) {  // two x0 y0 chunks: A0 and B0 of chunk kc + t in term place t
-                            mbar_expect_tx(full, 2u * ((uint32_t)(a.rows * SW) + stageB));
-#pragma unroll
-                            for (int t = 0; t < 2; ++t) {
-                                tma_load_4d(base + t * stageA, src[0], full, (kc + t) * KCH, c1, c2, c3);
-                                tma_load_3d(base + PA * stageA + t * stageB, mB[0], full, (kc + t) * KCH, 0, oslot);
-                            }
-                        } else {
-                            int na = PA, nb = PB;
-                            if (kGradable && graded) {
-                                const int np = chunk_products(a.gchunks, kc);
-                                na = np == 3 ? 2 : 1;
-                                nb = np >= 2 ? 2 : 1;
-                            }
-                            mbar_expect_tx(full, (uint32_t)(na * a.rows * SW) + (uint32_t)nb * stageB);
-#pragma unroll
-                            for (int i = 0; i < PA; ++i)
-                                if (i < na) tma_load_4d(base + i * stageA, src[i], full, kc * KCH, c1, c2, c3);
-#pragma unroll
-                            for (int j = 0; j < PB; ++j)
-                                if (j < nb) tma_load_3d(base + PA * stageA + j * stageB, mB[j], full, kc * KCH, 0, oslot);
-                        }
+                        const uint32_t full = full0 + 8u * (uint32_t)s, base = smem0 + (uint32_t)s * stage_bytes;
+                        mbar_expect_tx(full, copy_bytes<KC, PA, PB, SW, false>(kind, np, rows_bytes, stageB));
+                        issue_copies<KC, PA, PB, SW, false>(maps, l2l, full, base, sa, stageA, stageB, kc, kind, np, fused,
+                                                            c1, c2, c3, zspan, 0, oslot, a.nslots);
                     }
                     __syncwarp();
-                    kc += nkc;
                     ++it;
                     if (++s == a.stages) {
                         s = 0;
-                        ++round;
+                        phase ^= 1u;
                     }
                 }
             };
@@ -766,15 +839,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             if (oi < o_begin || oi >= o_end) continue;
                             const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
                             const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-                            load_offset(mA, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w,
-                                        off_slot(dx, dy, dz, w), a.gchunks != 0u);
+                            load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w,
+                                        scls * np2 + z0 + (sz >> 1) + w, 8 * np2, off_slot(dx, dy, dz, w), true);
                         }
                 // fused L2L: the parents' local expansions (natural order, no halo)
                 if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
-                    load_offset(mL, x0, y0, z0, a.noff + 8 + cls, false);
+                    load_offset(true, x0, y0, z0, a.np, a.noff + 8 + cls, false);
             } else {
                 for (int o = o_begin; o < o_end && ok; ++o)
-                    load_offset(mA, x0 + a.ws, y0 + a.ws, o * a.src_np2 + z0 + a.ws, a.noff + o, false);
+                    load_offset(false, x0 + a.ws, y0 + a.ws, o * a.src_np2 + z0 + a.ws, 8 * a.src_np2, a.noff + o, false);
             }
             if (el) {
                 produced_sh = it;
@@ -823,7 +896,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             const uint32_t at = (uint32_t)s * (stage_bytes >> 4);
                             const int nk = NCH - K16 * kc < K16 ? NCH - K16 * kc : K16;
                             const int nk1 = NCH - K16 * (kc + 1) < K16 ? NCH - K16 * (kc + 1) : K16;
-                            issue_stage<PR, K16, SW, false>(tmem_d, a_lo0 + at, b_lo0 + at, stageA >> 4, stageB >> 4, nk, nk1,
+                            issue_stage<PR, K16, SW, false>(tmem_d, a_lo0 + at, b_lo0 + at, sa >> 4, stageB >> 4, nk, nk1,
                                                             kind, graded ? graded_plan.np[kc] : PR::n,
                                                             graded ? graded_plan.s2[kc] : K16, a.idesc, acc0);
                             mma_commit(empty0 + 8u * (uint32_t)s);
@@ -854,6 +927,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         // ---------------- epilogue warps: drain each group's accumulator into FP32 registers
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
+        load_scales(a, scale_sh, NCH * 16, quad * 32 + lane);
         // fused L2L offset: its A planes carry the gain gL instead of gM
         const float l2l_fac =
             a.amaxL ? pow2f(gain_m_exp(*a.amax) - gain_m_exp(*a.amaxL)) : 1.f;
@@ -885,14 +959,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             float *stage = reinterpret_cast<float *>(smem_dyn + (smem0 - smem_u32(smem_dyn)));
             const int srow = a.nc | 1;
             if (row < a.rows) {
-                // with the fp16 split undo the balancing: x^ = x~ post(j) / (gM gT)
-                const float g = a.post ? pow2f(-gain_m_exp(__ldcg(a.amax)) - GAIN_T_EXP) : 1.f;
 #pragma unroll
                 for (int i = 0; i < NCH * 16; ++i)
-                    if (i < a.nc) {
-                        const float v = a.post ? Lr[i] * (__ldg(a.post + i) * g) : Lr[i];
+                    if (i < (NCH - 1) * 16 || i < a.nc) {
+                        const float2 f = scale_sh[i];
+                        const float v = Lr[i] * f.x;
                         stage[row * srow + i] = v;
-                        if (a.amax_out) mx = fmaxf(mx, fabsf(v * __ldg(a.sx + i)));
+                        mx = fmaxf(mx, fabsf(v * f.y));
                     }
             }
             const int64_t np = a.np;
@@ -956,6 +1029,7 @@ struct PairBars {
     uint64_t tfull[2];
     uint64_t tempty[2];
     uint64_t done;
+    float2 scale[256];  // the epilogue's per-coefficient factors (load_scales)
 };
 
 // Pipeline positions of one role thread, carried from tile to tile when a pair runs several tiles (the
@@ -985,14 +1059,12 @@ __device__ __forceinline__ void pair_bars_init(PairBars &b, int stages)
 // issues no copies until every thread is done with this tile, so the epilogue may stage the output rows
 // in the ring (`stage`, generic address of its start); otherwise each thread writes its row directly.
 template <int NCH>
-__device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensorMap *mA1, const CUtensorMap *mB0,
-                                          const CUtensorMap *mB1, const CUtensorMap *mL0, const CUtensorMap *mL1,
-                                          const TcArgs &a, int pair, uint32_t rank, uint32_t smem0, float *stage,
+__device__ __forceinline__ void pair_tile(const TcMaps &maps, const TcArgs &a, int pair, uint32_t rank, uint32_t smem0, float *stage,
                                           bool staged, PairBars &bars, uint32_t tmem, volatile int *abort_flag,
                                           PairPipe &pp, uint32_t el)
 {
     constexpr int PA = 2, PB = 2, SW = 128;
-    constexpr int KCH = kchunk_of(SW), K16 = SW / 32;
+    constexpr int K16 = SW / 32, KC = (NCH + K16 - 1) / K16;
     using PR = Products<PA, PB>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool leader = rank == 0;
@@ -1019,56 +1091,37 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
     if (warp == 0) {
         {
             // ---------------- producer (both CTAs): own A brick, own half of B, completing on the leader's barrier
-            const CUtensorMap *mA[2] = {mA0, mA1};
-            const CUtensorMap *mL[2] = {mL0, mL1};
-            const CUtensorMap *mB[2] = {mB0, mB1};
+            const ChunkPlan<KC> graded_plan(a.gchunks, a.gsteps, PR::n, K16);
+            const uint32_t full_local0 = smem_u32(&bars.full[0]), empty0 = smem_u32(&bars.empty[0]);
+            const uint32_t full_lead0 = warp_uniform(map_shared(full_local0, 0));
+            int it = pp.it, s = pp.s;
+            uint32_t phase = (pp.round & 1u) ^ 1u;
             bool ok = true;
-            auto load_offset = [&](const CUtensorMap *const *src, int c1, int c2, int c3, int oslot, bool graded) {
-                for (int kc = 0; kc < a.kchunks && ok;) {
-                    if (pp.it >= a.stages &&
-                        !mbar_wait_warp(smem_u32(&bars.empty[pp.s]), (pp.round & 1u) ^ 1u, abort_flag, a.wait_ns)) {
+            auto load_offset = [&](bool l2l, int c1, int c2, int c3, int zspan, int oslot, bool graded) {
+#pragma unroll
+                for (int kc = 0; kc < KC; ++kc) {
+                    const int kind = graded ? graded_plan.kind[kc] : 1;
+                    const int np = graded ? graded_plan.np[kc] : 3;
+                    if (kind == 0 || !ok) continue;
+                    if (it >= a.stages && !mbar_wait_warp(empty0 + 8u * (uint32_t)s, phase, abort_flag, a.wait_ns)) {
                         ok = false;
-                        break;
+                        continue;
                     }
-                    const uint32_t full_local = smem_u32(&bars.full[pp.s]);
-                    const uint32_t full = map_shared(full_local, 0);
-                    const uint32_t base = smem0 + (uint32_t)pp.s * stage_bytes;
-                    const int nkc = graded ? stage_chunks(a.gchunks, kc, a.kchunks) : 1;
                     if (el) {
-                        if (nkc == 2) {  // two x0 y0 chunks: A0 and B0 of chunk kc + t in term place t
-                            // the leader's barrier counts both CTAs' copies (the same boxes in each)
-                            if (leader) mbar_expect_tx(full_local, 2u * 2u * ((uint32_t)(a.rows * SW) + stageB));
-#pragma unroll
-                            for (int t = 0; t < 2; ++t) {
-                                tma_load_4d_pair(base + t * stageA, src[0], full, (kc + t) * KCH, c1, c2, c3);
-                                tma_load_3d_pair(base + PA * stageA + t * stageB, mB[0], full, (kc + t) * KCH,
-                                                 (int)(rank * halfN), oslot);
-                            }
-                        } else {
-                            int na = PA, nb = PB;
-                            if (graded) {
-                                const int np = chunk_products(a.gchunks, kc);
-                                na = np == 3 ? 2 : 1;
-                                nb = np >= 2 ? 2 : 1;
-                            }
-                            if (leader)
-                                mbar_expect_tx(full_local, 2u * ((uint32_t)(na * a.rows * SW) + (uint32_t)nb * stageB));
-#pragma unroll
-                            for (int i = 0; i < PA; ++i)
-                                if (i < na) tma_load_4d_pair(base + i * stageA, src[i], full, kc * KCH, c1, c2, c3);
-#pragma unroll
-                            for (int j = 0; j < PB; ++j)
-                                if (j < nb)
-                                    tma_load_3d_pair(base + PA * stageA + j * stageB, mB[j], full, kc * KCH,
-                                                     (int)(rank * halfN), oslot);
-                        }
+                        const uint32_t base = smem0 + (uint32_t)s * stage_bytes;
+                        // the leader's barrier counts both CTAs' copies (the same boxes in each)
+                        if (leader)
+                            mbar_expect_tx(full_local0 + 8u * (uint32_t)s,
+                                           2u * copy_bytes<KC, PA, PB, SW, true>(kind, np, stageA, stageB));
+                        issue_copies<KC, PA, PB, SW, true>(maps, l2l, full_lead0 + 8u * (uint32_t)s, base, stageA, stageA,
+                                                           stageB, kc, kind, np, true, c1, c2, c3, zspan,
+                                                           (int)(rank * halfN), oslot, a.nslots);
                     }
                     __syncwarp();
-                    kc += nkc;
-                    ++pp.it;
-                    if (++pp.s == a.stages) {
-                        pp.s = 0;
-                        ++pp.round;
+                    if (it < a.stages) ++it;
+                    if (++s == a.stages) {
+                        s = 0;
+                        phase ^= 1u;
                     }
                 }
             };
@@ -1082,11 +1135,14 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
                         if (oi < o_begin || oi >= o_end) continue;
                         const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
                         const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-                        load_offset(mA, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w,
-                                    off_slot(dx, dy, dz, w), a.gchunks != 0u);
+                        load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w,
+                                    8 * np2, off_slot(dx, dy, dz, w), true);
                     }
             if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
-                load_offset(mL, x0, y0, z0, a.noff + 8 + cls, false);
+                load_offset(true, x0, y0, z0, a.np, a.noff + 8 + cls, false);
+            pp.it = it;
+            pp.s = s;
+            pp.round = phase ^ 1u;
             if (!ok && el) {
                 *abort_flag = 1;
                 atomicOr(a.err, ERRF_TIMEOUT);
@@ -1096,7 +1152,6 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
     } else if (warp == 1) {
         if (leader) {
             // ---------------- MMA issuer (even CTA): 256-row MMAs over both CTAs' operands
-            constexpr int KC = (NCH + K16 - 1) / K16;
             const ChunkPlan<KC> graded_plan(a.gchunks, a.gsteps, PR::n, K16);
             const uint32_t a_lo0 = sdesc_lo(smem0), b_lo0 = sdesc_lo(smem0 + PA * stageA);
             const uint32_t full0 = smem_u32(&bars.full[0]), empty0 = smem_u32(&bars.empty[0]);
@@ -1158,6 +1213,7 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
         // ---------------- epilogue warps (both CTAs): drain this CTA's 128 rows
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
+        load_scales(a, bars.scale, NCH * 16, row);
         const float l2l_fac = a.amaxL ? pow2f(gain_m_exp(__ldcg(a.amax)) - gain_m_exp(__ldcg(a.amaxL))) : 1.f;
         float Lr[NCH * 16];
 #pragma unroll
@@ -1190,11 +1246,11 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
         } else if (!staged) {
             // the ring may already hold the next tile's copies: the rows are transposed across each warp in
             // registers for coalesced stores
-            const float g = pow2f(-gain_m_exp(__ldcg(a.amax)) - GAIN_T_EXP);
 #pragma unroll
             for (int i = 0; i < NCH * 16; ++i) {
-                Lr[i] = i < a.nc ? Lr[i] * (__ldg(a.post + i) * g) : 0.f;
-                if (a.amax_out && row < a.rows && i < a.nc) mx = fmaxf(mx, fabsf(Lr[i] * __ldg(a.sx + i)));
+                const float2 f = bars.scale[i];  // zeros beyond nc
+                Lr[i] = (i < (NCH - 1) * 16 || i < a.nc) ? Lr[i] * f.x : 0.f;
+                mx = fmaxf(mx, fabsf(Lr[i] * f.y));
             }
             const int64_t np = a.np;
             float *out = a.groups == 1 ? a.L : a.Lpart + (int64_t)grp * 8 * np * np * np * a.nc;
@@ -1205,16 +1261,14 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
             // every MMA of the tile has completed and no copy is pending, so the stage ring is idle: the rows
             // go through shared memory (stride srow, odd) and leave in coalesced stores, a warp per 32 rows
             const int srow = a.nc | 1;
-            const float g = pow2f(-gain_m_exp(__ldcg(a.amax)) - GAIN_T_EXP);
-            if (row < a.rows) {
 #pragma unroll
-                for (int i = 0; i < NCH * 16; ++i)
-                    if (i < a.nc) {
-                        const float v = Lr[i] * (__ldg(a.post + i) * g);
-                        stage[row * srow + i] = v;
-                        if (a.amax_out) mx = fmaxf(mx, fabsf(v * __ldg(a.sx + i)));
-                    }
-            }
+            for (int i = 0; i < NCH * 16; ++i)
+                if (i < (NCH - 1) * 16 || i < a.nc) {
+                    const float2 f = bars.scale[i];
+                    const float v = Lr[i] * f.x;
+                    stage[row * srow + i] = v;
+                    mx = fmaxf(mx, fabsf(v * f.y));
+                }
             const int64_t np = a.np;
             float *out = a.groups == 1 ? a.L : a.Lpart + (int64_t)grp * 8 * np * np * np * a.nc;
             const int tx = row % a.bx, ty = (row / a.bx) % a.by, tz = row / (a.bx * a.by);
@@ -1231,9 +1285,7 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap *mA0, const CUtensor
 
 template <int NCH>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
-    k_m2l_tc_pair(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
-                  const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1,
-                  const __grid_constant__ CUtensorMap mL0, const __grid_constant__ CUtensorMap mL1, TcArgs a)
+    k_m2l_tc_pair(const __grid_constant__ TcMaps maps, TcArgs a)
 {
     extern __shared__ uint8_t smem_dyn[];
     __shared__ __align__(8) PairBars bars;
@@ -1261,7 +1313,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
     const uint32_t el = elect_one();
     PairPipe pp;
     float *stage = reinterpret_cast<float *>(smem_dyn + (smem0 - smem_u32(smem_dyn)));
-    pair_tile<NCH>(&mA0, &mA1, &mB0, &mB1, &mL0, &mL1, a, (int)(blockIdx.x >> 1), rank, smem0, stage, true, bars,
+    pair_tile<NCH>(maps, a, (int)(blockIdx.x >> 1), rank, smem0, stage, true, bars,
                    tmem, &abort_sh, pp, el);
     if (warp == 1 && el && rank == 0)
         mma_commit_pair(smem_u32(&bars.done));  // arrives in both CTAs once every MMA has completed
@@ -1317,19 +1369,22 @@ __global__ void k_absmax(const float *__restrict__ M, int64_t ncell, int nc, con
     if (lane == 0 && m > 0.f) atomicMax(amax, __float_as_uint(m));  // positive floats order as integers
 }
 
-// FP32 class-layout moments -> split planes [part][class][hz][hy][hx][k] with a
-// periodic halo; rows kp wide (zero beyond nc).  fp16: balanced by s(k) gM.
-// One warp per halo cell, lanes over the coefficients.
-template <bool F16>
+// element of coefficient k of cell (or operator row) `cell` of `ncell` in one term of an operand array, chunks
+// of kch coefficients outermost
+__device__ __forceinline__ int64_t chunk_at(int64_t cell, int64_t ncell, int k, int kch)
+{
+    return ((int64_t)(k / kch) * ncell + cell) * kch + k % kch;
+}
+
+// FP32 class-layout moments -> bf16 split planes [part][chunk][class][hz][hy][hx][k] with a
+// periodic halo; rows kp wide (zero beyond nc).  One warp per halo cell, lanes over the coefficients.
 __global__ void k_split_halo(const float *__restrict__ M, int np, int hw, int nc, int kp, int parts,
-                             const float *__restrict__ s, const unsigned *__restrict__ amax,
-                             uint16_t *__restrict__ planes, size_t part_elems)
+                             int kch, uint16_t *__restrict__ planes, size_t part_elems)
 {
     const int np2 = np + 2 * hw;
     const int64_t ncell = 8 * (int64_t)np2 * np2 * np2;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const float g = F16 ? pow2f(gain_m_exp(*amax)) : 1.f;
     for (int64_t cell = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); cell < ncell; cell += warps) {
         const int hx = (int)(cell % np2);
         const int hy = (int)((cell / np2) % np2);
@@ -1337,20 +1392,13 @@ __global__ void k_split_halo(const float *__restrict__ M, int np, int hw, int nc
         const int c = hzc / np2, hz = hzc % np2;
         const int px = ((hx - hw) % np + np) % np, py = ((hy - hw) % np + np) % np, pz = ((hz - hw) % np + np) % np;
         const float *row = M + ((int64_t)c * np * np * np + px + (int64_t)np * (py + (int64_t)np * pz)) * nc;
-        uint16_t *out = planes + cell * kp;
-        for (int k = lane; k < kp; k += 32) {
-            float v = 0.f;
-            if (k < nc) {
-                v = row[k];
-                if (F16) v *= __ldg(s + k) * g;
-            }
-            split_terms<F16>(v, parts, out + k, part_elems);
-        }
+        for (int k = lane; k < kp; k += 32)
+            split_terms<false>(k < nc ? row[k] : 0.f, parts, planes + chunk_at(cell, ncell, k, kch), part_elems);
     }
 }
 
 // FP32 class-layout local expansion of level `lev` (side n = 2^lev) -> fp16
-// split planes in natural order [part][z][y][x][k], balanced L~ = L^ / s(k) gL
+// split planes in natural order [part][chunk][z][y][x][k], balanced L~ = L^ / s(k) gL
 // (the A operand of the fused L2L): natural cell `cell`, lanes over the coefficients.
 __device__ __forceinline__ void split_L_cell(const float *__restrict__ L, int lev, int nc, int kp,
                                              const float *__restrict__ sinv, float g, uint16_t *__restrict__ planes,
@@ -1362,10 +1410,10 @@ __device__ __forceinline__ void split_L_cell(const float *__restrict__ L, int le
                                  : (int64_t)((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)) * h * h * h + (x >> 1) +
                                        (int64_t)h * ((y >> 1) + (int64_t)h * (z >> 1));
     const float *row = L + src * nc;
-    uint16_t *out = planes + cell * kp;
+    const int64_t ncell = (int64_t)n * n * n;
     for (int k = lane; k < kp; k += 32) {
         const float v = k < nc ? __ldcg(row + k) * (__ldg(sinv + k) * g) : 0.f;
-        split_terms<true>(v, 2, out + k, part_elems);
+        split_terms<true>(v, 2, planes + chunk_at(cell, ncell, k, kchunk_of(128)), part_elems);
     }
 }
 
@@ -1382,7 +1430,7 @@ __global__ void k_split_L(const float *__restrict__ L, int lev, int nc, int kp, 
         split_L_cell(L, lev, nc, kp, sinv, g, planes, part_elems, cell, lane);
 }
 
-// FP64 operators -> split B tables [part][slot][j][k] (K-major, rows kp wide):
+// FP64 operators -> split B tables [part][chunk][slot][j][k] (K-major, rows kp wide in chunks of kch):
 // slots < noff the M2L operators T[slot][k][j] (input-major), then per child
 // octant o the M2M operator (M2M[j][o nc + k], parent output j) and the L2L
 // operator (L2L[o nc + j][k], child output j).  fp16: balanced with gT,
@@ -1390,7 +1438,7 @@ __global__ void k_split_L(const float *__restrict__ L, int lev, int nc, int kp, 
 // bf16: the translation slots stay zero (unused).
 template <bool F16>
 __global__ void k_split_ops(int noff, const double *__restrict__ T, const double *__restrict__ m2m,
-                            const double *__restrict__ l2l, int nc, int npad, int kp, int parts,
+                            const double *__restrict__ l2l, int nc, int npad, int kp, int kch, int parts,
                             const double *__restrict__ s, uint16_t *__restrict__ ops, size_t part_elems)
 {
     const int64_t total = (int64_t)(noff + 16) * npad * kp;
@@ -1412,14 +1460,15 @@ __global__ void k_split_ops(int noff, const double *__restrict__ T, const double
                 r = l2l[((int64_t)o * nc + j) * nc + k] * s[k] / s[j] * gT;
             }
         }
+        const int64_t at = chunk_at((int64_t)slot * npad + j, (int64_t)(noff + 16) * npad, k, kch);
         for (int i = 0; i < parts; ++i) {
             if (F16) {
                 const __half t = __float2half_rn((float)r);
-                ops[e + i * part_elems] = __half_as_ushort(t);
+                ops[at + i * part_elems] = __half_as_ushort(t);
                 r -= (double)__half2float(t);
             } else {
                 const __nv_bfloat16 t = __float2bfloat16_rn((float)r);
-                ops[e + i * part_elems] = __bfloat16_as_ushort(t);
+                ops[at + i * part_elems] = __bfloat16_as_ushort(t);
                 r -= (double)__bfloat162float(t);
             }
         }
@@ -1519,7 +1568,7 @@ __global__ void k_split_halo16(const float *__restrict__ M, int np, int hw, int 
             hi[i] = (uint32_t)h2[0] | ((uint32_t)h2[1] << 16);
             lo[i] = (uint32_t)l2[0] | ((uint32_t)l2[1] << 16);
         }
-        uint16_t *out = planes + cell * kp + k0;
+        uint16_t *out = planes + chunk_at(cell, total / G, k0, kchunk_of(128));
         *reinterpret_cast<uint4 *>(out) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
         *reinterpret_cast<uint4 *>(out + part_elems) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
@@ -1544,7 +1593,7 @@ constexpr int SWEEP_P_CELLS = 512;         // parent cells per P item
 constexpr int64_t SWEEP_G_ELEMS = 1 << 16;  // L elements per G item
 
 struct SweepLevel {
-    CUtensorMap mA[2], mB[2], mL[2];  // the level's pair-kernel tensor maps
+    TcMaps maps;                      // the level's pair-kernel tensor maps
     TcArgs a;                         // the level's pair-kernel arguments
     const float *Lprev;               // P: L of level l - 1 (class layout)
     const float *sinv;                // P: 1 / s(k)
@@ -1671,11 +1720,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
             // by other pairs through the generic proxy
             if (warp == 0 && el) {
 #pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&e.mA[m]) : "memory");
-                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&e.mB[m]) : "memory");
-                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&e.mL[m]) : "memory");
-                }
+                for (int m = 0; m < (int)(sizeof(TcMaps) / sizeof(CUtensorMap)); ++m)
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&e.maps.aS + m) : "memory");
                 asm volatile("fence.proxy.async.global;" ::: "memory");
             }
             __syncwarp();
@@ -1683,7 +1729,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
             // the last group's epilogue stages its rows in the ring
             for (int g = 0; g < e.gpi; ++g) {
                 if (*(volatile int *)&abort_sh) break;  // a wait ran out: the remaining groups are skipped
-                pair_tile<NCH>(&e.mA[0], &e.mA[1], &e.mB[0], &e.mB[1], &e.mL[0], &e.mL[1], e.a, it.z * e.gpi + g,
+                pair_tile<NCH>(e.maps, e.a, it.z * e.gpi + g,
                                rank, smem0, stage, g == e.gpi - 1, bars, tmem, &abort_sh, pp, el);
             }
         } else if (it.x == 0) {
@@ -1771,9 +1817,7 @@ size_t tc_smem_bytes(int pa, int pb, int npad, int sw)
     return need < 120 * 1024 ? 120 * 1024 : need;
 }
 
-typedef void (*TcKernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
-                         CUtensorMap, TcArgs);
-typedef void (*TcPairKernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcArgs);
+typedef void (*TcKernel)(TcMaps, TcArgs);  // single CTAs and CTA pairs alike
 
 // CTA-pair kernel (fp16, 128-byte rows): stage = 2 A terms of 128 rows + 2 B terms of npad / 2 rows
 int tc_pair_stages(int npad)
@@ -1790,11 +1834,11 @@ size_t tc_pair_smem_bytes(int npad)
     return need < 120 * 1024 ? 120 * 1024 : need;
 }
 
-TcPairKernel pick_pair_kernel(int nch)
+TcKernel pick_pair_kernel(int nch)
 {
     switch (nch) {
 #define FMM_TC_CASE(n) \
-    case n: return (TcPairKernel)k_m2l_tc_pair<n>;
+    case n: return (TcKernel)k_m2l_tc_pair<n>;
         FMM_TC_CASE(1) FMM_TC_CASE(2) FMM_TC_CASE(3) FMM_TC_CASE(4) FMM_TC_CASE(6) FMM_TC_CASE(7) FMM_TC_CASE(8)
         FMM_TC_CASE(9) FMM_TC_CASE(11) FMM_TC_CASE(13) FMM_TC_CASE(15) FMM_TC_CASE(16)
 #undef FMM_TC_CASE
@@ -1872,25 +1916,88 @@ void split_offsets(int n_off, int tiles, int max_groups, int sms, int &groups, i
 
 CUtensorMapSwizzle swizzle_of(int sw) { return sw == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B; }
 
-fmm_status encode_planes(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap *map, CUtensorMapDataType dt, void *base,
-                         int kp, int64_t d1, int64_t d2, int64_t d3, int b1, int b2, int b3, int sw)
+// One map over `base`: rank-n extents, strides (bytes) of all but the innermost, box
+fmm_status encode_map(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap *map, CUtensorMapDataType dt, void *base,
+                      int rank, const cuuint64_t *dims, const cuuint64_t *strides, const cuuint32_t *box, int sw)
 {
-    cuuint64_t dims[4] = {(cuuint64_t)kp, (cuuint64_t)d1, (cuuint64_t)d2, (cuuint64_t)d3};
-    cuuint64_t strides[3] = {(cuuint64_t)kp * 2, (cuuint64_t)kp * 2 * d1, (cuuint64_t)kp * 2 * d1 * d2};
-    cuuint32_t box[4] = {(cuuint32_t)kchunk_of(sw), (cuuint32_t)b1, (cuuint32_t)b2, (cuuint32_t)b3};
-    cuuint32_t es[4] = {1, 1, 1, 1};
-    return enc(map, dt, 4, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(sw),
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    return enc(map, dt, (cuuint32_t)rank, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(sw),
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
                ? FMM_OK
                : FMM_ERR_INTERNAL;
+}
+
+// The S, P and C maps (TcMaps) of a cell array [terms][kc chunks][d3][d2][d1][KCH], boxes b1 x b2 x b3 cells
+fmm_status encode_planes(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap *mS, CUtensorMap *mP, CUtensorMap *mC,
+                         CUtensorMapDataType dt, void *base, int kc, int terms, int64_t d1, int64_t d2, int64_t d3,
+                         int b1, int b2, int b3, int sw)
+{
+    const cuuint64_t row = (cuuint64_t)sw, k = (cuuint64_t)kchunk_of(sw), chunk = row * d1 * d2 * d3;
+    const cuuint32_t box[5] = {(cuuint32_t)k, (cuuint32_t)b1, (cuuint32_t)b2, (cuuint32_t)b3, 2};
+    const cuuint64_t dS[4] = {k, (cuuint64_t)d1, (cuuint64_t)d2, (cuuint64_t)(d3 * kc * terms)};
+    const cuuint64_t dP[5] = {k, (cuuint64_t)d1, (cuuint64_t)d2, (cuuint64_t)(d3 * kc), (cuuint64_t)terms};
+    const cuuint64_t dC[5] = {k, (cuuint64_t)d1, (cuuint64_t)d2, (cuuint64_t)d3, (cuuint64_t)(kc * terms)};
+    const cuuint64_t sP[4] = {row, row * d1, row * d1 * d2, chunk * kc}, sC[4] = {row, row * d1, row * d1 * d2, chunk};
+    fmm_status st = encode_map(enc, mS, dt, base, 4, dS, sP, box, sw);
+    if (st == FMM_OK && mP) st = encode_map(enc, mP, dt, base, 5, dP, sP, box, sw);
+    if (st == FMM_OK && mC) st = encode_map(enc, mC, dt, base, 5, dC, sC, box, sw);
+    return st;
+}
+
+// The same of the operator tables [terms][kc chunks][slots][npad][KCH], boxes of n rows of one slot
+fmm_status encode_operators(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap *mS, CUtensorMap *mP, CUtensorMap *mC,
+                            CUtensorMapDataType dt, void *base, int kc, int terms, int npad, int slots, int n, int sw)
+{
+    const cuuint64_t row = (cuuint64_t)sw, k = (cuuint64_t)kchunk_of(sw), slot = row * npad, chunk = slot * slots;
+    const cuuint32_t box[4] = {(cuuint32_t)k, (cuuint32_t)n, 1, 2};
+    const cuuint64_t dS[3] = {k, (cuuint64_t)npad, (cuuint64_t)slots * kc * terms};
+    const cuuint64_t dP[4] = {k, (cuuint64_t)npad, (cuuint64_t)slots * kc, (cuuint64_t)terms};
+    const cuuint64_t dC[4] = {k, (cuuint64_t)npad, (cuuint64_t)slots, (cuuint64_t)(kc * terms)};
+    const cuuint64_t sP[3] = {row, slot, chunk * kc}, sC[3] = {row, slot, chunk};
+    fmm_status st = encode_map(enc, mS, dt, base, 3, dS, sP, box, sw);
+    if (st == FMM_OK && mP) st = encode_map(enc, mP, dt, base, 4, dP, sP, box, sw);
+    if (st == FMM_OK && mC) st = encode_map(enc, mC, dt, base, 4, dC, sC, box, sw);
+    return st;
+}
+
+int chunks_of(const TcState *S) { return S->kp / kchunk_of(S->sw); }
+
+CUtensorMapDataType type_of(const TcState *S)
+{
+    return S->f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+}
+
+// level l's A and L maps for tiles of bx x by x bz cells (np a class side, hw the halo width)
+fmm_status encode_level(PFN_cuTensorMapEncodeTiled_v12000 enc, const TcState *S, int l, int np, int hw, int bx, int by,
+                        int bz, TcMaps *m)
+{
+    const int64_t np2 = np + 2 * hw;
+    const int kc = chunks_of(S);
+    fmm_status st = encode_planes(enc, &m->aS, S->f16 ? &m->aP : nullptr, S->f16 ? &m->aC : nullptr, type_of(S),
+                                  S->planes[l], kc, S->parts, np2, np2, 8 * np2, bx, by, bz, S->sw);
+    // L of level l - 1 (side np) in natural order, boxed like the level-l bricks; all levels share one buffer,
+    // used one level at a time
+    if (st == FMM_OK && S->f16)
+        st = encode_planes(enc, &m->lS, &m->lP, nullptr, type_of(S), S->planesL, kc, 2, np, np, np, bx, by, bz, S->sw);
+    if (!S->f16) m->aP = m->aC = m->lS = m->lP = m->aS;  // unused kernel parameters
+    return st;
+}
+
+// level l's maps for the CTA-pair kernel: half operator tiles
+TcMaps pair_maps(const TcState *S, int l)
+{
+    TcMaps m = S->maps[l];
+    m.bS = S->mapB2[0];
+    m.bP = S->mapB2[1];
+    m.bC = S->mapB2[2];
+    return m;
 }
 
 void fill_common(const Plan &P, const TcState *S, int pa, int pb, TcArgs &a)
 {
     a.nc = P.nc;
     a.npad = S->npad;
-    a.kchunks = (S->kp + kchunk_of(S->sw) - 1) / kchunk_of(S->sw);
-    a.ksteps = (P.nc + 15) / 16;
+    a.nslots = S->noff + 16;
     a.stages = tc_stages(pa, pb, S->npad, S->sw);
     // instruction descriptor: FP32 accumulator, A and B both bf16 (format 1) or both fp16 (format 0),
     // K-major, N >> 3 at bit 17, M >> 4 at bit 24
@@ -1921,7 +2028,7 @@ void fill_common(const Plan &P, const TcState *S, int pa, int pb, TcArgs &a)
     };
     if (S->f16 && pa == 2 && pb == 2 && (d2 > 0 || d1 > 0)) {
         const int kch = kchunk_of(S->sw);
-        for (int kc = 0; kc < a.kchunks && kc < 10; ++kc) {
+        for (int kc = 0; kc < chunks_of(S) && kc < 10; ++kc) {
             const int lam = lowest_degree(kch * kc);
             const int np = (d1 > 0 && lam >= d1) ? 1 : (d2 > 0 && lam >= d2) ? 2 : 3;
             if (np < 3) a.gchunks |= (uint32_t)np << (2 * kc);
@@ -1967,7 +2074,6 @@ fmm_status tc_prepare(Plan &P)
     // rows padded to whole copy boxes (aligned pieces); the MMAs stop at (p+1)^2 padded to 16
     S->sw = S->f16 ? 128 : 64;
     S->kp = (P.nc + kchunk_of(S->sw) - 1) / kchunk_of(S->sw) * kchunk_of(S->sw);
-    const CUtensorMapDataType dt = S->f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     if (S->f16) {
         // s(n,m) = sqrt((n+m)! (n-m)!) per real coefficient
         double h_s[(TC_PMAX + 1) * (TC_PMAX + 1)];
@@ -2000,34 +2106,21 @@ fmm_status tc_prepare(Plan &P)
     FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_part_elems * S->parts));
     if (S->f16)
         k_split_ops<true><<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.tab.m2m64, P.tab.l2l64, P.nc, S->npad, S->kp,
-                                                      S->parts, S->s64, S->ops, S->ops_part_elems);
+                                                      kchunk_of(S->sw), S->parts, S->s64, S->ops, S->ops_part_elems);
     else
-        k_split_ops<false><<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, nullptr, nullptr, P.nc, S->npad, S->kp, S->parts,
-                                                       nullptr, S->ops, S->ops_part_elems);
+        k_split_ops<false><<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, nullptr, nullptr, P.nc, S->npad, S->kp,
+                                                       kchunk_of(S->sw), S->parts, nullptr, S->ops, S->ops_part_elems);
     FMM_LAUNCH_CHECK(P);
-    for (int j = 0; j < S->parts; ++j) {
-        cuuint64_t dims[3] = {(cuuint64_t)S->kp, (cuuint64_t)S->npad, (cuuint64_t)(S->noff + 16)};
-        cuuint64_t strides[2] = {(cuuint64_t)S->kp * 2, (cuuint64_t)S->kp * 2 * S->npad};
-        cuuint32_t box[3] = {(cuuint32_t)kchunk_of(S->sw), (cuuint32_t)S->npad, 1};
-        cuuint32_t es[3] = {1, 1, 1};
-        if (enc(&S->mapB[j], dt, 3, S->ops + j * S->ops_part_elems, dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(S->sw), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return FMM_ERR_INTERNAL;
+    {
+        TcMaps &m = S->maps[0];  // the operator maps, the same on every level
+        TRY_TC(encode_operators(enc, &m.bS, S->f16 ? &m.bP : nullptr, S->f16 ? &m.bC : nullptr, type_of(S), S->ops,
+                                chunks_of(S), S->parts, S->npad, S->noff + 16, S->npad, S->sw));
+        if (!S->f16) m.bP = m.bC = m.bS;  // unused kernel parameters
     }
-    for (int j = S->parts; j < 3; ++j) S->mapB[j] = S->mapB[0];  // unused kernel parameters
     if (S->f16) {
-        for (int j = 0; j < 2; ++j) {
-            cuuint64_t dims[3] = {(cuuint64_t)S->kp, (cuuint64_t)S->npad, (cuuint64_t)(S->noff + 16)};
-            cuuint64_t strides[2] = {(cuuint64_t)S->kp * 2, (cuuint64_t)S->kp * 2 * S->npad};
-            cuuint32_t box[3] = {(cuuint32_t)kchunk_of(S->sw), (cuuint32_t)(S->npad / 2), 1};
-            cuuint32_t es[3] = {1, 1, 1};
-            if (enc(&S->mapB2[j], dt, 3, S->ops + j * S->ops_part_elems, dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_of(S->sw), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-                return FMM_ERR_INTERNAL;
-        }
-        TcPairKernel kp2 = pick_pair_kernel(S->npad / 16);
+        TRY_TC(encode_operators(enc, &S->mapB2[0], &S->mapB2[1], &S->mapB2[2], type_of(S), S->ops, chunks_of(S), S->parts,
+                                S->npad, S->noff + 16, S->npad / 2, S->sw));
+        TcKernel kp2 = pick_pair_kernel(S->npad / 16);
         if (!kp2) return FMM_ERR_INTERNAL;
         FMM_CUDA_TRY(cudaFuncSetAttribute((const void *)kp2, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)tc_pair_smem_bytes(S->npad)));
@@ -2052,19 +2145,8 @@ fmm_status tc_prepare(Plan &P)
         S->bz[l] = tile_dim(np, TC_ROWS / (S->bx[l] * S->by[l]));
         S->part_elems[l] = (size_t)8 * np2 * np2 * np2 * S->kp;
         FMM_CUDA_TRY(cudaMalloc(&S->planes[l], sizeof(uint16_t) * S->part_elems[l] * S->parts));
-        for (int i = 0; i < S->parts; ++i)
-            TRY_TC(encode_planes(enc, &S->mapA[l][i], dt, S->planes[l] + i * S->part_elems[l], S->kp, np2, np2,
-                                 8 * np2, S->bx[l], S->by[l], S->bz[l], S->sw));
-        for (int i = S->parts; i < 3; ++i) S->mapA[l][i] = S->mapA[l][0];
-        if (S->f16) {
-            // L of level l - 1 (side np) in natural order, boxed like the level-l bricks; all levels share
-            // one buffer, used one level at a time
-            for (int i = 0; i < 2; ++i)
-                TRY_TC(encode_planes(enc, &S->mapL[l][i], dt, S->planesL + (size_t)i * np * np * np * S->kp, S->kp,
-                                     np, np, np, S->bx[l], S->by[l], S->bz[l], S->sw));
-        } else {
-            S->mapL[l][0] = S->mapL[l][1] = S->mapA[l][0];  // unused kernel parameters
-        }
+        S->maps[l] = S->maps[0];
+        TRY_TC(encode_level(enc, S, l, np, P.ws, S->bx[l], S->by[l], S->bz[l], &S->maps[l]));
         const int tiles = 8 * (np / S->bx[l]) * (np / S->by[l]) * (np / S->bz[l]);
         split_offsets(n_il(P.ws) + (S->f16 ? 1 : 0), tiles, 27, sms, S->groups[l], S->per_group[l]);
         if (S->groups[l] > 1) {
@@ -2170,9 +2252,7 @@ fmm_status launch_m2m_tc(Plan &P, int l)
     TcKernel k = pick_kernel(S->pa, S->pb, S->npad / 16, S->sw);
     if (!k) return FMM_ERR_INTERNAL;
     const unsigned grid = (unsigned)a.tiles_per_class * (unsigned)a.groups;
-    k<<<grid, TC_THREADS, tc_smem_bytes(S->pa, S->pb, S->npad, S->sw), P.stream>>>(
-        S->mapA[src][0], S->mapA[src][1], S->mapA[src][2], S->mapB[0], S->mapB[1], S->mapB[2], S->mapA[src][0],
-        S->mapA[src][0], a);
+    k<<<grid, TC_THREADS, tc_smem_bytes(S->pa, S->pb, S->npad, S->sw), P.stream>>>(S->maps[src], a);
     FMM_LAUNCH_CHECK(P);
     if (a.groups > 1) {
         const int64_t cnt = (int64_t)n * n * n * P.nc;
@@ -2246,8 +2326,8 @@ fmm_status launch_m2l_tc(Plan &P, int l, bool precise, bool split)
         FMM_LAUNCH_CHECK(P);
     } else {
         const int64_t nhalo = 8 * np2 * np2 * np2;
-        k_split_halo<false><<<(unsigned)((nhalo + 7) / 8 < 4864 ? (nhalo + 7) / 8 : 4864), 256, 0, P.stream>>>(
-            (const float *)P.M[l], np, P.ws, P.nc, S->kp, pa, nullptr, nullptr, S->planes[l], S->part_elems[l]);
+        k_split_halo<<<(unsigned)((nhalo + 7) / 8 < 4864 ? (nhalo + 7) / 8 : 4864), 256, 0, P.stream>>>(
+            (const float *)P.M[l], np, P.ws, P.nc, S->kp, pa, kchunk_of(S->sw), S->planes[l], S->part_elems[l]);
         FMM_LAUNCH_CHECK(P);
     }
     if (S->f16)  // level l's largest |L^ / s|, for the fused L2L of level l + 1
@@ -2258,16 +2338,13 @@ fmm_status launch_m2l_tc(Plan &P, int l, bool precise, bool split)
     const bool time_it = P.timings_on && l == P.d && P.ev_top[0] && !precise;
     if (time_it) cudaEventRecord(P.ev_top[0], P.stream);
     if (pair) {
-        TcPairKernel k2 = pick_pair_kernel(S->npad / 16);
+        TcKernel k2 = pick_pair_kernel(S->npad / 16);
         if (!k2) return FMM_ERR_INTERNAL;
-        k2<<<grid, TC_THREADS, tc_pair_smem_bytes(S->npad), P.stream>>>(S->mapA[l][0], S->mapA[l][1], S->mapB2[0],
-                                                                         S->mapB2[1], S->mapL[l][0], S->mapL[l][1], a);
+        k2<<<grid, TC_THREADS, tc_pair_smem_bytes(S->npad), P.stream>>>(pair_maps(S, l), a);
     } else {
         TcKernel k = pick_kernel(pa, pb, S->npad / 16, S->sw);
         if (!k) return FMM_ERR_INTERNAL;
-        k<<<grid, TC_THREADS, tc_smem_bytes(pa, pb, S->npad, S->sw), P.stream>>>(
-            S->mapA[l][0], S->mapA[l][1], S->mapA[l][2], S->mapB[0], S->mapB[1], S->mapB[2], S->mapL[l][0],
-            S->mapL[l][1], a);
+        k<<<grid, TC_THREADS, tc_smem_bytes(pa, pb, S->npad, S->sw), P.stream>>>(S->maps[l], a);
     }
     FMM_LAUNCH_CHECK(P);
     if (time_it) {
@@ -2360,12 +2437,7 @@ fmm_status sweep_create(Plan *const *plans, int n, Sweep **out)
                 return FMM_ERR_INTERNAL;
             }
             sw->stages = e.a.stages;
-            e.mA[0] = S->mapA[l][0];
-            e.mA[1] = S->mapA[l][1];
-            e.mB[0] = S->mapB2[0];
-            e.mB[1] = S->mapB2[1];
-            e.mL[0] = S->mapL[l][0];
-            e.mL[1] = S->mapL[l][1];
+            e.maps = pair_maps(S, l);
             const int64_t ncl = (int64_t)1 << (3 * (l - 1));  // cells of level l - 1
             e.Lprev = (const float *)P.L[l - 1];
             e.sinv = S->s32inv;
@@ -2493,22 +2565,9 @@ fmm_status tc_set_brick(Plan &P, int l, int bx, int by, int bz)
         return FMM_ERR_INVALID_ARG;
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return FMM_ERR_INTERNAL;
-    const CUtensorMapDataType dt = S->f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    const int64_t np2 = np + 2 * P.ws;
-    CUtensorMap a[3], lm[2];
-    for (int i = 0; i < S->parts; ++i)
-        TRY_TC(encode_planes(enc, &a[i], dt, S->planes[l] + i * S->part_elems[l], S->kp, np2, np2, 8 * np2, bx, by,
-                             bz, S->sw));
-    for (int i = S->parts; i < 3; ++i) a[i] = a[0];
-    if (S->f16)
-        for (int i = 0; i < 2; ++i)
-            TRY_TC(encode_planes(enc, &lm[i], dt, S->planesL + (size_t)i * np * np * np * S->kp, S->kp, np, np, np,
-                                 bx, by, bz, S->sw));
-    else
-        lm[0] = lm[1] = a[0];
-    for (int i = 0; i < 3; ++i) S->mapA[l][i] = a[i];
-    S->mapL[l][0] = lm[0];
-    S->mapL[l][1] = lm[1];
+    TcMaps m = S->maps[l];
+    TRY_TC(encode_level(enc, S, l, np, P.ws, bx, by, bz, &m));
+    S->maps[l] = m;
     S->bx[l] = bx;
     S->by[l] = by;
     S->bz[l] = bz;
@@ -2539,7 +2598,11 @@ fmm_status tc_share_operators(Plan &dst, const Plan &src)
     if (!D->ops_borrowed) cudaFree(D->ops);
     D->ops = S->ops;
     D->ops_borrowed = true;
-    memcpy((void *)D->mapB, (const void *)S->mapB, sizeof(D->mapB));
+    for (TcMaps &m : D->maps) {
+        m.bS = S->maps[0].bS;
+        m.bP = S->maps[0].bP;
+        m.bC = S->maps[0].bC;
+    }
     memcpy((void *)D->mapB2, (const void *)S->mapB2, sizeof(D->mapB2));
     return FMM_OK;
 }
