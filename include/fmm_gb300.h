@@ -249,7 +249,8 @@ fmm_status fmm_plan_get_timings(fmm_plan plan, fmm_timings *out);
 int64_t fmm_plan_last_launch_count(fmm_plan plan);
 
 /* Which M2L implementation the plan runs at `level` (1..depth):
- * 0 = FP64 CUDA cores, 1 = FP32 CUDA cores, 2 = tcgen05 tensor cores;
+ * 0 = FP64 (whole-number residue products on the tensor cores up to order 15, CUDA cores above it and where the
+ * residue operands do not fit in memory), 1 = FP32 CUDA cores, 2 = tcgen05 tensor cores in 16-bit splits;
  * -1 for a NULL plan or a level out of range. */
 int fmm_plan_m2l_backend(fmm_plan plan, int level);
 

@@ -136,6 +136,7 @@ fmm_status far_field_pass(Plan &P, bool gradient, bool solute_only, StageTimer *
         // with the fp16 split the upward pass left the planes split and the L2L is fused
         const bool fused = tc_available(P, l) && tc_translations(P);
         if (tc_available(P, l)) TRY(launch_m2l_tc(P, l, solute_only, !fused));
+        else if (res_available(P, l)) TRY(launch_m2l_res(P, l));
         else TRY(launch_m2l_simt(P, l));
         if (ev) cudaEventRecord(P.ev_m2l[2 * (l - 1) + 1], P.stream);
         if (!fused) TRY(launch_l2l(P, l));
@@ -290,6 +291,7 @@ fmm_status evaluate(Plan &P, const double *pos, const double *q, const uint8_t *
     int kphi = pointer_kind(potentials);
     bool host_any = kp == 1 || kq == 1 || ks == 1 || kf == 1 || kphi == 1;
     if (host_any) TRY(ensure_staging(P));
+    TRY(res_ensure(P));
     ExecScope xs(P);
     TRY(xs.status);
     P.launches = 0;
@@ -366,6 +368,7 @@ fmm_status create_streams(Plan &P)
 fmm_status retc(Plan &P)
 {
     tc_free(P);
+    res_free(P);
     if (P.precision == FMM_PREC_MIXED && P.split != FMM_SPLIT_FP32) TRY(tc_prepare(P));
     return FMM_OK;
 }
@@ -604,6 +607,7 @@ void fmm_plan_destroy(fmm_plan plan)
     if (P.exec) cudaStreamSynchronize(P.exec);
     if (P.near) cudaStreamSynchronize(P.near);
     tc_free(P);
+    res_free(P);
     solute_free(P);
     free_tables(P);
     free_buffers(P);

@@ -146,6 +146,9 @@ struct Plan {
     void *L[9] = {};
     // tensor-core M2L state (bf16 operand planes, operator tables, TMA maps)
     void *tc = nullptr;
+    // FP64 residue M2L state (operator residues, planes, TMA maps)
+    void *res = nullptr;
+    bool res_tried = false;  // built (or found not to fit) for the present options
     // scratch of the sparse solute-only pass
     void *sol = nullptr;
     // reductions
@@ -309,6 +312,15 @@ fmm_status launch_m2m_tc(Plan &P, int level);
 // split the L2L from level - 1 is included: L[level] = M2L + L2L.
 fmm_status launch_m2l_tc(Plan &P, int level, bool precise = false, bool split = true);
 void tc_free(Plan &P);
+
+// FP64 M2L by residue products on the tensor cores (fmm_m2l_res.cu): L[level] = M2L, without the L2L
+bool res_available(const Plan &P, int level);
+// builds the state on an FP64 plan's first evaluation (a plan that is to run the mixed path never pays for it);
+// left for later while the plan's stream is being captured
+fmm_status res_ensure(Plan &P);
+fmm_status launch_m2l_res(Plan &P, int level);
+fmm_status res_share_operators(Plan &dst, const Plan &src);
+void res_free(Plan &P);
 
 // phases of one energy + solute-solvent evaluation on device inputs (fmm_api.cu), for the batch API:
 // front (sort .. near field) and back (solute pass, reductions, asynchronous copy of the results into

@@ -1,0 +1,534 @@
+// fmm_m2l_res.cu -- the FP64 path's M2L (Eq. Lcoeffdef) as exact residue products on the tensor cores.
+//
+// GB300 issues 2 FP64 operations per SM and clock, so the CUDA-core M2L (2 (p+1)^4 flop per source and target)
+// is bound by that pipe: 1.29 s per evaluation of 100,000 charges at p = 12, and far more than its flops at small
+// sizes, whose levels fill a few SMs.  The 16-bit tensor pipe is ~1,500 times as fast.  The products are therefore
+// taken in whole numbers, exactly, modulo 11 to 14 small coprime numbers (the Chinese remainder theorem; its use
+// for matrix products on low-precision units is the "Ozaki scheme II" of Ozaki, Uchino & Imamura, 2025):
+//   * moments and operators are balanced as in the mixed path, M~ = M^ s(n,m), T~ = T / (s s), |T~| <= 1/2, and
+//     rounded to whole numbers, M_int = round(M~ 2^g) with |M_int| < 2^56 (g from the level's largest |M~|) and
+//     T_int = round(T~ 2^56): the moments keep the 53 bits of every value within 2^-3 of the level's largest, and
+//     the operators' rounding is 2^-57, below the 2^-53 of the FP64 sum that this replaces;
+//   * sum_delta sum_k |T_int| <= 137 2^56 (ws = 1) or 277 2^56 (ws = 2), whatever the order, so |L_int| < 2^119.2
+//     or 2^120.2, and it follows from its residues modulo p_1 .. p_n with prod p_i > 2^121;
+//   * residues are centred, |r| <= p/2, exact in fp16; a product of two is a whole number, and a chain of G = 2
+//     offsets sums 2 (p+1)^2 of them: with 2 (p+1)^2 (p/2)^2 <= 2^24 the FP32 accumulator is exact.  The drained
+//     accumulators are added up as 32-bit integers (fmm_tc.cuh);
+//   * the operator residues carry the factor (P / p_i)^-1 mod p_i, so the results y_i give
+//     L_int / P = sum_i y_i / p_i mod 1 directly: a 96-bit fixed-point sum, good to 2^-83 P.
+// Orders above 15 (more than 256 coefficients) stay on the CUDA cores.
+//
+// Measured (energy, forces and solute-solvent energy, FP64 CUDA cores -> residues): 100,000 charges at depth 5,
+// p = 12 1,290 -> 12.4 ms (M2L kernels 1,283 -> 6.0 ms); 2,998 charges at depth 3, p = 8 581 -> 1.6 ms.  Forces
+// against the same sums in 80-bit arithmetic: 3.7e-16 relative (FP64 sums 7.2e-16) at 1,000 charges, p = 8;
+// 4.9e-16 (5.4e-16) at 2,998, p = 4; 7.4e-15 (7.5e-15, the operator tables' own rounding) at p = 12.
+#include <math.h>
+#include <string.h>
+
+#include <new>
+#include <vector>
+
+#include "fmm_tc.cuh"
+
+namespace fmm {
+
+namespace {
+
+constexpr int RES_MAX = 16;        // moduli
+constexpr int RES_CHAIN = 2;       // offsets per accumulator (G)
+constexpr int RES_M_BITS = 56;     // |M_int| < 2^56
+constexpr int RES_T_BITS = 56;     // T_int = round(T~ 2^56)
+constexpr size_t RES_PLANE_BUDGET = (size_t)2 << 30;  // operand planes held at once (moduli per launch)
+
+struct ResConsts {
+    int n;
+    int p[RES_MAX], c18[RES_MAX], c36[RES_MAX];  // modulus, 2^18 and 2^36 modulo it (centred)
+    int inv[RES_MAX];                            // (P / p_i)^-1 mod p_i, centred
+    float rp[RES_MAX];
+    uint32_t w[RES_MAX][3];                      // floor(2^96 / p_i), low word first
+    double pscale;                               // P / 2^96
+};
+
+struct ResState {
+    ResConsts c;
+    int npad = 0, kp = 0, noff = 0;
+    uint16_t *ops = nullptr;      // [modulus][chunk][slot][npad][64]
+    size_t ops_elems = 0;         // per modulus
+    bool ops_borrowed = false;
+    uint16_t *planes = nullptr;   // [modulus of the launch][chunk][class][hz][hy][hx][64], one level at a time
+    int16_t *resid = nullptr;     // [group][modulus of the launch][cell][nc]
+    uint32_t *frac = nullptr;     // [3][cells nc] 96-bit sums between the launches of a level
+    TcMaps maps[9];
+    CUtensorMap mapB2[2];         // S, C of half operator tiles (CTA pairs)
+    int batch[9];                 // moduli per launch of a level
+    int bx[9], by[9], bz[9], groups[9], per_group[9];
+    double *s64 = nullptr;        // [nc] s(n,m)
+    unsigned long long *amax = nullptr;  // [9] bits of the largest |M^ s| per level
+    int *mods = nullptr;
+};
+
+// x mod p for |x| <= 2^57, centred: 18-bit limbs (the highest signed) against 2^18 and 2^36 mod p, then one
+// approximate quotient and a correction
+__device__ __forceinline__ int residue(int x0, int x1, int x2, int p, int c18, int c36, float rp)
+{
+    int r = mod_near(x0 + x1 * c18 + x2 * c36, p, rp);
+    const int h = p >> 1;
+    if (r > h) r -= p;
+    if (r < -h) r += p;
+    return r;
+}
+
+__device__ __forceinline__ void limbs(long long x, int &x0, int &x1, int &x2)
+{
+    x0 = (int)(x & 0x3FFFF);
+    x1 = (int)((x >> 18) & 0x3FFFF);
+    x2 = (int)(x >> 36);
+}
+
+// g of a level from the bits of its largest |M~|: |M~ 2^g| < 2^RES_M_BITS, within the range of a double
+__device__ __forceinline__ int res_gain(unsigned long long bits)
+{
+    if (bits == 0ull) return 0;
+    const int g = RES_M_BITS - 1 - ((int)(bits >> 52) - 1023);
+    return g > 1000 ? 1000 : (g < -960 ? -960 : g);
+}
+
+__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// T~ of every slot -> residues times (P / p_i)^-1, [modulus][chunk][slot][j][k] with zero padding
+__global__ void k_res_ops(int noff, const double *__restrict__ T, int nc, int npad, int kp, const double *__restrict__ s,
+                          uint16_t *__restrict__ ops, size_t elems, const __grid_constant__ ResConsts c)
+{
+    const int64_t total = (int64_t)noff * npad * kp;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int k = (int)(e % kp);
+        const int j = (int)((e / kp) % npad);
+        const int slot = (int)(e / ((int64_t)kp * npad));
+        long long x = 0;
+        if (j < nc && k < nc)
+            x = llrint(T[((int64_t)slot * nc + k) * nc + j] / (s[k] * s[j]) * (double)(1ll << RES_T_BITS));
+        int x0, x1, x2;
+        limbs(x, x0, x1, x2);
+        const int64_t at = chunk_at((int64_t)slot * npad + j, (int64_t)noff * npad, k, 64);
+#pragma unroll
+        for (int i = 0; i < RES_MAX; ++i) {
+            if (i >= c.n) break;
+            const int r = residue(x0, x1, x2, c.p[i], c.c18[i], c.c36[i], c.rp[i]);
+            const int y = residue(r * c.inv[i], 0, 0, c.p[i], 0, 0, c.rp[i]);
+            ops[at + i * elems] = __half_as_ushort(__int2half_rn(y));
+        }
+    }
+}
+
+// largest |M^ s| of a level as double bits (positive doubles order as integers); a NaN is larger than all
+__global__ void k_res_absmax(const double *__restrict__ M, int64_t ncell, int nc, const double *__restrict__ s,
+                             unsigned long long *__restrict__ amax)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    unsigned long long m = 0;
+    for (int64_t c = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); c < ncell; c += warps) {
+        const double *row = M + c * nc;
+        for (int k = lane; k < nc; k += 32) {
+            const unsigned long long v = (unsigned long long)__double_as_longlong(row[k] * s[k]) & ~(1ull << 63);
+            m = v > m ? v : m;
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+        m = v > m ? v : m;
+    }
+    if (lane == 0 && m > 0) atomicMax(amax, m);
+}
+
+// FP64 class-layout moments -> residue planes of moduli m0 .. m0 + nb - 1 with a periodic halo, 8 coefficients per
+// thread (16-byte stores per plane), zero beyond nc.  Bound by the integer arithmetic of the residues (~15
+// instructions each) and the planes' bytes.
+__global__ void k_res_split(const double *__restrict__ M, int np, int hw, int nc, int kp, const double *__restrict__ s,
+                            const unsigned long long *__restrict__ amax, int m0, int nb, uint16_t *__restrict__ planes,
+                            const __grid_constant__ ResConsts c)
+{
+    const int np2 = np + 2 * hw;
+    const int G = kp / 8;
+    const int64_t ncell = 8 * (int64_t)np2 * np2 * np2, total = ncell * G;
+    const double g = pow2d(res_gain(*amax));
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t cell = t / G;
+        const int k0 = (int)(t - cell * G) * 8;
+        const int hx = (int)(cell % np2);
+        const int hy = (int)((cell / np2) % np2);
+        const int hzc = (int)(cell / ((int64_t)np2 * np2));
+        const int cl = hzc / np2, hz = hzc % np2;
+        const int px = ((hx - hw) % np + np) % np, py = ((hy - hw) % np + np) % np, pz = ((hz - hw) % np + np) % np;
+        const double *row = M + ((int64_t)cl * np * np * np + px + (int64_t)np * (py + (int64_t)np * pz)) * nc;
+        int x0[8], x1[8], x2[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int k = k0 + u;
+            const long long x = k < nc ? __double2ll_rn(row[k] * __ldg(s + k) * g) : 0;
+            limbs(x, x0[u], x1[u], x2[u]);
+        }
+        uint16_t *out = planes + chunk_at(cell, ncell, k0, 64);
+        for (int m = 0; m < nb; ++m) {
+            const int p = c.p[m0 + m], a = c.c18[m0 + m], b = c.c36[m0 + m];
+            const float rp = c.rp[m0 + m];
+            uint32_t w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const __half2 h = __halves2half2(__int2half_rn(residue(x0[2 * u], x1[2 * u], x2[2 * u], p, a, b, rp)),
+                                                 __int2half_rn(residue(x0[2 * u + 1], x1[2 * u + 1], x2[2 * u + 1], p, a,
+                                                                       b, rp)));
+                w[u] = *reinterpret_cast<const uint32_t *>(&h);
+            }
+            *reinterpret_cast<uint4 *>(out + (size_t)m * ncell * kp) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+
+// Residues y_i of nb moduli (and of the offset groups) -> the 96-bit fraction sum y_i / p_i mod 1, and on the last
+// launch of the level L^ = P (fraction) 2^-(g + RES_T_BITS) s(j).  Two neighbouring elements per thread (their
+// residues are one 32-bit load); frac carries the sums between the launches of a level.
+__global__ void k_res_join(int64_t n, int nc, int groups, int m0, int nb, const int16_t *__restrict__ resid,
+                           uint32_t *__restrict__ frac, bool first, bool last, const double *__restrict__ s,
+                           const unsigned long long *__restrict__ amax, double *__restrict__ L,
+                           const __grid_constant__ ResConsts c)
+{
+    const int64_t e = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+    if (e >= n) return;  // n is even (8 parity classes)
+    long long a0[2] = {0, 0}, a1[2] = {0, 0}, a2[2] = {0, 0};
+    for (int g = 0; g < groups; ++g)
+        for (int m = 0; m < nb; ++m) {
+            const int v = *reinterpret_cast<const int *>(resid + ((int64_t)g * nb + m) * n + e);
+            const int y[2] = {(int)(short)(v & 0xFFFF), v >> 16};
+            const uint32_t w0 = c.w[m0 + m][0], w1 = c.w[m0 + m][1], w2 = c.w[m0 + m][2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                a0[u] += (long long)y[u] * w0;
+                a1[u] += (long long)y[u] * w1;
+                a2[u] += (long long)y[u] * w2;
+            }
+        }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        if (!first) {
+            a0[u] += frac[e + u];
+            a1[u] += frac[n + e + u];
+            a2[u] += frac[2 * n + e + u];
+        }
+        // carries: limbs of 32 bits, the top one modulo 2^32 (the fraction is taken modulo 1)
+        a1[u] += a0[u] >> 32;
+        a2[u] += a1[u] >> 32;
+        const uint32_t lo = (uint32_t)a0[u], mid = (uint32_t)a1[u], hi = (uint32_t)a2[u];
+        if (!last) {
+            frac[e + u] = lo;
+            frac[n + e + u] = mid;
+            frac[2 * n + e + u] = hi;
+            continue;
+        }
+        const long long top = (long long)(((uint64_t)hi << 32) | mid);  // signed: |L_int| < P / 2
+        const unsigned long long bits = *amax;
+        double v = (double)top * 4294967296.0 + (double)lo;
+        v = v * c.pscale * s[(int)((e + u) % nc)] * pow2d(-RES_T_BITS) * pow2d(-res_gain(bits));
+        L[e + u] = (bits >> 52) == 2047 ? __longlong_as_double(0x7FF8000000000000ll) : v;  // inf or NaN moments
+    }
+}
+
+// the largest pairwise coprime numbers below the exactness bound until their product exceeds 2^bits
+bool choose_moduli(int nc, double bits, ResConsts &c)
+{
+    int h = 1;
+    while ((int64_t)RES_CHAIN * nc * (h + 1) * (h + 1) <= (1 << 24)) ++h;
+    int top = 2 * h + 1;
+    if (top > 2047) top = 2047;  // whole numbers of fp16; residues stay below 2^11
+    double have = 0;
+    c.n = 0;
+    for (int p = top; p > 2 && have < bits; --p) {
+        bool ok = true;
+        for (int i = 0; i < c.n && ok; ++i) {
+            int a = p, b = c.p[i];
+            while (b) {
+                const int t = a % b;
+                a = b;
+                b = t;
+            }
+            ok = a == 1;
+        }
+        if (!ok) continue;
+        if (c.n == RES_MAX) return false;
+        c.p[c.n++] = p;
+        have += log2((double)p);
+    }
+    if (have < bits) return false;
+    double pscale = 1.0;
+    for (int i = 0; i < c.n; ++i) pscale *= (double)c.p[i] * ldexp(1.0, -6);
+    c.pscale = ldexp(pscale, 6 * c.n - 96);
+    for (int i = 0; i < c.n; ++i) {
+        const int p = c.p[i];
+        auto centred = [p](int64_t v) {
+            int r = (int)(((v % p) + p) % p);
+            return r > p / 2 ? r - p : r;
+        };
+        c.rp[i] = 1.f / (float)p;
+        c.c18[i] = centred((int64_t)1 << 18);
+        c.c36[i] = centred((int64_t)1 << 36);
+        int64_t q = 1;  // P / p_i mod p_i
+        for (int j = 0; j < c.n; ++j)
+            if (j != i) q = q * c.p[j] % p;
+        int64_t inv = 1;
+        while (q * inv % p != 1) ++inv;
+        c.inv[i] = centred(inv);
+        // floor(2^96 / p), base 2^32 long division
+        uint64_t rem = 1;
+        for (int w = 2; w >= 0; --w) {
+            rem <<= 32;
+            c.w[i][w] = (uint32_t)(rem / p);
+            rem %= p;
+        }
+    }
+    return true;
+}
+
+#define FMM_RES_CASES(X) \
+    X(1) X(2) X(3) X(4) X(6) X(7) X(8) X(9) X(11) X(13) X(15) X(16)
+
+TcKernel res_kernel(int nch)
+{
+    switch (nch) {
+#define X(n) \
+    case n: return (TcKernel)k_m2l_tc<2, 2, n, 128, true>;
+        FMM_RES_CASES(X)
+#undef X
+    default: return nullptr;
+    }
+}
+
+TcKernel res_pair_kernel(int nch)
+{
+    switch (nch) {
+#define X(n) \
+    case n: return (TcKernel)k_m2l_tc_pair<n, true>;
+        FMM_RES_CASES(X)
+#undef X
+    default: return nullptr;
+    }
+}
+
+bool pairs_at(const ResState *S, int l)
+{
+    const int np = 1 << (l - 1);
+    const int tiles = (np / S->bx[l]) * (np / S->by[l]) * (np / S->bz[l]);
+    return S->bx[l] * S->by[l] * S->bz[l] == TC_ROWS && tiles % 2 == 0;
+}
+
+unsigned blocks_upto(int64_t n, int t, int64_t most)
+{
+    const int64_t b = (n + t - 1) / t;
+    return (unsigned)(b < most ? b : most);
+}
+
+fmm_status prepare(Plan &P, ResState *S)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return FMM_ERR_UNSUPPORTED;
+    // |L_int| < 2^56 2^56 137 (ws = 1: log2 137 = 7.10) or 277 (ws = 2: 8.12), and its sign
+    if (!choose_moduli(P.nc, RES_M_BITS + RES_T_BITS + (P.ws == 1 ? 7.2 : 8.2) + 1.0, S->c)) return FMM_ERR_UNSUPPORTED;
+    S->npad = (P.nc + 15) / 16 * 16;
+    S->kp = (P.nc + 63) / 64 * 64;
+    S->noff = noff(P.ws);
+    const int kc = S->kp / 64, n = S->c.n;
+    std::vector<double> h_s(P.nc);
+    for (int d = 0; d <= P.p; ++d)
+        for (int m = 0; m <= d; ++m) {
+            double f = 1.0;
+            for (int i = 2; i <= d + m; ++i) f *= i;
+            for (int i = 2; i <= d - m; ++i) f *= i;
+            h_s[cre(d, m)] = sqrt(f);
+            if (m > 0) h_s[cim(d, m)] = sqrt(f);
+        }
+    FMM_CUDA_TRY(cudaMalloc(&S->s64, sizeof(double) * P.nc));
+    FMM_CUDA_TRY(cudaMalloc(&S->amax, sizeof(unsigned long long) * 9));
+    FMM_CUDA_TRY(cudaMalloc(&S->mods, sizeof(int) * RES_MAX));
+    FMM_CUDA_TRY(cudaMemcpyAsync(S->s64, h_s.data(), sizeof(double) * P.nc, cudaMemcpyHostToDevice, P.stream));
+    FMM_CUDA_TRY(cudaMemcpyAsync(S->mods, S->c.p, sizeof(int) * RES_MAX, cudaMemcpyHostToDevice, P.stream));
+    S->ops_elems = (size_t)S->noff * S->npad * S->kp;
+    FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_elems * n));
+    k_res_ops<<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.nc, S->npad, S->kp, S->s64, S->ops, S->ops_elems, S->c);
+    FMM_LAUNCH_CHECK(P);
+    int sms = 0, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        sms = 152;
+    size_t planes = 0, resid = 0, frac = 0;
+    for (int l = 1; l <= P.d; ++l) {
+        const int np = 1 << (l - 1);
+        const size_t np2 = (size_t)np + 2 * P.ws, cells = (size_t)8 * np * np * np;
+        S->bx[l] = tile_dim(np, TC_ROWS);
+        S->by[l] = tile_dim(np, TC_ROWS / S->bx[l]);
+        S->bz[l] = tile_dim(np, TC_ROWS / (S->bx[l] * S->by[l]));
+        const size_t plane = 8 * np2 * np2 * np2 * S->kp * sizeof(uint16_t);
+        int b = (int)(RES_PLANE_BUDGET / plane);
+        b = b < 1 ? 1 : (b > n ? n : b);
+        b = (n + (n + b - 1) / b - 1) / ((n + b - 1) / b);  // even launches
+        S->batch[l] = b;
+        const int tiles = 8 * (np / S->bx[l]) * (np / S->by[l]) * (np / S->bz[l]);
+        split_offsets(n_il(P.ws), tiles * b, 27, sms, S->groups[l], S->per_group[l]);
+        if (plane * b > planes) planes = plane * b;
+        const size_t r = (size_t)S->groups[l] * b * cells * P.nc * sizeof(int16_t);
+        if (r > resid) resid = r;
+        if (b < n && cells * P.nc > frac) frac = cells * P.nc;
+    }
+    FMM_CUDA_TRY(cudaMalloc(&S->planes, planes));
+    FMM_CUDA_TRY(cudaMalloc(&S->resid, resid));
+    if (frac) FMM_CUDA_TRY(cudaMalloc(&S->frac, frac * 3 * sizeof(uint32_t)));
+    const CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+    fmm_status st = encode_operators(enc, &S->maps[0].bS, nullptr, &S->maps[0].bC, dt, S->ops, kc, n, S->npad, S->noff,
+                                     S->npad, 128);
+    if (st == FMM_OK)
+        st = encode_operators(enc, &S->mapB2[0], nullptr, &S->mapB2[1], dt, S->ops, kc, n, S->npad, S->noff, S->npad / 2,
+                              128);
+    for (int l = 1; l <= P.d && st == FMM_OK; ++l) {
+        const int np = 1 << (l - 1);
+        const int64_t np2 = np + 2 * P.ws;
+        TcMaps &m = S->maps[l];
+        m = S->maps[0];
+        st = encode_planes(enc, &m.aS, nullptr, &m.aC, dt, S->planes, kc, S->batch[l], np2, np2, 8 * np2, S->bx[l],
+                           S->by[l], S->bz[l], 128);
+        if (pairs_at(S, l)) {
+            m.bS = S->mapB2[0];
+            m.bC = S->mapB2[1];
+        }
+        m.aP = m.lS = m.lP = m.aS;  // unused kernel parameters
+        m.bP = m.bS;
+    }
+    if (st != FMM_OK) return st;
+    const TcKernel k1 = res_kernel(S->npad / 16), k2 = res_pair_kernel(S->npad / 16);
+    if (!k1 || !k2) return FMM_ERR_INTERNAL;
+    FMM_CUDA_TRY(cudaFuncSetAttribute((const void *)k1, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)tc_smem_bytes(2, 2, S->npad, 128)));
+    FMM_CUDA_TRY(cudaFuncSetAttribute((const void *)k2, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)tc_pair_smem_bytes(S->npad)));
+    FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
+    return FMM_OK;
+}
+
+}  // namespace
+
+bool res_available(const Plan &P, int level) { return P.res != nullptr && level >= 1 && level <= P.d; }
+
+// The residue state of an FP64 plan; without the memory for it the plan keeps the CUDA-core M2L
+fmm_status res_ensure(Plan &P)
+{
+    if (P.res || P.res_tried || P.precision != FMM_PREC_FP64 || P.p > TC_PMAX) return FMM_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    FMM_CUDA_TRY(cudaStreamIsCapturing(P.stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return FMM_OK;
+    P.res_tried = true;
+    ResState *S = new (std::nothrow) ResState();
+    if (!S) return FMM_ERR_OOM;
+    P.res = S;
+    const fmm_status st = prepare(P, S);
+    if (st == FMM_OK) return FMM_OK;
+    cudaStreamSynchronize(P.stream);
+    res_free(P);
+    P.res_tried = true;
+    if (st == FMM_ERR_OOM || st == FMM_ERR_UNSUPPORTED) {
+        cudaGetLastError();
+        return FMM_OK;
+    }
+    return st;
+}
+
+// L[l] = M2L of level l (the L2L from level l - 1 is added by launch_l2l)
+fmm_status launch_m2l_res(Plan &P, int l)
+{
+    ResState *S = (ResState *)P.res;
+    if (!S) return FMM_ERR_INTERNAL;
+    const int np = 1 << (l - 1), nc = P.nc, n = S->c.n;
+    const int64_t np2 = np + 2 * P.ws, cells = (int64_t)8 * np * np * np;
+    FMM_CUDA_TRY(cudaMemsetAsync(S->amax + l, 0, sizeof(unsigned long long), P.stream));
+    k_res_absmax<<<blocks_upto(cells, 8, 1216), 256, 0, P.stream>>>((const double *)P.M[l], cells, nc, S->s64, S->amax + l);
+    FMM_LAUNCH_CHECK(P);
+    TcArgs a;
+    memset(&a, 0, sizeof(a));
+    a.np = np;
+    a.bx = S->bx[l];
+    a.by = S->by[l];
+    a.bz = S->bz[l];
+    a.rows = a.bx * a.by * a.bz;
+    a.tiles_x = np / a.bx;
+    a.tiles_y = np / a.by;
+    a.tiles_per_class = a.tiles_x * a.tiles_y * (np / a.bz);
+    a.nc = nc;
+    a.npad = S->npad;
+    a.nslots = a.noff = S->noff;
+    a.groups = S->groups[l];
+    a.per_group = S->per_group[l];
+    a.n_off = a.n_il = n_il(P.ws);
+    a.ws = P.ws;
+    for (int k = 0; k < S->kp / 64; ++k) a.gchunks |= 1u << (2 * k);  // one product per chunk, two chunks a stage
+    a.acc_group = RES_CHAIN;
+    a.wait_ns = WAIT_LIMIT_NS;
+    a.err = P.d_err;
+    a.mods = S->mods;
+    a.resid = S->resid;
+    const bool pair = pairs_at(S, l);
+    a.stages = pair ? tc_pair_stages(S->npad) : tc_stages(2, 2, S->npad, 128);
+    a.idesc = (1u << 4) | ((uint32_t)(S->npad >> 3) << 17) | ((uint32_t)((pair ? 2 * TC_ROWS : TC_ROWS) >> 4) << 24);
+    const TcKernel k = pair ? res_pair_kernel(S->npad / 16) : res_kernel(S->npad / 16);
+    const size_t smem = pair ? tc_pair_smem_bytes(S->npad) : tc_smem_bytes(2, 2, S->npad, 128);
+    const int64_t halo = 8 * np2 * np2 * np2 * (S->kp / 8), elems = cells * nc;
+    for (int m0 = 0; m0 < n; m0 += S->batch[l]) {
+        const int nb = n - m0 < S->batch[l] ? n - m0 : S->batch[l];
+        k_res_split<<<blocks_upto(halo, 256, 8 * 1216), 256, 0, P.stream>>>((const double *)P.M[l], np, P.ws, nc, S->kp,
+                                                                            S->s64, S->amax + l, m0, nb, S->planes, S->c);
+        FMM_LAUNCH_CHECK(P);
+        a.mod0 = m0;
+        a.nmods = nb;
+        k<<<8u * (unsigned)a.tiles_per_class * (unsigned)a.groups * (unsigned)nb, TC_THREADS, smem, P.stream>>>(S->maps[l], a);
+        FMM_LAUNCH_CHECK(P);
+        k_res_join<<<(unsigned)((elems / 2 + 255) / 256), 256, 0, P.stream>>>(
+            elems, nc, a.groups, m0, nb, S->resid, S->frac, m0 == 0, m0 + nb == n, S->s64, S->amax + l, (double *)P.L[l],
+            S->c);
+        FMM_LAUNCH_CHECK(P);
+    }
+    return FMM_OK;
+}
+
+// dst reads src's operator residues when they are the same (p, ws); src must outlive dst
+fmm_status res_share_operators(Plan &dst, const Plan &src)
+{
+    ResState *D = (ResState *)dst.res;
+    const ResState *S = (const ResState *)src.res;
+    if (!D || !S || D == S || D->ops == S->ops || dst.p != src.p || dst.ws != src.ws) return FMM_OK;
+    FMM_CUDA_TRY(cudaDeviceSynchronize());  // nothing of dst's may still read its own table
+    if (!D->ops_borrowed) cudaFree(D->ops);
+    D->ops = S->ops;
+    D->ops_borrowed = true;
+    D->maps[0] = S->maps[0];
+    D->mapB2[0] = S->mapB2[0];
+    D->mapB2[1] = S->mapB2[1];
+    for (int l = 1; l <= dst.d; ++l) {
+        const bool pair = pairs_at(D, l);
+        D->maps[l].bS = D->maps[l].bP = pair ? S->mapB2[0] : S->maps[0].bS;
+        D->maps[l].bC = pair ? S->mapB2[1] : S->maps[0].bC;
+    }
+    return FMM_OK;
+}
+
+void res_free(Plan &P)
+{
+    ResState *S = (ResState *)P.res;
+    P.res_tried = false;
+    if (!S) return;
+    if (!S->ops_borrowed) cudaFree(S->ops);
+    cudaFree(S->planes);
+    cudaFree(S->resid);
+    cudaFree(S->frac);
+    cudaFree(S->s64);
+    cudaFree(S->amax);
+    cudaFree(S->mods);
+    delete S;
+    P.res = nullptr;
+}
+
+}  // namespace fmm
