@@ -300,10 +300,11 @@ fmm_status tc_prepare(Plan &P);
 // amax_ready: the kernel that wrote M[level] has already folded the level's largest |Mhat s| into
 // tc_amax(P, level) (else it is computed here)
 fmm_status tc_split_moments(Plan &P, int level, bool amax_ready);
-// fp16 split: the device word of level l's largest |Mhat s| (float bits), cleared by tc_clear_amax before
-// the kernel that produces M[l] folds its maximum in; s(n,m) per real coefficient
+// fp16 split: the device word of level l's largest |Mhat s| (float bits), into which the kernel that produces
+// M[l] folds its maximum; tc_clear_amax clears the words of all levels (M and L) at the start of a far-field
+// pass; s(n,m) per real coefficient
 unsigned *tc_amax(Plan &P, int level);
-fmm_status tc_clear_amax(Plan &P, int level);
+fmm_status tc_clear_amax(Plan &P);
 const float *tc_scale(const Plan &P);
 // fp16 split: M2M into level (< d) from the planes of level + 1
 fmm_status launch_m2m_tc(Plan &P, int level);
@@ -318,6 +319,7 @@ bool res_available(const Plan &P, int level);
 // builds the state on an FP64 plan's first evaluation (a plan that is to run the mixed path never pays for it);
 // left for later while the plan's stream is being captured
 fmm_status res_ensure(Plan &P);
+fmm_status res_clear_amax(Plan &P);  // at the start of a far-field pass
 fmm_status launch_m2l_res(Plan &P, int level);
 fmm_status res_share_operators(Plan &dst, const Plan &src);
 void res_free(Plan &P);

@@ -65,6 +65,7 @@ struct ResState {
     double *s64 = nullptr;        // [nc] s(n,m)
     unsigned long long *amax = nullptr;  // [9] bits of the largest |M^ s| per level
     int *mods = nullptr;
+    int *il = nullptr;            // interaction lists (upload_il)
 };
 
 // x mod p for |x| <= 2^57, centred: 18-bit limbs (the highest signed) against 2^18 and 2^36 mod p, then one
@@ -350,6 +351,8 @@ fmm_status prepare(Plan &P, ResState *S)
     FMM_CUDA_TRY(cudaMalloc(&S->mods, sizeof(int) * RES_MAX));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->s64, h_s.data(), sizeof(double) * P.nc, cudaMemcpyHostToDevice, P.stream));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->mods, S->c.p, sizeof(int) * RES_MAX, cudaMemcpyHostToDevice, P.stream));
+    fmm_status st = upload_il(P.ws, P.stream, &S->il);
+    if (st != FMM_OK) return st;
     S->ops_elems = (size_t)S->noff * S->npad * S->kp;
     FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_elems * n));
     k_res_ops<<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.nc, S->npad, S->kp, S->s64, S->ops, S->ops_elems, S->c);
@@ -381,7 +384,7 @@ fmm_status prepare(Plan &P, ResState *S)
     FMM_CUDA_TRY(cudaMalloc(&S->resid, resid));
     if (frac) FMM_CUDA_TRY(cudaMalloc(&S->frac, frac * 3 * sizeof(uint32_t)));
     const CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-    fmm_status st = encode_operators(enc, &S->maps[0].bS, nullptr, &S->maps[0].bC, dt, S->ops, kc, n, S->npad, S->noff,
+    st = encode_operators(enc, &S->maps[0].bS, nullptr, &S->maps[0].bC, dt, S->ops, kc, n, S->npad, S->noff,
                                      S->npad, 128);
     if (st == FMM_OK)
         st = encode_operators(enc, &S->mapB2[0], nullptr, &S->mapB2[1], dt, S->ops, kc, n, S->npad, S->noff, S->npad / 2,
@@ -438,6 +441,13 @@ fmm_status res_ensure(Plan &P)
     return st;
 }
 
+fmm_status res_clear_amax(Plan &P)
+{
+    ResState *S = (ResState *)P.res;
+    if (S) FMM_CUDA_TRY(cudaMemsetAsync(S->amax, 0, sizeof(unsigned long long) * 9, P.stream));
+    return FMM_OK;
+}
+
 // L[l] = M2L of level l (the L2L from level l - 1 is added by launch_l2l)
 fmm_status launch_m2l_res(Plan &P, int l)
 {
@@ -445,7 +455,6 @@ fmm_status launch_m2l_res(Plan &P, int l)
     if (!S) return FMM_ERR_INTERNAL;
     const int np = 1 << (l - 1), nc = P.nc, n = S->c.n;
     const int64_t np2 = np + 2 * P.ws, cells = (int64_t)8 * np * np * np;
-    FMM_CUDA_TRY(cudaMemsetAsync(S->amax + l, 0, sizeof(unsigned long long), P.stream));
     k_res_absmax<<<blocks_upto(cells, 8, 1216), 256, 0, P.stream>>>((const double *)P.M[l], cells, nc, S->s64, S->amax + l);
     FMM_LAUNCH_CHECK(P);
     TcArgs a;
@@ -470,6 +479,7 @@ fmm_status launch_m2l_res(Plan &P, int l)
     a.wait_ns = WAIT_LIMIT_NS;
     a.err = P.d_err;
     a.mods = S->mods;
+    a.il = S->il;
     a.resid = S->resid;
     const bool pair = pairs_at(S, l);
     a.stages = pair ? tc_pair_stages(S->npad) : tc_stages(2, 2, S->npad, 128);
@@ -527,6 +537,7 @@ void res_free(Plan &P)
     cudaFree(S->s64);
     cudaFree(S->amax);
     cudaFree(S->mods);
+    cudaFree(S->il);
     delete S;
     P.res = nullptr;
 }

@@ -84,7 +84,8 @@ struct TcState {
     float *s32inv = nullptr;        // [nc] 1 / s(n,m)
     double *s64 = nullptr;
     unsigned *amax = nullptr;       // [9] bits of the largest |M^ s| per level (fp16 split)
-    unsigned *amaxL = nullptr;      // [9] bits of the largest |L^ / s| per level
+    unsigned *amaxL = nullptr;      // [9] bits of the largest |L^ / s| per level (behind amax: one clear per pass)
+    int *il = nullptr;              // interaction lists (upload_il)
 };
 
 // ------------------------------------------------------------------ operand preparation
@@ -631,6 +632,10 @@ void fill_common(const Plan &P, const TcState *S, int pa, int pb, TcArgs &a)
     const uint32_t ab = S->f16 ? 0u : 1u;
     a.idesc = (1u << 4) | (ab << 7) | (ab << 10) | ((uint32_t)(S->npad >> 3) << 17) | ((uint32_t)(TC_ROWS >> 4) << 24);
     a.Lpart = S->Lpart;
+    a.il = S->il;
+    a.mod0 = a.nmods = 0;
+    a.mods = nullptr;
+    a.resid = nullptr;
     a.err = P.d_err;
     a.amax_out = nullptr;
     a.sx = nullptr;
@@ -722,12 +727,13 @@ fmm_status tc_prepare(Plan &P)
         FMM_CUDA_TRY(cudaMalloc(&S->s64, sizeof(double) * P.nc));
         FMM_CUDA_TRY(cudaMalloc(&S->s32, sizeof(float) * P.nc));
         FMM_CUDA_TRY(cudaMalloc(&S->s32inv, sizeof(float) * P.nc));
-        FMM_CUDA_TRY(cudaMalloc(&S->amax, sizeof(unsigned) * 9));
-        FMM_CUDA_TRY(cudaMalloc(&S->amaxL, sizeof(unsigned) * 9));
+        FMM_CUDA_TRY(cudaMalloc(&S->amax, sizeof(unsigned) * 18));
+        S->amaxL = S->amax + 9;
         FMM_CUDA_TRY(cudaMemcpyAsync(S->s64, h_s, sizeof(double) * P.nc, cudaMemcpyHostToDevice, P.stream));
         FMM_CUDA_TRY(cudaMemcpyAsync(S->s32, h_s32, sizeof(float) * P.nc, cudaMemcpyHostToDevice, P.stream));
         FMM_CUDA_TRY(cudaMemcpyAsync(S->s32inv, h_inv, sizeof(float) * P.nc, cudaMemcpyHostToDevice, P.stream));
     }
+    TRY_TC(upload_il(P.ws, P.stream, &S->il));
     // operator tables
     S->ops_part_elems = (size_t)(S->noff + 16) * S->npad * S->kp;
     FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_part_elems * S->parts));
@@ -809,11 +815,10 @@ unsigned *tc_amax(Plan &P, int l)
     return S && S->f16 && l >= 0 && l <= P.d ? S->amax + l : nullptr;
 }
 
-fmm_status tc_clear_amax(Plan &P, int l)
+fmm_status tc_clear_amax(Plan &P)
 {
-    unsigned *a = tc_amax(P, l);
-    if (!a) return FMM_ERR_INTERNAL;
-    FMM_CUDA_TRY(cudaMemsetAsync(a, 0, sizeof(unsigned), P.stream));
+    TcState *S = (TcState *)P.tc;
+    if (S && S->f16) FMM_CUDA_TRY(cudaMemsetAsync(S->amax, 0, sizeof(unsigned) * 18, P.stream));
     return FMM_OK;
 }
 
@@ -833,7 +838,6 @@ fmm_status tc_split_moments(Plan &P, int l, bool amax_ready)
     const int64_t np2 = np + 2 * P.ws;
     const int64_t ncell = (int64_t)8 * np * np * np;
     if (!amax_ready) {
-        FMM_CUDA_TRY(cudaMemsetAsync(S->amax + l, 0, sizeof(unsigned), P.stream));
         k_absmax<<<(unsigned)((ncell + 7) / 8 < 1216 ? (ncell + 7) / 8 : 1216), 256, 0, P.stream>>>(
             (const float *)P.M[l], ncell, P.nc, S->s32, S->amax + l);
         FMM_LAUNCH_CHECK(P);
@@ -873,7 +877,6 @@ fmm_status launch_m2m_tc(Plan &P, int l)
     a.post = S->s32inv;
     a.amax = S->amax + src;
     // level l's largest |M^ s| (the gain of its planes) is folded in by whoever writes M[l]
-    FMM_CUDA_TRY(cudaMemsetAsync(S->amax + l, 0, sizeof(unsigned), P.stream));
     a.amax_out = a.groups == 1 ? S->amax + l : nullptr;
     a.sx = S->s32;
     TcKernel k = pick_kernel(S->pa, S->pb, S->npad / 16, S->sw);
@@ -943,7 +946,6 @@ fmm_status launch_m2l_tc(Plan &P, int l, bool precise, bool split)
         // l - 1 launch (levels run in order), except at level 0 (the lattice operator's output)
         const int64_t ncl = (int64_t)np * np * np;
         if (l == 1) {
-            FMM_CUDA_TRY(cudaMemsetAsync(S->amaxL, 0, sizeof(unsigned), P.stream));
             k_absmax<<<1, 256, 0, P.stream>>>((const float *)P.L[0], 1, P.nc, S->s32inv, S->amaxL);
             FMM_LAUNCH_CHECK(P);
         }
@@ -957,8 +959,6 @@ fmm_status launch_m2l_tc(Plan &P, int l, bool precise, bool split)
             (const float *)P.M[l], np, P.ws, P.nc, S->kp, pa, kchunk_of(S->sw), S->planes[l], S->part_elems[l]);
         FMM_LAUNCH_CHECK(P);
     }
-    if (S->f16)  // level l's largest |L^ / s|, for the fused L2L of level l + 1
-        FMM_CUDA_TRY(cudaMemsetAsync(S->amaxL + l, 0, sizeof(unsigned), P.stream));
     TcArgs a;
     const bool pair = m2l_args(P, S, l, precise, pa, pb, a);
     unsigned grid = 8u * (unsigned)a.tiles_per_class * (unsigned)a.groups;
@@ -1245,7 +1245,7 @@ void tc_free(Plan &P)
     cudaFree(S->s32inv);
     cudaFree(S->s64);
     cudaFree(S->amax);
-    cudaFree(S->amaxL);
+    cudaFree(S->il);
     cudaFree(S->planesL);
     delete S;
     P.tc = nullptr;

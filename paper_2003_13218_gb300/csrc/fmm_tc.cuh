@@ -24,6 +24,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <vector>
+
 #include "fmm_internal.cuh"
 
 namespace fmm {
@@ -63,6 +65,7 @@ struct TcArgs {
     int src_np2;            // M2M: halo'd side of the child level's planes
     int ws, n_il, noff;     // well-separatedness, interaction-list length, M2L operator slots
     int out_np;             // M2M: class-layout side of the parent level (0 at level 0)
+    const int *il;          // M2L: the interaction list of each class, [8][n_il] packed offsets (il_pack)
     uint32_t idesc;
     uint32_t gchunks;       // fp16x2 M2L offsets: products per K chunk, 2 bits per chunk (0 = all 3), FMM_OPT_M2L_GRADE
     uint32_t gsteps;        // in a 3-product chunk, the first K16 step from which x1 y0 is dropped, 3 bits per chunk
@@ -107,6 +110,35 @@ __device__ inline int gain_m_exp(unsigned bits)
     const int e = GAIN_M_EXP - exp_of_bits(bits);
     return e < -100 ? -100 : (e > 100 ? 100 : e);
 }
+
+// An offset of an interaction list: delta per axis in [-2 ws - c, 2 ws + 1 - c], the near (2 ws + 1)^3 block left
+// out, in z, y, x order.  The producers read the list from a table: stepping through the cube and skipping what
+// is not theirs took ~160 cycles a position, up to 17 us before and after the copies of a small launch (2,998
+// charges at depth 3, p = 8: 682 -> 533 us a call; 100,000 at ws = 2: 2.9 -> 2.3 ms).
+__host__ __device__ inline int il_pack(int dx, int dy, int dz) { return (dx + 16) | ((dy + 16) << 8) | ((dz + 16) << 16); }
+
+// A producer warp's walk through offsets o .. end of one class's list: 32 entries per load, one load ahead
+struct IlWalk {
+    const int *list;
+    int o, end, lane, cur, next;
+    __device__ __forceinline__ IlWalk(const int *l, int begin, int e, int ln) : list(l), o(begin), end(e), lane(ln)
+    {
+        cur = o + lane < end ? __ldg(list + o + lane) : 0;
+        next = o + 32 + lane < end ? __ldg(list + o + 32 + lane) : 0;
+    }
+    // the offset of step k = 0, 1, .. (all lanes)
+    __device__ __forceinline__ void get(int k, int &dx, int &dy, int &dz)
+    {
+        if (k > 0 && (k & 31) == 0) {
+            cur = next;
+            next = o + k + 32 + lane < end ? __ldg(list + o + k + 32 + lane) : 0;
+        }
+        const int e = __shfl_sync(0xffffffffu, cur, k & 31);
+        dx = (e & 255) - 16;
+        dy = ((e >> 8) & 255) - 16;
+        dz = ((e >> 16) & 255) - 16;
+    }
+};
 
 // Accumulation groups of one CTA's offsets: the M2L (or M2M) offsets, local indices 0 .. nm - 1, in runs
 // of G that share one TMEM accumulator; the fused L2L offset (when present it is the CTA's last) alone,
@@ -679,6 +711,28 @@ __device__ __forceinline__ void load_scales(const TcArgs &a, float2 *sc, int n, 
     asm volatile("bar.sync 1, 128;" ::: "memory");
 }
 
+// One row of results, scaled, to its place in the staging tile; returns its largest |value f.y|.  The factors of
+// 16 columns are read before their values are stored (the compiler cannot move shared-memory reads over stores).
+template <int NCH>
+__device__ __forceinline__ float stage_row(const float (&Lr)[NCH * 16], const float2 *sc, float *dst, int nc)
+{
+    float mx = 0.f;
+#pragma unroll
+    for (int i0 = 0; i0 < NCH * 16; i0 += 16) {
+        float2 f[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) f[i] = sc[i0 + i];
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (i0 < (NCH - 1) * 16 || i0 + i < nc) {
+                const float v = Lr[i0 + i] * f[i].x;
+                dst[i0 + i] = v;
+                mx = fmaxf(mx, fabsf(v * f[i].y));
+            }
+    }
+    return mx;
+}
+
 // The end of a residue tile: sums taken modulo p, staged as 16-bit rows in the idle ring, stored
 template <int NCH>
 __device__ __forceinline__ void finish_residues(int (&acc)[NCH * 16], const TcArgs &a, int mod, int grp, int p, float rp,
@@ -825,21 +879,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
             };
             if (a.mode == 0) {
-                int oi = -1;  // position of the offset in the interaction-list order
-                // delta per axis in [-2 ws - c, 2 ws + 1 - c], the near (2 ws + 1)^3 block left out;
                 // the source brick sits at parent offset (c + delta) >> 1 in [-ws, ws], halo width ws
-                const int w = a.ws;
-                for (int dz = -2 * w - cz; dz <= 2 * w + 1 - cz && ok; ++dz)
-                    for (int dy = -2 * w - cy; dy <= 2 * w + 1 - cy && ok; ++dy)
-                        for (int dx = -2 * w - cx; dx <= 2 * w + 1 - cx && ok; ++dx) {
-                            if (dx >= -w && dx <= w && dy >= -w && dy <= w && dz >= -w && dz <= w) continue;
-                            ++oi;
-                            if (oi < o_begin || oi >= o_end) continue;
-                            const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
-                            const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-                            load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w,
-                                        scls * np2 + z0 + (sz >> 1) + w, 8 * np2, off_slot(dx, dy, dz, w), true);
-                        }
+                const int w = a.ws, o_il = o_end < a.n_il ? o_end : a.n_il;
+                IlWalk walk(a.il + cls * a.n_il, o_begin, o_il, lane);
+                for (int k = 0; k < o_il - o_begin && ok; ++k) {
+                    int dx, dy, dz;
+                    walk.get(k, dx, dy, dz);
+                    const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
+                    const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
+                    load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w, 8 * np2,
+                                off_slot(dx, dy, dz, w), true);
+                }
                 // fused L2L: the parents' local expansions (natural order, no halo)
                 if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
                     load_offset(true, x0, y0, z0, a.np, a.noff + 8 + cls, false);
@@ -991,14 +1041,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             float *stage = reinterpret_cast<float *>(smem_dyn + (smem0 - smem_u32(smem_dyn)));
             const int srow = a.nc | 1;
             if (row < a.rows) {
-#pragma unroll
-                for (int i = 0; i < NCH * 16; ++i)
-                    if (i < (NCH - 1) * 16 || i < a.nc) {
-                        const float2 f = scale_sh[i];
-                        const float v = Lr[i] * f.x;
-                        stage[row * srow + i] = v;
-                        mx = fmaxf(mx, fabsf(v * f.y));
-                    }
+                mx = stage_row<NCH>(Lr, scale_sh, stage + row * srow, a.nc);
             }
             const int64_t np = a.np;
             const int64_t level_cells = a.mode == 0 ? 8 * np * np * np : np * np * np;
@@ -1161,19 +1204,16 @@ __device__ __forceinline__ void pair_tile(const TcMaps &maps, const TcArgs &a, i
                     }
                 }
             };
-            int oi = -1;
-            const int w = a.ws;
-            for (int dz = -2 * w - cz; dz <= 2 * w + 1 - cz && ok; ++dz)
-                for (int dy = -2 * w - cy; dy <= 2 * w + 1 - cy && ok; ++dy)
-                    for (int dx = -2 * w - cx; dx <= 2 * w + 1 - cx && ok; ++dx) {
-                        if (dx >= -w && dx <= w && dy >= -w && dy <= w && dz >= -w && dz <= w) continue;
-                        ++oi;
-                        if (oi < o_begin || oi >= o_end) continue;
-                        const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
-                        const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-                        load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w,
-                                    8 * np2, off_slot(dx, dy, dz, w), true);
-                    }
+            const int w = a.ws, o_il = o_end < a.n_il ? o_end : a.n_il;
+            IlWalk walk(a.il + cls * a.n_il, o_begin, o_il, lane);
+            for (int k = 0; k < o_il - o_begin && ok; ++k) {
+                int dx, dy, dz;
+                walk.get(k, dx, dy, dz);
+                const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
+                const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
+                load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w, 8 * np2,
+                            off_slot(dx, dy, dz, w), true);
+            }
             if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
                 load_offset(true, x0, y0, z0, a.np, a.noff + 8 + cls, false);
             pp.it = it;
@@ -1336,14 +1376,7 @@ __device__ __forceinline__ void pair_tile(const TcMaps &maps, const TcArgs &a, i
             // every MMA of the tile has completed and no copy is pending, so the stage ring is idle: the rows
             // go through shared memory (stride srow, odd) and leave in coalesced stores, a warp per 32 rows
             const int srow = a.nc | 1;
-#pragma unroll
-            for (int i = 0; i < NCH * 16; ++i)
-                if (i < (NCH - 1) * 16 || i < a.nc) {
-                    const float2 f = bars.scale[i];
-                    const float v = Lr[i] * f.x;
-                    stage[row * srow + i] = v;
-                    mx = fmaxf(mx, fabsf(v * f.y));
-                }
+            mx = stage_row<NCH>(Lr, bars.scale, stage + row * srow, a.nc);
             const int64_t np = a.np;
             float *out = a.groups == 1 ? a.L : a.Lpart + (int64_t)grp * 8 * np * np * np * a.nc;
             const int tx = row % a.bx, ty = (row / a.bx) % a.by, tz = row / (a.bx * a.by);
@@ -1418,6 +1451,26 @@ __device__ __forceinline__ int64_t chunk_at(int64_t cell, int64_t ncell, int k, 
 }
 
 // ------------------------------------------------------------------ host helpers
+// the interaction lists of the 8 parity classes in device memory
+fmm_status upload_il(int ws, cudaStream_t st, int **out)
+{
+    const int n = n_il(ws);
+    std::vector<int> h;
+    h.reserve((size_t)8 * n);
+    for (int c = 0; c < 8; ++c) {
+        const int cx = c & 1, cy = (c >> 1) & 1, cz = (c >> 2) & 1;
+        for (int dz = -2 * ws - cz; dz <= 2 * ws + 1 - cz; ++dz)
+            for (int dy = -2 * ws - cy; dy <= 2 * ws + 1 - cy; ++dy)
+                for (int dx = -2 * ws - cx; dx <= 2 * ws + 1 - cx; ++dx)
+                    if (!(dx >= -ws && dx <= ws && dy >= -ws && dy <= ws && dz >= -ws && dz <= ws))
+                        h.push_back(il_pack(dx, dy, dz));
+    }
+    if (h.size() != (size_t)8 * n) return FMM_ERR_INTERNAL;
+    FMM_CUDA_TRY(cudaMalloc(out, sizeof(int) * h.size()));
+    FMM_CUDA_TRY(cudaMemcpyAsync(*out, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, st));
+    return cudaStreamSynchronize(st) == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
