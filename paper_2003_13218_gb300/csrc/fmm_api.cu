@@ -20,7 +20,7 @@ void free_buffers(Plan &P)
 {
     void *bufs[] = {P.in_pos, P.in_q,   P.out_forces, P.out_phi, P.in_sol, P.wpos,    P.key,    P.perm,   P.sleaf,
                     P.cell_start, P.cell_fill, P.scan_tmp, P.sorted, P.sorted_u, P.sorted_sol, P.phi_nf, P.phi_ff,
-                    P.phi_u, P.f_nf, P.g_ff, P.red_partial, P.red_out, P.d_err, P.sc_out, P.sc_lambda};
+                    P.phi_u, P.f_nf, P.g_ff, P.red_partial, P.red_out, P.d_err, P.sc_out, P.sc_lambda, P.d_M};
     for (void *b : bufs) cudaFree(b);
     for (int l = 0; l <= 8; ++l) {
         cudaFree(P.M[l]);
@@ -39,6 +39,7 @@ void free_buffers(Plan &P)
     P.phi_nf = P.phi_ff = P.phi_u = P.f_nf = P.g_ff = nullptr;
     P.red_partial = P.red_out = P.h_out = nullptr;
     P.d_err = nullptr;
+    P.d_M = nullptr;
 }
 
 template <typename X>
@@ -67,14 +68,16 @@ fmm_status alloc_buffers(Plan &P)
     FMM_CUDA_TRY(dalloc(&P.phi_u, sizeof(double) * N));
     FMM_CUDA_TRY(dalloc(&P.f_nf, sizeof(double) * 3 * N));
     FMM_CUDA_TRY(dalloc(&P.g_ff, sizeof(double) * 3 * N));
-    for (int l = 0; l <= P.d; ++l) {
+    for (int l = 1; l <= P.d; ++l) {  // the root is part of the top operator
         size_t cells = (size_t)1 << (3 * l);
         FMM_CUDA_TRY(dalloc(&P.M[l], sizeof(double) * cells * nc));
         FMM_CUDA_TRY(dalloc(&P.L[l], sizeof(double) * cells * nc));
     }
     FMM_CUDA_TRY(dalloc(&P.red_partial, reduction_scratch_bytes()));
     FMM_CUDA_TRY(dalloc(&P.red_out, sizeof(double) * 48));
-    FMM_CUDA_TRY(dalloc(&P.d_err, sizeof(int)));
+    FMM_CUDA_TRY(dalloc(&P.d_err, sizeof(int) * 2));
+    FMM_CUDA_TRY(dalloc(&P.d_M, sizeof(P.M)));
+    FMM_CUDA_TRY(cudaMemcpy(P.d_M, P.M, sizeof(P.M), cudaMemcpyHostToDevice));
     FMM_CUDA_TRY(cudaMallocHost((void **)&P.h_out, sizeof(double) * 40));
     return FMM_OK;
 }
@@ -121,17 +124,14 @@ struct StageTimer {
 fmm_status far_field_pass(Plan &P, bool gradient, bool solute_only, StageTimer *tm, bool fork_solute = false)
 {
     TRY(launch_upward(P, solute_only));
-    if (fork_solute) {
-        TRY(solute_prologue(P));
-        TRY(solute_sparse_fork(P));
-    }
+    if (fork_solute) TRY(solute_active(P));
     if (tm) tm->mark();
-    TRY(launch_lattice(P));
+    TRY(launch_top(P));
     if (tm) tm->mark();
     bool ev = tm && P.timings_on;
     // a batch's persistent sweep runs the levels >= sweep_from of the full pass, and its L2P after that
     const int last = (!solute_only && P.sweep_from > 0) ? P.sweep_from - 1 : P.d;
-    for (int l = 1; l <= last; ++l) {
+    for (int l = 2; l <= last; ++l) {
         if (ev) cudaEventRecord(P.ev_m2l[2 * (l - 1)], P.stream);
         // with the fp16 split the upward pass left the planes split and the L2L is fused
         const bool fused = tc_available(P, l) && tc_translations(P);
@@ -180,7 +180,7 @@ fmm_status eval_front(Plan &P, const double *dpos, const double *dq, const uint8
                       bool gradient, StageTimer *tm)
 {
     if (tm) tm->mark();
-    FMM_CUDA_TRY(cudaMemsetAsync(P.d_err, 0, sizeof(int), P.stream));
+    FMM_CUDA_TRY(cudaMemsetAsync(P.d_err, 0, sizeof(int) * 2, P.stream));
     if (want_uv && P.sc_c > 0)  // the soft-core lambda as it is when the call runs
         FMM_CUDA_TRY(cudaMemcpyAsync(P.sc_lambda, P.h_sc_lambda, sizeof(double), cudaMemcpyHostToDevice, P.stream));
     P.near_forked = P.near_p2p = false;
@@ -189,6 +189,7 @@ fmm_status eval_front(Plan &P, const double *dpos, const double *dq, const uint8
     if (tm) tm->mark();
     if (P.overlap && P.near) TRY(fork_near_field(P, dq, dsol, gradient, want_uv));
     else TRY(launch_bc_moments(P, dq, dsol));
+    if (want_uv) TRY(solute_fork(P));
     TRY(far_field_pass(P, gradient, false, tm, want_uv));
     if (!P.near_p2p) TRY(launch_p2p(P, gradient));
     if (tm) tm->mark();
@@ -269,6 +270,7 @@ struct ExecScope {
     ~ExecScope()
     {
         if (!active) return;
+        solute_join(P);       // a failed call's
         if (P.near_forked) {  // a failed call
             cudaEventRecord(P.ev_near, P.near);
             cudaStreamWaitEvent(P.exec, P.ev_near, 0);
@@ -337,7 +339,7 @@ fmm_status evaluate(Plan &P, const double *pos, const double *q, const uint8_t *
         P.last.reduce = t[7];
         cudaEventElapsedTime(&P.last.total, P.ev[0], P.ev[tm.k - 1]);
         float m = 0;
-        for (int l = 1; l <= P.d; ++l) {
+        for (int l = 2; l <= P.d; ++l) {
             float x = 0;
             cudaEventElapsedTime(&x, P.ev_m2l[2 * (l - 1)], P.ev_m2l[2 * (l - 1) + 1]);
             m += x;

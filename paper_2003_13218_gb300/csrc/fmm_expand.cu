@@ -9,7 +9,10 @@
 // C_n^{-m} = (-1)^m conj C_n^m, so only m >= 0 is stored.
 #include <math.h>
 
+#include <stdlib.h>
+
 #include <type_traits>
+#include <vector>
 
 #include "fmm_internal.cuh"
 
@@ -450,19 +453,6 @@ void launch_p2m(Plan &P, const Particle<T> *sp, T inv_h)
     else k_p2m<T, P_MAX><<<blocks, 128, 0, P.stream>>>(p, nside, P.cell_start, sp, inv_h, P.d, (T *)P.M[P.d]);
 }
 
-// ------------------------------------------------------------------ lattice apply
-// Lbar(0) = T0 . Mhat(0) (Eq. 12 in place of I in Eq. Lcoeffdef), in FP64
-template <typename T>
-__global__ void k_lattice_apply(int p, const double *__restrict__ T0, const T *__restrict__ M0, T *__restrict__ L0)
-{
-    int nc = ncoef(p);
-    int j = threadIdx.x;
-    if (j >= nc) return;
-    double acc = 0;
-    for (int k = 0; k < nc; ++k) acc += T0[(size_t)k * nc + j] * (double)M0[k];
-    L0[j] = (T)acc;
-}
-
 // ------------------------------------------------------------------ M2L (CUDA cores)
 // Eq. Lcoeffdef over the 189-cell interaction list of each target, as dense
 // real operators per offset.  Block: TT targets of one parity class, one
@@ -736,7 +726,7 @@ fmm_status upward_t(Plan &P, bool solute_only)
         launch_p2m<T>(P, sp, inv_h);
     }
     FMM_LAUNCH_CHECK(P);
-    for (int l = P.d - 1; l >= 0; --l) {
+    for (int l = P.d - 1; l >= 1; --l) {  // the top operator starts from level 1
         // the tensor-core M2M into level l folds level l's maximum in (amax of level l + 1 is ready from
         // the P2M or the previous M2M)
         fmm_status st = tc ? tc_split_moments(P, l + 1, amax_ready) : FMM_OK;
@@ -761,6 +751,20 @@ fmm_status build_tables(Plan &P)
     FMM_CUDA_TRY(cudaMalloc(&P.tab.T0, sizeof(double) * nc * nc));
     FMM_CUDA_TRY(cudaMalloc(&P.tab.Top64, sizeof(double) * (size_t)noff(P.ws) * nc * nc));
     FMM_CUDA_TRY(cudaMalloc(&P.tab.Top32, sizeof(float) * (size_t)noff(P.ws) * nc * nc));
+    {
+        const int n = n_il(P.ws), ws = P.ws;
+        std::vector<int> h;
+        h.reserve((size_t)8 * n);
+        for (int c = 0; c < 8; ++c)
+            for (int dz = -2 * ws - (c >> 2); dz <= 2 * ws + 1 - (c >> 2); ++dz)
+                for (int dy = -2 * ws - ((c >> 1) & 1); dy <= 2 * ws + 1 - ((c >> 1) & 1); ++dy)
+                    for (int dx = -2 * ws - (c & 1); dx <= 2 * ws + 1 - (c & 1); ++dx)
+                        if (!(abs(dx) <= ws && abs(dy) <= ws && abs(dz) <= ws)) h.push_back(il_pack(dx, dy, dz));
+        if (h.size() != (size_t)8 * n) return FMM_ERR_INTERNAL;
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.il, sizeof(int) * h.size()));
+        FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.il, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, P.stream));
+        FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
+    }
     k_octant_table<<<1, 32, 0, P.stream>>>(p, P.tab.Rw64, P.tab.Rw32);
     FMM_LAUNCH_CHECK(P);
     {
@@ -778,8 +782,7 @@ fmm_status build_tables(Plan &P)
     FMM_LAUNCH_CHECK(P);
     k_lattice_operator<<<1, 256, shI, P.stream>>>(p, P.tab.S, P.tab.T0);
     FMM_LAUNCH_CHECK(P);
-    FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
-    return FMM_OK;
+    return build_top(P);
 }
 
 fmm_status build_lattice(Plan &P)
@@ -795,8 +798,7 @@ fmm_status build_lattice(Plan &P)
     FMM_LAUNCH_CHECK(P);
     k_lattice_operator<<<1, 256, sizeof(Cx<double>) * ntri2, P.stream>>>(p, P.tab.S, P.tab.T0);
     FMM_LAUNCH_CHECK(P);
-    FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
-    return FMM_OK;
+    return build_top(P);
 }
 
 void free_tables(Plan &P)
@@ -813,24 +815,15 @@ void free_tables(Plan &P)
     cudaFree(P.tab.m2m32);
     cudaFree(P.tab.m2mP32);
     cudaFree(P.tab.l2lP32);
+    cudaFree(P.tab.il);
+    cudaFree(P.tab.G64);
+    cudaFree(P.tab.G32);
     P.tab = Tables{};
 }
 
 fmm_status launch_upward(Plan &P, bool solute_only)
 {
     return P.precision == FMM_PREC_FP64 ? upward_t<double>(P, solute_only) : upward_t<float>(P, solute_only);
-}
-
-fmm_status launch_lattice(Plan &P)
-{
-    if (P.precision == FMM_PREC_FP64)
-        k_lattice_apply<double><<<1, ((P.nc + 31) / 32) * 32, 0, P.stream>>>(P.p, P.tab.T0, (const double *)P.M[0],
-                                                                            (double *)P.L[0]);
-    else
-        k_lattice_apply<float><<<1, ((P.nc + 31) / 32) * 32, 0, P.stream>>>(P.p, P.tab.T0, (const float *)P.M[0],
-                                                                           (float *)P.L[0]);
-    FMM_LAUNCH_CHECK(P);
-    return FMM_OK;
 }
 
 fmm_status launch_m2l_simt(Plan &P, int l)

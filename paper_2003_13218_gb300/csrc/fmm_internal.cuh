@@ -51,6 +51,15 @@ __host__ __device__ inline int off_slot(int dx, int dy, int dz, int ws)
     return (dx + h) + side * ((dy + h) + side * (dz + h));
 }
 
+// an offset of an interaction list in one word
+__host__ __device__ inline int il_pack(int dx, int dy, int dz) { return (dx + 16) | ((dy + 16) << 8) | ((dz + 16) << 16); }
+__host__ __device__ inline void il_unpack(int e, int &dx, int &dy, int &dz)
+{
+    dx = (e & 255) - 16;
+    dy = ((e >> 8) & 255) - 16;
+    dz = ((e >> 16) & 255) - 16;
+}
+
 __host__ __device__ inline int64_t cell_index(int l, int x, int y, int z)
 {
     if (l == 0) return 0;
@@ -85,6 +94,9 @@ struct Tables {
     float *m2m32 = nullptr;
     float *m2mP32 = nullptr;  // M2M with each octant's K padded to a multiple of 8
     float *l2lP32 = nullptr;  // L2L with K padded likewise
+    int *il = nullptr;        // [8][n_il(ws)] interaction list of each parity class, packed offsets (il_pack)
+    double *G64 = nullptr;    // [8 NC][8 NC] top operator: M(1) -> L(1), input-major (fmm_top.cu)
+    float *G32 = nullptr;
 };
 
 struct Plan {
@@ -144,6 +156,7 @@ struct Plan {
     // expansions per level (T, class layout)
     void *M[9] = {};
     void *L[9] = {};
+    void **d_M = nullptr;  // the M pointers in device memory (kernels that take all levels)
     // tensor-core M2L state (bf16 operand planes, operator tables, TMA maps)
     void *tc = nullptr;
     // FP64 residue M2L state (operator residues, planes, TMA maps)
@@ -155,7 +168,7 @@ struct Plan {
     double *red_partial = nullptr;  // partial sums
     double *red_out = nullptr;      // [32] final FP64 scalars
     double *h_out = nullptr;        // pinned host mirror
-    int *d_err = nullptr;
+    int *d_err = nullptr;  // [0] error flags, [1] solute charges of the call
     Tables tab;
     cudaEvent_t ev[12] = {};
     cudaEvent_t ev_m2l[18] = {};  // around each level's M2L launch (full pass)
@@ -260,7 +273,11 @@ fmm_status build_tables(Plan &P);
 fmm_status build_lattice(Plan &P);  // the kappa-dependent lattice table only
 void free_tables(Plan &P);
 fmm_status launch_upward(Plan &P, bool solute_only);
-fmm_status launch_lattice(Plan &P);
+// L(1) from M(1): level 1's M2L and everything above it (fmm_top.cu)
+fmm_status build_top(Plan &P);
+fmm_status launch_top(Plan &P);
+fmm_status launch_top_solute(Plan &P, cudaStream_t st, const void *MU1, const int *cells, const int *ncells, void *Lu1);
+fmm_status launch_top_active(Plan &P, cudaStream_t st, const void *MU1, const int *cells, const int *ncells, double *Lt1);
 fmm_status launch_m2l_simt(Plan &P, int level);
 
 // M2M / L2L as dense products (fmm_translate.cu)
@@ -276,19 +293,20 @@ fmm_status launch_p2p_uv(Plan &P);
 // sparse solute-only pass of Eq. FMMcalc (fmm_solute.cu)
 fmm_status solute_prepare(Plan &P);
 void solute_free(Plan &P);
-// right after the sort: count the solute charges and copy the count to the host asynchronously
+// where the sort lists the solute slots (at most *cap; their count is P.d_err[1])
+int *solute_list(Plan &P, int *cap);
+// right after the sort: copy the solute count to the host asynchronously
 fmm_status solute_count(Plan &P);
-// the host copy of the last solute count (valid once the plan's stream has passed the copy); -1 when the
-// plan has no sparse pass
+// the host copy of the last solute count (valid once the plan's stream has passed the copy)
 int solute_count_host(const Plan &P);
-// after the full pass's upward sweep: the pass's prologue (active cells, solute moments, FP64 solvent
-// expansions at the active cells) on a high-priority side stream, overlapping the full pass's M2L
-fmm_status solute_prologue(Plan &P);
-// right after the prologue (P.overlap): the rest of the sparse pass on the side stream (it touches none of
-// the full pass's expansions) and Phi_u at every charge on the near stream when that is forked; grids
-// cover the largest count and the device count decides
-fmm_status solute_sparse_fork(Plan &P);
-// joins the prologue (or the forked sparse pass) and runs the rest; *done = false when the dense pass must run
+// right after the sort (P.overlap): the solute-only expansions on the pass's side stream, Phi_u at every charge on
+// the near stream when that is forked; grids cover the largest count and the device count decides
+fmm_status solute_fork(Plan &P);
+// after the full pass's upward sweep (P.overlap): the solvent's FP64 field at the active cells on the side stream
+fmm_status solute_active(Plan &P);
+// the side stream's work of the call, if any, into the plan's stream (also after a failed call)
+fmm_status solute_join(Plan &P);
+// joins the forked pass (or runs it) and finishes it; *done = false when the dense pass must run
 fmm_status launch_solute_pass(Plan &P, bool *done);
 
 // tensor-core M2L, and with the fp16 split also M2M and L2L (fmm_m2l_tc.cu)
@@ -305,6 +323,8 @@ fmm_status tc_split_moments(Plan &P, int level, bool amax_ready);
 // pass; s(n,m) per real coefficient
 unsigned *tc_amax(Plan &P, int level);
 fmm_status tc_clear_amax(Plan &P);
+// the same for L (largest |Lhat / s|) with the factors 1 / s; null without the fp16 split
+unsigned *tc_amaxL(Plan &P, int level, const float **sx);
 const float *tc_scale(const Plan &P);
 // fp16 split: M2M into level (< d) from the planes of level + 1
 fmm_status launch_m2m_tc(Plan &P, int level);

@@ -65,7 +65,6 @@ struct ResState {
     double *s64 = nullptr;        // [nc] s(n,m)
     unsigned long long *amax = nullptr;  // [9] bits of the largest |M^ s| per level
     int *mods = nullptr;
-    int *il = nullptr;            // interaction lists (upload_il)
 };
 
 // x mod p for |x| <= 2^57, centred: 18-bit limbs (the highest signed) against 2^18 and 2^36 mod p, then one
@@ -351,8 +350,6 @@ fmm_status prepare(Plan &P, ResState *S)
     FMM_CUDA_TRY(cudaMalloc(&S->mods, sizeof(int) * RES_MAX));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->s64, h_s.data(), sizeof(double) * P.nc, cudaMemcpyHostToDevice, P.stream));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->mods, S->c.p, sizeof(int) * RES_MAX, cudaMemcpyHostToDevice, P.stream));
-    fmm_status st = upload_il(P.ws, P.stream, &S->il);
-    if (st != FMM_OK) return st;
     S->ops_elems = (size_t)S->noff * S->npad * S->kp;
     FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_elems * n));
     k_res_ops<<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.nc, S->npad, S->kp, S->s64, S->ops, S->ops_elems, S->c);
@@ -362,7 +359,7 @@ fmm_status prepare(Plan &P, ResState *S)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         sms = 152;
     size_t planes = 0, resid = 0, frac = 0;
-    for (int l = 1; l <= P.d; ++l) {
+    for (int l = 2; l <= P.d; ++l) {  // level 1 is part of the top operator
         const int np = 1 << (l - 1);
         const size_t np2 = (size_t)np + 2 * P.ws, cells = (size_t)8 * np * np * np;
         S->bx[l] = tile_dim(np, TC_ROWS);
@@ -384,12 +381,12 @@ fmm_status prepare(Plan &P, ResState *S)
     FMM_CUDA_TRY(cudaMalloc(&S->resid, resid));
     if (frac) FMM_CUDA_TRY(cudaMalloc(&S->frac, frac * 3 * sizeof(uint32_t)));
     const CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-    st = encode_operators(enc, &S->maps[0].bS, nullptr, &S->maps[0].bC, dt, S->ops, kc, n, S->npad, S->noff,
+    fmm_status st = encode_operators(enc, &S->maps[0].bS, nullptr, &S->maps[0].bC, dt, S->ops, kc, n, S->npad, S->noff,
                                      S->npad, 128);
     if (st == FMM_OK)
         st = encode_operators(enc, &S->mapB2[0], nullptr, &S->mapB2[1], dt, S->ops, kc, n, S->npad, S->noff, S->npad / 2,
                               128);
-    for (int l = 1; l <= P.d && st == FMM_OK; ++l) {
+    for (int l = 2; l <= P.d && st == FMM_OK; ++l) {
         const int np = 1 << (l - 1);
         const int64_t np2 = np + 2 * P.ws;
         TcMaps &m = S->maps[l];
@@ -479,7 +476,7 @@ fmm_status launch_m2l_res(Plan &P, int l)
     a.wait_ns = WAIT_LIMIT_NS;
     a.err = P.d_err;
     a.mods = S->mods;
-    a.il = S->il;
+    a.il = P.tab.il;
     a.resid = S->resid;
     const bool pair = pairs_at(S, l);
     a.stages = pair ? tc_pair_stages(S->npad) : tc_stages(2, 2, S->npad, 128);
@@ -517,7 +514,7 @@ fmm_status res_share_operators(Plan &dst, const Plan &src)
     D->maps[0] = S->maps[0];
     D->mapB2[0] = S->mapB2[0];
     D->mapB2[1] = S->mapB2[1];
-    for (int l = 1; l <= dst.d; ++l) {
+    for (int l = 2; l <= dst.d; ++l) {
         const bool pair = pairs_at(D, l);
         D->maps[l].bS = D->maps[l].bP = pair ? S->mapB2[0] : S->maps[0].bS;
         D->maps[l].bC = pair ? S->mapB2[1] : S->maps[0].bC;
@@ -537,7 +534,6 @@ void res_free(Plan &P)
     cudaFree(S->s64);
     cudaFree(S->amax);
     cudaFree(S->mods);
-    cudaFree(S->il);
     delete S;
     P.res = nullptr;
 }

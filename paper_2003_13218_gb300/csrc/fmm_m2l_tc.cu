@@ -85,7 +85,6 @@ struct TcState {
     double *s64 = nullptr;
     unsigned *amax = nullptr;       // [9] bits of the largest |M^ s| per level (fp16 split)
     unsigned *amaxL = nullptr;      // [9] bits of the largest |L^ / s| per level (behind amax: one clear per pass)
-    int *il = nullptr;              // interaction lists (upload_il)
 };
 
 // ------------------------------------------------------------------ operand preparation
@@ -632,7 +631,7 @@ void fill_common(const Plan &P, const TcState *S, int pa, int pb, TcArgs &a)
     const uint32_t ab = S->f16 ? 0u : 1u;
     a.idesc = (1u << 4) | (ab << 7) | (ab << 10) | ((uint32_t)(S->npad >> 3) << 17) | ((uint32_t)(TC_ROWS >> 4) << 24);
     a.Lpart = S->Lpart;
-    a.il = S->il;
+    a.il = P.tab.il;
     a.mod0 = a.nmods = 0;
     a.mods = nullptr;
     a.resid = nullptr;
@@ -733,7 +732,6 @@ fmm_status tc_prepare(Plan &P)
         FMM_CUDA_TRY(cudaMemcpyAsync(S->s32, h_s32, sizeof(float) * P.nc, cudaMemcpyHostToDevice, P.stream));
         FMM_CUDA_TRY(cudaMemcpyAsync(S->s32inv, h_inv, sizeof(float) * P.nc, cudaMemcpyHostToDevice, P.stream));
     }
-    TRY_TC(upload_il(P.ws, P.stream, &S->il));
     // operator tables
     S->ops_part_elems = (size_t)(S->noff + 16) * S->npad * S->kp;
     FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_part_elems * S->parts));
@@ -770,7 +768,7 @@ fmm_status tc_prepare(Plan &P)
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
                                                  cudaSuccess || sms < 1)
         sms = 152;
-    for (int l = 1; l <= P.d; ++l) {
+    for (int l = 2; l <= P.d; ++l) {  // level 1 is part of the top operator
         int np = 1 << (l - 1);
         int64_t np2 = np + 2 * P.ws;  // periodic halo of ws cells
         S->bx[l] = tile_dim(np, TC_ROWS);
@@ -822,6 +820,14 @@ fmm_status tc_clear_amax(Plan &P)
     return FMM_OK;
 }
 
+unsigned *tc_amaxL(Plan &P, int l, const float **sx)
+{
+    TcState *S = (TcState *)P.tc;
+    if (!S || !S->f16) return nullptr;
+    *sx = S->s32inv;
+    return S->amaxL + l;
+}
+
 const float *tc_scale(const Plan &P)
 {
     const TcState *S = (const TcState *)P.tc;
@@ -833,7 +839,7 @@ const float *tc_scale(const Plan &P)
 fmm_status tc_split_moments(Plan &P, int l, bool amax_ready)
 {
     TcState *S = (TcState *)P.tc;
-    if (!S || !S->f16 || l < 1 || l > P.d) return FMM_ERR_INTERNAL;
+    if (!S || !S->f16 || l < 2 || l > P.d) return FMM_ERR_INTERNAL;
     const int np = 1 << (l - 1);
     const int64_t np2 = np + 2 * P.ws;
     const int64_t ncell = (int64_t)8 * np * np * np;
@@ -853,7 +859,7 @@ fmm_status tc_split_moments(Plan &P, int l, bool amax_ready)
 fmm_status launch_m2m_tc(Plan &P, int l)
 {
     TcState *S = (TcState *)P.tc;
-    if (!S || !S->f16 || l < 0 || l >= P.d) return FMM_ERR_INTERNAL;
+    if (!S || !S->f16 || l < 1 || l >= P.d) return FMM_ERR_INTERNAL;
     const int src = l + 1;
     const int n = 1 << l;  // natural side of level l = parent side of the level-(l+1) planes
     TcArgs a;
@@ -872,7 +878,7 @@ fmm_status launch_m2m_tc(Plan &P, int l)
     a.per_group = S->mper_group[l];
     a.n_off = 8;
     a.src_np2 = n + 2 * P.ws;
-    a.out_np = l == 0 ? 0 : n >> 1;
+    a.out_np = n >> 1;
     a.L = (float *)P.M[l];
     a.post = S->s32inv;
     a.amax = S->amax + src;
@@ -943,12 +949,8 @@ fmm_status launch_m2l_tc(Plan &P, int l, bool precise, bool split)
             if (st != FMM_OK) return st;
         }
         // parent-level local expansion for the fused L2L; its largest |L^ / s| was folded in by the level
-        // l - 1 launch (levels run in order), except at level 0 (the lattice operator's output)
+        // l - 1 launch (levels run in order)
         const int64_t ncl = (int64_t)np * np * np;
-        if (l == 1) {
-            k_absmax<<<1, 256, 0, P.stream>>>((const float *)P.L[0], 1, P.nc, S->s32inv, S->amaxL);
-            FMM_LAUNCH_CHECK(P);
-        }
         k_split_L<<<(unsigned)((ncl + 7) / 8 < 1216 ? (ncl + 7) / 8 : 1216), 256, 0, P.stream>>>(
             (const float *)P.L[l - 1], l - 1, P.nc, S->kp, S->s32inv, S->amaxL + l - 1, S->planesL,
             (size_t)ncl * S->kp);
@@ -992,7 +994,7 @@ int tc_sweep_first_level(const Plan &P)
 {
     const TcState *S = (const TcState *)P.tc;
     if (!S || !S->f16 || !P.tc_pair || P.precision != FMM_PREC_MIXED) return 0;
-    for (int l = 2; l <= P.d; ++l) {  // level 1 reads the lattice's L[0]: it stays on its own launches
+    for (int l = 2; l <= P.d; ++l) {
         const int np = 1 << (l - 1);
         const int tpc = (np / S->bx[l]) * (np / S->by[l]) * (np / S->bz[l]);
         if (S->bx[l] * S->by[l] * S->bz[l] == TC_ROWS && tpc % 2 == 0) return l;  // and every deeper level
@@ -1245,7 +1247,6 @@ void tc_free(Plan &P)
     cudaFree(S->s32inv);
     cudaFree(S->s64);
     cudaFree(S->amax);
-    cudaFree(S->il);
     cudaFree(S->planesL);
     delete S;
     P.tc = nullptr;

@@ -4,22 +4,29 @@
 //
 // With a handful of solute charges only the leaves holding them and their
 // ancestors carry solute moments.  The pass therefore
-//  * builds the list of active cells per level (at most NU_MAX per level),
-//    P2M at the active leaves and M2M along the active ancestors;
-//  * on the coarse levels 1..LD (few cells) computes the local expansion of
-//    every cell in the pass's own arrays: the level-0 lattice operator, then
-//    per level the M2L terms of the active cells (one block per active cell and
-//    offset, every periodic image counted) summed per target with the L2L of
-//    its parent, giving the full local expansion at level LD;
+//  * builds the list of active cells per level (at most NU_MAX per level) and
+//    their solute moments, each straight from the charges (Eq. P2M about that
+//    cell's centre, which is what M2M would carry up, up to rounding);
+//  * on the coarse levels 1..ld, ld = min(3, depth), computes the local
+//    expansion of every cell in the pass's own arrays: level 1 by the top
+//    operator, then per level the M2L terms of the active cells (one block per
+//    active cell and offset, every periodic image counted) summed per target
+//    with the L2L of its parent, giving the full local expansion at level ld;
 //  * on the finer levels evaluates M2L only onto the targets whose interaction
-//    list contains an active source (at most n_il(ws) per source), kept as a
-//    sorted list per level;
-//  * evaluates Phi_u at every charge as the level-LD expansion plus the sparse
+//    list contains an active source (at most n_il(ws) per source);
+//  * evaluates Phi_u at every charge as the level-ld expansion plus the sparse
 //    contributions found at its finer ancestors.  A local expansion is a
 //    polynomial of degree p, so evaluating it at a charge directly equals
 //    shifting it to the leaf with L2L first (Appendix B) up to rounding.
-// When more than NU_MAX charges are solute, or the tree has no finer levels,
-// the caller runs the dense pass instead.
+// The work of all levels that does not depend on another level shares one
+// launch (grids of blocks that take work items in turn, since the host does not
+// know the number of active cells): the pass is a chain of small kernels, and
+// as ~60 of them, level by level, it took 0.57 ms of a call on 100,000 charges.
+// None of it needs more than the sort, so it starts beside the upward pass.  At
+// depth 3 and less, where the dense pass used to run, it saves a second far-field
+// pass.  Calls with E_uv: 100,000 charges from host arrays 1.87 -> 1.18 ms, 16
+// coupling windows 6.96 -> 5.48 ms, 2,998 charges in FP64 1.36 -> 1.02 ms.
+// When more than NU_MAX charges are solute the caller runs the dense pass instead.
 #include <math.h>
 
 #include <new>
@@ -32,31 +39,35 @@ namespace fmm {
 namespace {
 
 constexpr int NU_MAX = 64;      // solute charges handled by the sparse pass
-constexpr int LD = 3;           // levels 0..LD treated densely
+constexpr int LD_MAX = 3;       // levels 1..min(3, depth) treated densely
+constexpr int ACT_OFFS = 3;     // interaction-list offsets per block of the solvent field (n_il is a multiple of it
+                                // or the last block takes fewer)
+constexpr int ITEM_BLOCKS = 912;  // 6 x 152 SMs: blocks of the launches that loop over work items
 // targets per fine level: at most NU_MAX * n_il(ws) (mt below)
 __host__ __device__ inline int max_tgt(int ws) { return NU_MAX * n_il(ws); }
+__host__ __device__ inline int act_groups(int ws) { return (n_il(ws) + ACT_OFFS - 1) / ACT_OFFS; }
 
 struct SoluteScratch {
-    int *list = nullptr;     // [NU_MAX] sorted slots of solute charges; [NU_MAX] = count
+    int *list = nullptr;     // [NU_MAX] sorted slots of solute charges as found; the count is P.d_err[1]
+    int *slots = nullptr;    // [NU_MAX] the same in slot order
     int *cells = nullptr;    // [9][NU_MAX] active cell (linear index) per level
-    int *ncells = nullptr;   // [9]
+    int *ncells = nullptr;   // [9] active cells, [16 + l] targets of fine level l
     void *MU = nullptr;      // [9][NU_MAX][nc] solute moments of the active cells
-    int *flags = nullptr;    // [8^d] target marks of one level
-    int *pos = nullptr;      // [8^d + 1] exclusive scan of the marks
-    int *scan_tmp = nullptr;
-    int *tlist = nullptr;    // [9][mt] sorted targets per fine level
-    void *contrib = nullptr; // [9][mt][nc] M2L sums at those targets
+    int *map = nullptr;      // per fine level [8^l]: 1 + index of a target cell in tlist, 0: no target
+    size_t map_bytes = 0;
+    int *tlist = nullptr;    // [9][mt] targets per fine level, in no particular order
+    void *contrib = nullptr; // [9][mt][nc] M2L sums at those targets; rows of levels 0..ld: M2L terms of the dense levels
     int *h_count = nullptr;  // pinned
-    cudaStream_t side = nullptr;       // high-priority stream of the prologue (overlaps the full pass's M2L)
+    cudaStream_t side = nullptr;       // high-priority stream of the pass (overlaps the full pass)
     cudaEvent_t ev_count = nullptr;    // count copied to h_count
-    cudaEvent_t ev_up = nullptr;       // full upward pass done (fork)
-    cudaEvent_t ev_act = nullptr;      // prologue done (join)
-    cudaEvent_t ev_ready = nullptr;    // forked pass's expansions ready (Phi_u on the near stream waits)
-    cudaEvent_t ev_sparse = nullptr;   // forked sparse pass done (join)
-    bool count_pending = false, prologue_pending = false, sparse_forked = false;
-    void *Lt = nullptr;      // [9][NU_MAX][nc] full local expansions at the active cells (FP64)
-    void *Lu = nullptr;      // solute-only local expansions of every cell of levels 0..LD (class layout), T
-    double *part = nullptr;  // [NU_MAX][n_il][nc] their M2L terms, one per offset
+    cudaEvent_t ev_sort = nullptr;     // sort done (fork)
+    cudaEvent_t ev_up = nullptr;       // full upward pass done
+    cudaEvent_t ev_ready = nullptr;    // expansions ready (Phi_u on the near stream waits)
+    cudaEvent_t ev_done = nullptr;     // everything on the side stream done (join)
+    bool count_pending = false, forked = false, act_done = false;
+    double *Lt = nullptr;    // [9][NU_MAX][nc] the solvent's M2L sums at the active cells (FP64)
+    void *Lu = nullptr;      // solute-only local expansions of every cell of levels 1..ld (class layout), T
+    double *part = nullptr;  // [level][NU_MAX][act_groups][nc] partial sums of Lt
 };
 
 inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -68,146 +79,116 @@ __device__ inline void cell_xyz(int64_t lin, int n, int &x, int &y, int &z)
     z = (int)(lin / ((int64_t)n * n));
 }
 
-// collect the sorted slots of the solute charges (list order is irrelevant:
-// the active cells are sorted afterwards); list[NU_MAX] counts all of them
-__global__ void k_sol_list(int64_t N, const uint8_t *__restrict__ sol, int *__restrict__ list)
+// One block of 64 threads: the solute slots in order, then per level the active cells -- the leaves of the solute
+// charges and their ancestors, each list sorted by linear index and without repeats.  Every thread ranks its own
+// key among the at most 64 (a serial sort by one thread took 7 us with one charge and far more with 64).
+__global__ void __launch_bounds__(NU_MAX) k_sol_cells(int d, const int *__restrict__ count, const int *__restrict__ list,
+                                                      const int *__restrict__ sleaf, int *__restrict__ slots,
+                                                      int *__restrict__ cells, int *__restrict__ ncells)
 {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= N || !sol[s]) return;
-    int idx = atomicAdd(&list[NU_MAX], 1);
-    if (idx < NU_MAX) list[idx] = (int)s;
-}
-
-// active cells per level: leaves of the solute charges and their ancestors,
-// each list sorted by linear index and without repeats (one thread)
-__global__ void k_sol_cells(int d, const int *__restrict__ list, const int *__restrict__ sleaf, int *__restrict__ cells,
-                            int *__restrict__ ncells)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int n = list[NU_MAX];
+    __shared__ int key[NU_MAX], first[NU_MAX];
+    const int i = threadIdx.x;
+    int n = *count;
     if (n > NU_MAX) n = 0;  // the dense pass runs instead: no active cells
-    int cur[NU_MAX], cnt = 0;
-    for (int i = 0; i < n; ++i) cur[cnt++] = sleaf[list[i]];
-    for (int l = d; l >= 0; --l) {
-        // sort + unique
-        for (int i = 1; i < cnt; ++i) {
-            int v = cur[i], j = i - 1;
-            while (j >= 0 && cur[j] > v) {
-                cur[j + 1] = cur[j];
-                --j;
-            }
-            cur[j + 1] = v;
+    key[i] = i < n ? list[i] : 0;
+    __syncthreads();
+    int x = 0, y = 0, z = 0;
+    if (i < n) {
+        int r = 0;
+        for (int j = 0; j < n; ++j) r += key[j] < key[i];
+        slots[r] = key[i];
+        cell_xyz(sleaf[key[i]], 1 << d, x, y, z);
+    }
+    for (int l = d; l >= 1; --l) {
+        const int nl = 1 << l;
+        __syncthreads();
+        const int k = x + nl * (y + nl * z);
+        key[i] = k;
+        __syncthreads();
+        int f = i < n;
+        for (int j = 0; j < i && f; ++j) f = key[j] != k;
+        first[i] = f;
+        const int cnt = __syncthreads_count(f);
+        if (f) {
+            int r = 0;
+            for (int j = 0; j < n; ++j) r += first[j] && key[j] < k;
+            cells[l * NU_MAX + r] = k;
         }
-        int u = 0;
-        for (int i = 0; i < cnt; ++i)
-            if (u == 0 || cur[i] != cur[u - 1]) cur[u++] = cur[i];
-        cnt = u;
-        for (int i = 0; i < cnt; ++i) cells[l * NU_MAX + i] = cur[i];
-        ncells[l] = cnt;
-        if (l == 0) break;
-        int nl = 1 << l;
-        for (int i = 0; i < cnt; ++i) {
-            int x, y, z;
-            cell_xyz(cur[i], nl, x, y, z);
-            cur[i] = (x >> 1) + (nl >> 1) * ((y >> 1) + (nl >> 1) * (z >> 1));
+        if (i == 0) {
+            ncells[l] = cnt;
+            ncells[16 + l] = 0;
         }
+        x >>= 1;
+        y >>= 1;
+        z >>= 1;
     }
 }
 
-// P2M of the solute charges of active leaf blockIdx.x; thread m = column m
+// reciprocals of the harmonics' recurrences, once per block: -1/(2m) and 1/((n+m)(n-m))
 template <typename T>
-__global__ void k_sol_p2m(int p, int d, const int *__restrict__ cells, const int *__restrict__ ncells,
-                          const int *__restrict__ start, const Particle<T> *__restrict__ spu, T inv_h, T *__restrict__ MU)
+__device__ __forceinline__ void recurrence_tables(int p, T *s_half, T *s_inv)
 {
-    int i = blockIdx.x;
-    if (i >= ncells[d]) return;
-    int m = threadIdx.x;
+    for (int e = threadIdx.x; e < (p + 1) * (p + 1); e += blockDim.x) {
+        const int n = e / (p + 1), mm = e % (p + 1);
+        s_inv[e] = n > mm ? T(1) / T((n + mm) * (n - mm)) : T(0);
+        if (e <= p) s_half[e] = e > 0 ? T(-0.5) / T(e) : T(0);
+    }
+}
+
+// Solute moments of active cell blockIdx.x of level blockIdx.y + 1 about the cell's centre; thread m = column m
+template <typename T>
+__global__ void k_sol_p2m(int p, int d, T h, const int *__restrict__ count, const int *__restrict__ slots,
+                          const int *__restrict__ sleaf, const int *__restrict__ cells, const int *__restrict__ ncells,
+                          const Particle<T> *__restrict__ sp, T *__restrict__ MU)
+{
+    __shared__ T s_half[P_MAX + 1], s_inv[(P_MAX + 1) * (P_MAX + 1)];
+    const int i = blockIdx.x, l = blockIdx.y + 1;
+    if (i >= ncells[l]) return;
+    recurrence_tables<T>(p, s_half, s_inv);
+    __syncthreads();
+    const int m = threadIdx.x;
     if (m > p) return;
-    int nc = ncoef(p);
-    int leaf = cells[d * NU_MAX + i];
+    const int nc = ncoef(p), nu = *count, sh = d - l;
+    int cx, cy, cz;
+    cell_xyz(cells[l * NU_MAX + i], 1 << l, cx, cy, cz);
+    const T inv_h = T(1) / (h * T(1 << sh));
     T accr[P_MAX + 1], acci[P_MAX + 1];
     for (int n = 0; n <= p; ++n) accr[n] = acci[n] = 0;
-    for (int s = start[leaf]; s < start[leaf + 1]; ++s) {
-        Particle<T> pt = spu[s];
-        if (pt.q == T(0)) continue;
-        T vx = -pt.x * inv_h, vy = -pt.y * inv_h, vz = -pt.z * inv_h;
-        T r2 = vx * vx + vy * vy + vz * vz;
-        T dre = 1, dim = 0;
+    for (int u = 0; u < nu; ++u) {
+        const int s = slots[u];
+        int x, y, z;
+        cell_xyz(sleaf[s], 1 << d, x, y, z);
+        if ((x >> sh) != cx || (y >> sh) != cy || (z >> sh) != cz) continue;
+        const Particle<T> pt = sp[s];
+        // the leaf's centre relative to the cell's, in leaf units
+        const T ox = T((x - (cx << sh)) + 0.5) - T(0.5) * T(1 << sh), oy = T((y - (cy << sh)) + 0.5) - T(0.5) * T(1 << sh),
+                oz = T((z - (cz << sh)) + 0.5) - T(0.5) * T(1 << sh);
+        const T vx = -(pt.x + ox * h) * inv_h, vy = -(pt.y + oy * h) * inv_h, vz = -(pt.z + oz * h) * inv_h;
+        const T r2 = vx * vx + vy * vy + vz * vz;
+        T dre = pt.q, dim = 0;
         for (int k = 1; k <= m; ++k) {
-            T sc = T(-0.5) / T(k);
-            T nre = sc * (vx * dre - vy * dim), nim = sc * (vx * dim + vy * dre);
+            const T nre = s_half[k] * (vx * dre - vy * dim), nim = s_half[k] * (vx * dim + vy * dre);
             dre = nre;
             dim = nim;
         }
         T p2re = 0, p2im = 0, p1re = dre, p1im = dim;
-        accr[m] += pt.q * dre;
-        acci[m] += pt.q * dim;
+        accr[m] += dre;
+        acci[m] += dim;
         for (int n = m + 1; n <= p; ++n) {
-            T a = T(2 * n - 1) * vz, inv = T(1) / T((n + m) * (n - m));
-            T cr = (a * p1re - r2 * p2re) * inv, ci = (a * p1im - r2 * p2im) * inv;
-            accr[n] += pt.q * cr;
-            acci[n] += pt.q * ci;
+            const T a = T(2 * n - 1) * vz, inv = s_inv[n * (p + 1) + m];
+            const T cr = (a * p1re - r2 * p2re) * inv, ci = (a * p1im - r2 * p2im) * inv;
+            accr[n] += cr;
+            acci[n] += ci;
             p2re = p1re;
             p2im = p1im;
             p1re = cr;
             p1im = ci;
         }
     }
-    T *out = MU + ((size_t)d * NU_MAX + i) * nc;
+    T *out = MU + ((size_t)l * NU_MAX + i) * nc;
     for (int n = m; n <= p; ++n) {
         out[cre(n, m)] = accr[n];
         if (m > 0) out[cim(n, m)] = acci[n];
-    }
-}
-
-// M2M from the active children at level l+1 into active cell blockIdx.x of
-// level l.  One warp (blockDim 32) per output (n, m) = blockIdx.y; lane = the
-// child degree k, then a fixed shuffle tree.
-template <typename T>
-__global__ void k_sol_m2m(int p, int l, const int *__restrict__ cells, const int *__restrict__ ncells,
-                          const T *__restrict__ Rw, T *__restrict__ MU)
-{
-    const int i = blockIdx.x;
-    if (i >= ncells[l]) return;
-    const int nc = ncoef(p);
-    const int nl = 1 << l;
-    const int kk = threadIdx.x;
-    int px, py, pz;
-    cell_xyz(cells[l * NU_MAX + i], nl, px, py, pz);
-    const int t = blockIdx.y;
-    int n = 0;
-    while (tri(n + 1, 0) <= t) ++n;
-    const int m = t - tri(n, 0);
-    T accr = 0, acci = 0;
-    if (kk <= n) {
-        const int dn = n - kk;
-        const T sgn = (dn & 1) ? T(-1) : T(1);
-        T scale = 1;
-        for (int s = 0; s < kk; ++s) scale *= T(0.5);
-        for (int k = 0; k < ncells[l + 1]; ++k) {
-            int cx, cy, cz;
-            cell_xyz(cells[(l + 1) * NU_MAX + k], 2 * nl, cx, cy, cz);
-            if ((cx >> 1) != px || (cy >> 1) != py || (cz >> 1) != pz) continue;
-            const int oct = (cx & 1) | ((cy & 1) << 1) | ((cz & 1) << 2);
-            const T *Mch = MU + ((size_t)(l + 1) * NU_MAX + k) * nc;
-            const T *R = Rw + oct * nc;
-            for (int ll = -kk; ll <= kk; ++ll) {
-                const int dm = m - ll;
-                if (dm < -dn || dm > dn) continue;
-                Cx<T> pr = cmul(coef(R, dn, dm), coef(Mch, kk, ll));
-                accr += sgn * scale * pr.re;
-                acci += sgn * scale * pr.im;
-            }
-        }
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        accr += __shfl_xor_sync(0xffffffffu, accr, off);
-        acci += __shfl_xor_sync(0xffffffffu, acci, off);
-    }
-    if (kk == 0) {
-        T *out = MU + ((size_t)l * NU_MAX + i) * nc;
-        out[cre(n, m)] = accr;
-        if (m > 0) out[cim(n, m)] = acci;
     }
 }
 
@@ -229,62 +210,62 @@ __device__ inline int wrap_delta(int d, int n)  // representative of d mod n in 
     return d;
 }
 
-// offset of level l in the dense arrays of levels 0..LD (8^0 + ... + 8^(l-1) cells before it)
-__host__ __device__ inline int64_t dense_off(int l, int nc) { return (((int64_t)1 << (3 * l)) - 1) / 7 * nc; }
+// offset of level l >= 1 in the dense arrays of levels 1..ld (8^1 + ... + 8^(l-1) cells before it)
+__host__ __device__ inline int64_t dense_off(int l, int nc) { return ((((int64_t)1 << (3 * l)) - 1) / 7 - 1) * nc; }
 
-// solute-only expansion of the root: the lattice operator of Eq. 12 applied to the root's solute moments
-// (zero without solute charges)
-template <typename T>
-__global__ void k_sol_lattice(int p, const int *__restrict__ ncells, const double *__restrict__ T0,
-                              const T *__restrict__ MU, T *__restrict__ Lu0)
+// offset of fine level l in the target map (levels l0 + 1 .. l - 1 before it)
+__host__ __device__ inline int64_t map_off(int l, int l0)
 {
-    const int nc = ncoef(p);
-    const bool any = ncells[0] > 0;
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        double acc = 0;
-        if (any)
-            for (int k = 0; k < nc; ++k) acc += T0[(size_t)k * nc + j] * (double)MU[k];
-        Lu0[j] = (T)acc;
-    }
+    return ((((int64_t)1 << (3 * l)) - 1) / 7) - ((((int64_t)1 << (3 * (l0 + 1))) - 1) / 7);
 }
 
-// M2L terms of the dense levels 1..LD, one block per (active source a, offset d of the window
-// [-2ws-1, 2ws+1]^3): part[a][d] = T(d) . MU_a (Eq. Lcoeffdef) when the source lies in the interaction
+// M2L terms of the dense levels 2..ld, one work item per (level, active source a, offset d of the window
+// [-2ws-1, 2ws+1]^3): part[l - 2][a][d] = T(d) . MU_a (Eq. Lcoeffdef) when the source lies in the interaction
 // list of the target t = s_a - d (wrapped).  At coarse levels several offsets reach the same target (its
 // periodic images): each has its own term.
 template <typename T>
-__global__ void k_sol_dense_m2l(int p, int l, int ws, const int *__restrict__ cells, const int *__restrict__ ncells,
+__global__ void k_sol_dense_m2l(int p, int ld, int ws, const int *__restrict__ cells, const int *__restrict__ ncells,
                                 const T *__restrict__ Top, const T *__restrict__ MU, T *__restrict__ part)
 {
-    const int a = blockIdx.x, b = blockIdx.y;
-    if (a >= ncells[l]) return;
-    const int nc = ncoef(p), n = 1 << l, h = 2 * ws + 1, side = 2 * h + 1;
-    const int dx = b % side - h, dy = (b / side) % side - h, dz = b / (side * side) - h;
-    int sx, sy, sz;
-    cell_xyz(cells[l * NU_MAX + a], n, sx, sy, sz);
-    const int tx = (sx - dx + 4 * n) & (n - 1), ty = (sy - dy + 4 * n) & (n - 1), tz = (sz - dz + 4 * n) & (n - 1);
-    if (!in_il(dx, dy, dz, tx, ty, tz, ws)) return;
-    const T *Tp = Top + (size_t)off_slot(dx, dy, dz, ws) * nc * nc;
-    const T *Ms = MU + ((size_t)l * NU_MAX + a) * nc;
-    T *out = part + ((size_t)a * side * side * side + b) * nc;
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        T acc = 0;
-        for (int k = 0; k < nc; ++k) acc += Tp[(size_t)k * nc + j] * Ms[k];
-        out[j] = acc;
+    const int nc = ncoef(p), h = 2 * ws + 1, side = 2 * h + 1, W = side * side * side;
+    int total = 0;
+    for (int l = 2; l <= ld; ++l) total += ncells[l] * W;
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        int l = 2, r = it;
+        while (r >= ncells[l] * W) r -= ncells[l++] * W;
+        const int a = r / W, b = r - a * W, n = 1 << l;
+        const int dx = b % side - h, dy = (b / side) % side - h, dz = b / (side * side) - h;
+        int sx, sy, sz;
+        cell_xyz(cells[l * NU_MAX + a], n, sx, sy, sz);
+        const int tx = (sx - dx + 4 * n) & (n - 1), ty = (sy - dy + 4 * n) & (n - 1), tz = (sz - dz + 4 * n) & (n - 1);
+        if (!in_il(dx, dy, dz, tx, ty, tz, ws)) continue;
+        const T *Tp = Top + (size_t)off_slot(dx, dy, dz, ws) * nc * nc;
+        const T *Ms = MU + ((size_t)l * NU_MAX + a) * nc;
+        T *out = part + (((size_t)(l - 2) * NU_MAX + a) * W + b) * nc;
+        for (int j = threadIdx.x; j < nc; j += blockDim.x) {
+            T a0 = 0, a1 = 0;
+            int k = 0;
+            for (; k + 1 < nc; k += 2) {
+                a0 += Tp[(size_t)k * nc + j] * Ms[k];
+                a1 += Tp[(size_t)(k + 1) * nc + j] * Ms[k + 1];
+            }
+            if (k < nc) a0 += Tp[(size_t)k * nc + j] * Ms[k];
+            out[j] = a0 + a1;
+        }
     }
 }
 
-// dense level 1 <= l <= LD of the solute-only pass, every target cell (one block each, thread j =
-// coefficient j): the L2L of the parent's expansion (Eq. L2L: Lhat_k^m = 2^-(k+1) sum_{n >= k}
-// Lhat_n^q R_{n-k}^{q-m}(w_c)) plus the M2L terms of k_sol_dense_m2l whose target this is, summed in
-// the window's offset order (the sums do not depend on the schedule)
+// dense level 2 <= l <= ld of the solute-only pass, every target cell (one block each, thread j =
+// coefficient j): the L2L of the parent's expansion (the octant's operator, transposed [nc][8 nc]) plus the M2L
+// terms of k_sol_dense_m2l whose target this is, summed in the window's offset order (the sums do not depend on
+// the schedule)
 template <typename T>
 __global__ void k_sol_dense(int p, int l, int ws, const int *__restrict__ cells, const int *__restrict__ ncells,
-                            const T *__restrict__ part, const T *__restrict__ Rw, const T *__restrict__ Lpar,
+                            const T *__restrict__ part, const T *__restrict__ l2lT, const T *__restrict__ Lpar,
                             T *__restrict__ Lout)
 {
     __shared__ short hit[(4 * WS_MAX + 3) * (4 * WS_MAX + 3) * (4 * WS_MAX + 3)];
-    __shared__ T sL[NC_MAX], sR[NC_MAX];
+    __shared__ T sL[NC_MAX];
     const int nc = ncoef(p), n = 1 << l, h = 2 * ws + 1, side = 2 * h + 1, W = side * side * side;
     int tx, ty, tz;
     cell_xyz(blockIdx.x, n, tx, ty, tz);
@@ -292,10 +273,7 @@ __global__ void k_sol_dense(int p, int l, int ws, const int *__restrict__ cells,
     const int *act = cells + l * NU_MAX;
     const int oct = (tx & 1) | ((ty & 1) << 1) | ((tz & 1) << 2);
     const T *Lp = Lpar + cell_index(l - 1, tx >> 1, ty >> 1, tz >> 1) * nc;
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        sL[j] = Lp[j];
-        sR[j] = Rw[oct * nc + j];
-    }
+    for (int j = threadIdx.x; j < nc; j += blockDim.x) sL[j] = Lp[j];
     for (int b = threadIdx.x; b < W; b += blockDim.x) {
         const int dx = b % side - h, dy = (b / side) % side - h, dz = b / (side * side) - h;
         int a = -1;
@@ -313,254 +291,233 @@ __global__ void k_sol_dense(int p, int l, int ws, const int *__restrict__ cells,
         hit[b] = (short)a;
     }
     __syncthreads();
+    const T *pl = part + (size_t)(l - 2) * NU_MAX * W * nc;
     for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        // output coefficient j = (k, m, real or imaginary part)
+        T a0 = 0, a1 = 0;
         int k = 0;
-        while ((k + 1) * (k + 1) <= j) ++k;
-        const int r = j - k * k;
-        const int m = (r + 1) >> 1;
-        const bool imag = r > 0 && (r & 1) == 0;
-        T accr = 0, acci = 0;
-        for (int nn = k; nn <= p; ++nn) {
-            const int dn = nn - k;
-            for (int q = m - dn; q <= m + dn; ++q) {
-                if (q < -nn || q > nn) continue;
-                Cx<T> pr = cmul(coef(sL, nn, q), coef(sR, dn, q - m));
-                accr += pr.re;
-                acci += pr.im;
-            }
+        for (; k + 1 < nc; k += 2) {
+            a0 += l2lT[(size_t)k * (8 * nc) + oct * nc + j] * sL[k];
+            a1 += l2lT[(size_t)(k + 1) * (8 * nc) + oct * nc + j] * sL[k + 1];
         }
-        T scale = 1;
-        for (int e = 0; e <= k; ++e) scale *= T(0.5);
-        T acc = scale * (imag ? acci : accr);
+        if (k < nc) a0 += l2lT[(size_t)k * (8 * nc) + oct * nc + j] * sL[k];
+        T acc = a0 + a1;
         for (int b = 0; b < W; ++b) {
             const int a = hit[b];
-            if (a >= 0) acc += part[((size_t)a * W + b) * nc + j];
+            if (a >= 0) acc += pl[((size_t)a * W + b) * nc + j];
         }
         Lout[cell_index(l, tx, ty, tz) * nc + j] = acc;
     }
 }
 
-// mark the targets of active source blockIdx.x at level l (threads over the candidate offsets)
-__global__ void k_sol_mark(int l, int ws, const int *__restrict__ cells, const int *__restrict__ ncells,
-                           int *__restrict__ flags)
+// the targets of active source blockIdx.x at fine level ld + 1 + blockIdx.y (threads over the candidate offsets):
+// the first source to reach a cell gives it a place in the level's target list
+__global__ void k_sol_mark(int ld, int ws, int mt, const int *__restrict__ cells, int *__restrict__ ncells,
+                           int *__restrict__ map, int *__restrict__ tlist)
 {
-    int i = blockIdx.x;
+    const int i = blockIdx.x, l = ld + 1 + blockIdx.y;
     if (i >= ncells[l]) return;
     const int side = off_side(ws), h = 2 * ws + 1;
-    int n = 1 << l;
+    const int n = 1 << l;
+    int *mp = map + map_off(l, ld);
     int sx, sy, sz;
     cell_xyz(cells[l * NU_MAX + i], n, sx, sy, sz);
     for (int o = threadIdx.x; o < side * side * side; o += blockDim.x) {
-        int dx = o % side - h, dy = (o / side) % side - h, dz = o / (side * side) - h;
-        int tx = (sx - dx + 2 * n) & (n - 1), ty = (sy - dy + 2 * n) & (n - 1), tz = (sz - dz + 2 * n) & (n - 1);
-        if (in_il(dx, dy, dz, tx, ty, tz, ws)) flags[tx + n * (ty + n * tz)] = 1;
+        const int dx = o % side - h, dy = (o / side) % side - h, dz = o / (side * side) - h;
+        const int tx = (sx - dx + 2 * n) & (n - 1), ty = (sy - dy + 2 * n) & (n - 1), tz = (sz - dz + 2 * n) & (n - 1);
+        if (!in_il(dx, dy, dz, tx, ty, tz, ws)) continue;
+        const int t = tx + n * (ty + n * tz);
+        if (atomicCAS(mp + t, 0, -1) != 0) continue;
+        const int k = atomicAdd(ncells + 16 + l, 1);  // below mt: n_il targets per source
+        tlist[(size_t)l * mt + k] = t;
+        mp[t] = k + 1;
     }
 }
 
-__global__ void k_sol_compact(int64_t n, int mt, const int *__restrict__ flags, const int *__restrict__ pos,
-                              int *__restrict__ tlist)
-{
-    int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (c < n && flags[c]) {
-        int k = pos[c];
-        if (k < mt) tlist[k] = (int)c;
-    }
-}
-
-// contribution of every active source to target tlist[blockIdx.x] (Eq. Lcoeffdef)
+// contribution of every active source to the targets of the fine levels (Eq. Lcoeffdef), one target per work item,
+// the sources in the order of their list
 template <typename T>
-__global__ void k_sol_m2l(int p, int l, int ws, const int *__restrict__ cells, const int *__restrict__ ncells,
-                          const int *__restrict__ tlist, const int *__restrict__ tcount, const T *__restrict__ Top,
-                          const T *__restrict__ MU, T *__restrict__ contrib)
+__global__ void k_sol_m2l(int p, int d, int ld, int ws, const int *__restrict__ cells, const int *__restrict__ ncells,
+                          const int *__restrict__ tlist, const T *__restrict__ Top, const T *__restrict__ MU,
+                          T *__restrict__ contrib)
 {
-    int b = blockIdx.x;
-    const int mt = max_tgt(ws);
-    int cnt = *tcount;
-    if (cnt > mt) cnt = mt;
-    if (b >= cnt) return;
-    int nc = ncoef(p);
-    int n = 1 << l;
-    int tx, ty, tz;
-    cell_xyz(tlist[b], n, tx, ty, tz);
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        T acc = 0;
-        for (int s = 0; s < ncells[l]; ++s) {
-            int sx, sy, sz;
-            cell_xyz(cells[l * NU_MAX + s], n, sx, sy, sz);
-            int dx = wrap_delta(sx - tx, n), dy = wrap_delta(sy - ty, n), dz = wrap_delta(sz - tz, n);
-            if (!in_il(dx, dy, dz, tx, ty, tz, ws)) continue;
-            const T *Tp = Top + (size_t)off_slot(dx, dy, dz, ws) * nc * nc + j;
-            const T *Ms = MU + ((size_t)l * NU_MAX + s) * nc;
-            for (int k = 0; k < nc; ++k) acc += Tp[(size_t)k * nc] * Ms[k];
-        }
-        contrib[((size_t)l * mt + b) * nc + j] = acc;
-    }
-}
-
-// ---- full-field potential at the solute charges (the A of Eq. FMMcalc), as
-// the oracle evaluates one sampled charge: M2L over the interaction list of
-// each active cell from the full pass's moments (CUDA cores, no operand
-// splitting), then the level-0 lattice expansion shifted down the active
-// ancestors by L2L, then L2P.  The few solute charges cannot average out the
-// split-operand rounding of the tensor-core M2L, so A is taken from here.
-
-// FP64 throughout, on the solvent moments M - M_u (the field of the solvent
-// at the solute charges): Lt[0][0] = T0 . (M(0) - M_u(0))
-template <typename T>
-__global__ void k_act_lattice(int p, const int *__restrict__ ncells, const double *__restrict__ T0,
-                              const T *__restrict__ M0, const T *__restrict__ MU0, double *__restrict__ Lt)
-{
-    if (ncells[0] == 0) return;
-    int nc = ncoef(p);
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        double acc = 0;
-        for (int k = 0; k < nc; ++k) acc += T0[(size_t)k * nc + j] * ((double)M0[k] - (double)MU0[k]);
-        Lt[j] = acc;
-    }
-}
-
-// part[i][o] = the M2L term of the o-th interaction-list offset of active cell
-// i at level l (one block per (cell, offset))
-template <typename T>
-__global__ void k_act_m2l(int p, int l, int ws, const int *__restrict__ cells, const int *__restrict__ ncells,
-                          const double *__restrict__ Top, const T *__restrict__ M, const T *__restrict__ MU,
-                          double *__restrict__ part)
-{
-    int i = blockIdx.x, o = blockIdx.y;
-    if (i >= ncells[l]) return;
-    int nc = ncoef(p);
-    int n = 1 << l;
-    int tx, ty, tz;
-    cell_xyz(cells[l * NU_MAX + i], n, tx, ty, tz);
-    int cx = tx & 1, cy = ty & 1, cz = tz & 1;
-    int dx = 0, dy = 0, dz = 0, c = -1;
-    for (int z = -2 * ws - cz; z <= 2 * ws + 1 - cz && c < o; ++z)
-        for (int y = -2 * ws - cy; y <= 2 * ws + 1 - cy && c < o; ++y)
-            for (int x = -2 * ws - cx; x <= 2 * ws + 1 - cx && c < o; ++x) {
-                if (x >= -ws && x <= ws && y >= -ws && y <= ws && z >= -ws && z <= ws) continue;
-                if (++c == o) {
-                    dx = x;
-                    dy = y;
-                    dz = z;
+    const int nc = ncoef(p), mt = max_tgt(ws);
+    int total = 0;
+    for (int l = ld + 1; l <= d; ++l) total += ncells[16 + l];
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        int l = ld + 1, b = it;
+        while (b >= ncells[16 + l]) b -= ncells[16 + l++];
+        const int n = 1 << l;
+        int tx, ty, tz;
+        cell_xyz(tlist[(size_t)l * mt + b], n, tx, ty, tz);
+        for (int j = threadIdx.x; j < nc; j += blockDim.x) {
+            T a0 = 0, a1 = 0;
+            for (int s = 0; s < ncells[l]; ++s) {
+                int sx, sy, sz;
+                cell_xyz(cells[l * NU_MAX + s], n, sx, sy, sz);
+                const int dx = wrap_delta(sx - tx, n), dy = wrap_delta(sy - ty, n), dz = wrap_delta(sz - tz, n);
+                if (!in_il(dx, dy, dz, tx, ty, tz, ws)) continue;
+                const T *Tp = Top + (size_t)off_slot(dx, dy, dz, ws) * nc * nc + j;
+                const T *Ms = MU + ((size_t)l * NU_MAX + s) * nc;
+                int k = 0;
+                for (; k + 1 < nc; k += 2) {
+                    a0 += Tp[(size_t)k * nc] * Ms[k];
+                    a1 += Tp[(size_t)(k + 1) * nc] * Ms[k + 1];
                 }
+                if (k < nc) a0 += Tp[(size_t)k * nc] * Ms[k];
             }
-    int sx = ((tx + dx) % n + n) % n, sy = ((ty + dy) % n + n) % n, sz = ((tz + dz) % n + n) % n;
-    const T *Ms = M + cell_index(l, sx, sy, sz) * nc;
-    // the solute part of this source, if it is an active cell
-    const T *Mu = nullptr;
-    int slin = sx + n * (sy + n * sz);
-    for (int k = 0; k < ncells[l]; ++k)
-        if (cells[l * NU_MAX + k] == slin) Mu = MU + ((size_t)l * NU_MAX + k) * nc;
-    const double *Tp = Top + (size_t)off_slot(dx, dy, dz, ws) * nc * nc;
-    const int nil = n_il(ws);
-    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-        double acc = 0;
-        if (Mu)
-            for (int k = 0; k < nc; ++k) acc += Tp[(size_t)k * nc + j] * ((double)Ms[k] - (double)Mu[k]);
-        else
-            for (int k = 0; k < nc; ++k) acc += Tp[(size_t)k * nc + j] * (double)Ms[k];
-        part[((size_t)i * nil + o) * nc + j] = acc;
+            contrib[((size_t)l * mt + b) * nc + j] = a0 + a1;
+        }
     }
 }
 
-// Lt[l][i] = sum of the n_il terms: one warp per (active cell, coefficient j),
-// lanes take every 32nd offset, then a fixed shuffle tree (deterministic)
-__global__ void k_act_sum(int p, int l, int nil, const int *__restrict__ ncells, const double *__restrict__ part,
+// ---- full-field potential at the solute charges (the A of Eq. FMMcalc): M2L over the interaction list of
+// each active cell from the full pass's moments in FP64 (CUDA cores, no operand splitting; level 1 and above by
+// the FP64 top operator), on the solvent moments M - M_u, and each level's sum evaluated at the charge itself.
+// The few solute charges cannot average out the split-operand rounding of the tensor-core M2L, so A is taken
+// from here.
+
+// part[l][i][g] = the M2L terms of ACT_OFFS offsets of active cell i at level l >= 2, one work item each.  Bound by
+// the FP64 pipe (2 operations per SM and clock): the moments are converted once per block, not per thread.
+template <typename T>
+__global__ void k_act_m2l(int p, int d, int ws, const int *__restrict__ il, const int *__restrict__ cells,
+                          const int *__restrict__ ncells, const double *__restrict__ Top, const T *const *__restrict__ Mlev,
+                          const T *__restrict__ MU, double *__restrict__ part)
+{
+    __shared__ double sM[NC_MAX];
+    const int nc = ncoef(p), nil = n_il(ws), ng = act_groups(ws);
+    int total = 0;
+    for (int l = 2; l <= d; ++l) total += ncells[l] * ng;
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        int l = 2, r = it;
+        while (r >= ncells[l] * ng) r -= ncells[l++] * ng;
+        const int i = r / ng, g = r - i * ng, n = 1 << l;
+        const T *M = Mlev[l];
+        int tx, ty, tz;
+        cell_xyz(cells[l * NU_MAX + i], n, tx, ty, tz);
+        const int cls = (tx & 1) | ((ty & 1) << 1) | ((tz & 1) << 2);
+        double acc[(NC_MAX + 191) / 192] = {};  // coefficients threadIdx.x, + blockDim.x, ...
+        for (int o = g * ACT_OFFS; o < nil && o < (g + 1) * ACT_OFFS; ++o) {
+            int dx, dy, dz;
+            il_unpack(il[cls * nil + o], dx, dy, dz);
+            const int sx = (tx + dx + 4 * n) & (n - 1), sy = (ty + dy + 4 * n) & (n - 1), sz = (tz + dz + 4 * n) & (n - 1);
+            const T *Ms = M + cell_index(l, sx, sy, sz) * nc;
+            const T *Mu = nullptr;  // the solute part of this source, if it is an active cell
+            const int slin = sx + n * (sy + n * sz);
+            for (int k = 0; k < ncells[l]; ++k)
+                if (cells[l * NU_MAX + k] == slin) Mu = MU + ((size_t)l * NU_MAX + k) * nc;
+            __syncthreads();
+            for (int k = threadIdx.x; k < nc; k += blockDim.x) sM[k] = Mu ? (double)Ms[k] - (double)Mu[k] : (double)Ms[k];
+            __syncthreads();
+            const double *Tp = Top + (size_t)off_slot(dx, dy, dz, ws) * nc * nc;
+#pragma unroll
+            for (int q = 0; q < (NC_MAX + 191) / 192; ++q) {
+                const int j = threadIdx.x + q * blockDim.x;
+                if (j >= nc) break;
+                double a0 = 0, a1 = 0;
+                int k = 0;
+                for (; k + 1 < nc; k += 2) {
+                    a0 += Tp[(size_t)k * nc + j] * sM[k];
+                    a1 += Tp[(size_t)(k + 1) * nc + j] * sM[k + 1];
+                }
+                if (k < nc) a0 += Tp[(size_t)k * nc + j] * sM[k];
+                acc[q] += a0 + a1;
+            }
+        }
+        double *out = part + ((size_t)((l - 2) * NU_MAX + i) * ng + g) * nc;
+#pragma unroll
+        for (int q = 0; q < (NC_MAX + 191) / 192; ++q) {
+            const int j = threadIdx.x + q * blockDim.x;
+            if (j < nc) out[j] = acc[q];
+        }
+    }
+}
+
+// Lt[l][i] = sum of the groups' terms, level 2 + blockIdx.z: one warp per (active cell, coefficient j), lanes take
+// every 32nd group, then a fixed shuffle tree (deterministic)
+__global__ void k_act_sum(int p, int ng, const int *__restrict__ ncells, const double *__restrict__ part,
                           double *__restrict__ Lt)
 {
-    const int i = blockIdx.x;
-    if (i >= ncells[l]) return;
-    const int nc = ncoef(p);
+    const int nc = ncoef(p), l = 2 + blockIdx.z;
     const int j = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (j >= nc) return;
-    double s = 0;
-    for (int o = lane; o < nil; o += 32) s += part[((size_t)i * nil + o) * nc + j];
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) Lt[((size_t)l * NU_MAX + i) * nc + j] = s;
+    for (int i = blockIdx.x; i < ncells[l]; i += gridDim.x) {
+        double s = 0;
+        for (int o = lane; o < ng; o += 32) s += part[((size_t)((l - 2) * NU_MAX + i) * ng + o) * nc + j];
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) Lt[((size_t)l * NU_MAX + i) * nc + j] = s;
+    }
 }
 
-// Lt[l][i] += L2L of the parent's full expansion (Lt[l-1] or, at level 1, the
-// lattice result L0): Lhat_k^m += sum_{n >= k} Lhat_n^q R_{n-k}^{q-m}(w_c) 2^{-(k+1)}.
-// One warp (blockDim 32) per output (k, m) = blockIdx.y; lane = n - k, then a
-// fixed shuffle tree.
-__global__ void k_act_l2l(int p, int l, const int *__restrict__ cells, const int *__restrict__ ncells,
-                          const double *__restrict__ Rw, const double *__restrict__ L0, double *__restrict__ Lt)
+// at solute charge blockIdx.x: phi_ff = (solvent field: every level's Lt at the charge) + phi_u (solute field of
+// the solute-only pass), so that A - B = sum_u q Phi_v holds term by term.  Warp w takes levels w + 1, w + 9, ...,
+// lane m the column m of the harmonics (one thread doing all of it, a division per term, took 66 us); the levels
+// are added in order.
+template <typename T>
+__global__ void __launch_bounds__(256) k_act_l2p(int p, int d, double h, const int *__restrict__ count,
+                                                 const int *__restrict__ slots, const int *__restrict__ cells,
+                                                 const int *__restrict__ ncells, const int *__restrict__ sleaf,
+                                                 const Particle<T> *__restrict__ sp, const double *__restrict__ Lt,
+                                                 const T *__restrict__ phi_u, T *__restrict__ phi)
 {
-    const int i = blockIdx.x;
-    if (i >= ncells[l]) return;
-    const int nc = ncoef(p);
-    const int nl = 1 << l;
-    const int lane = threadIdx.x;
+    __shared__ double s_half[P_MAX + 1], s_inv[(P_MAX + 1) * (P_MAX + 1)], s_lev[9];
+    const int n = *count;
+    if (n > NU_MAX || (int)blockIdx.x >= n) return;
+    recurrence_tables<double>(p, s_half, s_inv);
+    __syncthreads();
+    const int s = slots[blockIdx.x], nc = ncoef(p);
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int x, y, z;
-    cell_xyz(cells[l * NU_MAX + i], nl, x, y, z);
-    const double *Lp = L0;
-    if (l > 1) {
-        const int plin = (x >> 1) + (nl >> 1) * ((y >> 1) + (nl >> 1) * (z >> 1));
-        for (int k = 0; k < ncells[l - 1]; ++k)
-            if (cells[(l - 1) * NU_MAX + k] == plin) Lp = Lt + ((size_t)(l - 1) * NU_MAX + k) * nc;
-    }
-    const double *R = Rw + ((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)) * nc;
-    const int t = blockIdx.y;
-    int k = 0;
-    while (tri(k + 1, 0) <= t) ++k;
-    const int m = t - tri(k, 0);
-    double accr = 0, acci = 0;
-    const int n = k + lane;
-    if (n <= p) {
-        const int dn = n - k;
-        for (int q = -n; q <= n; ++q) {
-            const int dm = q - m;
-            if (dm < -dn || dm > dn) continue;
-            Cx<double> pr = cmul(coef(Lp, n, q), coef(R, dn, dm));
-            accr += pr.re;
-            acci += pr.im;
+    cell_xyz(sleaf[s], 1 << d, x, y, z);
+    const Particle<T> pt = sp[s];
+    for (int l = w + 1; l <= d; l += 8) {
+        const int sh = d - l, nl = 1 << l;
+        const int ax = x >> sh, ay = y >> sh, az = z >> sh, key = ax + nl * (ay + nl * az);
+        int i = 0;
+        while (i < ncells[l] - 1 && cells[l * NU_MAX + i] != key) ++i;
+        const double inv = 1.0 / (h * (double)(1 << sh));
+        const double vx = ((double)pt.x + ((x - (ax << sh)) + 0.5 - 0.5 * (1 << sh)) * h) * inv,
+                     vy = ((double)pt.y + ((y - (ay << sh)) + 0.5 - 0.5 * (1 << sh)) * h) * inv,
+                     vz = ((double)pt.z + ((z - (az << sh)) + 0.5 - 0.5 * (1 << sh)) * h) * inv;
+        const double r2 = vx * vx + vy * vy + vz * vz;
+        const double *Lc = Lt + ((size_t)l * NU_MAX + i) * nc;
+        double pot = 0;
+        if (lane <= p) {
+            const int m = lane;
+            double dre = 1, dim = 0;
+            for (int k = 1; k <= m; ++k) {
+                const double nre = s_half[k] * (vx * dre - vy * dim), nim = s_half[k] * (vx * dim + vy * dre);
+                dre = nre;
+                dim = nim;
+            }
+            double p2re = 0, p2im = 0, rre = dre, rim = dim;
+            for (int k = m; k <= p; ++k) {
+                if (k > m) {
+                    const double a = (2 * k - 1) * vz, iv = s_inv[k * (p + 1) + m];
+                    const double cr = (a * rre - r2 * p2re) * iv, ci = (a * rim - r2 * p2im) * iv;
+                    p2re = rre;
+                    p2im = rim;
+                    rre = cr;
+                    rim = ci;
+                }
+                const Cx<double> L = coef(Lc, k, m);
+                pot += L.re * rre - L.im * rim;
+            }
+            if (m > 0) pot *= 2.0;
         }
+        for (int o = 16; o > 0; o >>= 1) pot += __shfl_xor_sync(0xffffffffu, pot, o);
+        if (lane == 0) s_lev[l] = pot * inv;
     }
-    for (int off = 16; off > 0; off >>= 1) {
-        accr += __shfl_xor_sync(0xffffffffu, accr, off);
-        acci += __shfl_xor_sync(0xffffffffu, acci, off);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = 0;
+        for (int l = 1; l <= d; ++l) v += s_lev[l];
+        phi[s] = (T)(v + (double)phi_u[s]);
     }
-    if (lane == 0) {
-        double scale = 1;
-        for (int s = 0; s <= k; ++s) scale *= 0.5;
-        double *out = Lt + ((size_t)l * NU_MAX + i) * nc;
-        out[cre(k, m)] += scale * accr;
-        if (m > 0) out[cim(k, m)] += scale * acci;
-    }
-}
-
-template <typename T>
-__device__ T l2p_value(int p, const T *__restrict__ Lc, T vx, T vy, T vz, const T *s_half = nullptr,
-                       const T *s_inv = nullptr);
-
-// at each solute charge: phi_ff = (solvent field from Lt) + phi_u (solute field
-// of the solute-only pass), so that A - B = sum_u q Phi_v holds term by term
-template <typename T>
-__global__ void k_act_l2p(int p, int d, double inv_h, const int *__restrict__ list, const int *__restrict__ cells,
-                          const int *__restrict__ ncells, const int *__restrict__ sleaf,
-                          const Particle<T> *__restrict__ sp, const double *__restrict__ Lt,
-                          const T *__restrict__ phi_u, T *__restrict__ phi)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    int n = list[NU_MAX];
-    if (n > NU_MAX) n = NU_MAX;
-    if (k >= n) return;
-    int s = list[k];
-    int leaf = sleaf[s];
-    int i = 0;
-    while (i < ncells[d] && cells[d * NU_MAX + i] != leaf) ++i;
-    if (i >= ncells[d]) return;
-    Particle<T> pt = sp[s];
-    double v = l2p_value<double>(p, Lt + ((size_t)d * NU_MAX + i) * ncoef(p), (double)pt.x * inv_h,
-                                 (double)pt.y * inv_h, (double)pt.z * inv_h) *
-               inv_h;
-    phi[s] = (T)(v + (double)phi_u[s]);
 }
 
 // Phi at (v) from the real-layout local coefficients Lc (scaled), v in cell units;
-// s_half[m] = -1/(2m) and s_inv[n (p+1) + m] = 1/((n+m)(n-m)) when given
+// s_half[m] = -1/(2m) and s_inv[n (p+1) + m] = 1/((n+m)(n-m))
 template <typename T>
 __device__ T l2p_value(int p, const T *__restrict__ Lc, T vx, T vy, T vz, const T *s_half, const T *s_inv)
 {
@@ -568,7 +525,7 @@ __device__ T l2p_value(int p, const T *__restrict__ Lc, T vx, T vy, T vz, const 
     T pot = 0, dre = 1, dim = 0;
     for (int m = 0; m <= p; ++m) {
         if (m > 0) {
-            T sc = s_half ? s_half[m] : T(-0.5) / T(m);
+            T sc = s_half[m];
             T nre = sc * (vx * dre - vy * dim), nim = sc * (vx * dim + vy * dre);
             dre = nre;
             dim = nim;
@@ -577,7 +534,7 @@ __device__ T l2p_value(int p, const T *__restrict__ Lc, T vx, T vy, T vz, const 
         T p2re = 0, p2im = 0, rre = dre, rim = dim;
         for (int n = m; n <= p; ++n) {
             if (n > m) {
-                T a = T(2 * n - 1) * vz, inv = s_inv ? s_inv[n * (p + 1) + m] : T(1) / T((n + m) * (n - m));
+                T a = T(2 * n - 1) * vz, inv = s_inv[n * (p + 1) + m];
                 T cr = (a * rre - r2 * p2re) * inv, ci = (a * rim - r2 * p2im) * inv;
                 p2re = rre;
                 p2im = rim;
@@ -591,19 +548,15 @@ __device__ T l2p_value(int p, const T *__restrict__ Lc, T vx, T vy, T vz, const 
     return pot;
 }
 
-// Phi_u at every charge: level-LD expansion plus the sparse finer-level sums
+// Phi_u at every charge: level-ld expansion plus the sparse finer-level sums
 template <typename T>
-__global__ void k_sol_eval(int p, int d, int mt, int64_t N, T h_leaf, const int *__restrict__ sleaf,
-                           const Particle<T> *__restrict__ sp, const T *__restrict__ Lld, const int *__restrict__ tlist,
-                           const int *__restrict__ tcounts, const T *__restrict__ contrib, T *__restrict__ phi)
+__global__ void k_sol_eval(int p, int d, int ld, int mt, int64_t N, T h_leaf, const int *__restrict__ sleaf,
+                           const Particle<T> *__restrict__ sp, const T *__restrict__ Lld, const int *__restrict__ map,
+                           const T *__restrict__ contrib, T *__restrict__ phi)
 {
     __shared__ T s_half[P_MAX + 1];
     __shared__ T s_inv[(P_MAX + 1) * (P_MAX + 1)];
-    for (int e = threadIdx.x; e < (p + 1) * (p + 1); e += blockDim.x) {
-        const int n = e / (p + 1), mm = e % (p + 1);
-        s_inv[e] = n > mm ? T(1) / T((n + mm) * (n - mm)) : T(0);
-        if (e <= p) s_half[e] = e > 0 ? T(-0.5) / T(e) : T(0);
-    }
+    recurrence_tables<T>(p, s_half, s_inv);
     __syncthreads();
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= N) return;
@@ -614,187 +567,92 @@ __global__ void k_sol_eval(int p, int d, int mt, int64_t N, T h_leaf, const int 
     cell_xyz(leaf, nside, x, y, z);
     Particle<T> pt = sp[s];
     T total = 0;
-    for (int l = LD; l <= d; ++l) {
+    for (int l = ld; l <= d; ++l) {
         int sh = d - l;
         int ax = x >> sh, ay = y >> sh, az = z >> sh;
+        const T *Lc;
+        if (l == ld) Lc = Lld + cell_index(l, ax, ay, az) * nc;
+        else {
+            const int k = map[map_off(l, ld) + ax + (1 << l) * (ay + ((int64_t)az << l))];
+            if (k <= 0) continue;
+            Lc = contrib + ((size_t)l * mt + k - 1) * nc;
+        }
         // centre of the leaf relative to the centre of its level-l ancestor, in leaf units
         T ox = T((x - (ax << sh)) + 0.5) - T(0.5) * T(1 << sh);
         T oy = T((y - (ay << sh)) + 0.5) - T(0.5) * T(1 << sh);
         T oz = T((z - (az << sh)) + 0.5) - T(0.5) * T(1 << sh);
         T inv = T(1) / (h_leaf * T(1 << sh));
         T vx = (pt.x + ox * h_leaf) * inv, vy = (pt.y + oy * h_leaf) * inv, vz = (pt.z + oz * h_leaf) * inv;
-        if (l == LD) {
-            total += l2p_value<T>(p, Lld + cell_index(l, ax, ay, az) * nc, vx, vy, vz, s_half, s_inv) * inv;
-            continue;
-        }
-        int cnt = tcounts[l];
-        if (cnt > mt) cnt = mt;
-        int key = ax + (1 << l) * (ay + (1 << l) * az);
-        const int *tl = tlist + (size_t)l * mt;
-        int lo = 0, hi = cnt;
-        while (lo < hi) {
-            int mid = (lo + hi) >> 1;
-            if (tl[mid] < key) lo = mid + 1;
-            else hi = mid;
-        }
-        if (lo < cnt && tl[lo] == key)
-            total += l2p_value<T>(p, contrib + ((size_t)l * mt + lo) * nc, vx, vy, vz, s_half, s_inv) * inv;
+        total += l2p_value<T>(p, Lc, vx, vy, vz, s_half, s_inv) * inv;
     }
     phi[s] = total;
 }
 
-// exclusive scan (one block per 4096 flags), reusing the layout of the sort's scan
-__global__ void k_flag_scan_blocks(int64_t n, const int *__restrict__ in, int *__restrict__ out, int *__restrict__ sums)
-{
-    __shared__ int ws[32];
-    int64_t base = (int64_t)blockIdx.x * 4096 + threadIdx.x * 16;
-    int v[16], local = 0;
-    for (int k = 0; k < 16; ++k) {
-        int64_t idx = base + k;
-        v[k] = idx < n ? in[idx] : 0;
-        local += v[k];
-    }
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int x = local;
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        int t = lane < (int)(blockDim.x >> 5) ? ws[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        ws[lane] = t;
-    }
-    __syncthreads();
-    int excl = x - local + (wid > 0 ? ws[wid - 1] : 0);
-    for (int k = 0; k < 16; ++k) {
-        int64_t idx = base + k;
-        if (idx < n) out[idx] = excl;
-        excl += v[k];
-    }
-    if (threadIdx.x == blockDim.x - 1) sums[blockIdx.x] = excl;
-}
-
-__global__ void k_flag_scan_sums(int nb, int *__restrict__ sums, int *__restrict__ total)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        int acc = 0;
-        for (int b = 0; b < nb; ++b) {
-            int t = sums[b];
-            sums[b] = acc;
-            acc += t;
-        }
-        *total = acc;
-    }
-}
-
-__global__ void k_flag_scan_add(int64_t n, int *__restrict__ out, const int *__restrict__ sums)
-{
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] += sums[i / 4096];
-}
-
-// prologue on stream `st`: active cells, solute moments MU of the active cells
-// and the FP64 local expansions Lt of the solvent field there (from the full
-// pass's moments minus MU), before the rest of the pass overwrites the coarse
-// moments.  Grids cover NU_MAX cells; the device count decides (no cells when
-// the sparse pass does not apply).
+// the solute-only expansions, on stream `st` (needs the sort only); the device count decides how many cells are
+// active (none when the sparse pass does not apply)
 template <typename T>
-fmm_status solute_prologue_t(Plan &P, SoluteScratch &S, cudaStream_t st)
+fmm_status solute_expand_t(Plan &P, SoluteScratch &S, cudaStream_t st)
 {
-    const int p = P.p, d = P.d, nc = P.nc;
-    const int nside = 1 << d;
-    const double h = P.box / nside;
-    const int nu = NU_MAX;
-    const T *Rw = std::is_same<T, double>::value ? (const T *)P.tab.Rw64 : (const T *)P.tab.Rw32;
-    T *MU = (T *)S.MU;
-    k_sol_cells<<<1, 32, 0, st>>>(d, S.list, P.sleaf, S.cells, S.ncells);
+    const int p = P.p, d = P.d, nc = P.nc, ld = d < LD_MAX ? d : LD_MAX, mt = max_tgt(P.ws);
+    const bool f64 = std::is_same<T, double>::value;
+    const T h = (T)(P.box / (1 << d));
+    const T *Top = f64 ? (const T *)P.tab.Top64 : (const T *)P.tab.Top32;
+    const T *l2lT = (f64 ? (const T *)P.tab.l2l64 : (const T *)P.tab.l2l32) + (size_t)8 * nc * nc;
+    const int *count = P.d_err + 1;
+    T *MU = (T *)S.MU, *Lu = (T *)S.Lu, *part = (T *)S.contrib;
+    const int nth = ((nc + 31) / 32) * 32;
+    k_sol_cells<<<1, NU_MAX, 0, st>>>(d, count, S.list, P.sleaf, S.slots, S.cells, S.ncells);
     FMM_LAUNCH_CHECK(P);
-    k_sol_p2m<T><<<nu, 32, 0, st>>>(p, d, S.cells, S.ncells, P.cell_start, (const Particle<T> *)P.sorted_u,
-                                       (T)(1.0 / h), MU);
+    k_sol_p2m<T><<<dim3(NU_MAX, d), 32, 0, st>>>(p, d, h, count, S.slots, P.sleaf, S.cells, S.ncells,
+                                                 (const Particle<T> *)P.sorted, MU);
     FMM_LAUNCH_CHECK(P);
-    for (int l = d - 1; l >= 0; --l) {
-        k_sol_m2m<T><<<dim3(nu, (p + 1) * (p + 2) / 2), 32, 0, st>>>(p, l, S.cells, S.ncells, Rw, MU);
+    fmm_status s = launch_top_solute(P, st, MU + (size_t)NU_MAX * nc, S.cells + NU_MAX, S.ncells + 1, Lu + dense_off(1, nc));
+    if (s != FMM_OK) return s;
+    k_sol_dense_m2l<T><<<ITEM_BLOCKS, nth, 0, st>>>(p, ld, P.ws, S.cells, S.ncells, Top, MU, part);
+    FMM_LAUNCH_CHECK(P);
+    for (int l = 2; l <= ld; ++l) {
+        k_sol_dense<T><<<1u << (3 * l), nth, 0, st>>>(p, l, P.ws, S.cells, S.ncells, part, l2lT, Lu + dense_off(l - 1, nc),
+                                                      Lu + dense_off(l, nc));
         FMM_LAUNCH_CHECK(P);
     }
-    const int nth = ((nc + 31) / 32) * 32;
-    double *Lt = (double *)S.Lt;
-    k_act_lattice<T><<<1, nth, 0, st>>>(p, S.ncells, P.tab.T0, (const T *)P.M[0], MU, Lt);
-    FMM_LAUNCH_CHECK(P);
-    for (int l = 1; l <= d; ++l) {
-        k_act_m2l<T><<<dim3(nu, n_il(P.ws)), nth, 0, st>>>(p, l, P.ws, S.cells, S.ncells, P.tab.Top64,
-                                                            (const T *)P.M[l], MU, S.part);
+    if (d > ld) {
+        FMM_CUDA_TRY(cudaMemsetAsync(S.map, 0, S.map_bytes, st));
+        k_sol_mark<<<dim3(NU_MAX, d - ld), 256, 0, st>>>(ld, P.ws, mt, S.cells, S.ncells, S.map, S.tlist);
         FMM_LAUNCH_CHECK(P);
-        k_act_sum<<<dim3(nu, (nc + 7) / 8), 256, 0, st>>>(p, l, n_il(P.ws), S.ncells, S.part, Lt);
-        FMM_LAUNCH_CHECK(P);
-        k_act_l2l<<<dim3(nu, (p + 1) * (p + 2) / 2), 32, 0, st>>>(p, l, S.cells, S.ncells, P.tab.Rw64, Lt, Lt);
+        k_sol_m2l<T><<<ITEM_BLOCKS, nth, 0, st>>>(p, d, ld, P.ws, S.cells, S.ncells, S.tlist, Top, MU, (T *)S.contrib);
         FMM_LAUNCH_CHECK(P);
     }
     return FMM_OK;
 }
 
-// the rest of the pass (it reads only the prologue's active cells and moments): the dense coarse levels
-// into the pass's own arrays and the target lists and M2L sums of the sparse finer levels
+// the solvent's FP64 field at the active cells, on stream `st` (needs the full pass's moments of all levels)
 template <typename T>
-fmm_status solute_sparse_t(Plan &P, SoluteScratch &S, int nu)
+fmm_status solute_act_t(Plan &P, SoluteScratch &S, cudaStream_t st)
 {
-    const int p = P.p, d = P.d, nc = P.nc;
-    const T *Top = std::is_same<T, double>::value ? (const T *)P.tab.Top64 : (const T *)P.tab.Top32;
-    const T *Rw = std::is_same<T, double>::value ? (const T *)P.tab.Rw64 : (const T *)P.tab.Rw32;
-    T *MU = (T *)S.MU;
-    T *Lu = (T *)S.Lu;
-    const int nth = ((nc + 31) / 32) * 32;
-    // dense coarse levels 0..LD
-    k_sol_lattice<T><<<1, nth, 0, P.stream>>>(p, S.ncells, P.tab.T0, MU, Lu);
+    const int p = P.p, d = P.d, nc = P.nc, ng = act_groups(P.ws);
+    const T *MU = (const T *)S.MU;
+    const int nth = nc < 192 ? ((nc + 31) / 32) * 32 : 192;
+    k_act_m2l<T><<<ITEM_BLOCKS, nth, 0, st>>>(p, d, P.ws, P.tab.il, S.cells, S.ncells, P.tab.Top64,
+                                              (const T *const *)P.d_M, MU, S.part);
     FMM_LAUNCH_CHECK(P);
-    // the M2L terms of one dense level at a time in the (unused) level 0..LD part of the sparse sums
-    T *part = (T *)S.contrib;
-    const int win = off_side(P.ws) * off_side(P.ws) * off_side(P.ws);
-    for (int l = 1; l <= LD; ++l) {
-        k_sol_dense_m2l<T><<<dim3(nu, win), nth, 0, P.stream>>>(p, l, P.ws, S.cells, S.ncells, Top, MU, part);
-        FMM_LAUNCH_CHECK(P);
-        k_sol_dense<T><<<1u << (3 * l), nth, 0, P.stream>>>(p, l, P.ws, S.cells, S.ncells, part, Rw,
-                                                              Lu + dense_off(l - 1, nc), Lu + dense_off(l, nc));
-        FMM_LAUNCH_CHECK(P);
-    }
-    // sparse finer levels
-    for (int l = LD + 1; l <= d; ++l) {
-        int64_t n = (int64_t)1 << (3 * l);
-        FMM_CUDA_TRY(cudaMemsetAsync(S.flags, 0, sizeof(int) * n, P.stream));
-        k_sol_mark<<<nu, 256, 0, P.stream>>>(l, P.ws, S.cells, S.ncells, S.flags);
-        FMM_LAUNCH_CHECK(P);
-        int nb = (int)((n + 4095) / 4096);
-        k_flag_scan_blocks<<<nb, 256, 0, P.stream>>>(n, S.flags, S.pos, S.scan_tmp);
-        FMM_LAUNCH_CHECK(P);
-        k_flag_scan_sums<<<1, 32, 0, P.stream>>>(nb, S.scan_tmp, S.ncells + 16 + l);
-        FMM_LAUNCH_CHECK(P);
-        k_flag_scan_add<<<blocks_for(n, 256), 256, 0, P.stream>>>(n, S.pos, S.scan_tmp);
-        FMM_LAUNCH_CHECK(P);
-        k_sol_compact<<<blocks_for(n, 256), 256, 0, P.stream>>>(n, max_tgt(P.ws), S.flags, S.pos,
-                                                                 S.tlist + (size_t)l * max_tgt(P.ws));
-        FMM_LAUNCH_CHECK(P);
-        k_sol_m2l<T><<<nu * n_il(P.ws), ((nc + 31) / 32) * 32, 0, P.stream>>>(p, l, P.ws, S.cells, S.ncells,
-                                                                       S.tlist + (size_t)l * max_tgt(P.ws),
-                                                                       S.ncells + 16 + l, Top, MU, (T *)S.contrib);
-        FMM_LAUNCH_CHECK(P);
-    }
+    fmm_status s = launch_top_active(P, st, MU + (size_t)NU_MAX * nc, S.cells + NU_MAX, S.ncells + 1,
+                                     S.Lt + (size_t)NU_MAX * nc);
+    if (s != FMM_OK) return s;
+    k_act_sum<<<dim3(8, (nc + 7) / 8, d - 1), 256, 0, st>>>(p, ng, S.ncells, S.part, S.Lt);
+    FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
 
-// Phi_u at every charge: the level-LD expansion plus the sparse finer-level sums
+// Phi_u at every charge: the level-ld expansion plus the sparse finer-level sums
 template <typename T>
-fmm_status solute_eval_t(Plan &P, SoluteScratch &S)
+fmm_status solute_eval_t(Plan &P, SoluteScratch &S, cudaStream_t st)
 {
     const double h = P.box / (1 << P.d);
-    k_sol_eval<T><<<blocks_for(P.N, 128), 128, 0, P.stream>>>(P.p, P.d, max_tgt(P.ws), P.N, (T)h, P.sleaf,
-                                                              (const Particle<T> *)P.sorted,
-                                                              (const T *)S.Lu + dense_off(LD, P.nc), S.tlist,
-                                                              S.ncells + 16, (const T *)S.contrib, (T *)P.phi_u);
+    const int ld = P.d < LD_MAX ? P.d : LD_MAX;
+    k_sol_eval<T><<<blocks_for(P.N, 128), 128, 0, st>>>(P.p, P.d, ld, max_tgt(P.ws), P.N, (T)h, P.sleaf,
+                                                        (const Particle<T> *)P.sorted,
+                                                        (const T *)S.Lu + dense_off(ld, P.nc), S.map,
+                                                        (const T *)S.contrib, (T *)P.phi_u);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
@@ -805,44 +663,42 @@ template <typename T>
 fmm_status solute_act_l2p_t(Plan &P, SoluteScratch &S)
 {
     const double h = P.box / (1 << P.d);
-    k_act_l2p<T><<<1, NU_MAX, 0, P.stream>>>(P.p, P.d, 1.0 / h, S.list, S.cells, S.ncells, P.sleaf,
-                                             (const Particle<T> *)P.sorted, (const double *)S.Lt,
-                                             (const T *)P.phi_u, (T *)P.phi_ff);
+    k_act_l2p<T><<<NU_MAX, 256, 0, P.stream>>>(P.p, P.d, h, P.d_err + 1, S.slots, S.cells, S.ncells, P.sleaf,
+                                               (const Particle<T> *)P.sorted, S.Lt, (const T *)P.phi_u, (T *)P.phi_ff);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
+
+// the sparse pass applies to this call as far as the host knows
+bool solute_may_run(const Plan &P) { return P.known_count < 0 || (P.known_count > 0 && P.known_count <= NU_MAX); }
 
 }  // namespace
 
 fmm_status solute_prepare(Plan &P)
 {
     solute_free(P);
-    if (P.d <= LD) return FMM_OK;
     SoluteScratch *S = new (std::nothrow) SoluteScratch();
     if (!S) return FMM_ERR_OOM;
     P.sol = S;
-    int64_t nleaf = (int64_t)1 << (3 * P.d);
-    FMM_CUDA_TRY(cudaMalloc(&S->list, sizeof(int) * (NU_MAX + 4)));
+    const int ld = P.d < LD_MAX ? P.d : LD_MAX;
+    FMM_CUDA_TRY(cudaMalloc(&S->list, sizeof(int) * NU_MAX));
+    FMM_CUDA_TRY(cudaMalloc(&S->slots, sizeof(int) * NU_MAX));
     FMM_CUDA_TRY(cudaMalloc(&S->cells, sizeof(int) * 9 * NU_MAX));
     FMM_CUDA_TRY(cudaMalloc(&S->ncells, sizeof(int) * 32));
     FMM_CUDA_TRY(cudaMalloc(&S->MU, sizeof(double) * 9 * NU_MAX * P.nc));
-    FMM_CUDA_TRY(cudaMalloc(&S->flags, sizeof(int) * nleaf));
-    FMM_CUDA_TRY(cudaMalloc(&S->pos, sizeof(int) * (nleaf + 1)));
-    FMM_CUDA_TRY(cudaMalloc(&S->scan_tmp, sizeof(int) * (nleaf / 4096 + 2)));
+    S->map_bytes = sizeof(int) * (size_t)(P.d > ld ? map_off(P.d + 1, ld) : 0);
+    FMM_CUDA_TRY(cudaMalloc(&S->map, S->map_bytes + 16));
     FMM_CUDA_TRY(cudaMalloc(&S->tlist, sizeof(int) * 9 * max_tgt(P.ws)));
     FMM_CUDA_TRY(cudaMalloc(&S->contrib, sizeof(double) * (size_t)(P.d + 1) * max_tgt(P.ws) * P.nc));
     FMM_CUDA_TRY(cudaMallocHost((void **)&S->h_count, sizeof(int)));
     int lo = 0, hi = 0;
     FMM_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&lo, &hi));
     FMM_CUDA_TRY(cudaStreamCreateWithPriority(&S->side, cudaStreamNonBlocking, hi));
-    FMM_CUDA_TRY(cudaEventCreateWithFlags(&S->ev_count, cudaEventDisableTiming));
-    FMM_CUDA_TRY(cudaEventCreateWithFlags(&S->ev_up, cudaEventDisableTiming));
-    FMM_CUDA_TRY(cudaEventCreateWithFlags(&S->ev_act, cudaEventDisableTiming));
-    FMM_CUDA_TRY(cudaEventCreateWithFlags(&S->ev_ready, cudaEventDisableTiming));
-    FMM_CUDA_TRY(cudaEventCreateWithFlags(&S->ev_sparse, cudaEventDisableTiming));
+    for (cudaEvent_t *e : {&S->ev_count, &S->ev_sort, &S->ev_up, &S->ev_ready, &S->ev_done})
+        FMM_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     FMM_CUDA_TRY(cudaMalloc(&S->Lt, sizeof(double) * 9 * NU_MAX * P.nc));
-    FMM_CUDA_TRY(cudaMalloc(&S->Lu, sizeof(double) * dense_off(LD + 1, P.nc)));
-    FMM_CUDA_TRY(cudaMalloc(&S->part, sizeof(double) * NU_MAX * n_il(P.ws) * P.nc));
+    FMM_CUDA_TRY(cudaMalloc(&S->Lu, sizeof(double) * dense_off(ld + 1, P.nc)));
+    FMM_CUDA_TRY(cudaMalloc(&S->part, sizeof(double) * (size_t)(P.d - 1) * NU_MAX * act_groups(P.ws) * P.nc));
     return FMM_OK;
 }
 
@@ -851,12 +707,11 @@ void solute_free(Plan &P)
     SoluteScratch *S = (SoluteScratch *)P.sol;
     if (!S) return;
     cudaFree(S->list);
+    cudaFree(S->slots);
     cudaFree(S->cells);
     cudaFree(S->ncells);
     cudaFree(S->MU);
-    cudaFree(S->flags);
-    cudaFree(S->pos);
-    cudaFree(S->scan_tmp);
+    cudaFree(S->map);
     cudaFree(S->tlist);
     cudaFree(S->contrib);
     cudaFree(S->Lt);
@@ -867,11 +722,8 @@ void solute_free(Plan &P)
         cudaStreamSynchronize(S->side);
         cudaStreamDestroy(S->side);
     }
-    if (S->ev_count) cudaEventDestroy(S->ev_count);
-    if (S->ev_up) cudaEventDestroy(S->ev_up);
-    if (S->ev_act) cudaEventDestroy(S->ev_act);
-    if (S->ev_ready) cudaEventDestroy(S->ev_ready);
-    if (S->ev_sparse) cudaEventDestroy(S->ev_sparse);
+    for (cudaEvent_t e : {S->ev_count, S->ev_sort, S->ev_up, S->ev_ready, S->ev_done})
+        if (e) cudaEventDestroy(e);
     delete S;
     P.sol = nullptr;
 }
@@ -882,61 +734,65 @@ int solute_count_host(const Plan &P)
     return S ? *S->h_count : -1;
 }
 
+int *solute_list(Plan &P, int *cap)
+{
+    SoluteScratch *S = (SoluteScratch *)P.sol;
+    *cap = NU_MAX;
+    return S ? S->list : nullptr;
+}
+
 fmm_status solute_count(Plan &P)
 {
     SoluteScratch *S = (SoluteScratch *)P.sol;
-    if (!S) return FMM_OK;
-    S->sparse_forked = false;  // a new call (a failed one may have left it set)
-    FMM_CUDA_TRY(cudaMemsetAsync(S->list + NU_MAX, 0, sizeof(int), P.stream));
-    k_sol_list<<<blocks_for(P.N, 256), 256, 0, P.stream>>>(P.N, P.sorted_sol, S->list);
-    FMM_LAUNCH_CHECK(P);
-    FMM_CUDA_TRY(cudaMemcpyAsync(S->h_count, S->list + NU_MAX, sizeof(int), cudaMemcpyDeviceToHost, P.stream));
+    if (!S) return FMM_ERR_INTERNAL;
+    S->forked = S->act_done = false;  // a new call (a failed one may have left them set)
+    FMM_CUDA_TRY(cudaMemcpyAsync(S->h_count, P.d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, P.stream));
     FMM_CUDA_TRY(cudaEventRecord(S->ev_count, P.stream));
     S->count_pending = true;
     return FMM_OK;
 }
 
-fmm_status solute_prologue(Plan &P)
+fmm_status solute_fork(Plan &P)
 {
     SoluteScratch *S = (SoluteScratch *)P.sol;
-    if (!S) return FMM_OK;
-    if (!S->count_pending) {
-        fmm_status s = solute_count(P);
-        if (s != FMM_OK) return s;
+    if (!S || !P.overlap || !solute_may_run(P)) return FMM_OK;
+    FMM_CUDA_TRY(cudaEventRecord(S->ev_sort, P.stream));
+    FMM_CUDA_TRY(cudaStreamWaitEvent(S->side, S->ev_sort, 0));
+    S->forked = true;
+    fmm_status s = P.precision == FMM_PREC_FP64 ? solute_expand_t<double>(P, *S, S->side)
+                                                : solute_expand_t<float>(P, *S, S->side);
+    if (s != FMM_OK) return s;
+    // Phi_u at every charge (a full-size launch) on the near stream, where it fills idle SMs instead of taking
+    // them from the far field
+    cudaStream_t st = S->side;
+    if (P.near_forked) {
+        FMM_CUDA_TRY(cudaEventRecord(S->ev_ready, S->side));
+        FMM_CUDA_TRY(cudaStreamWaitEvent(P.near, S->ev_ready, 0));
+        st = P.near;
     }
-    FMM_CUDA_TRY(cudaEventRecord(S->ev_up, P.stream));
-    FMM_CUDA_TRY(cudaStreamWaitEvent(S->side, S->ev_up, 0));
-    fmm_status s = P.precision == FMM_PREC_FP64 ? solute_prologue_t<double>(P, *S, S->side)
-                                                : solute_prologue_t<float>(P, *S, S->side);
-    FMM_CUDA_TRY(cudaEventRecord(S->ev_act, S->side));
-    S->prologue_pending = true;
-    return s;
+    return P.precision == FMM_PREC_FP64 ? solute_eval_t<double>(P, *S, st) : solute_eval_t<float>(P, *S, st);
 }
 
-fmm_status solute_sparse_fork(Plan &P)
+fmm_status solute_active(Plan &P)
 {
     SoluteScratch *S = (SoluteScratch *)P.sol;
-    if (!S || !P.overlap || !S->prologue_pending || S->sparse_forked) return FMM_OK;
-    int nu = NU_MAX;  // unknown count: grids for the largest, the device count decides
-    if (P.known_count >= 0) {
-        if (P.known_count == 0 || P.known_count > NU_MAX) return FMM_OK;  // nothing to overlap
-        nu = P.known_count;
-    }
-    // behind the prologue on the side stream; Phi_u at every charge (a full-size launch) on the near
-    // stream, where it fills idle SMs instead of taking them from the far field
-    cudaStream_t main_stream = P.stream;
-    P.stream = S->side;
-    fmm_status s = P.precision == FMM_PREC_FP64 ? solute_sparse_t<double>(P, *S, nu) : solute_sparse_t<float>(P, *S, nu);
-    if (s == FMM_OK && P.near_forked) {
-        if (cudaEventRecord(S->ev_ready, S->side) != cudaSuccess || cudaStreamWaitEvent(P.near, S->ev_ready, 0) != cudaSuccess)
-            s = FMM_ERR_CUDA;
-        P.stream = P.near;
-    }
-    if (s == FMM_OK) s = P.precision == FMM_PREC_FP64 ? solute_eval_t<double>(P, *S) : solute_eval_t<float>(P, *S);
-    P.stream = main_stream;
+    if (!S || !S->forked) return FMM_OK;
+    FMM_CUDA_TRY(cudaEventRecord(S->ev_up, P.stream));
+    FMM_CUDA_TRY(cudaStreamWaitEvent(S->side, S->ev_up, 0));
+    fmm_status s = P.precision == FMM_PREC_FP64 ? solute_act_t<double>(P, *S, S->side)
+                                                : solute_act_t<float>(P, *S, S->side);
     if (s != FMM_OK) return s;
-    FMM_CUDA_TRY(cudaEventRecord(S->ev_sparse, S->side));
-    S->sparse_forked = true;
+    S->act_done = true;
+    return FMM_OK;
+}
+
+fmm_status solute_join(Plan &P)
+{
+    SoluteScratch *S = (SoluteScratch *)P.sol;
+    if (!S || !S->forked) return FMM_OK;
+    S->forked = false;
+    FMM_CUDA_TRY(cudaEventRecord(S->ev_done, S->side));
+    FMM_CUDA_TRY(cudaStreamWaitEvent(P.stream, S->ev_done, 0));
     return FMM_OK;
 }
 
@@ -945,45 +801,28 @@ fmm_status launch_solute_pass(Plan &P, bool *done)
 {
     *done = false;
     SoluteScratch *S = (SoluteScratch *)P.sol;
-    if (!S) return FMM_OK;
-    if (S->sparse_forked) {
-        // forked after the prologue (Phi_u on the near stream, joined before this call): join the side
-        // stream; the dense pass overwrites the (empty) result when the count is above NU_MAX
-        if (P.known_count < 0) FMM_CUDA_TRY(cudaEventSynchronize(S->ev_count));
-        FMM_CUDA_TRY(cudaStreamWaitEvent(P.stream, S->ev_sparse, 0));
-        S->count_pending = S->prologue_pending = S->sparse_forked = false;
-        int n = P.known_count >= 0 ? P.known_count : *S->h_count;
-        if (n > NU_MAX) return FMM_OK;
-        if (n == 0) {
-            size_t bytes = (P.precision == FMM_PREC_FP64 ? sizeof(double) : sizeof(float)) * P.N;
-            FMM_CUDA_TRY(cudaMemsetAsync(P.phi_u, 0, bytes, P.stream));
-            *done = true;
-            return FMM_OK;
-        }
-        fmm_status s = P.precision == FMM_PREC_FP64 ? solute_act_l2p_t<double>(P, *S) : solute_act_l2p_t<float>(P, *S);
-        if (s == FMM_OK) *done = true;
-        return s;
-    }
-    if (!S->prologue_pending) {
-        fmm_status s = solute_prologue(P);
-        if (s != FMM_OK) return s;
-    }
-    // the count was copied right after the sort (or the caller knows it); the join orders the
-    // prologue before the rest
+    if (!S) return FMM_ERR_INTERNAL;
+    const bool expanded = S->forked && S->act_done;
+    fmm_status s = solute_join(P);
+    if (s != FMM_OK) return s;
+    // the count was copied right after the sort, or the caller knows it
     if (P.known_count < 0) FMM_CUDA_TRY(cudaEventSynchronize(S->ev_count));
-    FMM_CUDA_TRY(cudaStreamWaitEvent(P.stream, S->ev_act, 0));
-    S->count_pending = S->prologue_pending = false;
-    int n = P.known_count >= 0 ? P.known_count : *S->h_count;
-    if (n > NU_MAX) return FMM_OK;
+    S->count_pending = S->act_done = false;
+    const int n = P.known_count >= 0 ? P.known_count : *S->h_count;
+    if (n > NU_MAX) return FMM_OK;  // the dense pass overwrites the (empty) result
     if (n == 0) {
         size_t bytes = (P.precision == FMM_PREC_FP64 ? sizeof(double) : sizeof(float)) * P.N;
         FMM_CUDA_TRY(cudaMemsetAsync(P.phi_u, 0, bytes, P.stream));
         *done = true;
         return FMM_OK;
     }
-    fmm_status s = P.precision == FMM_PREC_FP64 ? solute_sparse_t<double>(P, *S, n) : solute_sparse_t<float>(P, *S, n);
-    if (s == FMM_OK) s = P.precision == FMM_PREC_FP64 ? solute_eval_t<double>(P, *S) : solute_eval_t<float>(P, *S);
-    if (s == FMM_OK) s = P.precision == FMM_PREC_FP64 ? solute_act_l2p_t<double>(P, *S) : solute_act_l2p_t<float>(P, *S);
+    const bool f64 = P.precision == FMM_PREC_FP64;
+    if (!expanded) {  // in order on the plan's stream
+        s = f64 ? solute_expand_t<double>(P, *S, P.stream) : solute_expand_t<float>(P, *S, P.stream);
+        if (s == FMM_OK) s = f64 ? solute_act_t<double>(P, *S, P.stream) : solute_act_t<float>(P, *S, P.stream);
+        if (s == FMM_OK) s = f64 ? solute_eval_t<double>(P, *S, P.stream) : solute_eval_t<float>(P, *S, P.stream);
+    }
+    if (s == FMM_OK) s = f64 ? solute_act_l2p_t<double>(P, *S) : solute_act_l2p_t<float>(P, *S);
     if (s == FMM_OK) *done = true;
     return s;
 }

@@ -155,7 +155,8 @@ template <typename T>
 __global__ void k_gather(int64_t N, const int *__restrict__ perm, const int *__restrict__ key,
                          const double *__restrict__ wpos, const double *__restrict__ q, const uint8_t *__restrict__ sol,
                          double h, int nside, Particle<T> *__restrict__ out, Particle<T> *__restrict__ out_u,
-                         uint8_t *__restrict__ out_sol, int *__restrict__ sleaf)
+                         uint8_t *__restrict__ out_sol, int *__restrict__ sleaf, int *__restrict__ sol_list, int sol_cap,
+                         int *__restrict__ sol_count)
 {
     int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= N) return;
@@ -174,6 +175,10 @@ __global__ void k_gather(int64_t N, const int *__restrict__ perm, const int *__r
     if (sol) {
         uint8_t u = sol[i] ? 1 : 0;
         out_sol[s] = u;
+        if (u) {  // the first sol_cap solute slots in any order; all of them counted
+            const int idx = atomicAdd(sol_count, 1);
+            if (idx < sol_cap) sol_list[idx] = (int)s;
+        }
         Particle<T> ru = r;
         if (!u) ru.q = (T)0;
         out_u[s] = ru;
@@ -431,15 +436,17 @@ fmm_status launch_assign_sort(Plan &P, const double *pos, const double *q, const
     k_leaf_sort<<<blocks_for(P.nleaf, 256), 256, 0, P.stream>>>(P.nleaf, P.cell_start, P.perm);
     FMM_LAUNCH_CHECK(P);
     double h = P.box / nside;
+    int sol_cap = 0;
+    int *sol_list = solute_list(P, &sol_cap);
     if (P.precision == FMM_PREC_FP64)
         k_gather<double><<<blocks_for(P.N, 256), 256, 0, P.stream>>>(
             P.N, P.perm, P.key, P.wpos, q, sol, h, nside, (Particle<double> *)P.sorted,
-            (Particle<double> *)P.sorted_u, P.sorted_sol, P.sleaf);
+            (Particle<double> *)P.sorted_u, P.sorted_sol, P.sleaf, sol_list, sol_cap, P.d_err + 1);
     else
         k_gather<float><<<blocks_for(P.N, 256), 256, 0, P.stream>>>(P.N, P.perm, P.key, P.wpos, q, sol, h, nside,
                                                                     (Particle<float> *)P.sorted,
                                                                     (Particle<float> *)P.sorted_u, P.sorted_sol,
-                                                                    P.sleaf);
+                                                                    P.sleaf, sol_list, sol_cap, P.d_err + 1);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }

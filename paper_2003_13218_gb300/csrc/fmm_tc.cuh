@@ -24,8 +24,6 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include <vector>
-
 #include "fmm_internal.cuh"
 
 namespace fmm {
@@ -115,8 +113,6 @@ __device__ inline int gain_m_exp(unsigned bits)
 // out, in z, y, x order.  The producers read the list from a table: stepping through the cube and skipping what
 // is not theirs took ~160 cycles a position, up to 17 us before and after the copies of a small launch (2,998
 // charges at depth 3, p = 8: 682 -> 533 us a call; 100,000 at ws = 2: 2.9 -> 2.3 ms).
-__host__ __device__ inline int il_pack(int dx, int dy, int dz) { return (dx + 16) | ((dy + 16) << 8) | ((dz + 16) << 16); }
-
 // A producer warp's walk through offsets o .. end of one class's list: 32 entries per load, one load ahead
 struct IlWalk {
     const int *list;
@@ -134,9 +130,7 @@ struct IlWalk {
             next = o + k + 32 + lane < end ? __ldg(list + o + k + 32 + lane) : 0;
         }
         const int e = __shfl_sync(0xffffffffu, cur, k & 31);
-        dx = (e & 255) - 16;
-        dy = ((e >> 8) & 255) - 16;
-        dz = ((e >> 16) & 255) - 16;
+        il_unpack(e, dx, dy, dz);
     }
 };
 
@@ -1451,26 +1445,6 @@ __device__ __forceinline__ int64_t chunk_at(int64_t cell, int64_t ncell, int k, 
 }
 
 // ------------------------------------------------------------------ host helpers
-// the interaction lists of the 8 parity classes in device memory
-fmm_status upload_il(int ws, cudaStream_t st, int **out)
-{
-    const int n = n_il(ws);
-    std::vector<int> h;
-    h.reserve((size_t)8 * n);
-    for (int c = 0; c < 8; ++c) {
-        const int cx = c & 1, cy = (c >> 1) & 1, cz = (c >> 2) & 1;
-        for (int dz = -2 * ws - cz; dz <= 2 * ws + 1 - cz; ++dz)
-            for (int dy = -2 * ws - cy; dy <= 2 * ws + 1 - cy; ++dy)
-                for (int dx = -2 * ws - cx; dx <= 2 * ws + 1 - cx; ++dx)
-                    if (!(dx >= -ws && dx <= ws && dy >= -ws && dy <= ws && dz >= -ws && dz <= ws))
-                        h.push_back(il_pack(dx, dy, dz));
-    }
-    if (h.size() != (size_t)8 * n) return FMM_ERR_INTERNAL;
-    FMM_CUDA_TRY(cudaMalloc(out, sizeof(int) * h.size()));
-    FMM_CUDA_TRY(cudaMemcpyAsync(*out, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, st));
-    return cudaStreamSynchronize(st) == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
