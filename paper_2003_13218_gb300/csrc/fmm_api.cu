@@ -19,7 +19,7 @@ size_t reduction_scratch_bytes() { return sizeof(double) * 304 * 20 * 2; }
 void free_buffers(Plan &P)
 {
     void *bufs[] = {P.in_pos, P.in_q,   P.out_forces, P.out_phi, P.in_sol, P.wpos,    P.key,    P.perm,   P.sleaf,
-                    P.cell_start, P.cell_fill, P.scan_tmp, P.sorted, P.sorted_u, P.sorted_sol, P.phi_nf, P.phi_ff,
+                    P.cell_start, P.found, P.scan_tmp, P.sorted, P.sorted_u, P.sorted_sol, P.phi_nf, P.phi_ff,
                     P.phi_u, P.f_nf, P.g_ff, P.red_partial, P.red_out, P.d_err, P.sc_out, P.sc_lambda, P.d_M};
     for (void *b : bufs) cudaFree(b);
     for (int l = 0; l <= 8; ++l) {
@@ -33,7 +33,7 @@ void free_buffers(Plan &P)
     P.in_pos = P.in_q = P.out_forces = P.out_phi = nullptr;
     P.in_sol = nullptr;
     P.wpos = nullptr;
-    P.key = P.perm = P.sleaf = P.cell_start = P.cell_fill = P.scan_tmp = nullptr;
+    P.key = P.perm = P.found = P.sleaf = P.cell_start = P.cell_fill = P.scan_tmp = nullptr;
     P.sorted = P.sorted_u = nullptr;
     P.sorted_sol = nullptr;
     P.phi_nf = P.phi_ff = P.phi_u = P.f_nf = P.g_ff = nullptr;
@@ -58,7 +58,7 @@ fmm_status alloc_buffers(Plan &P)
     FMM_CUDA_TRY(dalloc(&P.perm, sizeof(int) * N));
     FMM_CUDA_TRY(dalloc(&P.sleaf, sizeof(int) * N));
     FMM_CUDA_TRY(dalloc(&P.cell_start, sizeof(int) * (P.nleaf + 1)));
-    FMM_CUDA_TRY(dalloc(&P.cell_fill, sizeof(int) * P.nleaf));
+    FMM_CUDA_TRY(dalloc(&P.found, sizeof(int) * N));
     FMM_CUDA_TRY(dalloc(&P.scan_tmp, sizeof(int) * (P.nleaf / 4096 + 2)));
     FMM_CUDA_TRY(dalloc(&P.sorted, sizeof(Particle<double>) * N));
     FMM_CUDA_TRY(dalloc(&P.sorted_u, sizeof(Particle<double>) * N));
@@ -75,7 +75,8 @@ fmm_status alloc_buffers(Plan &P)
     }
     FMM_CUDA_TRY(dalloc(&P.red_partial, reduction_scratch_bytes()));
     FMM_CUDA_TRY(dalloc(&P.red_out, sizeof(double) * 48));
-    FMM_CUDA_TRY(dalloc(&P.d_err, sizeof(int) * 2));
+    FMM_CUDA_TRY(dalloc(&P.d_err, sizeof(int) * (ERR_WORDS + P.nleaf)));
+    P.cell_fill = P.d_err + ERR_WORDS;
     FMM_CUDA_TRY(dalloc(&P.d_M, sizeof(P.M)));
     FMM_CUDA_TRY(cudaMemcpy(P.d_M, P.M, sizeof(P.M), cudaMemcpyHostToDevice));
     FMM_CUDA_TRY(cudaMallocHost((void **)&P.h_out, sizeof(double) * 40));
@@ -121,10 +122,24 @@ struct StageTimer {
         if (s_ != FMM_OK) return s_;         \
     } while (0)
 
-fmm_status far_field_pass(Plan &P, bool gradient, bool solute_only, StageTimer *tm, bool fork_solute = false)
+struct Forks {  // what a full pass sends to its side streams once its upward sweep is enqueued
+    const double *q;
+    const uint8_t *sol;
+    bool gradient, near, uv;
+};
+
+fmm_status fork_near_field(Plan &P, const Forks &f);
+
+fmm_status far_field_pass(Plan &P, bool gradient, bool solute_only, StageTimer *tm, const Forks *forks = nullptr)
 {
     TRY(launch_upward(P, solute_only));
-    if (fork_solute) TRY(solute_active(P));
+    // the far field is the critical chain: in small boxes the host's launches are, so its first part goes out first
+    // (the side streams wait for the sort's events, not for this)
+    if (forks && forks->near) TRY(fork_near_field(P, *forks));
+    if (forks && forks->uv) {
+        TRY(solute_fork(P));
+        TRY(solute_active(P));
+    }
     if (tm) tm->mark();
     TRY(launch_top(P));
     if (tm) tm->mark();
@@ -148,18 +163,17 @@ fmm_status far_field_pass(Plan &P, bool gradient, bool solute_only, StageTimer *
     return FMM_OK;
 }
 
-// the work of one call that needs only the sort, on the plan's near stream (P.overlap): the background
+// the work of one call that needs only the sort (ev_sorted), on the plan's near stream (P.overlap): the background
 // moments, the near field and the solute-solvent near-field sum
-fmm_status fork_near_field(Plan &P, const double *dq, const uint8_t *dsol, bool gradient, bool want_uv)
+fmm_status fork_near_field(Plan &P, const Forks &f)
 {
-    FMM_CUDA_TRY(cudaEventRecord(P.ev_sorted, P.stream));
     FMM_CUDA_TRY(cudaStreamWaitEvent(P.near, P.ev_sorted, 0));
     P.near_forked = P.near_p2p = true;
     cudaStream_t main_stream = P.stream;
     P.stream = P.near;
-    fmm_status s = launch_bc_moments(P, dq, dsol);
-    if (s == FMM_OK) s = launch_p2p(P, gradient);
-    if (s == FMM_OK && want_uv) s = launch_p2p_uv(P);
+    fmm_status s = launch_bc_moments(P, f.q, f.sol);
+    if (s == FMM_OK) s = launch_p2p(P, f.gradient);
+    if (s == FMM_OK && f.uv) s = launch_p2p_uv(P);
     P.stream = main_stream;
     return s;
 }
@@ -180,17 +194,16 @@ fmm_status eval_front(Plan &P, const double *dpos, const double *dq, const uint8
                       bool gradient, StageTimer *tm)
 {
     if (tm) tm->mark();
-    FMM_CUDA_TRY(cudaMemsetAsync(P.d_err, 0, sizeof(int) * 2, P.stream));
     if (want_uv && P.sc_c > 0)  // the soft-core lambda as it is when the call runs
         FMM_CUDA_TRY(cudaMemcpyAsync(P.sc_lambda, P.h_sc_lambda, sizeof(double), cudaMemcpyHostToDevice, P.stream));
     P.near_forked = P.near_p2p = false;
     TRY(launch_assign_sort(P, dpos, dq, dsol));
     if (want_uv) TRY(solute_count(P));
     if (tm) tm->mark();
-    if (P.overlap && P.near) TRY(fork_near_field(P, dq, dsol, gradient, want_uv));
+    const Forks forks{dq, dsol, gradient, P.overlap && P.near, want_uv};
+    if (forks.near) FMM_CUDA_TRY(cudaEventRecord(P.ev_sorted, P.stream));
     else TRY(launch_bc_moments(P, dq, dsol));
-    if (want_uv) TRY(solute_fork(P));
-    TRY(far_field_pass(P, gradient, false, tm, want_uv));
+    TRY(far_field_pass(P, gradient, false, tm, &forks));
     if (!P.near_p2p) TRY(launch_p2p(P, gradient));
     if (tm) tm->mark();
     return FMM_OK;
@@ -214,16 +227,14 @@ fmm_status eval_back(Plan &P, const double *dq, bool want_uv, double *dforces, S
     if (dforces) TRY(launch_forces_out(P, dq, dforces));
     if (dphi) TRY(launch_potentials_out(P, dphi));
     if (tm) tm->mark();
-    FMM_CUDA_TRY(cudaMemcpyAsync(P.h_out, P.red_out, sizeof(double) * 31, cudaMemcpyDeviceToHost, P.stream));
-    FMM_CUDA_TRY(cudaMemcpyAsync(P.h_out + 32, P.d_err, sizeof(int), cudaMemcpyDeviceToHost, P.stream));
+    FMM_CUDA_TRY(cudaMemcpyAsync(P.h_out, P.red_out, sizeof(double) * 32, cudaMemcpyDeviceToHost, P.stream));
     return FMM_OK;
 }
 
 // results of the last evaluation from P.h_out (the plan's stream synchronised)
 fmm_status eval_read(Plan &P, fmm_energy_terms *terms, fmm_uv_terms *uv)
 {
-    int err;
-    memcpy(&err, P.h_out + 32, sizeof(int));
+    const int err = (int)P.h_out[31];
     if (terms) {
         terms->near = P.h_out[16];
         terms->far = P.h_out[17];

@@ -335,30 +335,33 @@ __global__ void k_p2m(int p, int nside, const int *__restrict__ start, const Par
     }
 }
 
-// The same P2M at a compile-time order PP in FP32, one lane per leaf: a warp takes 32 leaves of one
-// parity class with consecutive parent coordinates (32 consecutive rows of the level's class layout),
-// each lane runs the recurrences of Eq. P2M for its leaf's charges with all (PP+1)^2 coefficients in
-// registers (indices fold into immediates).  The rows go through shared memory (row stride (PP+1)^2, odd,
+// The same P2M at a compile-time order PP in FP32, LPL lanes per leaf: a warp takes 32 / LPL leaves of one
+// parity class with consecutive parent coordinates (consecutive rows of the level's class layout),
+// each lane runs the recurrences of Eq. P2M for its share of its leaf's charges with all (PP+1)^2 coefficients in
+// registers (indices fold into immediates); the LPL lanes' sums are added in a fixed tree.  One lane per leaf is
+// best where the leaves fill the GPU (262,144 leaves of 4 charges: 85 us); small trees and dense leaves leave it
+// idle or serial, and take up to 8 (launch_p2m_fixed).  The rows go through shared memory (row stride (PP+1)^2, odd,
 // so the 32 lanes hit 32 banks) and leave as 32 contiguous rows.  When `amax` is set (fp16x2 split) the
 // warp also folds max_k |Mhat_k s(k)| into *amax (positive floats order as their bit patterns), which
 // the tensor-core operand split needs for the level gain.
 constexpr int P2M_WARPS = 4;
 
-template <int PP>
+template <int PP, int LPL>
 __global__ void __launch_bounds__(32 * P2M_WARPS) k_p2m_fixed(int d, const int *__restrict__ start,
                                                               const Particle<float> *__restrict__ sp, float inv_h,
                                                               float *__restrict__ M, const float *__restrict__ s,
                                                               unsigned *__restrict__ amax)
 {
     constexpr int NC = (PP + 1) * (PP + 1);
-    extern __shared__ float p2m_tile[];  // [P2M_WARPS][32][NC]
+    constexpr int ROWS = 32 / LPL;
+    extern __shared__ float p2m_tile[];  // [P2M_WARPS][ROWS][NC]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float *tile = p2m_tile + w * 32 * NC;
+    float *tile = p2m_tile + w * ROWS * NC;
     const int np = 1 << (d - 1);
     const int64_t ncls = (int64_t)np * np * np;
-    const int64_t row0 = ((int64_t)blockIdx.x * P2M_WARPS + w) * 32;
+    const int64_t row0 = ((int64_t)blockIdx.x * P2M_WARPS + w) * ROWS;
     if (row0 >= 8 * ncls) return;
-    const int64_t row = row0 + lane;
+    const int64_t row = row0 + lane / LPL;
     const bool valid = row < 8 * ncls;
     float acc[NC];
 #pragma unroll
@@ -371,7 +374,7 @@ __global__ void __launch_bounds__(32 * P2M_WARPS) k_p2m_fixed(int d, const int *
         const int nside = 2 * np;
         const int leaf = x + nside * (y + nside * z);
         const int b = start[leaf], e = start[leaf + 1];
-        for (int j = b; j < e; ++j) {
+        for (int j = b + lane % LPL; j < e; j += LPL) {
             const Particle<float> pt = sp[j];
             const float vx = -pt.x * inv_h, vy = -pt.y * inv_h, vz = -pt.z * inv_h;
             const float r2 = vx * vx + vy * vy + vz * vz;
@@ -408,14 +411,20 @@ __global__ void __launch_bounds__(32 * P2M_WARPS) k_p2m_fixed(int d, const int *
             }
         }
     }
-    float mx = 0.f;
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        tile[lane * NC + k] = acc[k];
-        if (amax) mx = fmaxf(mx, fabsf(acc[k] * __ldg(s + k)));
+    for (int o = LPL / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < NC; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    float mx = 0.f;
+    if (lane % LPL == 0) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            tile[(lane / LPL) * NC + k] = acc[k];
+            if (amax) mx = fmaxf(mx, fabsf(acc[k] * __ldg(s + k)));
+        }
     }
     __syncwarp();
-    const int64_t nrows = 8 * ncls - row0 < 32 ? 8 * ncls - row0 : 32;
+    const int64_t nrows = 8 * ncls - row0 < ROWS ? 8 * ncls - row0 : ROWS;
     float *dst = M + row0 * NC;
     for (int64_t e = lane; e < nrows * NC; e += 32) dst[e] = tile[e];
     if (amax) {
@@ -424,20 +433,34 @@ __global__ void __launch_bounds__(32 * P2M_WARPS) k_p2m_fixed(int d, const int *
     }
 }
 
+template <int PP, int LPL>
+fmm_status run_p2m_fixed(Plan &P, const Particle<float> *sp, float inv_h, unsigned *amax, const float *s)
+{
+    constexpr int NC = (PP + 1) * (PP + 1), ROWS = 32 / LPL;
+    const size_t sh = sizeof(float) * P2M_WARPS * ROWS * NC;
+    static bool attr = false;
+    if (!attr) {
+        FMM_CUDA_TRY(cudaFuncSetAttribute(k_p2m_fixed<PP, LPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
+        attr = true;
+    }
+    const unsigned blocks = (unsigned)((P.nleaf + ROWS * P2M_WARPS - 1) / (ROWS * P2M_WARPS));
+    k_p2m_fixed<PP, LPL><<<blocks, 32 * P2M_WARPS, sh, P.stream>>>(P.d, P.cell_start, sp, inv_h, (float *)P.M[P.d], s, amax);
+    return FMM_OK;
+}
+
+// lanes per leaf: the fewest that give every SM 8 warps and no lane more than about 6 charges (beyond 8 the
+// shuffles of the (p+1)^2 sums cost more than the charges)
 template <int PP>
 fmm_status launch_p2m_fixed(Plan &P, const Particle<float> *sp, float inv_h, unsigned *amax, const float *s)
 {
-    constexpr int NC = (PP + 1) * (PP + 1);
-    const size_t sh = sizeof(float) * P2M_WARPS * 32 * NC;
-    static bool attr = false;
-    if (!attr) {
-        FMM_CUDA_TRY(cudaFuncSetAttribute(k_p2m_fixed<PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
-        attr = true;
+    int lpl = 1;
+    while (lpl < 8 && (P.nleaf * lpl < 32 * 1216 || (double)P.N > 6.0 * lpl * (double)P.nleaf)) lpl *= 2;
+    switch (lpl) {
+    case 1: return run_p2m_fixed<PP, 1>(P, sp, inv_h, amax, s);
+    case 2: return run_p2m_fixed<PP, 2>(P, sp, inv_h, amax, s);
+    case 4: return run_p2m_fixed<PP, 4>(P, sp, inv_h, amax, s);
+    default: return run_p2m_fixed<PP, 8>(P, sp, inv_h, amax, s);
     }
-    const int64_t rows = P.nleaf;
-    const unsigned blocks = (unsigned)((rows + 32 * P2M_WARPS - 1) / (32 * P2M_WARPS));
-    k_p2m_fixed<PP><<<blocks, 32 * P2M_WARPS, sh, P.stream>>>(P.d, P.cell_start, sp, inv_h, (float *)P.M[P.d], s, amax);
-    return FMM_OK;
 }
 
 template <typename T>
@@ -701,12 +724,10 @@ fmm_status upward_t(Plan &P, bool solute_only)
         fmm_status st = tc ? tc_clear_amax(P) : res_clear_amax(P);
         if (st != FMM_OK) return st;
     }
-    // fp16 split: the P2M at a compile-time order folds the level maximum of |Mhat s| in as it writes.  It
-    // runs one lane per leaf, so it is used for deep trees of sparse leaves (the benchmark boxes: 262,144
-    // leaves of ~4 charges); shallow trees of dense leaves keep the thread-per-(leaf, order) kernel
+    // fp16 split: the P2M at a compile-time order folds the level maximum of |Mhat s| in as it writes.  Leaves so
+    // full that 8 lanes each would run long keep the thread-per-(leaf, order) kernel
     bool amax_ready = false;
-    const bool lane_per_leaf = P.nleaf >= 32768 && (double)P.N <= 12.0 * (double)P.nleaf;
-    if (std::is_same<T, float>::value && lane_per_leaf &&
+    if (std::is_same<T, float>::value && (double)P.N <= 128.0 * (double)P.nleaf &&
         (P.p == 4 || P.p == 6 || P.p == 8 || P.p == 10 || P.p == 12)) {
         unsigned *amax = nullptr;
         if (tc) {

@@ -40,6 +40,7 @@ __host__ __device__ inline int n_il(int ws)
     return a * a * a - b * b * b;
 }
 
+constexpr int ERR_WORDS = 4;
 enum : int { ERRF_NONFINITE = 1, ERRF_INTERNAL = 2, ERRF_TIMEOUT = 4 };
 
 __host__ __device__ inline int ncoef(int p) { return (p + 1) * (p + 1); }
@@ -142,6 +143,7 @@ struct Plan {
     uint8_t *in_sol = nullptr;
     double *wpos = nullptr;        // [N][3] wrapped input positions (original order)
     int *key = nullptr;            // [N] leaf of each particle
+    int *found = nullptr;          // [N] particles by leaf, in any order within one
     int *perm = nullptr;           // [N] sorted slot -> original index
     int *sleaf = nullptr;          // [N] leaf of each sorted slot
     int *cell_start = nullptr;     // [nleaf + 1]
@@ -168,7 +170,8 @@ struct Plan {
     double *red_partial = nullptr;  // partial sums
     double *red_out = nullptr;      // [32] final FP64 scalars
     double *h_out = nullptr;        // pinned host mirror
-    int *d_err = nullptr;  // [0] error flags, [1] solute charges of the call
+    int *d_err = nullptr;  // [0] error flags, [1] solute charges of the call, [2], [3] blocks done (reductions);
+                           // cell_fill lies behind these ERR_WORDS words (one clear per call)
     Tables tab;
     cudaEvent_t ev[12] = {};
     cudaEvent_t ev_m2l[18] = {};  // around each level's M2L launch (full pass)
@@ -295,11 +298,11 @@ fmm_status solute_prepare(Plan &P);
 void solute_free(Plan &P);
 // where the sort lists the solute slots (at most *cap; their count is P.d_err[1])
 int *solute_list(Plan &P, int *cap);
-// right after the sort: copy the solute count to the host asynchronously
+// right after the sort: mark the fork of the solute pass and copy the solute count to the host asynchronously
 fmm_status solute_count(Plan &P);
 // the host copy of the last solute count (valid once the plan's stream has passed the copy)
 int solute_count_host(const Plan &P);
-// right after the sort (P.overlap): the solute-only expansions on the pass's side stream, Phi_u at every charge on
+// behind the sort (P.overlap): the solute-only expansions on the pass's side stream, Phi_u at every charge on
 // the near stream when that is forked; grids cover the largest count and the device count decides
 fmm_status solute_fork(Plan &P);
 // after the full pass's upward sweep (P.overlap): the solvent's FP64 field at the active cells on the side stream

@@ -193,38 +193,184 @@ __global__ void __launch_bounds__(P2P_THREADS) k_p2p_tile(int d, int ws, int bx,
     }
 }
 
-// near-field solute-solvent pair sum: out_i = q_i sum_{j in NF(i), j solvent} q_j / r_ij
-// for solute i, 0 otherwise
+// near-field solute-solvent pair sum of every solute slot: out_i = q_i sum_{j in NF(i), j solvent} q_j / r_ij (the
+// slots of the solvent are not read).  The sum runs over the neighbour leaves and their charges in order, in T: the
+// solute-solvent energy is a small difference of it and the far field, so another order would show.
+// A block looks at 128 slots.  Where only a few are solute, it takes them one at a time, all threads computing the
+// terms and one adding them up from shared memory: as one thread's whole work a lone ion's ~1,000 sources took
+// 31-127 us, each term a chain of loads.  Where many are, each of their threads sums its own.
+// SC: also the soft-core form of these pairs, r -> reff = (alpha lambda A^c + r^c)^(1/c) (the paper's soft-core
+// form, which it notes applies to the electrostatic NF term), in FP64 from the stored coordinates:
+// sc[s] = q_i sum_j q_j / reff and sc[N + s] = -(alpha A^c / c) q_i sum_j q_j / (reff (alpha lambda A^c + r^c)).
+// alpha_Ac = alpha A^c; lambda is read from device memory.
+constexpr int UV_THREADS = 128;
+constexpr int UV_FEW = 6;       // solute slots of a block up to which it works on one at a time
+constexpr int UV_CHUNK = 1024;  // terms staged at once
+
+struct UvSoft {
+    int c;
+    double b0, ic;  // alpha lambda A^c and 1/c
+};
+
 template <typename T>
-__global__ void k_p2p_uv(int64_t N, int d, int ws, T h, const int *__restrict__ start, const int *__restrict__ sleaf,
-                         const Particle<T> *__restrict__ sp, const uint8_t *__restrict__ sol, T *__restrict__ out)
+__device__ __forceinline__ void uv_soft_term(const Particle<T> &pi, const Particle<T> &pj, int dx, int dy, int dz, T h,
+                                             const UvSoft &f, double &e, double &de)
 {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= N) return;
-    if (!sol[s]) {
-        out[s] = 0;
+    const double ux = (double)pi.x - (double)dx * (double)h - (double)pj.x,
+                 uy = (double)pi.y - (double)dy * (double)h - (double)pj.y,
+                 uz = (double)pi.z - (double)dz * (double)h - (double)pj.z;
+    const double base = f.b0 + pow(sqrt(ux * ux + uy * uy + uz * uz), (double)f.c);
+    const double reff = pow(base, f.ic);
+    e += (double)pj.q / reff;
+    de += (double)pj.q / (reff * base);
+}
+
+template <typename T>
+__device__ __forceinline__ T uv_term(const Particle<T> &pj, T ox, T oy, T oz)
+{
+    const T rx = ox - pj.x, ry = oy - pj.y, rz = oz - pj.z;
+    return pj.q * inv_sqrt<T>(rx * rx + ry * ry + rz * rz);
+}
+
+__device__ __forceinline__ double uv_block_sum(double v, double *part, int lane, int w)
+{
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) part[w] = v;
+    __syncthreads();
+    double a = part[0];
+    for (int k = 1; k < UV_THREADS / 32; ++k) a += part[k];
+    __syncthreads();
+    return a;
+}
+
+template <typename T, bool SC>
+__global__ void __launch_bounds__(UV_THREADS) k_p2p_uv(int64_t N, int d, int ws, T h, const int *__restrict__ start,
+                                                       const int *__restrict__ sleaf, const Particle<T> *__restrict__ sp,
+                                                       const uint8_t *__restrict__ sol, T *__restrict__ out, int c,
+                                                       double alpha_Ac, const double *__restrict__ lambda,
+                                                       double *__restrict__ sc)
+{
+    constexpr int NL_MAX = (2 * WS_MAX + 1) * (2 * WS_MAX + 1) * (2 * WS_MAX + 1);
+    __shared__ unsigned found[UV_THREADS / 32];
+    __shared__ int first[NL_MAX], pre[NL_MAX + 1];  // a neighbour leaf's first charge; charges of the leaves before it
+    __shared__ T term[UV_CHUNK];
+    __shared__ double part[UV_THREADS / 32];
+    const int64_t s0 = blockIdx.x * (int64_t)UV_THREADS;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool mine = s0 + threadIdx.x < N && sol[s0 + threadIdx.x];
+    const unsigned m = __ballot_sync(0xffffffffu, mine);
+    if (lane == 0) found[w] = m;
+    const int nsol = __syncthreads_count(mine);
+    if (nsol == 0) return;
+    const int side = 2 * ws + 1, nl = side * side * side, nside = 1 << d;
+    UvSoft f{};
+    if (SC) f = {c, alpha_Ac * *lambda, 1.0 / (double)c};
+    auto neighbour = [&](int leaf, int l, int &dx, int &dy, int &dz) {  // l-th neighbour leaf, x fastest
+        dx = l % side - ws;
+        dy = (l / side) % side - ws;
+        dz = l / (side * side) - ws;
+        const int x = leaf & (nside - 1), y = (leaf >> d) & (nside - 1), z = leaf >> (2 * d);
+        return ((x + dx) & (nside - 1)) + nside * (((y + dy) & (nside - 1)) + nside * ((z + dz) & (nside - 1)));
+    };
+    if (nsol > UV_FEW) {
+        if (!mine) return;
+        const int64_t s = s0 + threadIdx.x;
+        const int leaf = sleaf[s];
+        const Particle<T> pi = sp[s];
+        T acc = 0;
+        double e = 0.0, de = 0.0;
+        for (int l = 0; l < nl; ++l) {
+            int dx, dy, dz;
+            const int lc = neighbour(leaf, l, dx, dy, dz);
+            const T ox = pi.x - T(dx) * h, oy = pi.y - T(dy) * h, oz = pi.z - T(dz) * h;
+            for (int j = start[lc]; j < start[lc + 1]; ++j) {
+                if (sol[j]) continue;
+                const Particle<T> pj = sp[j];
+                acc += uv_term<T>(pj, ox, oy, oz);
+                if (SC) uv_soft_term<T>(pi, pj, dx, dy, dz, h, f, e, de);
+            }
+        }
+        out[s] = pi.q * acc;
+        if (SC) {
+            sc[s] = (double)pi.q * e;
+            sc[N + s] = -(alpha_Ac * f.ic) * (double)pi.q * de;
+        }
         return;
     }
-    int nside = 1 << d;
-    int leaf = sleaf[s];
-    int x = leaf % nside, y = (leaf / nside) % nside, z = leaf / (nside * nside);
-    Particle<T> pi = sp[s];
-    T acc = 0;
-    for (int dz = -ws; dz <= ws; ++dz)
-        for (int dy = -ws; dy <= ws; ++dy)
-            for (int dx = -ws; dx <= ws; ++dx) {
-                int xx = (x + dx + nside) & (nside - 1), yy = (y + dy + nside) & (nside - 1),
-                    zz = (z + dz + nside) & (nside - 1);
-                int c = xx + nside * (yy + nside * zz);
-                T ox = pi.x - T(dx) * h, oy = pi.y - T(dy) * h, oz = pi.z - T(dz) * h;
-                for (int j = start[c]; j < start[c + 1]; ++j) {
-                    if (sol[j]) continue;
-                    Particle<T> pj = sp[j];
-                    T rx = ox - pj.x, ry = oy - pj.y, rz = oz - pj.z;
-                    acc += pj.q * inv_sqrt<T>(rx * rx + ry * ry + rz * rz);
+    for (int v = 0; v < UV_THREADS / 32; ++v)
+        for (unsigned fm = found[v]; fm; fm &= fm - 1) {
+            const int64_t s = s0 + 32 * v + __ffs(fm) - 1;
+            const int leaf = sleaf[s];
+            const Particle<T> pi = sp[s];
+            for (int l = threadIdx.x; l < nl; l += UV_THREADS) {
+                int dx, dy, dz;
+                const int lc = neighbour(leaf, l, dx, dy, dz);
+                first[l] = start[lc];
+                pre[l + 1] = start[lc + 1] - start[lc];
+            }
+            if (threadIdx.x == 0) pre[0] = 0;
+            __syncthreads();
+            if (w == 0) {  // counts -> exclusive prefix
+                int base = 0;
+                for (int l0 = 0; l0 < nl; l0 += 32) {
+                    const int l = l0 + lane;
+                    int x = l < nl ? pre[l + 1] : 0;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, x, o);
+                        if (lane >= o) x += y;
+                    }
+                    if (l < nl) pre[l + 1] = base + x;
+                    base += __shfl_sync(0xffffffffu, x, 31);
                 }
             }
-    out[s] = pi.q * acc;
+            __syncthreads();
+            const int total = pre[nl];
+            T acc = 0;
+            double e = 0.0, de = 0.0;
+            for (int t0 = 0; t0 < total; t0 += UV_CHUNK) {
+                const int n = total - t0 < UV_CHUNK ? total - t0 : UV_CHUNK;
+                for (int t = threadIdx.x; t < n; t += UV_THREADS) {
+                    int lo = 0, hi = nl;  // the leaf of term t0 + t
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if (pre[mid] <= t0 + t) lo = mid;
+                        else hi = mid;
+                    }
+                    int dx, dy, dz;
+                    neighbour(leaf, lo, dx, dy, dz);
+                    const int j = first[lo] + t0 + t - pre[lo];
+                    const Particle<T> pj = sp[j];
+                    const T g = uv_term<T>(pj, pi.x - T(dx) * h, pi.y - T(dy) * h, pi.z - T(dz) * h);
+                    const bool solvent = !sol[j];
+                    term[t] = solvent ? g : T(0);
+                    if (SC && solvent) uv_soft_term<T>(pi, pj, dx, dy, dz, h, f, e, de);
+                }
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    int t = 0;
+                    for (; t + 8 <= n; t += 8) {
+                        T g[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) g[u] = term[t + u];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) acc += g[u];
+                    }
+                    for (; t < n; ++t) acc += term[t];
+                }
+                __syncthreads();
+            }
+            if (SC) {
+                e = uv_block_sum(e, part, lane, w);
+                de = uv_block_sum(de, part, lane, w);
+            }
+            if (threadIdx.x == 0) {
+                out[s] = pi.q * acc;
+                if (SC) {
+                    sc[s] = (double)pi.q * e;
+                    sc[N + s] = -(alpha_Ac * f.ic) * (double)pi.q * de;
+                }
+            }
+        }
 }
 
 }  // namespace
@@ -260,59 +406,6 @@ fmm_status launch_p2p_tile(Plan &P, T h, T *phi, T *field)
     return FMM_OK;
 }
 
-// The same sum together with the soft-core form of the solute-solvent near-field pairs, r -> reff =
-// (alpha lambda A^c + r^c)^(1/c) (the paper's soft-core form, which it notes applies to the electrostatic
-// NF term), in FP64 from the stored coordinates: sc[s] = q_i sum_j q_j / reff and
-// sc[N + s] = -(alpha A^c / c) q_i sum_j q_j / (reff (alpha lambda A^c + r^c)) for solute slot s, 0 elsewhere.
-// alpha_Ac = alpha A^c; lambda is read from device memory.
-template <typename T>
-__global__ void k_p2p_uv_sc(int64_t N, int d, int ws, T h, const int *__restrict__ start, const int *__restrict__ sleaf,
-                            const Particle<T> *__restrict__ sp, const uint8_t *__restrict__ sol, T *__restrict__ out,
-                            int c, double alpha_Ac, const double *__restrict__ lambda, double *__restrict__ sc)
-{
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= N) return;
-    if (!sol[s]) {
-        out[s] = 0;
-        sc[s] = 0.0;
-        sc[N + s] = 0.0;
-        return;
-    }
-    const double b0 = alpha_Ac * *lambda;
-    const double ic = 1.0 / (double)c;
-    int nside = 1 << d;
-    int leaf = sleaf[s];
-    int x = leaf % nside, y = (leaf / nside) % nside, z = leaf / (nside * nside);
-    Particle<T> pi = sp[s];
-    T acc = 0;
-    double e = 0.0, de = 0.0;
-    for (int dz = -ws; dz <= ws; ++dz)
-        for (int dy = -ws; dy <= ws; ++dy)
-            for (int dx = -ws; dx <= ws; ++dx) {
-                int xx = (x + dx + nside) & (nside - 1), yy = (y + dy + nside) & (nside - 1),
-                    zz = (z + dz + nside) & (nside - 1);
-                int cidx = xx + nside * (yy + nside * zz);
-                T ox = pi.x - T(dx) * h, oy = pi.y - T(dy) * h, oz = pi.z - T(dz) * h;
-                const double dox = (double)pi.x - (double)dx * (double)h, doy = (double)pi.y - (double)dy * (double)h,
-                             doz = (double)pi.z - (double)dz * (double)h;
-                for (int j = start[cidx]; j < start[cidx + 1]; ++j) {
-                    if (sol[j]) continue;
-                    Particle<T> pj = sp[j];
-                    T rx = ox - pj.x, ry = oy - pj.y, rz = oz - pj.z;
-                    acc += pj.q * inv_sqrt<T>(rx * rx + ry * ry + rz * rz);
-                    const double ux = dox - (double)pj.x, uy = doy - (double)pj.y, uz = doz - (double)pj.z;
-                    const double r = sqrt(ux * ux + uy * uy + uz * uz);
-                    const double base = b0 + pow(r, (double)c);
-                    const double reff = pow(base, ic);
-                    e += (double)pj.q / reff;
-                    de += (double)pj.q / (reff * base);
-                }
-            }
-    out[s] = pi.q * acc;
-    sc[s] = (double)pi.q * e;
-    sc[N + s] = -(alpha_Ac * ic) * (double)pi.q * de;
-}
-
 }  // namespace
 
 fmm_status launch_p2p(Plan &P, bool forces)
@@ -329,31 +422,26 @@ fmm_status launch_p2p(Plan &P, bool forces)
     return FMM_OK;
 }
 
+template <typename T>
+static void run_p2p_uv(Plan &P, T h)
+{
+    const unsigned blocks = blocks_for(P.N, UV_THREADS);
+    const Particle<T> *sp = (const Particle<T> *)P.sorted;
+    T *out = (T *)P.phi_nf + P.N;
+    if (P.sc_c > 0)
+        k_p2p_uv<T, true><<<blocks, UV_THREADS, 0, P.stream>>>(P.N, P.d, P.ws, h, P.cell_start, P.sleaf, sp, P.sorted_sol,
+                                                               out, P.sc_c, P.sc_alpha * pow(P.sc_A, (double)P.sc_c),
+                                                               P.sc_lambda, P.sc_out);
+    else
+        k_p2p_uv<T, false><<<blocks, UV_THREADS, 0, P.stream>>>(P.N, P.d, P.ws, h, P.cell_start, P.sleaf, sp,
+                                                                P.sorted_sol, out, 0, 0.0, nullptr, nullptr);
+}
+
 fmm_status launch_p2p_uv(Plan &P)
 {
-    int nside = 1 << P.d;
-    double h = P.box / nside;
-    if (P.sc_c > 0) {
-        const double alpha_Ac = P.sc_alpha * pow(P.sc_A, (double)P.sc_c);
-        if (P.precision == FMM_PREC_FP64)
-            k_p2p_uv_sc<double><<<blocks_for(P.N, 128), 128, 0, P.stream>>>(
-                P.N, P.d, P.ws, h, P.cell_start, P.sleaf, (const Particle<double> *)P.sorted, P.sorted_sol,
-                (double *)P.phi_nf + P.N, P.sc_c, alpha_Ac, P.sc_lambda, P.sc_out);
-        else
-            k_p2p_uv_sc<float><<<blocks_for(P.N, 128), 128, 0, P.stream>>>(
-                P.N, P.d, P.ws, (float)h, P.cell_start, P.sleaf, (const Particle<float> *)P.sorted, P.sorted_sol,
-                (float *)P.phi_nf + P.N, P.sc_c, alpha_Ac, P.sc_lambda, P.sc_out);
-        FMM_LAUNCH_CHECK(P);
-        return FMM_OK;
-    }
-    if (P.precision == FMM_PREC_FP64)
-        k_p2p_uv<double><<<blocks_for(P.N, 128), 128, 0, P.stream>>>(
-            P.N, P.d, P.ws, h, P.cell_start, P.sleaf, (const Particle<double> *)P.sorted, P.sorted_sol,
-            (double *)P.phi_nf + P.N);
-    else
-        k_p2p_uv<float><<<blocks_for(P.N, 128), 128, 0, P.stream>>>(
-            P.N, P.d, P.ws, (float)h, P.cell_start, P.sleaf, (const Particle<float> *)P.sorted, P.sorted_sol,
-            (float *)P.phi_nf + P.N);
+    const double h = P.box / (1 << P.d);
+    if (P.precision == FMM_PREC_FP64) run_p2p_uv<double>(P, h);
+    else run_p2p_uv<float>(P, (float)h);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }

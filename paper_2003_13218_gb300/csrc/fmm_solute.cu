@@ -219,6 +219,30 @@ __host__ __device__ inline int64_t map_off(int l, int l0)
     return ((((int64_t)1 << (3 * l)) - 1) / 7) - ((((int64_t)1 << (3 * (l0 + 1))) - 1) / 7);
 }
 
+// sum_k a[k stride] b[k], k < n, in 4 partial sums with 8 loads in flight (a column of an operator against a row of
+// coefficients: the loads' latency is what these small kernels wait for)
+template <typename T>
+__device__ __forceinline__ T dot8(const T *__restrict__ a, size_t stride, const T *b, int n)
+{
+    T s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+    int k = 0;
+    for (; k + 8 <= n; k += 8) {
+        T v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = a[(size_t)(k + u) * stride];
+        s0 += v[0] * b[k];
+        s1 += v[1] * b[k + 1];
+        s2 += v[2] * b[k + 2];
+        s3 += v[3] * b[k + 3];
+        s0 += v[4] * b[k + 4];
+        s1 += v[5] * b[k + 5];
+        s2 += v[6] * b[k + 6];
+        s3 += v[7] * b[k + 7];
+    }
+    for (; k < n; ++k) s0 += a[(size_t)k * stride] * b[k];
+    return (s0 + s1) + (s2 + s3);
+}
+
 // M2L terms of the dense levels 2..ld, one work item per (level, active source a, offset d of the window
 // [-2ws-1, 2ws+1]^3): part[l - 2][a][d] = T(d) . MU_a (Eq. Lcoeffdef) when the source lies in the interaction
 // list of the target t = s_a - d (wrapped).  At coarse levels several offsets reach the same target (its
@@ -243,14 +267,7 @@ __global__ void k_sol_dense_m2l(int p, int ld, int ws, const int *__restrict__ c
         const T *Ms = MU + ((size_t)l * NU_MAX + a) * nc;
         T *out = part + (((size_t)(l - 2) * NU_MAX + a) * W + b) * nc;
         for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-            T a0 = 0, a1 = 0;
-            int k = 0;
-            for (; k + 1 < nc; k += 2) {
-                a0 += Tp[(size_t)k * nc + j] * Ms[k];
-                a1 += Tp[(size_t)(k + 1) * nc + j] * Ms[k + 1];
-            }
-            if (k < nc) a0 += Tp[(size_t)k * nc + j] * Ms[k];
-            out[j] = a0 + a1;
+            out[j] = dot8<T>(Tp + j, nc, Ms, nc);
         }
     }
 }
@@ -264,7 +281,9 @@ __global__ void k_sol_dense(int p, int l, int ws, const int *__restrict__ cells,
                             const T *__restrict__ part, const T *__restrict__ l2lT, const T *__restrict__ Lpar,
                             T *__restrict__ Lout)
 {
-    __shared__ short hit[(4 * WS_MAX + 3) * (4 * WS_MAX + 3) * (4 * WS_MAX + 3)];
+    constexpr int W_MAX = (4 * WS_MAX + 3) * (4 * WS_MAX + 3) * (4 * WS_MAX + 3);
+    __shared__ int hit[W_MAX];  // part rows of this target, in offset order
+    __shared__ int nhit;
     __shared__ T sL[NC_MAX];
     const int nc = ncoef(p), n = 1 << l, h = 2 * ws + 1, side = 2 * h + 1, W = side * side * side;
     int tx, ty, tz;
@@ -274,37 +293,43 @@ __global__ void k_sol_dense(int p, int l, int ws, const int *__restrict__ cells,
     const int oct = (tx & 1) | ((ty & 1) << 1) | ((tz & 1) << 2);
     const T *Lp = Lpar + cell_index(l - 1, tx >> 1, ty >> 1, tz >> 1) * nc;
     for (int j = threadIdx.x; j < nc; j += blockDim.x) sL[j] = Lp[j];
-    for (int b = threadIdx.x; b < W; b += blockDim.x) {
-        const int dx = b % side - h, dy = (b / side) % side - h, dz = b / (side * side) - h;
-        int a = -1;
-        if (in_il(dx, dy, dz, tx, ty, tz, ws)) {
-            const int key = ((tx + dx + 4 * n) & (n - 1)) + n * (((ty + dy + 4 * n) & (n - 1)) +
-                                                                 n * ((tz + dz + 4 * n) & (n - 1)));
-            int lo = 0, hi = na;  // active cells are sorted and unique
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (act[mid] < key) lo = mid + 1;
-                else hi = mid;
+    if (threadIdx.x < 32) {  // the first warp collects the hits in order
+        int cnt = 0;
+        for (int b0 = 0; b0 < W; b0 += 32) {
+            const int b = b0 + threadIdx.x;
+            const int dx = b % side - h, dy = (b / side) % side - h, dz = b / (side * side) - h;
+            int a = -1;
+            if (b < W && in_il(dx, dy, dz, tx, ty, tz, ws)) {
+                const int key = ((tx + dx + 4 * n) & (n - 1)) + n * (((ty + dy + 4 * n) & (n - 1)) +
+                                                                     n * ((tz + dz + 4 * n) & (n - 1)));
+                int lo = 0, hi = na;  // active cells are sorted and unique
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (act[mid] < key) lo = mid + 1;
+                    else hi = mid;
+                }
+                if (lo < na && act[lo] == key) a = lo;
             }
-            if (lo < na && act[lo] == key) a = lo;
+            const unsigned m = __ballot_sync(0xffffffffu, a >= 0);
+            if (a >= 0) hit[cnt + __popc(m & ((1u << threadIdx.x) - 1u))] = a * W + b;
+            cnt += __popc(m);
         }
-        hit[b] = (short)a;
+        if (threadIdx.x == 0) nhit = cnt;
     }
     __syncthreads();
     const T *pl = part + (size_t)(l - 2) * NU_MAX * W * nc;
     for (int j = threadIdx.x; j < nc; j += blockDim.x) {
+        T acc = dot8<T>(l2lT + oct * nc + j, 8 * nc, sL, nc);
+        const int nh = nhit;
         T a0 = 0, a1 = 0;
-        int k = 0;
-        for (; k + 1 < nc; k += 2) {
-            a0 += l2lT[(size_t)k * (8 * nc) + oct * nc + j] * sL[k];
-            a1 += l2lT[(size_t)(k + 1) * (8 * nc) + oct * nc + j] * sL[k + 1];
+        int b = 0;
+#pragma unroll 4
+        for (; b + 1 < nh; b += 2) {
+            a0 += pl[(size_t)hit[b] * nc + j];
+            a1 += pl[(size_t)hit[b + 1] * nc + j];
         }
-        if (k < nc) a0 += l2lT[(size_t)k * (8 * nc) + oct * nc + j] * sL[k];
-        T acc = a0 + a1;
-        for (int b = 0; b < W; ++b) {
-            const int a = hit[b];
-            if (a >= 0) acc += pl[((size_t)a * W + b) * nc + j];
-        }
+        if (b < nh) a0 += pl[(size_t)hit[b] * nc + j];
+        acc += a0 + a1;
         Lout[cell_index(l, tx, ty, tz) * nc + j] = acc;
     }
 }
@@ -350,7 +375,7 @@ __global__ void k_sol_m2l(int p, int d, int ld, int ws, const int *__restrict__ 
         int tx, ty, tz;
         cell_xyz(tlist[(size_t)l * mt + b], n, tx, ty, tz);
         for (int j = threadIdx.x; j < nc; j += blockDim.x) {
-            T a0 = 0, a1 = 0;
+            T acc = 0;
             for (int s = 0; s < ncells[l]; ++s) {
                 int sx, sy, sz;
                 cell_xyz(cells[l * NU_MAX + s], n, sx, sy, sz);
@@ -358,14 +383,9 @@ __global__ void k_sol_m2l(int p, int d, int ld, int ws, const int *__restrict__ 
                 if (!in_il(dx, dy, dz, tx, ty, tz, ws)) continue;
                 const T *Tp = Top + (size_t)off_slot(dx, dy, dz, ws) * nc * nc + j;
                 const T *Ms = MU + ((size_t)l * NU_MAX + s) * nc;
-                int k = 0;
-                for (; k + 1 < nc; k += 2) {
-                    a0 += Tp[(size_t)k * nc] * Ms[k];
-                    a1 += Tp[(size_t)(k + 1) * nc] * Ms[k + 1];
-                }
-                if (k < nc) a0 += Tp[(size_t)k * nc] * Ms[k];
+                acc += dot8<T>(Tp, nc, Ms, nc);
             }
-            contrib[((size_t)l * mt + b) * nc + j] = a0 + a1;
+            contrib[((size_t)l * mt + b) * nc + j] = acc;
         }
     }
 }
@@ -413,14 +433,7 @@ __global__ void k_act_m2l(int p, int d, int ws, const int *__restrict__ il, cons
             for (int q = 0; q < (NC_MAX + 191) / 192; ++q) {
                 const int j = threadIdx.x + q * blockDim.x;
                 if (j >= nc) break;
-                double a0 = 0, a1 = 0;
-                int k = 0;
-                for (; k + 1 < nc; k += 2) {
-                    a0 += Tp[(size_t)k * nc + j] * sM[k];
-                    a1 += Tp[(size_t)(k + 1) * nc + j] * sM[k + 1];
-                }
-                if (k < nc) a0 += Tp[(size_t)k * nc + j] * sM[k];
-                acc[q] += a0 + a1;
+                acc[q] += dot8<double>(Tp + j, nc, sM, nc);
             }
         }
         double *out = part + ((size_t)((l - 2) * NU_MAX + i) * ng + g) * nc;
@@ -746,6 +759,7 @@ fmm_status solute_count(Plan &P)
     SoluteScratch *S = (SoluteScratch *)P.sol;
     if (!S) return FMM_ERR_INTERNAL;
     S->forked = S->act_done = false;  // a new call (a failed one may have left them set)
+    FMM_CUDA_TRY(cudaEventRecord(S->ev_sort, P.stream));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->h_count, P.d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, P.stream));
     FMM_CUDA_TRY(cudaEventRecord(S->ev_count, P.stream));
     S->count_pending = true;
@@ -756,7 +770,6 @@ fmm_status solute_fork(Plan &P)
 {
     SoluteScratch *S = (SoluteScratch *)P.sol;
     if (!S || !P.overlap || !solute_may_run(P)) return FMM_OK;
-    FMM_CUDA_TRY(cudaEventRecord(S->ev_sort, P.stream));
     FMM_CUDA_TRY(cudaStreamWaitEvent(S->side, S->ev_sort, 0));
     S->forked = true;
     fmm_status s = P.precision == FMM_PREC_FP64 ? solute_expand_t<double>(P, *S, S->side)
