@@ -379,7 +379,9 @@ namespace {
 
 // staged-tile launch: rows of BX leaves, BX a power of two up to min(32, side) chosen so that a row holds
 // about 128 target charges at the mean leaf occupancy (dense leaves: short rows, more blocks); the staging
-// capacity is twice the expected particle count of a tile's rows (at least 512 records), within 96 KB of
+// capacity is 1.25 times the expected particle count of a tile's rows plus 256 (a tile beyond it reads global memory;
+// twice the count plus 512 left room for one block less per SM: 10M charges 23.1 -> 22.2 ms, 100k at ws = 2 1.62 ->
+// 1.53 ms), within 96 KB of
 // shared memory
 template <typename T>
 fmm_status launch_p2p_tile(Plan &P, T h, T *phi, T *field)
@@ -397,7 +399,7 @@ fmm_status launch_p2p_tile(Plan &P, T h, T *phi, T *field)
     const int side = 2 * P.ws + 1, F = side * side * (bx + 2 * P.ws);
     const size_t head = ((sizeof(int) * (2 * F + 1) + 15) / 16) * 16;
     const double expect = (double)P.N / (double)P.nleaf * F;
-    size_t cap = (size_t)(2.0 * expect) + 512;
+    size_t cap = (size_t)(1.25 * expect) + 256;
     const size_t cap_max = (smem_max - head) / sizeof(Particle<T>);
     if (cap > cap_max) cap = cap_max;
     const unsigned blocks = (unsigned)((int64_t)n * n * (n / bx));
