@@ -150,7 +150,7 @@ fmm_status far_field_pass(Plan &P, bool gradient, bool solute_only, StageTimer *
         if (ev) cudaEventRecord(P.ev_m2l[2 * (l - 1)], P.stream);
         // with the fp16 split the upward pass left the planes split and the L2L is fused
         const bool fused = tc_available(P, l) && tc_translations(P);
-        if (tc_available(P, l)) TRY(launch_m2l_tc(P, l, solute_only, !fused));
+        if (tc_available(P, l)) TRY(launch_m2l_tc(P, l, solute_only));
         else if (res_available(P, l)) TRY(launch_m2l_res(P, l));
         else TRY(launch_m2l_simt(P, l));
         if (ev) cudaEventRecord(P.ev_m2l[2 * (l - 1) + 1], P.stream);

@@ -748,14 +748,10 @@ fmm_status upward_t(Plan &P, bool solute_only)
     }
     FMM_LAUNCH_CHECK(P);
     for (int l = P.d - 1; l >= 1; --l) {  // the top operator starts from level 1
-        // the tensor-core M2M into level l folds level l's maximum in (amax of level l + 1 is ready from
-        // the P2M or the previous M2M)
-        fmm_status st = tc ? tc_split_moments(P, l + 1, amax_ready) : FMM_OK;
-        if (st == FMM_OK) st = tc ? launch_m2m_tc(P, l) : launch_m2m(P, l);
+        fmm_status st = launch_m2m(P, l);
         if (st != FMM_OK) return st;
-        amax_ready = tc;
     }
-    return FMM_OK;
+    return tc ? tc_split_moments(P, amax_ready) : FMM_OK;
 }
 
 }  // namespace
@@ -833,9 +829,12 @@ void free_tables(Plan &P)
     cudaFree(P.tab.l2l64);
     cudaFree(P.tab.l2l32);
     cudaFree(P.tab.m2m64);
-    cudaFree(P.tab.m2m32);
-    cudaFree(P.tab.m2mP32);
-    cudaFree(P.tab.l2lP32);
+    cudaFree(P.tab.m2m_fold64);
+    cudaFree(P.tab.m2m_fold32);
+    cudaFree(P.tab.l2l_fold64);
+    cudaFree(P.tab.l2l_fold32);
+    cudaFree(P.tab.fold_cnt);
+    cudaFree(P.tab.fold_beg);
     cudaFree(P.tab.il);
     cudaFree(P.tab.G64);
     cudaFree(P.tab.G32);

@@ -92,9 +92,9 @@ struct Tables {
     double *l2l64 = nullptr;  // [8 NC][NC] L2L operators of the 8 child octants (row-major)
     float *l2l32 = nullptr;
     double *m2m64 = nullptr;  // [NC][8 NC] M2M operators (row-major)
-    float *m2m32 = nullptr;
-    float *m2mP32 = nullptr;  // M2M with each octant's K padded to a multiple of 8
-    float *l2lP32 = nullptr;  // L2L with K padded likewise
+    void *m2m_fold64 = nullptr, *m2m_fold32 = nullptr;  // nonzeros of octant 0's operators (fmm_translate.cu)
+    void *l2l_fold64 = nullptr, *l2l_fold32 = nullptr;
+    int *fold_cnt = nullptr, *fold_beg = nullptr;
     int *il = nullptr;        // [8][n_il(ws)] interaction list of each parity class, packed offsets (il_pack)
     double *G64 = nullptr;    // [8 NC][8 NC] top operator: M(1) -> L(1), input-major (fmm_top.cu)
     float *G32 = nullptr;
@@ -312,15 +312,14 @@ fmm_status solute_join(Plan &P);
 // joins the forked pass (or runs it) and finishes it; *done = false when the dense pass must run
 fmm_status launch_solute_pass(Plan &P, bool *done);
 
-// tensor-core M2L, and with the fp16 split also M2M and L2L (fmm_m2l_tc.cu)
+// tensor-core M2L, and with the fp16 split also L2L (fmm_m2l_tc.cu)
 bool tc_available(const Plan &P, int level);
-// fp16 split: M2M on the tensor cores and L2L fused into each level's M2L
+// fp16 split: L2L fused into each level's M2L
 bool tc_translations(const Plan &P);
 fmm_status tc_prepare(Plan &P);
-// fp16 split: balanced halo planes of M[level] (done by the upward pass before the M2M into level - 1);
-// amax_ready: the kernel that wrote M[level] has already folded the level's largest |Mhat s| into
-// tc_amax(P, level) (else it is computed here)
-fmm_status tc_split_moments(Plan &P, int level, bool amax_ready);
+// fp16 split: balanced halo planes of all levels (the end of the upward pass); leaf_amax_ready: the P2M has
+// already folded the deepest level's largest |Mhat s| into tc_amax (else it is computed here)
+fmm_status tc_split_moments(Plan &P, bool leaf_amax_ready);
 // fp16 split: the device word of level l's largest |Mhat s| (float bits), into which the kernel that produces
 // M[l] folds its maximum; tc_clear_amax clears the words of all levels (M and L) at the start of a far-field
 // pass; s(n,m) per real coefficient
@@ -329,12 +328,9 @@ fmm_status tc_clear_amax(Plan &P);
 // the same for L (largest |Lhat / s|) with the factors 1 / s; null without the fp16 split
 unsigned *tc_amaxL(Plan &P, int level, const float **sx);
 const float *tc_scale(const Plan &P);
-// fp16 split: M2M into level (< d) from the planes of level + 1
-fmm_status launch_m2m_tc(Plan &P, int level);
-// precise: at least the accuracy of the 3 x 3 bf16 split whatever the plan's option (solute-only pass);
-// split: (re)build the planes of M[level] first (always done for the bf16 splits).  With the fp16
-// split the L2L from level - 1 is included: L[level] = M2L + L2L.
-fmm_status launch_m2l_tc(Plan &P, int level, bool precise = false, bool split = true);
+// precise: at least the accuracy of the 3 x 3 bf16 split whatever the plan's option (solute-only pass).
+// With the fp16 split the L2L from level - 1 is included: L[level] = M2L + L2L.
+fmm_status launch_m2l_tc(Plan &P, int level, bool precise);
 void tc_free(Plan &P);
 
 // FP64 M2L by residue products on the tensor cores (fmm_m2l_res.cu): L[level] = M2L, without the L2L
@@ -342,6 +338,8 @@ bool res_available(const Plan &P, int level);
 // builds the state on an FP64 plan's first evaluation (a plan that is to run the mixed path never pays for it);
 // left for later while the plan's stream is being captured
 fmm_status res_ensure(Plan &P);
+// where the M2M into a level leaves its largest |Mhat s|, and s (null without the state)
+unsigned long long *res_amax(Plan &P, int level, const double **s);
 fmm_status res_clear_amax(Plan &P);  // at the start of a far-field pass
 fmm_status launch_m2l_res(Plan &P, int level);
 fmm_status res_share_operators(Plan &dst, const Plan &src);

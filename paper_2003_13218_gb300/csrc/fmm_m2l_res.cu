@@ -445,6 +445,13 @@ fmm_status res_clear_amax(Plan &P)
     return FMM_OK;
 }
 
+unsigned long long *res_amax(Plan &P, int l, const double **s)
+{
+    ResState *S = (ResState *)P.res;
+    *s = S ? S->s64 : nullptr;
+    return S ? S->amax + l : nullptr;
+}
+
 // L[l] = M2L of level l (the L2L from level l - 1 is added by launch_l2l)
 fmm_status launch_m2l_res(Plan &P, int l)
 {
@@ -452,8 +459,11 @@ fmm_status launch_m2l_res(Plan &P, int l)
     if (!S) return FMM_ERR_INTERNAL;
     const int np = 1 << (l - 1), nc = P.nc, n = S->c.n;
     const int64_t np2 = np + 2 * P.ws, cells = (int64_t)8 * np * np * np;
-    k_res_absmax<<<blocks_upto(cells, 8, 1216), 256, 0, P.stream>>>((const double *)P.M[l], cells, nc, S->s64, S->amax + l);
-    FMM_LAUNCH_CHECK(P);
+    if (l == P.d) {  // the M2M into a level folds its maximum in
+        k_res_absmax<<<blocks_upto(cells, 8, 1216), 256, 0, P.stream>>>((const double *)P.M[l], cells, nc, S->s64,
+                                                                        S->amax + l);
+        FMM_LAUNCH_CHECK(P);
+    }
     TcArgs a;
     memset(&a, 0, sizeof(a));
     a.np = np;

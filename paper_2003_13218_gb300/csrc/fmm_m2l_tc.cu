@@ -58,10 +58,10 @@ namespace fmm {
 
 namespace {
 
-// operator slots of the B tables: the noff(ws) M2L offsets, then M2M and L2L per child octant
+// operator slots of the B tables: the noff(ws) M2L offsets, then the L2L per child octant
 
 struct TcState {
-    bool f16 = false;               // fp16x2 split with balanced scaling (and tensor-core translations)
+    bool f16 = false;               // fp16x2 split with balanced scaling (and fused L2L)
     int pa = 0, pb = 0;             // terms of the plan's split
     int parts = 0;                  // terms stored (3 for the bf16 splits: the solute pass uses 3 x 3)
     int npad = 0, kp = 0;
@@ -78,7 +78,6 @@ struct TcState {
     size_t partL_elems = 0;
     int bx[9], by[9], bz[9];
     int groups[9], per_group[9];    // offset groups per tile (small levels run more CTAs)
-    int mgroups[9], mper_group[9];  // the same for the M2M into level l
     float *Lpart = nullptr;         // partial sums of the offset groups
     float *s32 = nullptr;           // [nc] s(n,m) per real coefficient (fp16 split)
     float *s32inv = nullptr;        // [nc] 1 / s(n,m)
@@ -179,16 +178,14 @@ __global__ void k_split_L(const float *__restrict__ L, int lev, int nc, int kp, 
 
 // FP64 operators -> split B tables [part][chunk][slot][j][k] (K-major, rows kp wide in chunks of kch):
 // slots < noff the M2L operators T[slot][k][j] (input-major), then per child
-// octant o the M2M operator (M2M[j][o nc + k], parent output j) and the L2L
-// operator (L2L[o nc + j][k], child output j).  fp16: balanced with gT,
-//   M2L  T~ = T / (s(k) s(j)),  M2M  S~ = S s(j) / s(k),  L2L  U~ = U s(k) / s(j);
-// bf16: the translation slots stay zero (unused).
+// octant o the L2L operator (L2L[o nc + j][k], child output j).  fp16: balanced with gT,
+//   M2L  T~ = T / (s(k) s(j)),  L2L  U~ = U s(k) / s(j);
+// bf16: the L2L slots stay zero (unused).
 template <bool F16>
-__global__ void k_split_ops(int noff, const double *__restrict__ T, const double *__restrict__ m2m,
-                            const double *__restrict__ l2l, int nc, int npad, int kp, int kch, int parts,
+__global__ void k_split_ops(int noff, const double *__restrict__ T, const double *__restrict__ l2l, int nc, int npad, int kp, int kch, int parts,
                             const double *__restrict__ s, uint16_t *__restrict__ ops, size_t part_elems)
 {
-    const int64_t total = (int64_t)(noff + 16) * npad * kp;
+    const int64_t total = (int64_t)(noff + 8) * npad * kp;
     const double gT = (double)pow2f(GAIN_T_EXP);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int k = (int)(e % kp);
@@ -199,15 +196,12 @@ __global__ void k_split_ops(int noff, const double *__restrict__ T, const double
             if (slot < noff) {
                 r = T[((int64_t)slot * nc + k) * nc + j];
                 if (F16) r = r / (s[k] * s[j]) * gT;
-            } else if (F16 && slot < noff + 8) {
-                const int o = slot - noff;
-                r = m2m[(int64_t)j * 8 * nc + o * nc + k] * s[j] / s[k] * gT;
             } else if (F16) {
-                const int o = slot - noff - 8;
+                const int o = slot - noff;
                 r = l2l[((int64_t)o * nc + j) * nc + k] * s[k] / s[j] * gT;
             }
         }
-        const int64_t at = chunk_at((int64_t)slot * npad + j, (int64_t)(noff + 16) * npad, k, kch);
+        const int64_t at = chunk_at((int64_t)slot * npad + j, (int64_t)(noff + 8) * npad, k, kch);
         for (int i = 0; i < parts; ++i) {
             if (F16) {
                 const __half t = __float2half_rn((float)r);
@@ -282,15 +276,34 @@ __global__ void k_group_sum(int64_t n, int groups, const float *__restrict__ par
 }
 
 // fp16 split: FP32 class-layout moments -> the two balanced fp16 halo planes, 8 coefficients per thread
-// (16-byte stores per plane); rows kp wide, zero beyond nc
-__global__ void k_split_halo16(const float *__restrict__ M, int np, int hw, int nc, int kp, const float *__restrict__ s,
-                               const unsigned *__restrict__ amax, uint16_t *__restrict__ planes, size_t part_elems)
+// (16-byte stores per plane); rows kp wide, zero beyond nc.  One launch for all levels, the deepest first.
+struct SplitLevel {
+    const float *M;
+    const unsigned *amax;
+    uint16_t *planes;
+    size_t part_elems;
+    int64_t end;  // threads of this level and those before it
+    int np;
+};
+struct SplitLevels {
+    SplitLevel l[8];
+    int64_t total;
+};
+
+__global__ void k_split_halo16(const __grid_constant__ SplitLevels lv, int hw, int nc, int kp, const float *__restrict__ s)
 {
-    const int np2 = np + 2 * hw;
     const int G = kp / 8;
-    const int64_t total = 8 * (int64_t)np2 * np2 * np2 * G;
-    const float g = pow2f(gain_m_exp(*amax));
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t0 < lv.total;
+         t0 += (int64_t)gridDim.x * blockDim.x) {
+        int i = 0;
+        int64_t t = t0, total = lv.l[0].end;
+        while (t0 >= lv.l[i].end) {
+            t = t0 - lv.l[i].end;
+            total = lv.l[i + 1].end - lv.l[i].end;
+            ++i;
+        }
+        const int np = lv.l[i].np, np2 = np + 2 * hw;
+        const float g = pow2f(gain_m_exp(__ldg(lv.l[i].amax)));
         const int64_t cell = t / G;
         const int k0 = (int)(t - cell * G) * 8;
         const int hx = (int)(cell % np2);
@@ -298,26 +311,26 @@ __global__ void k_split_halo16(const float *__restrict__ M, int np, int hw, int 
         const int hzc = (int)(cell / ((int64_t)np2 * np2));
         const int c = hzc / np2, hz = hzc % np2;
         const int px = ((hx - hw) % np + np) % np, py = ((hy - hw) % np + np) % np, pz = ((hz - hw) % np + np) % np;
-        const float *row = M + ((int64_t)c * np * np * np + px + (int64_t)np * (py + (int64_t)np * pz)) * nc;
+        const float *row = lv.l[i].M + ((int64_t)c * np * np * np + px + (int64_t)np * (py + (int64_t)np * pz)) * nc;
         uint32_t hi[4], lo[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int w = 0; w < 4; ++w) {
             uint16_t h2[2], l2[2];
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const int k = k0 + 2 * i + u;
+                const int k = k0 + 2 * w + u;
                 const float v = k < nc ? row[k] * (__ldg(s + k) * g) : 0.f;
-                const __half t0 = __float2half_rn(v);
-                const __half t1 = __float2half_rn(v - __half2float(t0));
-                h2[u] = __half_as_ushort(t0);
-                l2[u] = __half_as_ushort(t1);
+                const __half t0h = __float2half_rn(v);
+                const __half t1h = __float2half_rn(v - __half2float(t0h));
+                h2[u] = __half_as_ushort(t0h);
+                l2[u] = __half_as_ushort(t1h);
             }
-            hi[i] = (uint32_t)h2[0] | ((uint32_t)h2[1] << 16);
-            lo[i] = (uint32_t)l2[0] | ((uint32_t)l2[1] << 16);
+            hi[w] = (uint32_t)h2[0] | ((uint32_t)h2[1] << 16);
+            lo[w] = (uint32_t)l2[0] | ((uint32_t)l2[1] << 16);
         }
-        uint16_t *out = planes + chunk_at(cell, total / G, k0, kchunk_of(128));
+        uint16_t *out = lv.l[i].planes + chunk_at(cell, total / G, k0, kchunk_of(128));
         *reinterpret_cast<uint4 *>(out) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4 *>(out + part_elems) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        *reinterpret_cast<uint4 *>(out + lv.l[i].part_elems) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
 }
 
@@ -624,7 +637,7 @@ void fill_common(const Plan &P, const TcState *S, int pa, int pb, TcArgs &a)
 {
     a.nc = P.nc;
     a.npad = S->npad;
-    a.nslots = S->noff + 16;
+    a.nslots = S->noff + 8;
     a.stages = tc_stages(pa, pb, S->npad, S->sw);
     // instruction descriptor: FP32 accumulator, A and B both bf16 (format 1) or both fp16 (format 0),
     // K-major, N >> 3 at bit 17, M >> 4 at bit 24
@@ -641,8 +654,6 @@ void fill_common(const Plan &P, const TcState *S, int pa, int pb, TcArgs &a)
     a.acc_group = P.acc_group;
     a.wait_ns = P.wait_ns;
     a.inject_stall = P.inject_stall ? 1 : 0;
-    a.src_np2 = 0;
-    a.out_np = 0;
     a.amaxL = nullptr;
     a.ws = P.ws;
     a.n_il = n_il(P.ws);
@@ -733,24 +744,24 @@ fmm_status tc_prepare(Plan &P)
         FMM_CUDA_TRY(cudaMemcpyAsync(S->s32inv, h_inv, sizeof(float) * P.nc, cudaMemcpyHostToDevice, P.stream));
     }
     // operator tables
-    S->ops_part_elems = (size_t)(S->noff + 16) * S->npad * S->kp;
+    S->ops_part_elems = (size_t)(S->noff + 8) * S->npad * S->kp;
     FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_part_elems * S->parts));
     if (S->f16)
-        k_split_ops<true><<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.tab.m2m64, P.tab.l2l64, P.nc, S->npad, S->kp,
+        k_split_ops<true><<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.tab.l2l64, P.nc, S->npad, S->kp,
                                                       kchunk_of(S->sw), S->parts, S->s64, S->ops, S->ops_part_elems);
     else
-        k_split_ops<false><<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, nullptr, nullptr, P.nc, S->npad, S->kp,
+        k_split_ops<false><<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, nullptr, P.nc, S->npad, S->kp,
                                                        kchunk_of(S->sw), S->parts, nullptr, S->ops, S->ops_part_elems);
     FMM_LAUNCH_CHECK(P);
     {
         TcMaps &m = S->maps[0];  // the operator maps, the same on every level
         TRY_TC(encode_operators(enc, &m.bS, S->f16 ? &m.bP : nullptr, S->f16 ? &m.bC : nullptr, type_of(S), S->ops,
-                                chunks_of(S), S->parts, S->npad, S->noff + 16, S->npad, S->sw));
+                                chunks_of(S), S->parts, S->npad, S->noff + 8, S->npad, S->sw));
         if (!S->f16) m.bP = m.bC = m.bS;  // unused kernel parameters
     }
     if (S->f16) {
         TRY_TC(encode_operators(enc, &S->mapB2[0], &S->mapB2[1], &S->mapB2[2], type_of(S), S->ops, chunks_of(S), S->parts,
-                                S->npad, S->noff + 16, S->npad / 2, S->sw));
+                                S->npad, S->noff + 8, S->npad / 2, S->sw));
         TcKernel kp2 = pick_pair_kernel(S->npad / 16);
         if (!kp2) return FMM_ERR_INTERNAL;
         FMM_CUDA_TRY(cudaFuncSetAttribute((const void *)kp2, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -782,13 +793,6 @@ fmm_status tc_prepare(Plan &P)
         split_offsets(n_il(P.ws) + (S->f16 ? 1 : 0), tiles, 27, sms, S->groups[l], S->per_group[l]);
         if (S->groups[l] > 1) {
             size_t need = (size_t)S->groups[l] * 8 * np * np * np * P.nc;
-            if (need > lpart_elems) lpart_elems = need;
-        }
-        // M2M into level l - 1 (natural side np, bricks of the level-l planes)
-        const int mtiles = (np / S->bx[l]) * (np / S->by[l]) * (np / S->bz[l]);
-        split_offsets(8, mtiles, 8, sms, S->mgroups[l - 1], S->mper_group[l - 1]);
-        if (S->f16 && S->mgroups[l - 1] > 1) {
-            size_t need = (size_t)S->mgroups[l - 1] * np * np * np * P.nc;
             if (need > lpart_elems) lpart_elems = need;
         }
     }
@@ -834,68 +838,30 @@ const float *tc_scale(const Plan &P)
     return S && S->f16 ? S->s32 : nullptr;
 }
 
-// fp16 split: the balanced halo planes of M[l]; the level's largest |M^ s| is computed first unless the
-// kernel that wrote M[l] folded it in already
-fmm_status tc_split_moments(Plan &P, int l, bool amax_ready)
+// fp16 split: the balanced halo planes of every level; a level's largest |M^ s| was folded in by the M2M that wrote
+// it, the deepest one's by the P2M (leaf_amax_ready) or it is computed here
+fmm_status tc_split_moments(Plan &P, bool leaf_amax_ready)
 {
     TcState *S = (TcState *)P.tc;
-    if (!S || !S->f16 || l < 2 || l > P.d) return FMM_ERR_INTERNAL;
-    const int np = 1 << (l - 1);
-    const int64_t np2 = np + 2 * P.ws;
-    const int64_t ncell = (int64_t)8 * np * np * np;
-    if (!amax_ready) {
+    if (!S || !S->f16) return FMM_ERR_INTERNAL;
+    if (!leaf_amax_ready) {
+        const int64_t ncell = (int64_t)1 << (3 * P.d);
         k_absmax<<<(unsigned)((ncell + 7) / 8 < 1216 ? (ncell + 7) / 8 : 1216), 256, 0, P.stream>>>(
-            (const float *)P.M[l], ncell, P.nc, S->s32, S->amax + l);
+            (const float *)P.M[P.d], ncell, P.nc, S->s32, S->amax + P.d);
         FMM_LAUNCH_CHECK(P);
     }
-    const int64_t nthr = 8 * np2 * np2 * np2 * (S->kp / 8);
-    k_split_halo16<<<(unsigned)((nthr + 255) / 256 < 8 * 1216 ? (nthr + 255) / 256 : 8 * 1216), 256, 0, P.stream>>>(
-        (const float *)P.M[l], np, P.ws, P.nc, S->kp, S->s32, S->amax + l, S->planes[l], S->part_elems[l]);
-    FMM_LAUNCH_CHECK(P);
-    return FMM_OK;
-}
-
-// fp16 split: M2M into level l (< d) from the split planes of level l + 1
-fmm_status launch_m2m_tc(Plan &P, int l)
-{
-    TcState *S = (TcState *)P.tc;
-    if (!S || !S->f16 || l < 1 || l >= P.d) return FMM_ERR_INTERNAL;
-    const int src = l + 1;
-    const int n = 1 << l;  // natural side of level l = parent side of the level-(l+1) planes
-    TcArgs a;
-    fill_common(P, S, S->pa, S->pb, a);
-    a.mode = 1;
-    a.gchunks = a.gsteps = 0;  // translations keep every product
-    a.np = n;
-    a.bx = S->bx[src];
-    a.by = S->by[src];
-    a.bz = S->bz[src];
-    a.rows = a.bx * a.by * a.bz;
-    a.tiles_x = n / a.bx;
-    a.tiles_y = n / a.by;
-    a.tiles_per_class = a.tiles_x * a.tiles_y * (n / a.bz);
-    a.groups = S->mgroups[l];
-    a.per_group = S->mper_group[l];
-    a.n_off = 8;
-    a.src_np2 = n + 2 * P.ws;
-    a.out_np = n >> 1;
-    a.L = (float *)P.M[l];
-    a.post = S->s32inv;
-    a.amax = S->amax + src;
-    // level l's largest |M^ s| (the gain of its planes) is folded in by whoever writes M[l]
-    a.amax_out = a.groups == 1 ? S->amax + l : nullptr;
-    a.sx = S->s32;
-    TcKernel k = pick_kernel(S->pa, S->pb, S->npad / 16, S->sw);
-    if (!k) return FMM_ERR_INTERNAL;
-    const unsigned grid = (unsigned)a.tiles_per_class * (unsigned)a.groups;
-    k<<<grid, TC_THREADS, tc_smem_bytes(S->pa, S->pb, S->npad, S->sw), P.stream>>>(S->maps[src], a);
-    FMM_LAUNCH_CHECK(P);
-    if (a.groups > 1) {
-        const int64_t cnt = (int64_t)n * n * n * P.nc;
-        k_group_sum<<<(unsigned)((cnt + 255) / 256 < 2048 ? (cnt + 255) / 256 : 2048), 256, 0, P.stream>>>(
-            cnt, a.groups, S->Lpart, a.L, P.nc, S->s32, S->amax + l);
-        FMM_LAUNCH_CHECK(P);
+    SplitLevels lv;
+    memset(&lv, 0, sizeof(lv));
+    int i = 0;
+    for (int l = P.d; l >= 2; --l, ++i) {
+        const int np = 1 << (l - 1);
+        const int64_t np2 = np + 2 * P.ws;
+        lv.total += 8 * np2 * np2 * np2 * (S->kp / 8);
+        lv.l[i] = {(const float *)P.M[l], S->amax + l, S->planes[l], S->part_elems[l], lv.total, np};
     }
+    const int64_t nb = (lv.total + 255) / 256;
+    k_split_halo16<<<(unsigned)(nb < 8 * 1216 ? nb : 8 * 1216), 256, 0, P.stream>>>(lv, P.ws, P.nc, S->kp, S->s32);
+    FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
 
@@ -906,7 +872,6 @@ static bool m2l_args(const Plan &P, const TcState *S, int l, bool precise, int p
     const int np = 1 << (l - 1);
     fill_common(P, S, pa, pb, a);
     if (precise) a.gchunks = a.gsteps = 0;  // the solute-only pass keeps every product
-    a.mode = 0;
     a.np = np;
     a.bx = S->bx[l];
     a.by = S->by[l];
@@ -934,7 +899,7 @@ static bool m2l_args(const Plan &P, const TcState *S, int l, bool precise, int p
     return pair;
 }
 
-fmm_status launch_m2l_tc(Plan &P, int l, bool precise, bool split)
+fmm_status launch_m2l_tc(Plan &P, int l, bool precise)
 {
     TcState *S = (TcState *)P.tc;
     if (!S) return FMM_ERR_INTERNAL;
@@ -944,10 +909,6 @@ fmm_status launch_m2l_tc(Plan &P, int l, bool precise, bool split)
     int np = 1 << (l - 1);
     int64_t np2 = np + 2 * P.ws;
     if (S->f16) {
-        if (split) {
-            fmm_status st = tc_split_moments(P, l, false);
-            if (st != FMM_OK) return st;
-        }
         // parent-level local expansion for the fused L2L; its largest |L^ / s| was folded in by the level
         // l - 1 launch (levels run in order)
         const int64_t ncl = (int64_t)np * np * np;

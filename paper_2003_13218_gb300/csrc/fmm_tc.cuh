@@ -54,16 +54,13 @@ struct TcMaps {
 };
 
 struct TcArgs {
-    int mode;               // 0: M2L (+ fused L2L), 1: M2M
     int np, bx, by, bz, rows, tiles_x, tiles_y, tiles_per_class;
     int nc, npad, stages;
     int nslots;             // operator slots of the B tables
     int groups, per_group;  // the offsets split over `groups` CTAs per tile (small levels)
-    int n_off;              // offsets: 189 (+1 with the fused L2L) or 8 (M2M)
-    int src_np2;            // M2M: halo'd side of the child level's planes
+    int n_off;              // offsets: 189 or 875 (+1 with the fused L2L)
     int ws, n_il, noff;     // well-separatedness, interaction-list length, M2L operator slots
-    int out_np;             // M2M: class-layout side of the parent level (0 at level 0)
-    const int *il;          // M2L: the interaction list of each class, [8][n_il] packed offsets (il_pack)
+    const int *il;          // the interaction list of each class, [8][n_il] packed offsets (il_pack)
     uint32_t idesc;
     uint32_t gchunks;       // fp16x2 M2L offsets: products per K chunk, 2 bits per chunk (0 = all 3), FMM_OPT_M2L_GRADE
     uint32_t gsteps;        // in a 3-product chunk, the first K16 step from which x1 y0 is dropped, 3 bits per chunk
@@ -73,7 +70,7 @@ struct TcArgs {
     int inject_stall;       // test hook (single-CTA kernel): the MMA issuer first waits on a barrier nothing arrives on
     float *L;               // output level array (L of the level, or M of the parent level)
     float *Lpart;           // [groups][level cells][nc] partial sums when groups > 1
-    const float *post;      // fp16 split: s(j) (M2L) or 1 / s(j) (M2M) per output coefficient, else null
+    const float *post;      // fp16 split: s(j) per output coefficient, else null
     const unsigned *amax;   // fp16 split: largest |M^ s| of the A planes (gM follows from it)
     const unsigned *amaxL;  // fused L2L: largest |L^ / s| of the parent planes (gL), else null
     // residue products (FP64 path): modulus mod0 + m of `mods` in block order, planes and results by m
@@ -82,7 +79,7 @@ struct TcArgs {
     int16_t *resid;         // [groups][moduli of the launch][level cells][nc]
     int nmods;
     unsigned *amax_out;     // fp16 split, one offset group: fold max_i |out_i sx(i)| of the written rows in here
-    const float *sx;        // with amax_out: s(i) (M2M output, |M^ s|) or 1 / s(i) (M2L output, |L^ / s|)
+    const float *sx;        // with amax_out: 1 / s(i)
     int *err;
 };
 
@@ -744,16 +741,12 @@ __device__ __forceinline__ void finish_residues(int (&acc)[NCH * 16], const TcAr
                       a.resid + ((int64_t)grp * a.nmods + mod) * cells * a.nc, a.nc, lane);
 }
 
-// One CTA sums, for 128 target rows, the products of a list of offsets:
-//   mode 0 (M2L): the 189 interaction-list offsets of parity class `cls`, A
-//     from the halo'd source planes of the level; with fused L2L (fp16 split)
-//     a 190th offset whose A is the parent level's local expansion at the
-//     targets' parents (natural-order planes) and whose B is the L2L operator
-//     of child octant `cls`; its accumulator is scaled by gM / gL.
-//   mode 1 (M2M): the 8 child octants o, A from class plane o of the child
-//     level's planes at the targets' own coordinates, B the M2M operator of o;
-//     targets are a brick of the parent level in natural order, written to its
-//     class layout.
+// One CTA sums, for 128 target rows, the products of a list of offsets: the
+// 189 (875) interaction-list offsets of parity class `cls`, A from the halo'd
+// source planes of the level; with fused L2L (fp16 split) one more offset whose
+// A is the parent level's local expansion at the targets' parents (natural-order
+// planes) and whose B is the L2L operator of child octant `cls`; its accumulator
+// is scaled by gM / gL.
 // PA, PB: terms of the A and B operands; NCH: output coefficients / 16 (the
 // accumulator width held in registers); SW: bytes per swizzled operand row.
 template <int PA, int PB, int NCH, int SW, bool RES = false>
@@ -787,12 +780,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const int mod = RES ? (int)blockIdx.x / per_mod : 0;
     const int block = (int)blockIdx.x - mod * per_mod;
     const int grp = block % a.groups;
-    const int cls = a.mode == 0 ? (block / a.groups) & 7 : 0;
-    const int tile = a.mode == 0 ? (block / a.groups) >> 3 : block / a.groups;
+    const int cls = (block / a.groups) & 7;
+    const int tile = (block / a.groups) >> 3;
     const int o_begin = grp * a.per_group;
     const int o_end = o_begin + a.per_group < a.n_off ? o_begin + a.per_group : a.n_off;
     const int nloc = o_end > o_begin ? o_end - o_begin : 0;
-    const bool has_l2l = a.mode == 0 && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end;
+    const bool has_l2l = a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end;
     const AccGroups groups(nloc, has_l2l, a.acc_group);
     const int x0 = (tile % a.tiles_x) * a.bx;
     const int y0 = ((tile / a.tiles_x) % a.tiles_y) * a.by;
@@ -840,8 +833,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         {
             // ---------------- producer: TMA loads of the A brick and the B operator
             constexpr int KC = (NCH + K16 - 1) / K16;
-            const ChunkPlan<KC> graded_plan(kGradable && a.mode == 0 ? a.gchunks : 0u,
-                                            kGradable && a.mode == 0 ? a.gsteps : 0u, PB == 2 ? 3 : PA + PB, K16);
+            const ChunkPlan<KC> graded_plan(kGradable ? a.gchunks : 0u,
+                                            kGradable ? a.gsteps : 0u, PB == 2 ? 3 : PA + PB, K16);
             const uint32_t full0 = smem_u32(&bar_full[0]), empty0 = smem_u32(&bar_empty[0]);
             int it = 0, s = 0;
             uint32_t phase = 1;
@@ -872,25 +865,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     }
                 }
             };
-            if (a.mode == 0) {
-                // the source brick sits at parent offset (c + delta) >> 1 in [-ws, ws], halo width ws
-                const int w = a.ws, o_il = o_end < a.n_il ? o_end : a.n_il;
-                IlWalk walk(a.il + cls * a.n_il, o_begin, o_il, lane);
-                for (int k = 0; k < o_il - o_begin && ok; ++k) {
-                    int dx, dy, dz;
-                    walk.get(k, dx, dy, dz);
-                    const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
-                    const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-                    load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w, 8 * np2,
-                                off_slot(dx, dy, dz, w), true);
-                }
-                // fused L2L: the parents' local expansions (natural order, no halo)
-                if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
-                    load_offset(true, x0, y0, z0, a.np, a.noff + 8 + cls, false);
-            } else {
-                for (int o = o_begin; o < o_end && ok; ++o)
-                    load_offset(false, x0 + a.ws, y0 + a.ws, o * a.src_np2 + z0 + a.ws, 8 * a.src_np2, a.noff + o, false);
+            // the source brick sits at parent offset (c + delta) >> 1 in [-ws, ws], halo width ws
+            const int w = a.ws, o_il = o_end < a.n_il ? o_end : a.n_il;
+            IlWalk walk(a.il + cls * a.n_il, o_begin, o_il, lane);
+            for (int k = 0; k < o_il - o_begin && ok; ++k) {
+                int dx, dy, dz;
+                walk.get(k, dx, dy, dz);
+                const int sx = cx + dx, sy = cy + dy, sz = cz + dz;
+                const int scls = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
+                load_offset(false, x0 + (sx >> 1) + w, y0 + (sy >> 1) + w, scls * np2 + z0 + (sz >> 1) + w, 8 * np2,
+                            off_slot(dx, dy, dz, w), true);
             }
+            // fused L2L: the parents' local expansions (natural order, no halo)
+            if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
+                load_offset(true, x0, y0, z0, a.np, a.noff + cls, false);
             if (el) {
                 produced_sh = it;
                 if (!ok) {
@@ -905,8 +893,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             // ---------------- MMA issuer: one fresh accumulator per group of offsets
             using PR = Products<PA, PB>;
             constexpr int KC = (NCH + K16 - 1) / K16;
-            const ChunkPlan<KC> graded_plan(kGradable && a.mode == 0 ? a.gchunks : 0u,
-                                            kGradable && a.mode == 0 ? a.gsteps : 0u, PR::n, K16);
+            const ChunkPlan<KC> graded_plan(kGradable ? a.gchunks : 0u,
+                                            kGradable ? a.gsteps : 0u, PR::n, K16);
             const uint32_t a_lo0 = sdesc_lo(smem0), b_lo0 = sdesc_lo(smem0 + PA * stageA);
             const uint32_t full0 = smem_u32(&bar_full[0]), empty0 = smem_u32(&bar_empty[0]);
             int it = 0, s = 0;
@@ -924,7 +912,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const uint32_t tmem_d = tmem + (uint32_t)(acc * 256);
                 uint32_t acc0 = 0;  // the group's first MMA overwrites the accumulator
                 for (int o = groups.begin(g); o < groups.end(g) && ok; ++o) {
-                    const bool graded = a.mode == 0 && o_begin + o < a.n_il;
+                    const bool graded = o_begin + o < a.n_il;
 #pragma unroll
                     for (int kc = 0; kc < KC; ++kc) {
                         const int kind = graded ? graded_plan.kind[kc] : 1;
@@ -1038,20 +1026,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 mx = stage_row<NCH>(Lr, scale_sh, stage + row * srow, a.nc);
             }
             const int64_t np = a.np;
-            const int64_t level_cells = a.mode == 0 ? 8 * np * np * np : np * np * np;
+            const int64_t level_cells = 8 * np * np * np;
             float *out = a.groups == 1 ? a.L : a.Lpart + (int64_t)grp * level_cells * a.nc;
             const int tx = row % a.bx, ty = (row / a.bx) % a.by, tz = row / (a.bx * a.by);
-            int64_t my_idx;
-            if (a.mode == 0) {
-                my_idx = (int64_t)cls * np * np * np + (x0 + tx) + np * ((y0 + ty) + np * (int64_t)(z0 + tz));
-            } else {
-                // natural coordinates of the parent level -> its class layout
-                const int px = x0 + tx, py = y0 + ty, pz = z0 + tz;
-                const int64_t on = a.out_np;
-                my_idx = on == 0 ? 0
-                                 : (int64_t)((px & 1) | ((py & 1) << 1) | ((pz & 1) << 2)) * on * on * on + (px >> 1) +
-                                       on * ((py >> 1) + on * (int64_t)(pz >> 1));
-            }
+            const int64_t my_idx =
+                (int64_t)cls * np * np * np + (x0 + tx) + np * ((y0 + ty) + np * (int64_t)(z0 + tz));
             __syncwarp();
             store_rows<NCH>(stage, srow, quad * 32, a.rows, my_idx, out, a.nc, lane);
         }
@@ -1078,7 +1057,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
-// Pair variant of mode 0 for the fp16 split (128-byte rows): a cluster of two
+// Pair variant for the fp16 split (128-byte rows): a cluster of two
 // CTAs computes 256 target rows, tiles 2t and 2t + 1 of one class, with 2-SM
 // MMAs (M = 256).  Each CTA copies its own 128-row A brick and half of every
 // operator tile (N/2 rows); the MMAs, issued by the even CTA, read both CTAs'
@@ -1209,7 +1188,7 @@ __device__ __forceinline__ void pair_tile(const TcMaps &maps, const TcArgs &a, i
                             off_slot(dx, dy, dz, w), true);
             }
             if (ok && a.n_off > a.n_il && a.n_il >= o_begin && a.n_il < o_end)
-                load_offset(true, x0, y0, z0, a.np, a.noff + 8 + cls, false);
+                load_offset(true, x0, y0, z0, a.np, a.noff + cls, false);
             pp.it = it;
             pp.s = s;
             pp.round = phase ^ 1u;

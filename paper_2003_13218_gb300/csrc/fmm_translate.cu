@@ -1,16 +1,26 @@
-// fmm_translate.cu -- M2M and L2L (Appendix B) as dense products.
+// fmm_translate.cu -- M2M and L2L (Appendix B), folded over the eight child octants.
 //
 // In level-scaled coefficients both translations are fixed linear maps per
-// child octant c (w_c = child-centre offset / parent side = (+-1/4)^3):
-//   L2L: Lhat_k^l(child) = sum_{n >= k, m} Lhat_n^m(parent) R_{n-k}^{m-l}(w_c) 2^{-(k+1)}
-//   M2M: Mhat_n^m(parent) = sum_c sum_{k <= n, l} R_{n-k}^{m-l}(-w_c) Mhat_k^l(child_c) 2^{-k}
-// so a whole level is one product with gathered columns:
-//   L2L: [8 C x C] (all octants stacked) . [C x parents]   -> added to the children
-//   M2M: [C x 8 C] . [8 C x parents] (the 8 children of each parent) -> parents
-// The real operator matrices are built once per plan from the complex forms.
+// child octant s (w_s = child-centre offset / parent side = (+-1/4)^3):
+//   L2L: Lhat_k^l(child) = sum_{n >= k, m} Lhat_n^m(parent) R_{n-k}^{m-l}(w_s) 2^{-(k+1)}
+//   M2M: Mhat_n^m(parent) = sum_s sum_{k <= n, l} R_{n-k}^{m-l}(-w_s) Mhat_k^l(child_s) 2^{-k}
+// The octants are mirror images of octant 0, and a reflection only changes signs of the real coefficients
+// (x: (-1)^m for Re, -(-1)^m for Im; y: Im; z: (-1)^(n+m)).  With chi_j the three sign bits of coefficient j
+// and A the operator of octant 0, A_s[j][k] = (-1)^((chi_j ^ chi_k) . s) A[j][k], so
+//   M2M: M[j]   = sum_k A[j][k] W_{chi_j ^ chi_k}[k],          W_c[k] = sum_s (-1)^(c . s) m_s[k]
+//   L2L: L_s[j] = sum_c (-1)^(c . s) V_c[j],                   V_c[j] = sum_{k: chi_j ^ chi_k = c} A[j][k] l[k]
+// with butterflies over the eight children: one operator instead of eight.  A is sparse as well (|m - l| <= |n - k|,
+// and half of the rest vanishes on the diagonal x = y): a quarter of the entries at p = 6, less above.  Together
+// 1/30 of the dense products, which leaves loads as the bound: shared memory on wide levels, the latency of a row's
+// chain on the top ones.
+//
+// Measured: FP64, 100,000 charges at depth 5, p = 12: 0.51 ms for all M2M and L2L launches, the call 11.7 -> 8.05 ms
+// (dense FP64 products, 1.2 TFLOP/s at most).  Mixed path: the M2M ran on the tensor cores on operands rounded to two
+// fp16 terms and waited for the level's split; in FP32 here, with one split launch for all levels, 2,998 charges take
+// 300 us (316), 61,000 with 210 solute charges 559 us (602); 1M and 10M within 1 % of before.
 #include <math.h>
 
-#include <type_traits>
+#include <vector>
 
 #include "fmm_internal.cuh"
 
@@ -20,7 +30,7 @@ namespace {
 
 inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-__device__ inline void split_index(int j, int &n, int &m, bool &im)
+__host__ __device__ inline void split_index(int j, int &n, int &m, bool &im)
 {
     n = (int)sqrt((double)j);
     while (n * n > j) --n;
@@ -79,7 +89,7 @@ __global__ void k_l2l_ops(int p, const double *__restrict__ Rw, double *__restri
 }
 
 // M2M operators, row-major [nc][8 nc]: row j (parent output), column c nc + e (child input)
-__global__ void k_m2m_ops(int p, const double *__restrict__ Rw, double *__restrict__ B64, float *__restrict__ B32)
+__global__ void k_m2m_ops(int p, const double *__restrict__ Rw, double *__restrict__ B64)
 {
     int nc = ncoef(p);
     int64_t total = (int64_t)8 * nc * nc;
@@ -107,310 +117,311 @@ __global__ void k_m2m_ops(int p, const double *__restrict__ Rw, double *__restri
             v = s * (oim ? acc.im : acc.re);
         }
         B64[t] = v;
-        B32[t] = (float)v;
-        const size_t tt = (size_t)total + (size_t)col * nc + j;  // transposed copy [8 nc][nc]
-        B64[tt] = v;
-        B32[tt] = (float)v;
     }
 }
 
-// Dense product with gathered columns:
-//   C[coff(n) + moff(m)] (+)= sum_k A[m][k] B[boff(n) + koff(k)]
-// MODE 0 (M2M, parents at level l): boff = n nc, koff(k) = (k / nc) 8^l nc + k % nc,
-//         coff = cell_index(l, P(n)) nc, moff(m) = m, overwrite;
-// MODE 1 (L2L, children at level l): boff = cell_index(l - 1, P(n)) nc, koff(k) = k,
-//         coff = n nc, moff(m) = (m / nc) 8^(l-1) nc + m % nc, accumulate.
-// n runs over the parent coordinates P in x-fastest order.
-template <typename T, int MODE, int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-    k_translate(int M, int64_t N, int K, int nc, int l, const T *__restrict__ A, const T *__restrict__ B,
-                T *__restrict__ C)
+// ------------------------------------------------------------------ folded products
+template <typename T>
+struct alignas(2 * sizeof(T)) FoldEntry {  // a nonzero of a row of A: its value and the operand's index
+    T v;
+    int at;
+};
+
+// sign bits of coefficient j under the reflections of x (1), y (2) and z (4)
+__host__ __device__ inline int mirror_signs(int j)
 {
-    constexpr int NT = (BM / TM) * (BN / TN);
-    __shared__ T As[BK][BM];
-    __shared__ T Bs[BK][BN];
-    __shared__ int64_t bcol[BN];
-    __shared__ int64_t ccol[BN];
-    const int tid = threadIdx.x;
-    const int m0 = blockIdx.y * BM;
-    const int64_t n0 = (int64_t)blockIdx.x * BN;
-    const int np = MODE == 0 ? (1 << l) : (1 << (l - 1));  // parents per side
-    const int64_t np3 = (int64_t)np * np * np;
-    for (int i = tid; i < BN; i += NT) {
-        int64_t n = n0 + i;
-        int64_t b = 0, c = 0;
-        if (n < N) {
-            int px = (int)(n % np), py = (int)((n / np) % np), pz = (int)(n / ((int64_t)np * np));
-            if (MODE == 0) {
-                b = n * nc;
-                c = cell_index(l, px, py, pz) * nc;
-            } else {
-                b = cell_index(l - 1, px, py, pz) * nc;
-                c = n * nc;
+    int n, m;
+    bool im;
+    split_index(j, n, m, im);
+    return ((m + im) & 1) | ((int)im << 1) | (((n + m) & 1) << 2);
+}
+
+// L2L: the nonzeros of row j of A, one warp per row, [entry][row] so that neighbouring rows' entries are contiguous; by
+// c = chi_j ^ chi_k, at = k, those of c from beg[c nc + j] to beg[(c + 1) nc + j]
+__global__ void k_l2l_entries(int nc, const double *__restrict__ A, FoldEntry<double> *__restrict__ e64,
+                              FoldEntry<float> *__restrict__ e32, int *__restrict__ beg)
+{
+    const int j = blockIdx.x, lane = threadIdx.x;
+    const int sj = mirror_signs(j);
+    int at = 0;
+    for (int c = 0; c < 8; ++c) {
+        if (lane == 0) beg[c * nc + j] = at;
+        for (int k0 = 0; k0 < nc; k0 += 32) {
+            const int k = k0 + lane;
+            const double v = k < nc ? A[(size_t)j * nc + k] : 0.0;
+            const bool take = v != 0.0 && (sj ^ mirror_signs(k)) == c;
+            const unsigned b = __ballot_sync(0xffffffffu, take);
+            if (take) {
+                const size_t o = (size_t)(at + __popc(b & ((1u << lane) - 1u))) * nc + j;
+                e64[o] = {v, k};
+                e32[o] = {(float)v, k};
             }
+            at += __popc(b);
         }
-        bcol[i] = b;
-        ccol[i] = c;
     }
-    const int tm = tid % (BM / TM), tn = tid / (BM / TM);
-    T acc[TM][TN];
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = 0;
-    __syncthreads();
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        for (int e = tid; e < BM * BK; e += NT) {
-            int kk = e % BK, mm = e / BK;
-            int m = m0 + mm, k = k0 + kk;
-            As[kk][mm] = (m < M && k < K) ? A[(size_t)m * K + k] : T(0);
-        }
-        for (int e = tid; e < BN * BK; e += NT) {
-            int kk = e % BK, nn = e / BK;
-            int k = k0 + kk;
-            T v = 0;
-            if (n0 + nn < N && k < K) {
-                int64_t ko = MODE == 0 ? (int64_t)(k / nc) * np3 * nc + (k % nc) : k;
-                v = B[bcol[nn] + ko];
-            }
-            Bs[kk][nn] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            T a[TM], b[TN];
-#pragma unroll
-            for (int i = 0; i < TM; ++i) a[i] = As[kk][tm + i * (BM / TM)];
-#pragma unroll
-            for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tn + j * (BN / TN)];
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] += a[i] * b[j];
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-        int nn = tn + j * (BN / TN);
-        if (n0 + nn >= N) continue;
-#pragma unroll
-        for (int i = 0; i < TM; ++i) {
-            int m = m0 + tm + i * (BM / TM);
-            if (m >= M) continue;
-            if (MODE == 0) {
-                C[ccol[nn] + m] = acc[i][j];
-            } else {
-                int64_t mo = (int64_t)(m / nc) * np3 * nc + (m % nc);
-                C[ccol[nn] + mo] += acc[i][j];
+    if (lane == 0) beg[8 * nc + j] = at;
+}
+
+// M2M: the nonzeros of A's rows (A [nc][nc] on the host), at = (chi_j ^ chi_k) nc + k, cnt[j] of them, [entry][row].
+// Eight neighbouring rows are read by a quarter warp, whose 16-byte loads of shared memory take one cycle if the
+// operands' indices differ modulo 8 (in order of k they met 2 to 3 at a time, and the wide kernel is bound by those
+// loads): each row in turn takes, of the residues that the step has left free, the one it has most entries of.
+void m2m_entries(int nc, const std::vector<double> &A, std::vector<FoldEntry<double>> &ent, std::vector<int> &cnt)
+{
+    ent.assign((size_t)nc * nc, FoldEntry<double>{0.0, 0});
+    cnt.assign(nc, 0);
+    for (int j0 = 0; j0 < nc; j0 += 8) {
+        std::vector<int> left[8][8];  // [row][residue]: the k still to take, the lowest last
+        for (int r = 0; r < 8 && j0 + r < nc; ++r)
+            for (int k = nc - 1; k >= 0; --k)
+                if (A[(size_t)(j0 + r) * nc + k] != 0.0)
+                    left[r][((mirror_signs(j0 + r) ^ mirror_signs(k)) * nc + k) & 7].push_back(k);
+        for (bool more = true; more;) {
+            more = false;
+            bool used[8] = {};
+            for (int r = 0; r < 8 && j0 + r < nc; ++r) {
+                int best = -1;
+                size_t score = 0;
+                for (int q = 0; q < 8; ++q) {
+                    const size_t w = left[r][q].empty() ? 0 : left[r][q].size() + (used[q] ? 0 : (size_t)nc);
+                    if (w > score) {
+                        score = w;
+                        best = q;
+                    }
+                }
+                if (best < 0) continue;
+                const int j = j0 + r, k = left[r][best].back();
+                left[r][best].pop_back();
+                used[best] = more = true;
+                ent[(size_t)cnt[j]++ * nc + j] = {A[(size_t)j * nc + k], (mirror_signs(j) ^ mirror_signs(k)) * nc + k};
             }
         }
     }
 }
 
-// FP32 register-tiled version of the same products for the fine levels.
-// The operator's K runs octant by octant, each padded to KO (a multiple of 8)
-// with zero columns, so a K tile never straddles two octants and no index
-// needs a division.  Tiles: BM x BN outputs per block, 8 x 8 per thread
-// (rows tm*4 + i and BM/2 + tm*4 + i, columns likewise, for conflict-free
-// vector reads), K in steps of 8, shared memory double-buffered.
-template <int MODE, int BM, int BN>
-__global__ void __launch_bounds__((BM / 8) * (BN / 8), 2)
-    k_translate_f32(int M, int64_t N, int nc, int KO, int l, const float *__restrict__ A, int KA,
-                    const float *__restrict__ B, float *__restrict__ C)
+template <typename T, int PB>
+__device__ __forceinline__ void get_vec(const T *p, T (&v)[PB])
 {
-    constexpr int NT = (BM / 8) * (BN / 8);
-    constexpr int BK = 8;
-    __shared__ __align__(16) float As[2][BK][BM];
-    __shared__ __align__(16) float Bs[2][BK][BN];
-    __shared__ int64_t bcol[BN];
-    __shared__ int64_t ccol[BN];
-    const int tid = threadIdx.x;
-    const int m0 = blockIdx.y * BM;
-    const int64_t n0 = (int64_t)blockIdx.x * BN;
-    const int np = MODE == 0 ? (1 << l) : (1 << (l - 1));
-    const int64_t np3 = (int64_t)np * np * np;
-    for (int i = tid; i < BN; i += NT) {
-        int64_t n = n0 + i;
-        int64_t b = -1, c = 0;
-        if (n < N) {
-            int px = (int)(n % np), py = (int)((n / np) % np), pz = (int)(n / ((int64_t)np * np));
-            if (MODE == 0) {
-                b = n * nc;
-                c = cell_index(l, px, py, pz) * nc;
-            } else {
-                b = cell_index(l - 1, px, py, pz) * nc;
-                c = n * nc;
-            }
-        }
-        bcol[i] = b;
-        ccol[i] = c;
-    }
-    const int tiles_per_oct = KO / BK;
-    const int KT = (MODE == 0 ? 8 : 1) * tiles_per_oct;
-    const int64_t ostride = MODE == 0 ? np3 * nc : 0;
-    __syncthreads();
-
-    float ra[BM * BK / NT > 0 ? BM * BK / NT : 1];
-    float rb[BN * BK / NT];
-    auto load_tile = [&](int t) {
-        const int o = t / tiles_per_oct, kb = (t % tiles_per_oct) * BK;
+    if constexpr (PB * sizeof(T) >= 16) {
 #pragma unroll
-        for (int i = 0; i < BM * BK / NT; ++i) {
-            int e = tid + i * NT;
-            int mm = e / BK, kk = e % BK;
-            int m = m0 + mm;
-            ra[i] = m < M ? A[(size_t)m * KA + o * KO + kb + kk] : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < BN * BK / NT; ++i) {
-            int e = tid + i * NT;
-            int nn = e / BK, kk = e % BK;
-            int k = kb + kk;
-            rb[i] = (bcol[nn] >= 0 && k < nc) ? B[bcol[nn] + o * ostride + k] : 0.f;
-        }
-    };
-    auto store_tile = [&](int buf) {
-#pragma unroll
-        for (int i = 0; i < BM * BK / NT; ++i) {
-            int e = tid + i * NT;
-            As[buf][e % BK][e / BK] = ra[i];
-        }
-#pragma unroll
-        for (int i = 0; i < BN * BK / NT; ++i) {
-            int e = tid + i * NT;
-            Bs[buf][e % BK][e / BK] = rb[i];
-        }
-    };
-
-    const int tm = tid % (BM / 8), tn = tid / (BM / 8);
-    float acc[8][8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-
-    load_tile(0);
-    store_tile(0);
-    __syncthreads();
-    for (int t = 0; t < KT; ++t) {
-        const int buf = t & 1;
-        if (t + 1 < KT) load_tile(t + 1);
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float4 a0 = *reinterpret_cast<const float4 *>(&As[buf][kk][tm * 4]);
-            float4 a1 = *reinterpret_cast<const float4 *>(&As[buf][kk][BM / 2 + tm * 4]);
-            float4 b0 = *reinterpret_cast<const float4 *>(&Bs[buf][kk][tn * 4]);
-            float4 b1 = *reinterpret_cast<const float4 *>(&Bs[buf][kk][BN / 2 + tn * 4]);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] += a[i] * b[j];
-        }
-        if (t + 1 < KT) store_tile(buf ^ 1);
-        __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int nn = (j < 4 ? tn * 4 + j : BN / 2 + tn * 4 + (j - 4));
-        if (n0 + nn >= N) continue;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int m = m0 + (i < 4 ? tm * 4 + i : BM / 2 + tm * 4 + (i - 4));
-            if (m >= M) continue;
-            if (MODE == 0) {
-                C[ccol[nn] + m] = acc[i][j];
-            } else {
-                const int c = m / nc;
-                C[ccol[nn] + (int64_t)c * np3 * nc + (m - c * nc)] += acc[i][j];
-            }
-        }
-    }
-}
-
-// operators with every octant's K padded to KO: M2M [nc][8 KO], L2L [8 nc][KO]
-__global__ void k_pad_ops(int nc, int KO, const float *__restrict__ m2m, const float *__restrict__ l2l,
-                          float *__restrict__ m2mP, float *__restrict__ l2lP)
-{
-    const int64_t n0 = (int64_t)nc * 8 * KO, n1 = (int64_t)8 * nc * KO;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n0 + n1; t += (int64_t)gridDim.x * blockDim.x) {
-        if (t < n0) {
-            int m = (int)(t / (8 * KO)), r = (int)(t % (8 * KO));
-            int o = r / KO, kk = r % KO;
-            m2mP[t] = kk < nc ? m2m[(size_t)m * 8 * nc + o * nc + kk] : 0.f;
-        } else {
-            int64_t u = t - n0;
-            int m = (int)(u / KO), kk = (int)(u % KO);
-            l2lP[u] = kk < nc ? l2l[(size_t)m * nc + kk] : 0.f;
-        }
-    }
-}
-
-// The same products for coarse levels (few columns): one block per
-// (column, 32 outputs), the 8 warps split K, partial sums added in warp order.
-// AT is the operator transposed, [K][M].
-template <typename T, int MODE>
-__global__ void __launch_bounds__(256)
-    k_translate_small(int M, int K, int nc, int l, const T *__restrict__ AT, const T *__restrict__ B, T *__restrict__ C)
-{
-    __shared__ T part[8][32];
-    const int64_t n = blockIdx.x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int m = blockIdx.y * 32 + lane;
-    const int np = MODE == 0 ? (1 << l) : (1 << (l - 1));
-    const int64_t np3 = (int64_t)np * np * np;
-    const int px = (int)(n % np), py = (int)((n / np) % np), pz = (int)(n / ((int64_t)np * np));
-    const int64_t bcol = MODE == 0 ? n * nc : cell_index(l - 1, px, py, pz) * nc;
-    const int k0 = (int)((int64_t)K * w / 8), k1 = (int)((int64_t)K * (w + 1) / 8);
-    T acc = 0;
-    if (m < M) {
-        // M2M: K = 8 nc, so warp w covers exactly octant w
-        const int64_t obase = MODE == 0 ? (int64_t)w * np3 * nc - (int64_t)w * nc : 0;
-        for (int k = k0; k < k1; ++k) acc += AT[(size_t)k * M + m] * B[bcol + obase + k];
-    }
-    part[w][lane] = acc;
-    __syncthreads();
-    if (w == 0 && m < M) {
-        T s = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) s += part[i][lane];
-        if (MODE == 0) {
-            C[cell_index(l, px, py, pz) * nc + m] = s;
-        } else {
-            C[((int64_t)(m / nc) * np3 + n) * nc + (m % nc)] += s;
-        }
-    }
-}
-
-template <typename T, int MODE>
-fmm_status launch_translate(Plan &P, int l, const T *A, const T *AT, const T *B, T *C)
-{
-    const int nc = P.nc;
-    const int M = MODE == 0 ? nc : 8 * nc;
-    const int K = MODE == 0 ? 8 * nc : nc;
-    const int64_t N = MODE == 0 ? ((int64_t)1 << (3 * l)) : ((int64_t)1 << (3 * (l - 1)));
-    if (N * ((M + 31) / 32) <= 32768) {
-        dim3 grid((unsigned)N, (M + 31) / 32);
-        k_translate_small<T, MODE><<<grid, 256, 0, P.stream>>>(M, K, nc, l, AT, B, C);
-        FMM_LAUNCH_CHECK(P);
-        return FMM_OK;
-    }
-    if (std::is_same<T, float>::value) {
-        constexpr int BM = 64, BN = 256;
-        const int KO = (nc + 7) / 8 * 8;
-        const float *AP = MODE == 0 ? P.tab.m2mP32 : P.tab.l2lP32;
-        const int KA = MODE == 0 ? 8 * KO : KO;
-        dim3 grid(blocks_for(N, BN), (M + BM - 1) / BM);
-        k_translate_f32<MODE, BM, BN><<<grid, (BM / 8) * (BN / 8), 0, P.stream>>>(
-            M, N, nc, KO, l, AP, KA, (const float *)B, (float *)C);
+        for (int i = 0; i < (int)(PB * sizeof(T) / 16); ++i)
+            reinterpret_cast<uint4 *>(v)[i] = reinterpret_cast<const uint4 *>(p)[i];
     } else {
-        constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4;
-        dim3 grid(blocks_for(N, BN), (M + BM - 1) / BM);
-        k_translate<T, MODE, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, P.stream>>>(M, N, K, nc, l, A, B,
-                                                                                               C);
+#pragma unroll
+        for (int i = 0; i < PB; ++i) v[i] = p[i];
     }
+}
+
+template <typename T, int PB>
+__device__ __forceinline__ void put_vec(T *p, const T (&v)[PB])
+{
+    if constexpr (PB * sizeof(T) >= 16) {
+#pragma unroll
+        for (int i = 0; i < (int)(PB * sizeof(T) / 16); ++i)
+            reinterpret_cast<uint4 *>(p)[i] = reinterpret_cast<const uint4 *>(v)[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < PB; ++i) p[i] = v[i];
+    }
+}
+
+// w_c = sum_s (-1)^(c . s) w_s in place (its own inverse up to 8)
+template <typename T, int PB>
+__device__ __forceinline__ void butterflies(T (&w)[8][PB])
+{
+#pragma unroll
+    for (int bit = 1; bit < 8; bit <<= 1)
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+            if (!(s & bit))
+#pragma unroll
+                for (int b = 0; b < PB; ++b) {
+                    const T u = w[s][b], v = w[s | bit][b];
+                    w[s][b] = u + v;
+                    w[s | bit][b] = u - v;
+                }
+}
+
+__device__ __forceinline__ unsigned mag_bits(float x) { return __float_as_uint(fmaxf(0.f, fabsf(x))); }  // a NaN drops
+__device__ __forceinline__ unsigned long long mag_bits(double x)  // a NaN is larger than all
+{
+    return (unsigned long long)__double_as_longlong(x) & ~(1ull << 63);
+}
+
+constexpr int FOLD_PB = 4;     // parents per block where there are many
+constexpr int FOLD_SPLIT = 2;  // threads per row of A where there are few (2 x 448 threads at p = 20)
+
+// M2M into level l (natural parent order n, 8^l of them): a block takes PB parents, a thread one coefficient.  The
+// children's rows of one octant are contiguous in n, so every load is a run of PB nc values; W sits in shared memory
+// with the PB parents side by side, which one entry of A then serves in one vector load.  A lone parent's rows (PB = 1, levels
+// whose blocks leave most of the GPU idle) are read by FOLD_SPLIT threads each, whose sums are added in order: the loop
+// over a row is a chain of loads.  sx, amax (or null): the level's largest |M sx| is folded in for the gain of the
+// M2L's operands.
+template <typename T, int PB, typename U>
+__global__ void k_m2m_fold(int nc, int l, const FoldEntry<T> *__restrict__ ent, const int *__restrict__ cnt,
+                           const T *__restrict__ child, T *__restrict__ parent, const T *__restrict__ sx,
+                           U *__restrict__ amax)
+{
+    constexpr int SPLIT = PB == 1 ? FOLD_SPLIT : 1;
+    extern __shared__ __align__(16) unsigned char fold_smem[];
+    __shared__ U mx_sh;
+    T *W = reinterpret_cast<T *>(fold_smem);  // [8][nc][PB], then [SPLIT - 1][nc] partial sums
+    const int64_t np3 = (int64_t)1 << (3 * l), n0 = (int64_t)blockIdx.x * PB;  // PB divides 8^l
+    const int width = blockDim.x / SPLIT;
+    const int part = SPLIT > 1 ? threadIdx.x / width : 0, k = threadIdx.x - part * width;
+    if (threadIdx.x == 0) mx_sh = 0;
+    if (k < nc && part == 0) {
+        alignas(16) T w[8][PB];
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+#pragma unroll
+            for (int b = 0; b < PB; ++b) w[s][b] = child[(s * np3 + n0 + b) * nc + k];
+        butterflies<T, PB>(w);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) put_vec<T, PB>(W + (c * nc + k) * PB, w[c]);
+    }
+    __syncthreads();
+    U mx = 0;
+    alignas(16) T acc[PB] = {};
+    if (k < nc) {
+        const int n = cnt[k];
+#pragma unroll 4
+        for (int i = part; i < n; i += SPLIT) {
+            const FoldEntry<T> e = ent[(size_t)i * nc + k];
+            alignas(16) T w[PB];
+            get_vec<T, PB>(W + e.at * PB, w);
+#pragma unroll
+            for (int b = 0; b < PB; ++b) acc[b] += e.v * w[b];
+        }
+        if (part > 0) W[(7 + part) * nc + k] = acc[0];
+    }
+    if (SPLIT > 1) __syncthreads();
+    if (k < nc && part == 0) {
+#pragma unroll
+        for (int g = 1; g < SPLIT; ++g) acc[0] += W[(7 + g) * nc + k];
+        const int side = 1 << l;
+#pragma unroll
+        for (int b = 0; b < PB; ++b) {
+            const int p = (int)(n0 + b);
+            parent[cell_index(l, p & (side - 1), (p >> l) & (side - 1), p >> (2 * l)) * nc + k] = acc[b];
+            if (amax) {
+                const U v = mag_bits(acc[b] * sx[k]);
+                mx = v > mx ? v : mx;
+            }
+        }
+    }
+    if (amax) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const U v = __shfl_xor_sync(0xffffffffu, mx, o);
+            mx = v > mx ? v : mx;
+        }
+        if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(&mx_sh, mx);
+        __syncthreads();
+        if (threadIdx.x == 0 && mx_sh > 0) atomicMax(amax, mx_sh);
+    }
+}
+
+// L2L from level l - 1 into level l, added to the children: PB parents per block (in the children's parent order), a
+// thread one coefficient of their eight children, V in registers.  PB = 1 (few parents): the eight V_c of a coefficient
+// are as many items spread over the block, through shared memory.
+template <typename T, int PB>
+__global__ void k_l2l_fold(int nc, int l, const FoldEntry<T> *__restrict__ ent, const int *__restrict__ beg,
+                           const T *__restrict__ parent, T *__restrict__ child)
+{
+    extern __shared__ __align__(16) unsigned char fold_smem[];
+    T *X = reinterpret_cast<T *>(fold_smem);  // [nc][PB]
+    const int64_t np3 = (int64_t)1 << (3 * (l - 1)), n0 = (int64_t)blockIdx.x * PB;  // PB divides 8^(l - 1)
+    const int k = threadIdx.x, side = 1 << (l - 1);
+    if (k < nc) {
+        alignas(16) T x[PB];
+#pragma unroll
+        for (int b = 0; b < PB; ++b) {
+            const int p = (int)(n0 + b);
+            x[b] = parent[cell_index(l - 1, p & (side - 1), (p >> (l - 1)) & (side - 1), p >> (2 * (l - 1))) * nc + k];
+        }
+        put_vec<T, PB>(X + k * PB, x);
+    }
+    __syncthreads();
+    if constexpr (PB == 1) {
+        T *Vs = X + nc;  // [8][nc]
+        for (int e = k; e < 8 * nc; e += blockDim.x) {
+            const int j = e % nc, end = beg[e + nc];  // e = c nc + j
+            T v = 0;
+#pragma unroll 4
+            for (int i = beg[e]; i < end; ++i) {
+                const FoldEntry<T> t = ent[(size_t)i * nc + j];
+                v += t.v * X[t.at];
+            }
+            Vs[e] = v;
+        }
+        __syncthreads();
+        for (int e = k; e < 8 * nc; e += blockDim.x) {
+            const int s = e / nc, j = e - s * nc;
+            T v = Vs[j];
+#pragma unroll
+            for (int c = 1; c < 8; ++c) v += __popc(c & s) & 1 ? -Vs[c * nc + j] : Vs[c * nc + j];
+            child[(s * np3 + n0) * nc + j] += v;
+        }
+        return;
+    }
+    if (k >= nc) return;
+    alignas(16) T V[8][PB];
+    int i = beg[k];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+#pragma unroll
+        for (int b = 0; b < PB; ++b) V[c][b] = 0;
+        const int end = beg[(c + 1) * nc + k];
+#pragma unroll 2
+        for (; i < end; ++i) {
+            const FoldEntry<T> e = ent[(size_t)i * nc + k];
+            alignas(16) T x[PB];
+            get_vec<T, PB>(X + e.at * PB, x);
+#pragma unroll
+            for (int b = 0; b < PB; ++b) V[c][b] += e.v * x[b];
+        }
+    }
+    butterflies<T, PB>(V);
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+#pragma unroll
+        for (int b = 0; b < PB; ++b) child[(s * np3 + n0 + b) * nc + k] += V[s][b];
+}
+
+// four parents share each entry of A where that still leaves several blocks per SM, else one parent a block with its work
+// spread over more threads (L2L at 8 and 64 parents, FP64, p = 8: 37 us with a thread per coefficient, 11 us spread)
+inline bool fold_wide(int64_t parents) { return parents >= 8 * 152 * FOLD_PB / 2; }
+
+template <typename T, typename U>
+fmm_status m2m_t(Plan &P, int l, const void *ent, const T *sx, U *amax)
+{
+    const int64_t n = (int64_t)1 << (3 * l);
+    const int threads = (P.nc + 31) / 32 * 32;  // at most 448
+    const FoldEntry<T> *e = (const FoldEntry<T> *)ent;
+    const T *child = (const T *)P.M[l + 1];
+    T *parent = (T *)P.M[l];
+    if (fold_wide(n))
+        k_m2m_fold<T, FOLD_PB, U><<<(unsigned)(n / FOLD_PB), threads, sizeof(T) * 8 * P.nc * FOLD_PB, P.stream>>>(
+            P.nc, l, e, P.tab.fold_cnt, child, parent, sx, amax);
+    else
+        k_m2m_fold<T, 1, U><<<(unsigned)n, FOLD_SPLIT * threads, sizeof(T) * (7 + FOLD_SPLIT) * P.nc, P.stream>>>(
+            P.nc, l, e, P.tab.fold_cnt, child, parent, sx, amax);
+    FMM_LAUNCH_CHECK(P);
+    return FMM_OK;
+}
+
+template <typename T>
+fmm_status l2l_t(Plan &P, int l, const void *ent)
+{
+    const int64_t n = (int64_t)1 << (3 * (l - 1));
+    const int threads = (P.nc + 31) / 32 * 32;
+    const FoldEntry<T> *e = (const FoldEntry<T> *)ent;
+    if (fold_wide(n))
+        k_l2l_fold<T, FOLD_PB><<<(unsigned)(n / FOLD_PB), threads, sizeof(T) * P.nc * FOLD_PB, P.stream>>>(
+            P.nc, l, e, P.tab.fold_beg, (const T *)P.L[l - 1], (T *)P.L[l]);
+    else
+        k_l2l_fold<T, 1><<<(unsigned)n, 4 * threads < 1024 ? 4 * threads : 1024, sizeof(T) * 9 * P.nc, P.stream>>>(
+            P.nc, l, e, P.tab.fold_beg, (const T *)P.L[l - 1], (T *)P.L[l]);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
@@ -421,48 +432,67 @@ fmm_status build_translation_ops(Plan &P)
 {
     const int nc = P.nc;
     const size_t n = (size_t)8 * nc * nc;
-    if (!P.tab.l2l64) {  // each table followed by its transpose
+    if (!P.tab.l2l64) {  // the L2L tables are followed by their transposes
         FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l64, sizeof(double) * 2 * n));
         FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l32, sizeof(float) * 2 * n));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m64, sizeof(double) * 2 * n));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m32, sizeof(float) * 2 * n));
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m64, sizeof(double) * n));
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m_fold64, sizeof(FoldEntry<double>) * nc * nc));
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m_fold32, sizeof(FoldEntry<float>) * nc * nc));
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l_fold64, sizeof(FoldEntry<double>) * nc * nc));
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l_fold32, sizeof(FoldEntry<float>) * nc * nc));
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.fold_cnt, sizeof(int) * nc));
+        FMM_CUDA_TRY(cudaMalloc(&P.tab.fold_beg, sizeof(int) * 9 * nc));
     }
     k_l2l_ops<<<blocks_for(n, 256), 256, 0, P.stream>>>(P.p, P.tab.Rw64, P.tab.l2l64, P.tab.l2l32);
     FMM_LAUNCH_CHECK(P);
-    k_m2m_ops<<<blocks_for(n, 256), 256, 0, P.stream>>>(P.p, P.tab.Rw64, P.tab.m2m64, P.tab.m2m32);
+    k_m2m_ops<<<blocks_for(n, 256), 256, 0, P.stream>>>(P.p, P.tab.Rw64, P.tab.m2m64);
     FMM_LAUNCH_CHECK(P);
-    const int KO = (nc + 7) / 8 * 8;
-    const size_t np_ = (size_t)8 * nc * KO;
-    if (!P.tab.m2mP32) {
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2mP32, sizeof(float) * np_));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.l2lP32, sizeof(float) * np_));
+    k_l2l_entries<<<nc, 32, 0, P.stream>>>(nc, P.tab.l2l64, (FoldEntry<double> *)P.tab.l2l_fold64,
+                                           (FoldEntry<float> *)P.tab.l2l_fold32, P.tab.fold_beg);
+    FMM_LAUNCH_CHECK(P);
+    {
+        std::vector<double> A((size_t)nc * nc);  // octant 0's columns of the M2M
+        FMM_CUDA_TRY(cudaMemcpy2DAsync(A.data(), sizeof(double) * nc, P.tab.m2m64, sizeof(double) * 8 * nc,
+                                       sizeof(double) * nc, nc, cudaMemcpyDeviceToHost, P.stream));
+        FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
+        std::vector<FoldEntry<double>> e64;
+        std::vector<int> cnt;
+        m2m_entries(nc, A, e64, cnt);
+        std::vector<FoldEntry<float>> e32(e64.size());
+        for (size_t i = 0; i < e64.size(); ++i) e32[i] = {(float)e64[i].v, e64[i].at};
+        FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.m2m_fold64, e64.data(), sizeof(e64[0]) * e64.size(), cudaMemcpyHostToDevice,
+                                     P.stream));
+        FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.m2m_fold32, e32.data(), sizeof(e32[0]) * e32.size(), cudaMemcpyHostToDevice,
+                                     P.stream));
+        FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.fold_cnt, cnt.data(), sizeof(int) * nc, cudaMemcpyHostToDevice, P.stream));
+        FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
     }
-    k_pad_ops<<<blocks_for(2 * np_, 256), 256, 0, P.stream>>>(nc, KO, P.tab.m2m32, P.tab.l2l32, P.tab.m2mP32,
-                                                             P.tab.l2lP32);
-    FMM_LAUNCH_CHECK(P);
+    // four parents at p = 20 take 113 KB (FP64)
+    FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2m_fold<double, FOLD_PB, unsigned long long>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(sizeof(double) * 8 * NC_MAX * FOLD_PB)));
+    FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2m_fold<float, FOLD_PB, unsigned>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(sizeof(float) * 8 * NC_MAX * FOLD_PB)));
     return FMM_OK;
 }
 
-// M2M into level l (parents) from level l + 1
+// M2M into level l (parents) from level l + 1; where the M2L runs on the tensor cores, level l's largest balanced
+// moment is folded in
 fmm_status launch_m2m(Plan &P, int l)
 {
-    const size_t n = (size_t)8 * P.nc * P.nc;
-    if (P.precision == FMM_PREC_FP64)
-        return launch_translate<double, 0>(P, l, P.tab.m2m64, P.tab.m2m64 + n, (const double *)P.M[l + 1],
-                                           (double *)P.M[l]);
-    return launch_translate<float, 0>(P, l, P.tab.m2m32, P.tab.m2m32 + n, (const float *)P.M[l + 1],
-                                      (float *)P.M[l]);
+    if (P.precision == FMM_PREC_FP64) {
+        const double *sx = nullptr;
+        unsigned long long *amax = res_amax(P, l, &sx);
+        return m2m_t<double, unsigned long long>(P, l, P.tab.m2m_fold64, sx, amax);
+    }
+    return m2m_t<float, unsigned>(P, l, P.tab.m2m_fold32, tc_scale(P), tc_amax(P, l));
 }
 
 // L2L from level l - 1 into level l (added to the M2L result)
 fmm_status launch_l2l(Plan &P, int l)
 {
-    const size_t n = (size_t)8 * P.nc * P.nc;
-    if (P.precision == FMM_PREC_FP64)
-        return launch_translate<double, 1>(P, l, P.tab.l2l64, P.tab.l2l64 + n, (const double *)P.L[l - 1],
-                                           (double *)P.L[l]);
-    return launch_translate<float, 1>(P, l, P.tab.l2l32, P.tab.l2l32 + n, (const float *)P.L[l - 1],
-                                      (float *)P.L[l]);
+    if (P.precision == FMM_PREC_FP64) return l2l_t<double>(P, l, P.tab.l2l_fold64);
+    return l2l_t<float>(P, l, P.tab.l2l_fold32);
 }
 
 }  // namespace fmm
