@@ -268,70 +268,126 @@ __global__ void k_lattice_operator(int p, const double *__restrict__ S, double *
 
 // ------------------------------------------------------------------ P2M
 // Eq. P2M in level-scaled form: Mhat_n^m = sum_j q_j R_n^m((r_M - r_j)/h).
-// One thread per (leaf, m): the column n = m..p of every particle.  PM >= p is
-// a compile-time bound so that the column accumulators stay in registers
-// (the loops over n are unrolled and predicated on m <= n <= p).
-template <typename T, int PM>
-__global__ void k_p2m(int p, int nside, const int *__restrict__ start, const Particle<T> *__restrict__ sp,
-                      T inv_h, int d, T *__restrict__ M)
-{
-    // reciprocals of the recurrences, once per block: -1/(2k) and 1/((n+m)(n-m))
-    __shared__ T s_half[PM + 1];
-    __shared__ T s_inv[(PM + 1) * (PM + 1)];
-    for (int e = threadIdx.x; e < (PM + 1) * (PM + 1); e += blockDim.x) {
-        const int n = e / (PM + 1), mm = e % (PM + 1);
-        s_inv[e] = n > mm ? T(1) / T((n + mm) * (n - mm)) : T(0);
-        if (e <= PM) s_half[e] = e > 0 ? T(-0.5) / T(e) : T(0);
-    }
-    __syncthreads();
-    int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t nleaf = (int64_t)nside * nside * nside;
-    if (tid >= nleaf * (p + 1)) return;
-    int64_t leaf = tid / (p + 1);
-    int m = (int)(tid % (p + 1));
-    int x = (int)(leaf % nside), y = (int)((leaf / nside) % nside), z = (int)(leaf / ((int64_t)nside * nside));
-    T acc_re[PM + 1], acc_im[PM + 1];
-#pragma unroll
-    for (int n = 0; n <= PM; ++n) acc_re[n] = acc_im[n] = 0;
-    for (int s = start[leaf]; s < start[leaf + 1]; ++s) {
-        Particle<T> pt = sp[s];
-        T vx = -pt.x * inv_h, vy = -pt.y * inv_h, vz = -pt.z * inv_h;
-        T r2 = vx * vx + vy * vy + vz * vz;
-        T dre = 1, dim = 0;
-        for (int k = 1; k <= m; ++k) {
-            T sc = s_half[k];
-            T nre = sc * (vx * dre - vy * dim);
-            T nim = sc * (vx * dim + vy * dre);
-            dre = nre;
-            dim = nim;
+// factors of the recurrences R_n^m = (a_nm z R_{n-1}^m - b_nm r^2 R_{n-2}^m) and R_m^m = c_m (x + iy) R_{m-1}^{m-1}
+template <typename T>
+struct ExpandFactors {
+    T a[(P_MAX + 1) * (P_MAX + 1)], b[(P_MAX + 1) * (P_MAX + 1)], c[P_MAX + 1];
+    constexpr ExpandFactors() : a{}, b{}, c{}
+    {
+        for (int m = 0; m <= P_MAX; ++m) {
+            c[m] = m > 0 ? T(-0.5) / T(m) : T(0);
+            for (int n = m + 1; n <= P_MAX; ++n) {
+                a[m * (P_MAX + 1) + n] = T(2 * n - 1) / T((n + m) * (n - m));
+                b[m * (P_MAX + 1) + n] = T(1) / T((n + m) * (n - m));
+            }
         }
-        T p2re = 0, p2im = 0, p1re = dre, p1im = dim;
-#pragma unroll
-        for (int n = 0; n <= PM; ++n) {
-            if (n == m) {
-                acc_re[n] += pt.q * dre;
-                acc_im[n] += pt.q * dim;
-            } else if (n > m && n <= p) {
-                T a = T(2 * n - 1) * vz;
-                T inv = s_inv[n * (PM + 1) + m];
-                T cr = (a * p1re - r2 * p2re) * inv;
-                T ci = (a * p1im - r2 * p2im) * inv;
-                acc_re[n] += pt.q * cr;
-                acc_im[n] += pt.q * ci;
+    }
+};
+__constant__ ExpandFactors<double> expand_factors64 = ExpandFactors<double>();
+__constant__ ExpandFactors<float> expand_factors32 = ExpandFactors<float>();
+template <typename T>
+__device__ __forceinline__ const ExpandFactors<T> &expand_factors();
+template <>
+__device__ __forceinline__ const ExpandFactors<double> &expand_factors<double>() { return expand_factors64; }
+template <>
+__device__ __forceinline__ const ExpandFactors<float> &expand_factors<float>() { return expand_factors32; }
+
+__device__ __forceinline__ unsigned p2m_bits(float x) { return __float_as_uint(fmaxf(0.f, fabsf(x))); }  // a NaN drops
+__device__ __forceinline__ unsigned long long p2m_bits(double x)  // a NaN is larger than all
+{
+    return (unsigned long long)__double_as_longlong(x) & ~(1ull << 63);
+}
+
+// Any order, FP64 or FP32: a warp takes `lb` consecutive leaves, whose charges are contiguous, and runs the recurrences
+// with one charge per lane, 32 at a time; the columns m of the 32 charges go through shared memory, where the lanes
+// take one coefficient each and add up every leaf's charges in order.  GB300's FP64 pipe takes 16 cycles per warp
+// instruction however many lanes are active, so what counts is that no lane idles: with one thread per (leaf, m), whose
+// loops run to the longest column and fullest leaf of the warp, 100,000 charges at p = 12 took 776 us and 2,998 at
+// p = 8 109 us; here 302 us and, shared, 22 us.  The warps of a block share the same charges and take the columns m in
+// turn (small systems: one warp, on one of an SM's four FP64 pipes, took 46 us for the latter).  sx, amax (or null): the
+// level's largest |M sx| is folded in.
+constexpr int P2M_SHARE = 4;  // warps that share 32 charges in small systems
+
+template <typename T, typename U>
+__global__ void __launch_bounds__(32 * P2M_SHARE) k_p2m(int p, int d, int lb, const int *__restrict__ start,
+                                            const Particle<T> *__restrict__ sp, T inv_h, T *__restrict__ M,
+                                            const T *__restrict__ sx, U *__restrict__ amax)
+{
+    extern __shared__ __align__(16) unsigned char p2m_smem[];
+    const ExpandFactors<T> &F = expand_factors<T>();
+    const int nc = ncoef(p), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, share = blockDim.x >> 5, nside = 1 << d;
+    const int64_t nleaf = (int64_t)1 << (3 * d), leaf0 = (int64_t)blockIdx.x * lb;
+    const int nl = (int)(nleaf - leaf0 < lb ? nleaf - leaf0 : lb);
+    T *rows = reinterpret_cast<T *>(p2m_smem);  // [lb][nc]
+    T *col = rows + lb * nc + warp * 2 * (p + 1) * 33;  // [2 (p + 1)][33]: the column's (n, Re | Im) of the 32 charges
+    int *st = reinterpret_cast<int *>(rows + lb * nc + share * 2 * (p + 1) * 33);
+    for (int i = threadIdx.x; i <= nl; i += blockDim.x) st[i] = start[leaf0 + i];
+    for (int e = threadIdx.x; e < nl * nc; e += blockDim.x) rows[e] = 0;
+    __syncthreads();
+    const int s1 = st[nl];
+    for (int c0 = st[0]; c0 < s1; c0 += 32) {
+        Particle<T> pt = {};
+        if (c0 + lane < s1) pt = sp[c0 + lane];
+        const T vx = -pt.x * inv_h, vy = -pt.y * inv_h, vz = -pt.z * inv_h;
+        const T r2 = vx * vx + vy * vy + vz * vz;
+        T dre = pt.q, dim = 0;  // q R_m^m
+        for (int m = 0; m <= p; ++m) {
+            if (m > 0) {
+                const T cx = F.c[m] * vx, cy = F.c[m] * vy;
+                const T nre = cx * dre - cy * dim;
+                dim = cx * dim + cy * dre;
+                dre = nre;
+            }
+            if (m % share != warp) continue;  // another warp's column
+            T p2re = 0, p2im = 0, p1re = dre, p1im = dim;
+            col[lane] = dre;
+            col[33 + lane] = dim;
+            for (int n = m + 1; n <= p; ++n) {
+                const T a = F.a[m * (P_MAX + 1) + n] * vz, b = F.b[m * (P_MAX + 1) + n] * r2;
+                const T cr = a * p1re - b * p2re, ci = a * p1im - b * p2im;
+                col[(2 * (n - m)) * 33 + lane] = cr;
+                col[(2 * (n - m) + 1) * 33 + lane] = ci;
                 p2re = p1re;
                 p2im = p1im;
                 p1re = cr;
                 p1im = ci;
             }
+            __syncwarp();
+            for (int v = lane; v < 2 * (p - m + 1); v += 32) {
+                const int n = m + (v >> 1);
+                if (m == 0 && (v & 1)) continue;
+                const int idx = v & 1 ? cim(n, m) : cre(n, m);
+                for (int i = 0; i < nl; ++i) {
+                    const int b = st[i] > c0 ? st[i] - c0 : 0, e = st[i + 1] < c0 + 32 ? st[i + 1] - c0 : 32;
+                    if (b >= e) continue;
+                    T acc = rows[i * nc + idx];
+                    for (int j = b; j < e; ++j) acc += col[v * 33 + j];
+                    rows[i * nc + idx] = acc;
+                }
+            }
+            __syncwarp();
         }
     }
-    int nc = ncoef(p);
-    T *out = M + cell_index(d, x, y, z) * nc;
-#pragma unroll
-    for (int n = 0; n <= PM; ++n) {
-        if (n < m || n > p) continue;
-        out[cre(n, m)] = acc_re[n];
-        if (m > 0) out[cim(n, m)] = acc_im[n];
+    __syncthreads();
+    U mx = 0;
+    for (int i = warp; i < nl; i += share) {
+        const int leaf = (int)(leaf0 + i);
+        T *out = M + cell_index(d, leaf & (nside - 1), (leaf >> d) & (nside - 1), leaf >> (2 * d)) * nc;
+        for (int k = lane; k < nc; k += 32) {
+            const T v = rows[i * nc + k];
+            out[k] = v;
+            if (amax) {
+                const U b = p2m_bits(v * sx[k]);
+                mx = b > mx ? b : mx;
+            }
+        }
+    }
+    if (amax) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const U v = __shfl_xor_sync(0xffffffffu, mx, o);
+            mx = v > mx ? v : mx;
+        }
+        if (lane == 0 && mx > 0) atomicMax(amax, mx);
     }
 }
 
@@ -445,6 +501,7 @@ fmm_status run_p2m_fixed(Plan &P, const Particle<float> *sp, float inv_h, unsign
     }
     const unsigned blocks = (unsigned)((P.nleaf + ROWS * P2M_WARPS - 1) / (ROWS * P2M_WARPS));
     k_p2m_fixed<PP, LPL><<<blocks, 32 * P2M_WARPS, sh, P.stream>>>(P.d, P.cell_start, sp, inv_h, (float *)P.M[P.d], s, amax);
+    FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
 
@@ -463,17 +520,22 @@ fmm_status launch_p2m_fixed(Plan &P, const Particle<float> *sp, float inv_h, uns
     }
 }
 
-template <typename T>
-void launch_p2m(Plan &P, const Particle<T> *sp, T inv_h)
+// leaves per warp: about 28 charges, so that mostly one round of 32 does, within 24 KB of rows and 32 leaves
+template <typename T, typename U>
+fmm_status launch_p2m(Plan &P, const Particle<T> *sp, T inv_h, const T *sx, U *amax)
 {
-    const int p = P.p, nside = 1 << P.d;
-    const int64_t nthr = P.nleaf * (p + 1);
-    const unsigned blocks = (unsigned)((nthr + 127) / 128);
-    if (p <= 4) k_p2m<T, 4><<<blocks, 128, 0, P.stream>>>(p, nside, P.cell_start, sp, inv_h, P.d, (T *)P.M[P.d]);
-    else if (p <= 8) k_p2m<T, 8><<<blocks, 128, 0, P.stream>>>(p, nside, P.cell_start, sp, inv_h, P.d, (T *)P.M[P.d]);
-    else if (p <= 12) k_p2m<T, 12><<<blocks, 128, 0, P.stream>>>(p, nside, P.cell_start, sp, inv_h, P.d, (T *)P.M[P.d]);
-    else if (p <= 16) k_p2m<T, 16><<<blocks, 128, 0, P.stream>>>(p, nside, P.cell_start, sp, inv_h, P.d, (T *)P.M[P.d]);
-    else k_p2m<T, P_MAX><<<blocks, 128, 0, P.stream>>>(p, nside, P.cell_start, sp, inv_h, P.d, (T *)P.M[P.d]);
+    const double occ = (double)P.N / (double)P.nleaf;
+    const int fit = (int)(24576 / (sizeof(T) * P.nc)), most = fit < 32 ? fit : 32;
+    int lb = (int)(28.0 / occ < most ? 28.0 / occ : most);
+    if (lb < 1) lb = 1;
+    // a warp per charge group where those groups fill the SMs' pipes; a column buffer per warp, 48 KB in all
+    int share = P.N < 152 * 32 * 4 ? P2M_SHARE : 1;
+    if (sizeof(T) * 2 * (P.p + 1) * 33 * share > 23000) share = 2;
+    const size_t sh = sizeof(T) * ((size_t)lb * P.nc + 2 * (P.p + 1) * 33 * share) + sizeof(int) * (lb + 1);
+    k_p2m<T, U><<<(unsigned)((P.nleaf + lb - 1) / lb), 32 * share, sh, P.stream>>>(P.p, P.d, lb, P.cell_start, sp, inv_h,
+                                                                            (T *)P.M[P.d], sx, amax);
+    FMM_LAUNCH_CHECK(P);
+    return FMM_OK;
 }
 
 // ------------------------------------------------------------------ M2L (CUDA cores)
@@ -724,34 +786,30 @@ fmm_status upward_t(Plan &P, bool solute_only)
         fmm_status st = tc ? tc_clear_amax(P) : res_clear_amax(P);
         if (st != FMM_OK) return st;
     }
-    // fp16 split: the P2M at a compile-time order folds the level maximum of |Mhat s| in as it writes.  Leaves so
-    // full that 8 lanes each would run long keep the thread-per-(leaf, order) kernel
-    bool amax_ready = false;
-    if (std::is_same<T, float>::value && (double)P.N <= 128.0 * (double)P.nleaf &&
-        (P.p == 4 || P.p == 6 || P.p == 8 || P.p == 10 || P.p == 12)) {
-        unsigned *amax = nullptr;
-        if (tc) {
-            amax = tc_amax(P, P.d);
-        }
-        const Particle<float> *spf = (const Particle<float> *)sp;
-        const float ih = (float)inv_h;
+    // where the M2L runs on the tensor cores, the P2M folds the level maximum of |Mhat s| in as it writes.  FP32 at the
+    // usual orders keeps its coefficients in registers, unless leaves are so full that 8 lanes each would run long
+    fmm_status st;
+    if constexpr (std::is_same<T, float>::value) {
+        unsigned *amax = tc ? tc_amax(P, P.d) : nullptr;
         const float *sc = tc ? tc_scale(P) : nullptr;
-        fmm_status st = P.p == 4    ? launch_p2m_fixed<4>(P, spf, ih, amax, sc)
-                        : P.p == 6  ? launch_p2m_fixed<6>(P, spf, ih, amax, sc)
-                        : P.p == 8  ? launch_p2m_fixed<8>(P, spf, ih, amax, sc)
-                        : P.p == 10 ? launch_p2m_fixed<10>(P, spf, ih, amax, sc)
-                                    : launch_p2m_fixed<12>(P, spf, ih, amax, sc);
-        if (st != FMM_OK) return st;
-        amax_ready = tc;
+        const bool sparse = (double)P.N <= 128.0 * (double)P.nleaf;
+        st = sparse && P.p == 4    ? launch_p2m_fixed<4>(P, sp, inv_h, amax, sc)
+             : sparse && P.p == 6  ? launch_p2m_fixed<6>(P, sp, inv_h, amax, sc)
+             : sparse && P.p == 8  ? launch_p2m_fixed<8>(P, sp, inv_h, amax, sc)
+             : sparse && P.p == 10 ? launch_p2m_fixed<10>(P, sp, inv_h, amax, sc)
+             : sparse && P.p == 12 ? launch_p2m_fixed<12>(P, sp, inv_h, amax, sc)
+                                   : launch_p2m<float, unsigned>(P, sp, inv_h, sc, amax);
     } else {
-        launch_p2m<T>(P, sp, inv_h);
+        const double *sc = nullptr;
+        unsigned long long *amax = res_amax(P, P.d, &sc);
+        st = launch_p2m<double, unsigned long long>(P, sp, inv_h, sc, amax);
     }
-    FMM_LAUNCH_CHECK(P);
+    if (st != FMM_OK) return st;
     for (int l = P.d - 1; l >= 1; --l) {  // the top operator starts from level 1
         fmm_status st = launch_m2m(P, l);
         if (st != FMM_OK) return st;
     }
-    return tc ? tc_split_moments(P, amax_ready) : FMM_OK;
+    return tc ? tc_split_moments(P) : FMM_OK;
 }
 
 }  // namespace

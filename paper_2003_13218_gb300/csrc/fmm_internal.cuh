@@ -317,9 +317,9 @@ bool tc_available(const Plan &P, int level);
 // fp16 split: L2L fused into each level's M2L
 bool tc_translations(const Plan &P);
 fmm_status tc_prepare(Plan &P);
-// fp16 split: balanced halo planes of all levels (the end of the upward pass); leaf_amax_ready: the P2M has
-// already folded the deepest level's largest |Mhat s| into tc_amax (else it is computed here)
-fmm_status tc_split_moments(Plan &P, bool leaf_amax_ready);
+// fp16 split: balanced halo planes of all levels (the end of the upward pass); the P2M and M2M have folded each
+// level's largest |Mhat s| into tc_amax
+fmm_status tc_split_moments(Plan &P);
 // fp16 split: the device word of level l's largest |Mhat s| (float bits), into which the kernel that produces
 // M[l] folds its maximum; tc_clear_amax clears the words of all levels (M and L) at the start of a far-field
 // pass; s(n,m) per real coefficient
@@ -338,7 +338,7 @@ bool res_available(const Plan &P, int level);
 // builds the state on an FP64 plan's first evaluation (a plan that is to run the mixed path never pays for it);
 // left for later while the plan's stream is being captured
 fmm_status res_ensure(Plan &P);
-// where the M2M into a level leaves its largest |Mhat s|, and s (null without the state)
+// where the P2M and M2M leave a level's largest |Mhat s|, and s (null without the state)
 unsigned long long *res_amax(Plan &P, int level, const double **s);
 fmm_status res_clear_amax(Plan &P);  // at the start of a far-field pass
 fmm_status launch_m2l_res(Plan &P, int level);

@@ -120,27 +120,6 @@ __global__ void k_res_ops(int noff, const double *__restrict__ T, int nc, int np
     }
 }
 
-// largest |M^ s| of a level as double bits (positive doubles order as integers); a NaN is larger than all
-__global__ void k_res_absmax(const double *__restrict__ M, int64_t ncell, int nc, const double *__restrict__ s,
-                             unsigned long long *__restrict__ amax)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    unsigned long long m = 0;
-    for (int64_t c = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); c < ncell; c += warps) {
-        const double *row = M + c * nc;
-        for (int k = lane; k < nc; k += 32) {
-            const unsigned long long v = (unsigned long long)__double_as_longlong(row[k] * s[k]) & ~(1ull << 63);
-            m = v > m ? v : m;
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
-        m = v > m ? v : m;
-    }
-    if (lane == 0 && m > 0) atomicMax(amax, m);
-}
-
 // FP64 class-layout moments -> residue planes of moduli m0 .. m0 + nb - 1 with a periodic halo, 8 coefficients per
 // thread (16-byte stores per plane), zero beyond nc.  Bound by the integer arithmetic of the residues (~15
 // instructions each) and the planes' bytes.
@@ -459,11 +438,6 @@ fmm_status launch_m2l_res(Plan &P, int l)
     if (!S) return FMM_ERR_INTERNAL;
     const int np = 1 << (l - 1), nc = P.nc, n = S->c.n;
     const int64_t np2 = np + 2 * P.ws, cells = (int64_t)8 * np * np * np;
-    if (l == P.d) {  // the M2M into a level folds its maximum in
-        k_res_absmax<<<blocks_upto(cells, 8, 1216), 256, 0, P.stream>>>((const double *)P.M[l], cells, nc, S->s64,
-                                                                        S->amax + l);
-        FMM_LAUNCH_CHECK(P);
-    }
     TcArgs a;
     memset(&a, 0, sizeof(a));
     a.np = np;

@@ -106,22 +106,6 @@ __device__ __forceinline__ void split_terms(float v, int parts, uint16_t *o, siz
     }
 }
 
-// largest |M^ s(k)| of a level (fp16 split), as float bits into *amax; one
-// warp per cell, lanes over the coefficients
-__global__ void k_absmax(const float *__restrict__ M, int64_t ncell, int nc, const float *__restrict__ s,
-                         unsigned *__restrict__ amax)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    float m = 0.f;
-    for (int64_t c = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); c < ncell; c += warps) {
-        const float *row = M + c * nc;
-        for (int k = lane; k < nc; k += 32) m = fmaxf(m, fabsf(row[k] * __ldg(s + k)));
-    }
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0 && m > 0.f) atomicMax(amax, __float_as_uint(m));  // positive floats order as integers
-}
-
 // FP32 class-layout moments -> bf16 split planes [part][chunk][class][hz][hy][hx][k] with a
 // periodic halo; rows kp wide (zero beyond nc).  One warp per halo cell, lanes over the coefficients.
 __global__ void k_split_halo(const float *__restrict__ M, int np, int hw, int nc, int kp, int parts,
@@ -838,18 +822,11 @@ const float *tc_scale(const Plan &P)
     return S && S->f16 ? S->s32 : nullptr;
 }
 
-// fp16 split: the balanced halo planes of every level; a level's largest |M^ s| was folded in by the M2M that wrote
-// it, the deepest one's by the P2M (leaf_amax_ready) or it is computed here
-fmm_status tc_split_moments(Plan &P, bool leaf_amax_ready)
+// fp16 split: the balanced halo planes of every level, whose largest |M^ s| the P2M and M2M have folded in
+fmm_status tc_split_moments(Plan &P)
 {
     TcState *S = (TcState *)P.tc;
     if (!S || !S->f16) return FMM_ERR_INTERNAL;
-    if (!leaf_amax_ready) {
-        const int64_t ncell = (int64_t)1 << (3 * P.d);
-        k_absmax<<<(unsigned)((ncell + 7) / 8 < 1216 ? (ncell + 7) / 8 : 1216), 256, 0, P.stream>>>(
-            (const float *)P.M[P.d], ncell, P.nc, S->s32, S->amax + P.d);
-        FMM_LAUNCH_CHECK(P);
-    }
     SplitLevels lv;
     memset(&lv, 0, sizeof(lv));
     int i = 0;
