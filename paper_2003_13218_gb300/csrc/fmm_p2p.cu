@@ -21,7 +21,7 @@ __device__ inline T inv_sqrt(T x);
 template <>
 __device__ inline float inv_sqrt<float>(float x) { return rsqrtf(x); }
 template <>
-__device__ inline double inv_sqrt<double>(double x) { return 1.0 / sqrt(x); }
+__device__ inline double inv_sqrt<double>(double x) { return rsqrt(x); }  // within 1 ulp; 1.0 / sqrt(x) is twice the instructions
 
 // One source of the near field: adds q_j / r and q_j r / r^3 for r = (ox, oy, oz) - x_j.  A source at r = 0
 // (the target itself: the same stored coordinates) adds nothing; the near field never holds a charge's own
@@ -72,8 +72,55 @@ __device__ __forceinline__ void stage_copy(Particle<T> *dst, const Particle<T> *
     }
 }
 
+// The FP64 target loop.  GB300's FP64 pipe takes 16 cycles per warp instruction however many lanes are active, so the
+// loops run over whole rows of neighbours (the 2 WS + 1 leaves of a row are contiguous; which leaf, hence which shift, a
+// source is in follows from integer compares): the lanes of a warp differ by 14 sources in 9 where leaf by leaf they
+// wait for the fullest leaf, 6 in 3.  In small systems `split` neighbouring lanes share a target and take its rows in
+// turn.  100,000 charges at depth 5: 1,240 us leaf by leaf with 1 / sqrt, 631 us here; 2,998 at depth 3 278 and 88 us.
+template <int WS, bool STAGED>
+__device__ __forceinline__ void p2p_rows(int W, int it, int lane_of, int split, double h, const Particle<double> &pi,
+                                         const int *pre, const int *gst, const Particle<double> *stg,
+                                         const Particle<double> *__restrict__ sp, double (&out)[4])
+{
+    constexpr int SIDE = 2 * WS + 1;
+    double ox[SIDE];
+#pragma unroll
+    for (int t = 0; t < SIDE; ++t) ox[t] = pi.x - (double)(t - WS) * h;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k] = 0.0;
+    for (int r = lane_of; r < SIDE * SIDE; r += split) {
+        const double oy = pi.y - (double)(r % SIDE - WS) * h, oz = pi.z - (double)(r / SIDE - WS) * h;
+        const int f = r * W + it - WS;
+        int b[SIDE], off[SIDE];  // each leaf's first staged index and its distance from the sorted one
+#pragma unroll
+        for (int t = 0; t < SIDE; ++t) {
+            b[t] = pre[f + t];
+            off[t] = STAGED ? 0 : gst[f + t] - b[t];
+        }
+        const int je = pre[f + SIDE];
+        double acc = 0.0, ex = 0.0, ey = 0.0, ez = 0.0;
+        for (int j = b[0]; j < je; ++j) {
+            double x = ox[0];
+            int o = off[0];
+#pragma unroll
+            for (int t = 1; t < SIDE; ++t) {
+                x = j >= b[t] ? ox[t] : x;
+                o = j >= b[t] ? off[t] : o;
+            }
+            p2p_pair<double>(STAGED ? stg[j] : sp[j + o], x, oy, oz, acc, ex, ey, ez);
+        }
+        out[0] += acc;
+        out[1] += ex;
+        out[2] += ey;
+        out[3] += ez;
+    }
+    for (int o = 1; o < split; o <<= 1)  // the whole warp is here
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out[k] += __shfl_xor_sync(0xffffffffu, out[k], o);
+}
+
 template <typename T>
-__global__ void __launch_bounds__(P2P_THREADS) k_p2p_tile(int d, int ws, int bx, int cap, T h,
+__global__ void __launch_bounds__(P2P_THREADS) k_p2p_tile(int d, int ws, int bx, int cap, int split, T h,
                                                           const int *__restrict__ start,
                                                           const Particle<T> *__restrict__ sp, T *__restrict__ phi,
                                                           T *__restrict__ field)
@@ -139,56 +186,90 @@ __global__ void __launch_bounds__(P2P_THREADS) k_p2p_tile(int d, int ws, int bx,
     // 3. targets: the leaves x0 .. x0 + bx - 1 of the centre row
     const int rc = ws * side + ws;
     const int tb = pre[rc * W + ws], te = pre[rc * W + ws + bx];
-    for (int st = tb + (int)threadIdx.x; st < te; st += P2P_THREADS) {
-        int lo = rc * W + ws, hi = rc * W + ws + bx;  // the target's staged leaf
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (pre[mid] <= st) lo = mid;
-            else hi = mid;
+    if constexpr (sizeof(T) == 8) {
+        for (int u0 = 0; u0 < (te - tb) * split; u0 += P2P_THREADS) {
+            const int u = u0 + (int)threadIdx.x;
+            const bool on = u < (te - tb) * split;
+            const int st = on ? tb + u / split : te - 1;  // spare lanes redo the last target and store nothing
+            int lo = rc * W + ws, hi = rc * W + ws + bx;
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (pre[mid] <= st) lo = mid;
+                else hi = mid;
+            }
+            const int it = lo - rc * W, s = gst[lo] + (st - pre[lo]);
+            // a warp with no target of its own: nothing to do (the shuffles stay within a warp)
+            if (__ballot_sync(0xffffffffu, on) == 0) continue;
+            const Particle<T> pi = staged ? stg[st] : sp[s];
+            T v[4];
+            if (ws == 1) {
+                if (staged) p2p_rows<1, true>(W, it, u % split, split, h, pi, pre, gst, stg, sp, v);
+                else p2p_rows<1, false>(W, it, u % split, split, h, pi, pre, gst, stg, sp, v);
+            } else {
+                if (staged) p2p_rows<2, true>(W, it, u % split, split, h, pi, pre, gst, stg, sp, v);
+                else p2p_rows<2, false>(W, it, u % split, split, h, pi, pre, gst, stg, sp, v);
+            }
+            if (on && u % split == 0) {
+                phi[s] = v[0];
+                if (field) {
+                    field[3 * s] = v[1];
+                    field[3 * s + 1] = v[2];
+                    field[3 * s + 2] = v[3];
+                }
+            }
         }
-        const int it = lo - rc * W;  // index of the target leaf within its row
-        const int s = gst[lo] + (st - pre[lo]);  // sorted index of the target
-        const Particle<T> pi = staged ? stg[st] : sp[s];
-        // four independent partial sums (sources j, j + 1, j + 2, j + 3 of each leaf), so that the loads and
-        // the dependent additions of consecutive pairs overlap; added in a fixed order at the end
-        T a[4] = {0, 0, 0, 0}, fx[4] = {0, 0, 0, 0}, fy[4] = {0, 0, 0, 0}, fz[4] = {0, 0, 0, 0};
-        for (int dz = -ws; dz <= ws; ++dz)
-            for (int dy = -ws; dy <= ws; ++dy)
-                for (int dx = -ws; dx <= ws; ++dx) {
-                    const int f = ((dz + ws) * side + dy + ws) * W + it + dx;
-                    const T ox = pi.x - T(dx) * h, oy = pi.y - T(dy) * h, oz = pi.z - T(dz) * h;
-                    int jb, je;
-                    const Particle<T> *src;
-                    if (staged) {
-                        jb = pre[f];
-                        je = pre[f + 1];
-                        src = stg;
-                    } else {  // the leaf's records in the sorted array
-                        jb = gst[f];
-                        je = jb + (pre[f + 1] - pre[f]);
-                        src = sp;
-                    }
-                    int j = jb;
-                    for (; j + 4 <= je; j += 4) {
-                        Particle<T> q4[4];
+    } else {
+        for (int st = tb + (int)threadIdx.x; st < te; st += P2P_THREADS) {
+            int lo = rc * W + ws, hi = rc * W + ws + bx;  // the target's staged leaf
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (pre[mid] <= st) lo = mid;
+                else hi = mid;
+            }
+            const int it = lo - rc * W;  // index of the target leaf within its row
+            const int s = gst[lo] + (st - pre[lo]);  // sorted index of the target
+            const Particle<T> pi = staged ? stg[st] : sp[s];
+            // four independent partial sums (sources j, j + 1, j + 2, j + 3 of each leaf), so that the loads and
+            // the dependent additions of consecutive pairs overlap; added in a fixed order at the end
+            T a[4] = {0, 0, 0, 0}, fx[4] = {0, 0, 0, 0}, fy[4] = {0, 0, 0, 0}, fz[4] = {0, 0, 0, 0};
+            for (int dz = -ws; dz <= ws; ++dz)
+                for (int dy = -ws; dy <= ws; ++dy)
+                    for (int dx = -ws; dx <= ws; ++dx) {
+                        const int f = ((dz + ws) * side + dy + ws) * W + it + dx;
+                        const T ox = pi.x - T(dx) * h, oy = pi.y - T(dy) * h, oz = pi.z - T(dz) * h;
+                        int jb, je;
+                        const Particle<T> *src;
+                        if (staged) {
+                            jb = pre[f];
+                            je = pre[f + 1];
+                            src = stg;
+                        } else {  // the leaf's records in the sorted array
+                            jb = gst[f];
+                            je = jb + (pre[f + 1] - pre[f]);
+                            src = sp;
+                        }
+                        int j = jb;
+                        for (; j + 4 <= je; j += 4) {
+                            Particle<T> q4[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) q4[u] = src[j + u];
+                            for (int u = 0; u < 4; ++u) q4[u] = src[j + u];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) p2p_pair<T>(q4[u], ox, oy, oz, a[u], fx[u], fy[u], fz[u]);
-                    }
-                    if (j < je) {
-                        p2p_pair<T>(src[j], ox, oy, oz, a[0], fx[0], fy[0], fz[0]);
-                        if (j + 1 < je) {
-                            p2p_pair<T>(src[j + 1], ox, oy, oz, a[1], fx[1], fy[1], fz[1]);
-                            if (j + 2 < je) p2p_pair<T>(src[j + 2], ox, oy, oz, a[2], fx[2], fy[2], fz[2]);
+                            for (int u = 0; u < 4; ++u) p2p_pair<T>(q4[u], ox, oy, oz, a[u], fx[u], fy[u], fz[u]);
+                        }
+                        if (j < je) {
+                            p2p_pair<T>(src[j], ox, oy, oz, a[0], fx[0], fy[0], fz[0]);
+                            if (j + 1 < je) {
+                                p2p_pair<T>(src[j + 1], ox, oy, oz, a[1], fx[1], fy[1], fz[1]);
+                                if (j + 2 < je) p2p_pair<T>(src[j + 2], ox, oy, oz, a[2], fx[2], fy[2], fz[2]);
+                            }
                         }
                     }
-                }
-        phi[s] = (a[0] + a[1]) + (a[2] + a[3]);
-        if (field) {
-            field[3 * s] = (fx[0] + fx[1]) + (fx[2] + fx[3]);
-            field[3 * s + 1] = (fy[0] + fy[1]) + (fy[2] + fy[3]);
-            field[3 * s + 2] = (fz[0] + fz[1]) + (fz[2] + fz[3]);
+            phi[s] = (a[0] + a[1]) + (a[2] + a[3]);
+            if (field) {
+                field[3 * s] = (fx[0] + fx[1]) + (fx[2] + fx[3]);
+                field[3 * s + 1] = (fy[0] + fy[1]) + (fy[2] + fy[3]);
+                field[3 * s + 2] = (fz[0] + fz[1]) + (fz[2] + fz[3]);
+            }
         }
     }
 }
@@ -382,7 +463,7 @@ namespace {
 // capacity is 1.25 times the expected particle count of a tile's rows plus 256 (a tile beyond it reads global memory;
 // twice the count plus 512 left room for one block less per SM: 10M charges 23.1 -> 22.2 ms, 100k at ws = 2 1.62 ->
 // 1.53 ms), within 96 KB of
-// shared memory
+// shared memory.  The FP32 path keeps one thread per target: it runs beside the far field
 template <typename T>
 fmm_status launch_p2p_tile(Plan &P, T h, T *phi, T *field)
 {
@@ -394,8 +475,14 @@ fmm_status launch_p2p_tile(Plan &P, T h, T *phi, T *field)
     }
     const int n = 1 << P.d;
     const double occ = (double)P.N / (double)P.nleaf;
+    // FP64: lanes per target until every SM has 8 warps, and tiles for two blocks per SM
+    int split = 1;
+    if (sizeof(T) == 8)
+        while (split < 8 && P.N * split < 152 * 8 * 32) split *= 2;
     int bx = 1;
-    while (bx < 32 && bx < n && (double)(2 * bx) * occ <= 128.0) bx *= 2;
+    while (bx < 32 && bx < n && (double)(2 * bx) * occ * split <= 128.0) bx *= 2;
+    if (sizeof(T) == 8)
+        while (bx > 1 && (int64_t)n * n * (n / bx) < 304) bx /= 2;
     const int side = 2 * P.ws + 1, F = side * side * (bx + 2 * P.ws);
     const size_t head = ((sizeof(int) * (2 * F + 1) + 15) / 16) * 16;
     const double expect = (double)P.N / (double)P.nleaf * F;
@@ -404,7 +491,7 @@ fmm_status launch_p2p_tile(Plan &P, T h, T *phi, T *field)
     if (cap > cap_max) cap = cap_max;
     const unsigned blocks = (unsigned)((int64_t)n * n * (n / bx));
     k_p2p_tile<T><<<blocks, P2P_THREADS, head + cap * sizeof(Particle<T>), P.stream>>>(
-        P.d, P.ws, bx, (int)cap, h, P.cell_start, (const Particle<T> *)P.sorted, phi, field);
+        P.d, P.ws, bx, (int)cap, split, h, P.cell_start, (const Particle<T> *)P.sorted, phi, field);
     return FMM_OK;
 }
 
