@@ -603,64 +603,78 @@ __global__ void k_m2l_simt(int p, int l, int cls, int ws, const T *__restrict__ 
 // grad Phi = (1/h^2) sum_{n',m'} G_{n'}^{m'} R_{n'}^{m'}(v) with
 //   G^z = L_{n'+1}^{m'},  G^x = (L_{n'+1}^{m'-1} - L_{n'+1}^{m'+1})/2,
 //   G^y = -i (L_{n'+1}^{m'-1} + L_{n'+1}^{m'+1})/2.
+// Any order, `split` neighbouring lanes per charge, which take the columns m in turn: in small FP64 systems a charge's
+// whole sum by one thread is a long chain on few warps (an FP64 warp instruction holds one of an SM's four pipes for 64
+// cycles; 2,998 charges at p = 8: 44 us, here 29 us).  The sums over n of a column are formed without its weight (1 for m = 0, else
+// 2) and without the halves of G^x and G^y.
 template <typename T>
-__global__ void k_l2p(int p, int d, int64_t N, const int *__restrict__ sleaf, const Particle<T> *__restrict__ sp,
-                      T inv_h, const T *__restrict__ L, T *__restrict__ phi, T *__restrict__ grad)
+__global__ void __launch_bounds__(128) k_l2p(int p, int split, int d, int64_t N, const int *__restrict__ sleaf,
+                                             const Particle<T> *__restrict__ sp, T inv_h, const T *__restrict__ L,
+                                             T *__restrict__ phi, T *__restrict__ grad)
 {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= N) return;
-    int nside = 1 << d;
-    int leaf = sleaf[s];
-    int x = leaf % nside, y = (leaf / nside) % nside, z = leaf / (nside * nside);
-    const T *Lc = L + cell_index(d, x, y, z) * ncoef(p);
-    Particle<T> pt = sp[s];
-    T vx = pt.x * inv_h, vy = pt.y * inv_h, vz = pt.z * inv_h;
-    T r2 = vx * vx + vy * vy + vz * vz;
+    const ExpandFactors<T> &F = expand_factors<T>();
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool on = t < N * split;
+    const int64_t s = on ? t / split : N - 1;  // the spare lanes of the last warp take part in the shuffles
+    const int sub = (int)(t % split);
+    const int mask = (1 << d) - 1, leaf = sleaf[s];
+    const T *Lc = L + cell_index(d, leaf & mask, (leaf >> d) & mask, leaf >> (2 * d)) * ncoef(p);
+    const Particle<T> pt = sp[s];
+    const T vx = pt.x * inv_h, vy = pt.y * inv_h, vz = pt.z * inv_h;
+    const T r2 = vx * vx + vy * vy + vz * vz;
     T pot = 0, gx = 0, gy = 0, gz = 0;
     T dre = 1, dim = 0;
-    for (int m = 0; m <= p; ++m) {
-        if (m > 0) {
-            T sc = T(-0.5) / T(m);
-            T nre = sc * (vx * dre - vy * dim);
-            T nim = sc * (vx * dim + vy * dre);
+    int at = 0;  // (dre, dim) = R_at^at
+    for (int m = sub; m <= p; m += split) {
+        for (; at < m; ++at) {
+            const T cx = F.c[at + 1] * vx, cy = F.c[at + 1] * vy;
+            const T nre = cx * dre - cy * dim;
+            dim = cx * dim + cy * dre;
             dre = nre;
-            dim = nim;
         }
-        T w = m == 0 ? T(1) : T(2);
         T p2re = 0, p2im = 0, rre = dre, rim = dim;
+        T spot = 0, sx = 0, sy = 0, sz = 0;
         for (int n = m; n <= p; ++n) {
             if (n > m) {
-                T a = T(2 * n - 1) * vz;
-                T inv = T(1) / T((n + m) * (n - m));
-                T cr = (a * rre - r2 * p2re) * inv;
-                T ci = (a * rim - r2 * p2im) * inv;
+                const T a = F.a[m * (P_MAX + 1) + n] * vz, b = F.b[m * (P_MAX + 1) + n] * r2;
+                const T cr = a * rre - b * p2re, ci = a * rim - b * p2im;
                 p2re = rre;
                 p2im = rim;
                 rre = cr;
                 rim = ci;
             }
-            Cx<T> Lnm = coef(Lc, n, m);
-            pot += w * (Lnm.re * rre - Lnm.im * rim);
+            const Cx<T> Lnm = coef(Lc, n, m);
+            spot += Lnm.re * rre - Lnm.im * rim;
             if (grad && n < p) {
-                Cx<T> a = coef(Lc, n + 1, m - 1), b = coef(Lc, n + 1, m + 1), c = coef(Lc, n + 1, m);
-                Cx<T> Gx = {T(0.5) * (a.re - b.re), T(0.5) * (a.im - b.im)};
-                Cx<T> Gy = {T(0.5) * (a.im + b.im), -T(0.5) * (a.re + b.re)};
-                gx += w * (Gx.re * rre - Gx.im * rim);
-                gy += w * (Gy.re * rre - Gy.im * rim);
-                gz += w * (c.re * rre - c.im * rim);
+                const Cx<T> a = coef(Lc, n + 1, m - 1), b = coef(Lc, n + 1, m + 1), c = coef(Lc, n + 1, m);
+                sx += (a.re - b.re) * rre - (a.im - b.im) * rim;
+                sy += (a.im + b.im) * rre + (a.re + b.re) * rim;
+                sz += c.re * rre - c.im * rim;
             }
         }
+        const T w = m == 0 ? T(1) : T(2);
+        pot += w * spot;
+        gx += w * sx;
+        gy += w * sy;
+        gz += w * sz;
     }
+    for (int o = 1; o < split; o <<= 1) {
+        pot += __shfl_xor_sync(0xffffffffu, pot, o);
+        gx += __shfl_xor_sync(0xffffffffu, gx, o);
+        gy += __shfl_xor_sync(0xffffffffu, gy, o);
+        gz += __shfl_xor_sync(0xffffffffu, gz, o);
+    }
+    if (!on || sub != 0) return;
     phi[s] = pot * inv_h;
     if (grad) {
-        T s2 = inv_h * inv_h;
-        grad[3 * s] = gx * s2;
-        grad[3 * s + 1] = gy * s2;
+        const T s2 = inv_h * inv_h;
+        grad[3 * s] = T(0.5) * gx * s2;
+        grad[3 * s + 1] = T(0.5) * gy * s2;
         grad[3 * s + 2] = gz * s2;
     }
 }
 
-// The same L2P at a compile-time order PP: the loops unroll, the recurrences' reciprocals fold into
+// L2P at a compile-time order PP, one thread per charge: the loops unroll, the recurrences' reciprocals fold into
 // constants and the coefficient indices into immediates.  The expansions of the block's leaves
 // (consecutive in the sorted order) are staged in shared memory when at most L2P_LEAVES of them span
 // the block: a warp's particles sit in several leaves, and each of its coefficient loads would touch
@@ -758,19 +772,21 @@ fmm_status launch_l2p_fixed(Plan &P, T inv_h, const T *L, T *phi, T *grad)
     return FMM_OK;
 }
 
-// L2P of the plan at its order: the fixed-order kernel for the usual orders, else the generic one
+// L2P of the plan at its order: the fixed-order kernel for the usual orders, else the generic one, and that with four
+// lanes per charge in FP64 where one lane each would leave a pipe without a warp
 template <typename T>
 fmm_status l2p_t(Plan &P, T inv_h, const T *L, T *phi, T *grad)
 {
-    switch (P.p) {
+    const int split = std::is_same<T, double>::value && P.N < 152 * 32 * 4 ? 4 : 1;
+    switch (split > 1 ? -1 : P.p) {
     case 4: return launch_l2p_fixed<T, 4>(P, inv_h, L, phi, grad);
     case 6: return launch_l2p_fixed<T, 6>(P, inv_h, L, phi, grad);
     case 8: return launch_l2p_fixed<T, 8>(P, inv_h, L, phi, grad);
     case 10: return launch_l2p_fixed<T, 10>(P, inv_h, L, phi, grad);
     case 12: return launch_l2p_fixed<T, 12>(P, inv_h, L, phi, grad);
     default:
-        k_l2p<T><<<blocks_for(P.N, 128), 128, 0, P.stream>>>(P.p, P.d, P.N, P.sleaf, (const Particle<T> *)P.sorted,
-                                                             inv_h, L, phi, grad);
+        k_l2p<T><<<blocks_for(P.N * split, 128), 128, 0, P.stream>>>(P.p, split, P.d, P.N, P.sleaf,
+                                                                     (const Particle<T> *)P.sorted, inv_h, L, phi, grad);
         return FMM_OK;
     }
 }
