@@ -219,7 +219,10 @@ __device__ void block_reduce_store(const double (&acc)[NQ], double *__restrict__
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         double v = acc[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        // most warps have no solute charge: half of the quantities are zero in all lanes, and adding them up would
+        // only occupy the FP64 pipe
+        if (__any_sync(0xffffffffu, v != 0.0))
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) sh[w][q] = v;
     }
     __syncthreads();
@@ -261,10 +264,11 @@ __device__ void final_sum(const double *__restrict__ partial, int nb, double *ou
                 c[u] = b < nb ? __ldcg(partial + (b * NQ + q) * 2 + 1) : 0.0;
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                k.add(v[u]);
-                k.c += c[u];
-            }
+            for (int u = 0; u < 4; ++u)
+                if (b0 + 32 * u < nb) {
+                    k.add(v[u]);
+                    k.c += c[u];
+                }
         }
         k = warp_merge(k);
         if (lane == 0) out[q] = k.val();
@@ -450,12 +454,14 @@ __global__ void k_potentials_out(int64_t N, const int *__restrict__ perm, const 
 
 inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-// blocks of a reduction: twice the SMs, fewer below 311,296 charges (1,024 a block: each block's sum is one more for
-// the last block, whose part is a chain of FP64 latencies)
+// blocks of a reduction: one element per thread while that takes no more than a block per SM, then four, then two
+// blocks per SM
 inline unsigned red_blocks(int64_t n)
 {
-    const int64_t b = (n + 4 * RED_THREADS - 1) / (4 * RED_THREADS);
-    return (unsigned)(b < RED_BLOCKS ? b : RED_BLOCKS);
+    const int64_t one = (n + RED_THREADS - 1) / RED_THREADS, four = (one + 3) / 4;
+    if (one <= RED_BLOCKS / 2) return (unsigned)one;
+    if (four <= RED_BLOCKS / 2) return RED_BLOCKS / 2;
+    return (unsigned)(four < RED_BLOCKS ? four : RED_BLOCKS);
 }
 
 }  // namespace
