@@ -903,12 +903,7 @@ void free_tables(Plan &P)
     cudaFree(P.tab.l2l64);
     cudaFree(P.tab.l2l32);
     cudaFree(P.tab.m2m64);
-    cudaFree(P.tab.m2m_fold64);
-    cudaFree(P.tab.m2m_fold32);
-    cudaFree(P.tab.l2l_fold64);
-    cudaFree(P.tab.l2l_fold32);
-    cudaFree(P.tab.fold_cnt);
-    cudaFree(P.tab.fold_beg);
+    cudaFree(P.tab.m2m_fold64);  // and the other folded tables behind it
     cudaFree(P.tab.il);
     cudaFree(P.tab.G64);
     cudaFree(P.tab.G32);

@@ -20,6 +20,7 @@
 // 300 us (316), 61,000 with 210 solute charges 559 us (602); 1M and 10M within 1 % of before.
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "fmm_internal.cuh"
@@ -170,12 +171,14 @@ void m2m_entries(int nc, const std::vector<double> &A, std::vector<FoldEntry<dou
 {
     ent.assign((size_t)nc * nc, FoldEntry<double>{0.0, 0});
     cnt.assign(nc, 0);
+    std::vector<int> sign(nc);
+    for (int k = 0; k < nc; ++k) sign[k] = mirror_signs(k);
     for (int j0 = 0; j0 < nc; j0 += 8) {
         std::vector<int> left[8][8];  // [row][residue]: the k still to take, the lowest last
         for (int r = 0; r < 8 && j0 + r < nc; ++r)
             for (int k = nc - 1; k >= 0; --k)
                 if (A[(size_t)(j0 + r) * nc + k] != 0.0)
-                    left[r][((mirror_signs(j0 + r) ^ mirror_signs(k)) * nc + k) & 7].push_back(k);
+                    left[r][((sign[j0 + r] ^ sign[k]) * nc + k) & 7].push_back(k);
         for (bool more = true; more;) {
             more = false;
             bool used[8] = {};
@@ -193,7 +196,7 @@ void m2m_entries(int nc, const std::vector<double> &A, std::vector<FoldEntry<dou
                 const int j = j0 + r, k = left[r][best].back();
                 left[r][best].pop_back();
                 used[best] = more = true;
-                ent[(size_t)cnt[j]++ * nc + j] = {A[(size_t)j * nc + k], (mirror_signs(j) ^ mirror_signs(k)) * nc + k};
+                ent[(size_t)cnt[j]++ * nc + j] = {A[(size_t)j * nc + k], (sign[j] ^ sign[k]) * nc + k};
             }
         }
     }
@@ -436,12 +439,15 @@ fmm_status build_translation_ops(Plan &P)
         FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l64, sizeof(double) * 2 * n));
         FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l32, sizeof(float) * 2 * n));
         FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m64, sizeof(double) * n));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m_fold64, sizeof(FoldEntry<double>) * nc * nc));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.m2m_fold32, sizeof(FoldEntry<float>) * nc * nc));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l_fold64, sizeof(FoldEntry<double>) * nc * nc));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.l2l_fold32, sizeof(FoldEntry<float>) * nc * nc));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.fold_cnt, sizeof(int) * nc));
-        FMM_CUDA_TRY(cudaMalloc(&P.tab.fold_beg, sizeof(int) * 9 * nc));
+        const size_t n64 = sizeof(FoldEntry<double>) * nc * nc, n32 = sizeof(FoldEntry<float>) * nc * nc;
+        char *fold = nullptr;  // one allocation, m2m_fold64's
+        FMM_CUDA_TRY(cudaMalloc(&fold, 2 * n64 + 2 * n32 + sizeof(int) * 10 * nc));
+        P.tab.m2m_fold64 = fold;
+        P.tab.l2l_fold64 = fold + n64;
+        P.tab.m2m_fold32 = fold + 2 * n64;
+        P.tab.l2l_fold32 = fold + 2 * n64 + n32;
+        P.tab.fold_cnt = (int *)(fold + 2 * n64 + 2 * n32);
+        P.tab.fold_beg = P.tab.fold_cnt + nc;
     }
     k_l2l_ops<<<blocks_for(n, 256), 256, 0, P.stream>>>(P.p, P.tab.Rw64, P.tab.l2l64, P.tab.l2l32);
     FMM_LAUNCH_CHECK(P);
@@ -458,14 +464,15 @@ fmm_status build_translation_ops(Plan &P)
         std::vector<FoldEntry<double>> e64;
         std::vector<int> cnt;
         m2m_entries(nc, A, e64, cnt);
-        std::vector<FoldEntry<float>> e32(e64.size());
+        const size_t used = (size_t)nc * *std::max_element(cnt.begin(), cnt.end());  // entries of the longest row
+        e64.resize(used);
+        std::vector<FoldEntry<float>> e32(used);
         for (size_t i = 0; i < e64.size(); ++i) e32[i] = {(float)e64[i].v, e64[i].at};
         FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.m2m_fold64, e64.data(), sizeof(e64[0]) * e64.size(), cudaMemcpyHostToDevice,
                                      P.stream));
         FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.m2m_fold32, e32.data(), sizeof(e32[0]) * e32.size(), cudaMemcpyHostToDevice,
                                      P.stream));
         FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.fold_cnt, cnt.data(), sizeof(int) * nc, cudaMemcpyHostToDevice, P.stream));
-        FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
     }
     // four parents at p = 20 take 113 KB (FP64)
     FMM_CUDA_TRY(cudaFuncSetAttribute(k_m2m_fold<double, FOLD_PB, unsigned long long>,
