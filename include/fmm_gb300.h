@@ -132,9 +132,9 @@ enum {
                               products: ~2^-12 relative on those terms), the other steps keep all 3; 0 = never.  Contributions of high input
                               degrees to a well-separated cell's local expansion are small, so the error stays far
                               below the first-term precision of the low degrees.  D2, D1 in 0..20; default
-                              FMM_GRADE_DEFAULT.  M2M, the fused L2L and the solute-only pass always use 3
+                              FMM_GRADE_DEFAULT.  The fused L2L and the solute-only pass always use 3
                               products */,
-    FMM_OPT_M2L_ACC_GROUP = 11 /* ival in 1..64: tensor-core M2L / M2M offsets whose products are summed in
+    FMM_OPT_M2L_ACC_GROUP = 11 /* ival in 1..64: tensor-core M2L offsets whose products are summed in
                               one FP32 TMEM accumulator before it is drained into registers (the fused L2L
                               always alone); longer chains drain less often but carry more of the tensor
                               core's accumulation rounding; default FMM_ACC_GROUP_DEFAULT */,
@@ -156,7 +156,7 @@ enum {
                               evaluation returns FMM_ERR_TIMEOUT after the wait budget (use with
                               FMM_OPT_M2L_PAIR = 0 and a short budget) */
     FMM_OPT_M2L_BRICK = 17        /* ival = l | bx << 8 | by << 16 | bz << 24: the tiles of the tensor-core M2L of
-                              level l (2..depth; and the M2M from it) are bricks of bx x by x bz cells of one
+                              level l (2..depth) are bricks of bx x by x bz cells of one
                               parity class, bx by bz = 128, each dividing 2^(l-1), an even number per class.
                               Only the grouping of targets into tiles changes: results are bitwise the same.
                               FMM_ERR_UNSUPPORTED without the tensor-core path (FP64 plans); a WS, PRECISION

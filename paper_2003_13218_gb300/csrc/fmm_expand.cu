@@ -1,6 +1,6 @@
 // fmm_expand.cu -- the expansion operators of Appendix B on the GPU:
-// P2M (Eq. P2M), M2M, the level-0 lattice operator (Eq. 12), M2L over the
-// interaction lists (Eq. Lcoeffdef, CUDA-core version), L2L and L2P with its
+// P2M (Eq. P2M), the level-0 lattice operator (Eq. 12), M2L over the
+// interaction lists (Eq. Lcoeffdef, CUDA-core version) and L2P with its
 // gradient (Eq. EqFF); plus the per-plan operator tables.
 //
 // Solid harmonics (normalisation that makes the printed equations hold with

@@ -283,7 +283,7 @@ fmm_status launch_top_solute(Plan &P, cudaStream_t st, const void *MU1, const in
 fmm_status launch_top_active(Plan &P, cudaStream_t st, const void *MU1, const int *cells, const int *ncells, double *Lt1);
 fmm_status launch_m2l_simt(Plan &P, int level);
 
-// M2M / L2L as dense products (fmm_translate.cu)
+// M2M / L2L, folded over the child octants (fmm_translate.cu)
 fmm_status build_translation_ops(Plan &P);
 fmm_status launch_m2m(Plan &P, int level);  // level + 1 -> level
 fmm_status launch_l2l(Plan &P, int level);  // level - 1 -> level (accumulates)
@@ -353,7 +353,7 @@ fmm_status eval_enqueue_front(Plan &P, const double *dpos, const double *dq, con
 fmm_status eval_enqueue_far_tail(Plan &P);
 fmm_status eval_enqueue_back(Plan &P, const double *dq);
 
-// the level-l tile brick of the tensor-core M2L (and of the M2M from level l); see FMM_OPT_M2L_BRICK
+// the level-l tile brick of the tensor-core M2L; see FMM_OPT_M2L_BRICK
 fmm_status tc_set_brick(Plan &P, int l, int bx, int by, int bz);
 void tc_get_brick(const Plan &P, int l, int *bx, int *by, int *bz);
 

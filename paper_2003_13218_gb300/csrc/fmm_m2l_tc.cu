@@ -1149,7 +1149,7 @@ void tc_get_brick(const Plan &P, int l, int *bx, int *by, int *bz)
     *bz = S && l >= 1 && l <= P.d ? S->bz[l] : 0;
 }
 
-// The split operator tables depend only on p, ws and the split (the M2L, M2M and L2L operators are
+// The split operator tables depend only on p, ws and the split (the M2L and L2L operators are
 // built for unit cells), so plans that agree on those can read one copy: dst drops its own and reads
 // src's, which must outlive it.  A plan with another table is left alone.
 fmm_status tc_share_operators(Plan &dst, const Plan &src)

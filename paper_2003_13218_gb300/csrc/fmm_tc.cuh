@@ -1,4 +1,4 @@
-// fmm_tc.cuh -- the tensor-core (tcgen05) product kernels of the M2L, M2M and fused L2L, shared by the mixed path
+// fmm_tc.cuh -- the tensor-core (tcgen05) product kernels of the M2L and fused L2L, shared by the mixed path
 // (fmm_m2l_tc.cu: 16-bit operand splits) and the FP64 path (fmm_m2l_res.cu: exact residue products), with the
 // host helpers that lay out their launches and tensor maps.
 //
@@ -131,7 +131,7 @@ struct IlWalk {
     }
 };
 
-// Accumulation groups of one CTA's offsets: the M2L (or M2M) offsets, local indices 0 .. nm - 1, in runs
+// Accumulation groups of one CTA's offsets: the M2L offsets, local indices 0 .. nm - 1, in runs
 // of G that share one TMEM accumulator; the fused L2L offset (when present it is the CTA's last) alone,
 // since its drain is scaled by gM / gL.
 struct AccGroups {
