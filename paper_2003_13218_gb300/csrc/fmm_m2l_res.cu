@@ -85,15 +85,20 @@ __device__ __forceinline__ void limbs(long long x, int &x0, int &x1, int &x2)
     x2 = (int)(x >> 36);
 }
 
-// g of a level from the bits of its largest |M~|: |M~ 2^g| < 2^RES_M_BITS, within the range of a double
+// g of a level from the bits of its largest |M~|: |M~ 2^g| < 2^RES_M_BITS for every double, -968 <= g <= 1078
 __device__ __forceinline__ int res_gain(unsigned long long bits)
 {
-    if (bits == 0ull) return 0;
-    const int g = RES_M_BITS - 1 - ((int)(bits >> 52) - 1023);
-    return g > 1000 ? 1000 : (g < -960 ? -960 : g);
+    return bits == 0ull ? 0 : RES_M_BITS - 1 - ((int)(bits >> 52) - 1023);
 }
 
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// 2^e = a b with both factors normal (moments below 2^-967 have a gain that no double holds)
+__device__ __forceinline__ void pow2_factors(int e, double &a, double &b)
+{
+    a = pow2d(e / 2);
+    b = pow2d(e - e / 2);
+}
 
 // T~ of every slot -> residues times (P / p_i)^-1, [modulus][chunk][slot][j][k] with zero padding
 __global__ void k_res_ops(int noff, const double *__restrict__ T, int nc, int npad, int kp, const double *__restrict__ s,
@@ -130,7 +135,8 @@ __global__ void k_res_split(const double *__restrict__ M, int np, int hw, int nc
     const int np2 = np + 2 * hw;
     const int G = kp / 8;
     const int64_t ncell = 8 * (int64_t)np2 * np2 * np2, total = ncell * G;
-    const double g = pow2d(res_gain(*amax));
+    double g0, g1;
+    pow2_factors(res_gain(*amax), g0, g1);
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t cell = t / G;
         const int k0 = (int)(t - cell * G) * 8;
@@ -144,7 +150,7 @@ __global__ void k_res_split(const double *__restrict__ M, int np, int hw, int nc
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int k = k0 + u;
-            const long long x = k < nc ? __double2ll_rn(row[k] * __ldg(s + k) * g) : 0;
+            const long long x = k < nc ? __double2ll_rn(row[k] * __ldg(s + k) * g0 * g1) : 0;
             limbs(x, x0[u], x1[u], x2[u]);
         }
         uint16_t *out = planes + chunk_at(cell, ncell, k0, 64);
@@ -174,6 +180,9 @@ __global__ void k_res_join(int64_t n, int nc, int groups, int m0, int nb, const 
 {
     const int64_t e = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
     if (e >= n) return;  // n is even (8 parity classes)
+    const unsigned long long bits = *amax;
+    double g0, g1;
+    pow2_factors(-res_gain(bits), g0, g1);
     long long a0[2] = {0, 0}, a1[2] = {0, 0}, a2[2] = {0, 0};
     for (int g = 0; g < groups; ++g)
         for (int m = 0; m < nb; ++m) {
@@ -205,9 +214,8 @@ __global__ void k_res_join(int64_t n, int nc, int groups, int m0, int nb, const 
             continue;
         }
         const long long top = (long long)(((uint64_t)hi << 32) | mid);  // signed: |L_int| < P / 2
-        const unsigned long long bits = *amax;
         double v = (double)top * 4294967296.0 + (double)lo;
-        v = v * c.pscale * s[(int)((e + u) % nc)] * pow2d(-RES_T_BITS) * pow2d(-res_gain(bits));
+        v = v * c.pscale * s[(int)((e + u) % nc)] * pow2d(-RES_T_BITS) * g0 * g1;
         L[e + u] = (bits >> 52) == 2047 ? __longlong_as_double(0x7FF8000000000000ll) : v;  // inf or NaN moments
     }
 }
