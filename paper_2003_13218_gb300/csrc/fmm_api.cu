@@ -146,15 +146,20 @@ fmm_status far_field_pass(Plan &P, bool gradient, bool solute_only, StageTimer *
     bool ev = tm && P.timings_on;
     // a batch's persistent sweep runs the levels >= sweep_from of the full pass, and its L2P after that
     const int last = (!solute_only && P.sweep_from > 0) ? P.sweep_from - 1 : P.d;
+    const bool res = res_available(P, 2);
     for (int l = 2; l <= last; ++l) {
         if (ev) cudaEventRecord(P.ev_m2l[2 * (l - 1)], P.stream);
         // with the fp16 split the upward pass left the planes split and the L2L is fused
         const bool fused = tc_available(P, l) && tc_translations(P);
         if (tc_available(P, l)) TRY(launch_m2l_tc(P, l, solute_only));
-        else if (res_available(P, l)) TRY(launch_m2l_res(P, l));
+        else if (res) TRY(launch_m2l_res(P, l));
         else TRY(launch_m2l_simt(P, l));
         if (ev) cudaEventRecord(P.ev_m2l[2 * (l - 1) + 1], P.stream);
-        if (!fused) TRY(launch_l2l(P, l));
+        if (!fused && !res) TRY(launch_l2l(P, l));
+    }
+    if (res) {
+        TRY(launch_m2l_res_low(P));
+        for (int l = 2; l <= last; ++l) TRY(launch_l2l(P, l));
     }
     if (tm) tm->mark();
     if (last < P.d) return FMM_OK;

@@ -305,13 +305,14 @@ __device__ __forceinline__ unsigned long long p2m_bits(double x)  // a NaN is la
 // loops run to the longest column and fullest leaf of the warp, 100,000 charges at p = 12 took 776 us and 2,998 at
 // p = 8 109 us; here 302 us and, shared, 22 us.  The warps of a block share the same charges and take the columns m in
 // turn (small systems: one warp, on one of an SM's four FP64 pipes, took 46 us for the latter).  sx, amax (or null): the
-// level's largest |M sx| is folded in.
+// level's largest |M sx| is folded in; cmax (FP64, with amax): that of each leaf, the double's upper word.
 constexpr int P2M_SHARE = 4;  // warps that share 32 charges in small systems
 
 template <typename T, typename U>
 __global__ void __launch_bounds__(32 * P2M_SHARE) k_p2m(int p, int d, int lb, const int *__restrict__ start,
                                             const Particle<T> *__restrict__ sp, T inv_h, T *__restrict__ M,
-                                            const T *__restrict__ sx, U *__restrict__ amax)
+                                            const T *__restrict__ sx, U *__restrict__ amax,
+                                            uint32_t *__restrict__ cmax)
 {
     extern __shared__ __align__(16) unsigned char p2m_smem[];
     const ExpandFactors<T> &F = expand_factors<T>();
@@ -372,13 +373,22 @@ __global__ void __launch_bounds__(32 * P2M_SHARE) k_p2m(int p, int d, int lb, co
     U mx = 0;
     for (int i = warp; i < nl; i += share) {
         const int leaf = (int)(leaf0 + i);
-        T *out = M + cell_index(d, leaf & (nside - 1), (leaf >> d) & (nside - 1), leaf >> (2 * d)) * nc;
+        const int64_t cell = cell_index(d, leaf & (nside - 1), (leaf >> d) & (nside - 1), leaf >> (2 * d));
+        T *out = M + cell * nc;
+        U mc = 0;
         for (int k = lane; k < nc; k += 32) {
             const T v = rows[i * nc + k];
             out[k] = v;
             if (amax) {
                 const U b = p2m_bits(v * sx[k]);
-                mx = b > mx ? b : mx;
+                mc = b > mc ? b : mc;
+            }
+        }
+        mx = mc > mx ? mc : mx;
+        if constexpr (sizeof(U) == 8) {
+            if (cmax) {
+                const uint32_t h = __reduce_max_sync(0xffffffffu, (uint32_t)(mc >> 32));
+                if (lane == 0) cmax[cell] = h;
             }
         }
     }
@@ -522,7 +532,7 @@ fmm_status launch_p2m_fixed(Plan &P, const Particle<float> *sp, float inv_h, uns
 
 // leaves per warp: about 28 charges, so that mostly one round of 32 does, within 24 KB of rows and 32 leaves
 template <typename T, typename U>
-fmm_status launch_p2m(Plan &P, const Particle<T> *sp, T inv_h, const T *sx, U *amax)
+fmm_status launch_p2m(Plan &P, const Particle<T> *sp, T inv_h, const T *sx, U *amax, uint32_t *cmax)
 {
     const double occ = (double)P.N / (double)P.nleaf;
     const int fit = (int)(24576 / (sizeof(T) * P.nc)), most = fit < 32 ? fit : 32;
@@ -533,7 +543,7 @@ fmm_status launch_p2m(Plan &P, const Particle<T> *sp, T inv_h, const T *sx, U *a
     if (sizeof(T) * 2 * (P.p + 1) * 33 * share > 23000) share = 2;
     const size_t sh = sizeof(T) * ((size_t)lb * P.nc + 2 * (P.p + 1) * 33 * share) + sizeof(int) * (lb + 1);
     k_p2m<T, U><<<(unsigned)((P.nleaf + lb - 1) / lb), 32 * share, sh, P.stream>>>(P.p, P.d, lb, P.cell_start, sp, inv_h,
-                                                                            (T *)P.M[P.d], sx, amax);
+                                                                            (T *)P.M[P.d], sx, amax, cmax);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
@@ -814,11 +824,12 @@ fmm_status upward_t(Plan &P, bool solute_only)
              : sparse && P.p == 8  ? launch_p2m_fixed<8>(P, sp, inv_h, amax, sc)
              : sparse && P.p == 10 ? launch_p2m_fixed<10>(P, sp, inv_h, amax, sc)
              : sparse && P.p == 12 ? launch_p2m_fixed<12>(P, sp, inv_h, amax, sc)
-                                   : launch_p2m<float, unsigned>(P, sp, inv_h, sc, amax);
+                                   : launch_p2m<float, unsigned>(P, sp, inv_h, sc, amax, nullptr);
     } else {
         const double *sc = nullptr;
-        unsigned long long *amax = res_amax(P, P.d, &sc);
-        st = launch_p2m<double, unsigned long long>(P, sp, inv_h, sc, amax);
+        uint32_t *cmax = nullptr;
+        unsigned long long *amax = res_amax(P, P.d, &sc, &cmax);
+        st = launch_p2m<double, unsigned long long>(P, sp, inv_h, sc, amax, cmax);
     }
     if (st != FMM_OK) return st;
     for (int l = P.d - 1; l >= 1; --l) {  // the top operator starts from level 1

@@ -333,15 +333,18 @@ const float *tc_scale(const Plan &P);
 fmm_status launch_m2l_tc(Plan &P, int level, bool precise);
 void tc_free(Plan &P);
 
-// FP64 M2L by residue products on the tensor cores (fmm_m2l_res.cu): L[level] = M2L, without the L2L
+// FP64 M2L by residue products on the tensor cores (fmm_m2l_res.cu): L[level] = M2L, without the L2L; after all levels
+// launch_m2l_res_low computes the targets that need floating-point sums
 bool res_available(const Plan &P, int level);
 // builds the state on an FP64 plan's first evaluation (a plan that is to run the mixed path never pays for it);
 // left for later while the plan's stream is being captured
 fmm_status res_ensure(Plan &P);
-// where the P2M and M2M leave a level's largest |Mhat s|, and s (null without the state)
-unsigned long long *res_amax(Plan &P, int level, const double **s);
+// where the P2M and M2M leave a level's largest |Mhat s|, and that of each of its cells (upper word of the double), and
+// s (null without the state)
+unsigned long long *res_amax(Plan &P, int level, const double **s, uint32_t **cmax);
 fmm_status res_clear_amax(Plan &P);  // at the start of a far-field pass
 fmm_status launch_m2l_res(Plan &P, int level);
+fmm_status launch_m2l_res_low(Plan &P);
 fmm_status res_share_operators(Plan &dst, const Plan &src);
 void res_free(Plan &P);
 

@@ -3,14 +3,18 @@
 // GB300 issues 2 FP64 operations per SM and clock, so the CUDA-core M2L (2 (p+1)^4 flop per source and target)
 // is bound by that pipe: 1.29 s per evaluation of 100,000 charges at p = 12, and far more than its flops at small
 // sizes, whose levels fill a few SMs.  The 16-bit tensor pipe is ~1,500 times as fast.  The products are therefore
-// taken in whole numbers, exactly, modulo 11 to 14 small coprime numbers (the Chinese remainder theorem; its use
+// taken in whole numbers, exactly, modulo 11 to 15 small coprime numbers (the Chinese remainder theorem; its use
 // for matrix products on low-precision units is the "Ozaki scheme II" of Ozaki, Uchino & Imamura, 2025):
 //   * moments and operators are balanced as in the mixed path, M~ = M^ s(n,m), T~ = T / (s s), |T~| <= 1/2, and
-//     rounded to whole numbers, M_int = round(M~ 2^g) with |M_int| < 2^56 (g from the level's largest |M~|) and
-//     T_int = round(T~ 2^56): the moments keep the 53 bits of every value within 2^-3 of the level's largest, and
-//     the operators' rounding is 2^-57, below the 2^-53 of the FP64 sum that this replaces;
-//   * sum_delta sum_k |T_int| <= 137 2^56 (ws = 1) or 277 2^56 (ws = 2), whatever the order, so |L_int| < 2^119.2
-//     or 2^120.2, and it follows from its residues modulo p_1 .. p_n with prod p_i > 2^121;
+//     rounded to whole numbers, M_int = round(M~ 2^g) with |M_int| < 2^B (g from the level's largest |M~|) and
+//     T_int = round(T~ 2^C): B = 56 to 58, as the moduli allow, C = 56, or 58 at ws = 2 and up to order 3;
+//   * a whole number has the level's exponent, a double its own.  A target whose sources are all more than 2^(B - K)
+//     below the level's largest (far from a dominant charge) therefore takes the FP64 sum instead (k_res_low).  K = 54,
+//     53 from order 3, 52 from 5 and 51 from 12 on, where the FP64 sum rounds more: with one source in a list right at that
+//     line, the worst case, the gradients of the potential err by 0.5 to 0.95 times as much as with the FP64 sum and the
+//     potentials by 0.1 to 1.0 times (p = 0 to 12, against 64-bit mantissas); with 40 sources of the same size by 0.1;
+//   * sum_delta sum_k |T_int| <= 137 2^C (ws = 1) or 277 2^C (ws = 2), whatever the order, so |L_int| < 2^(B + C + 7.2)
+//     or 2^(B + C + 8.2), and it follows from its residues modulo p_1 .. p_n with prod p_i above twice that;
 //   * residues are centred, |r| <= p/2, exact in fp16; a product of two is a whole number, and a chain of G = 2
 //     offsets sums 2 (p+1)^2 of them: with 2 (p+1)^2 (p/2)^2 <= 2^24 the FP32 accumulator is exact.  The drained
 //     accumulators are added up as 32-bit integers (fmm_tc.cuh);
@@ -36,8 +40,8 @@ namespace {
 
 constexpr int RES_MAX = 16;        // moduli
 constexpr int RES_CHAIN = 2;       // offsets per accumulator (G)
-constexpr int RES_M_BITS = 56;     // |M_int| < 2^56
-constexpr int RES_T_BITS = 56;     // T_int = round(T~ 2^56)
+constexpr int RES_M_BITS = 56, RES_M_BITS_MAX = 58;  // |M_int| < 2^B, B as the moduli allow
+constexpr int JOIN_THREADS = 256;
 constexpr size_t RES_PLANE_BUDGET = (size_t)2 << 30;  // operand planes held at once (moduli per launch)
 
 struct ResConsts {
@@ -47,6 +51,7 @@ struct ResConsts {
     float rp[RES_MAX];
     uint32_t w[RES_MAX][3];                      // floor(2^96 / p_i), low word first
     double pscale;                               // P / 2^96
+    int mbits, tbits, keep;                      // B, C, K
 };
 
 struct ResState {
@@ -64,11 +69,15 @@ struct ResState {
     int bx[9], by[9], bz[9], groups[9], per_group[9];
     double *s64 = nullptr;        // [nc] s(n,m)
     unsigned long long *amax = nullptr;  // [9] bits of the largest |M^ s| per level
+    uint32_t *cmax = nullptr;            // the same per cell, upper words, levels 1 .. d behind one another
+    uint32_t *low = nullptr;             // targets that take the FP64 sum (numbered as in cmax)
+    int *low_count = nullptr;            // behind amax: their count, then [LOW_CELLS] blocks done
+    double *low_part = nullptr;          // [LOW_CELLS][LOW_GROUPS][nc]; the allocation that amax, cmax and low share
     int *mods = nullptr;
 };
 
-// x mod p for |x| <= 2^57, centred: 18-bit limbs (the highest signed) against 2^18 and 2^36 mod p, then one
-// approximate quotient and a correction
+// x mod p, centred: 18-bit limbs (the highest signed) against 2^18 and 2^36 mod p, then one approximate quotient and
+// a correction (limbs_fit: how large x may be)
 __device__ __forceinline__ int residue(int x0, int x1, int x2, int p, int c18, int c36, float rp)
 {
     int r = mod_near(x0 + x1 * c18 + x2 * c36, p, rp);
@@ -85,10 +94,10 @@ __device__ __forceinline__ void limbs(long long x, int &x0, int &x1, int &x2)
     x2 = (int)(x >> 36);
 }
 
-// g of a level from the bits of its largest |M~|: |M~ 2^g| < 2^RES_M_BITS for every double, -968 <= g <= 1078
-__device__ __forceinline__ int res_gain(unsigned long long bits)
+// g of a level from the bits of its largest |M~|: |M~ 2^g| < 2^mbits for every double, -968 <= g <= 1080
+__device__ __forceinline__ int res_gain(unsigned long long bits, int mbits)
 {
-    return bits == 0ull ? 0 : RES_M_BITS - 1 - ((int)(bits >> 52) - 1023);
+    return bits == 0ull ? 0 : mbits - 1 - ((int)(bits >> 52) - 1023);
 }
 
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
@@ -111,14 +120,15 @@ __global__ void k_res_ops(int noff, const double *__restrict__ T, int nc, int np
         const int slot = (int)(e / ((int64_t)kp * npad));
         long long x = 0;
         if (j < nc && k < nc)
-            x = llrint(T[((int64_t)slot * nc + k) * nc + j] / (s[k] * s[j]) * (double)(1ll << RES_T_BITS));
+            x = llrint(T[((int64_t)slot * nc + k) * nc + j] / (s[k] * s[j]) * (double)(1ll << c.tbits));
         int x0, x1, x2;
         limbs(x, x0, x1, x2);
         const int64_t at = chunk_at((int64_t)slot * npad + j, (int64_t)noff * npad, k, 64);
 #pragma unroll
         for (int i = 0; i < RES_MAX; ++i) {
             if (i >= c.n) break;
-            const int r = residue(x0, x1, x2, c.p[i], c.c18[i], c.c36[i], c.rp[i]);
+            const int t2 = mod_near(x2, c.p[i], c.rp[i]);  // |x2| up to 2^21
+            const int r = residue(x0, x1, t2, c.p[i], c.c18[i], c.c36[i], c.rp[i]);
             const int y = residue(r * c.inv[i], 0, 0, c.p[i], 0, 0, c.rp[i]);
             ops[at + i * elems] = __half_as_ushort(__int2half_rn(y));
         }
@@ -136,7 +146,7 @@ __global__ void k_res_split(const double *__restrict__ M, int np, int hw, int nc
     const int G = kp / 8;
     const int64_t ncell = 8 * (int64_t)np2 * np2 * np2, total = ncell * G;
     double g0, g1;
-    pow2_factors(res_gain(*amax), g0, g1);
+    pow2_factors(res_gain(*amax, c.mbits), g0, g1);
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t cell = t / G;
         const int k0 = (int)(t - cell * G) * 8;
@@ -170,21 +180,70 @@ __global__ void k_res_split(const double *__restrict__ M, int np, int hw, int nc
     }
 }
 
-// Residues y_i of nb moduli (and of the offset groups) -> the 96-bit fraction sum y_i / p_i mod 1, and on the last
-// launch of the level L^ = P (fraction) 2^-(g + RES_T_BITS) s(j).  Two neighbouring elements per thread (their
-// residues are one 32-bit load); frac carries the sums between the launches of a level.
-__global__ void k_res_join(int64_t n, int nc, int groups, int m0, int nb, const int16_t *__restrict__ resid,
-                           uint32_t *__restrict__ frac, bool first, bool last, const double *__restrict__ s,
-                           const unsigned long long *__restrict__ amax, double *__restrict__ L,
-                           const __grid_constant__ ResConsts c)
+// cell of the o-th source of target `cell` of a level with class side 2^lg, and its operator slot
+__device__ __forceinline__ int64_t res_source(const int *__restrict__ il, int n_il, int lg, int ws, int64_t cell, int o,
+                                              int &slot)
 {
-    const int64_t e = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
-    if (e >= n) return;  // n is even (8 parity classes)
+    const int c = (int)(cell >> (3 * lg)), mask = (1 << lg) - 1;
+    int dx, dy, dz;
+    il_unpack(__ldg(il + c * n_il + o), dx, dy, dz);
+    slot = off_slot(dx, dy, dz, ws);
+    const int sx = (c & 1) + dx, sy = ((c >> 1) & 1) + dy, sz = (c >> 2) + dz;
+    const int x = ((int)cell + (sx >> 1)) & mask, y = ((int)(cell >> lg) + (sy >> 1)) & mask,
+              z = ((int)(cell >> (2 * lg)) + (sz >> 1)) & mask;
+    return ((int64_t)((sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2)) << (3 * lg)) + x + (((int64_t)z << lg) + y << lg);
+}
+
+// Where the targets that take the FP64 sum are listed, and what tells them
+struct ResLow {
+    const uint32_t *cmax;  // the level's
+    const int *il;
+    int n_il, lg, ws;
+    uint32_t base;         // of the level in the list's numbers
+    uint32_t *list;
+    int *count;
+};
+
+// whether every source of a target is below the upper word `lim` and one is not zero (a whole warp; mostly the first
+// 32 sources settle it)
+__device__ __forceinline__ bool res_low_list(const ResLow &d, int64_t cell, uint32_t lim, int lane)
+{
+    bool any = false;
+    for (int o0 = 0; o0 < d.n_il; o0 += 32) {
+        int slot;
+        const uint32_t v = o0 + lane < d.n_il ? d.cmax[res_source(d.il, d.n_il, d.lg, d.ws, cell, o0 + lane, slot)] : 0u;
+        if (__any_sync(0xffffffffu, v >= lim)) return false;
+        any |= v > 0u;
+    }
+    return __any_sync(0xffffffffu, any) != 0;
+}
+
+// Residues y_i of nb moduli (and of the offset groups) -> the 96-bit fraction sum y_i / p_i mod 1, and on the last
+// launch of the level L^ = P (fraction) 2^-(g + C) s(j).  Two neighbouring elements per thread (their
+// residues are one 32-bit load); frac carries the sums between the launches of a level.  The last launch also lists the
+// targets whose sources are too far below the level's largest, all of them where that is inf or NaN.
+__global__ void __launch_bounds__(JOIN_THREADS) k_res_join(int64_t n, int nc, int groups, int m0, int nb,
+                                                           const int16_t *__restrict__ resid, uint32_t *__restrict__ frac,
+                                                           bool first, bool last, const double *__restrict__ s,
+                                                           const unsigned long long *__restrict__ amax,
+                                                           double *__restrict__ L, const ResLow d,
+                                                           const __grid_constant__ ResConsts c)
+{
+    const int64_t e0 = 2 * (blockIdx.x * (int64_t)JOIN_THREADS), e = e0 + 2 * threadIdx.x;
     const unsigned long long bits = *amax;
+    if (last) {  // a warp per cell that begins in the block
+        const int64_t e1 = e0 + 2 * JOIN_THREADS < n ? e0 + 2 * JOIN_THREADS : n;
+        const uint32_t hi = (uint32_t)(bits >> 32), down = (uint32_t)(c.mbits - c.keep) << 20;
+        for (int64_t cell = (e0 + nc - 1) / nc + (threadIdx.x >> 5); cell * nc < e1; cell += JOIN_THREADS / 32)
+            if ((bits >> 52) == 2047 || (hi > down && res_low_list(d, cell, hi - down, threadIdx.x & 31)))
+                if ((threadIdx.x & 31) == 0) d.list[atomicAdd(d.count, 1)] = d.base + (uint32_t)cell;
+    }
+    if (e >= n) return;  // n is even (8 parity classes)
     double g0, g1;
-    pow2_factors(-res_gain(bits), g0, g1);
+    pow2_factors(-res_gain(bits, c.mbits), g0, g1);
     long long a0[2] = {0, 0}, a1[2] = {0, 0}, a2[2] = {0, 0};
     for (int g = 0; g < groups; ++g)
+#pragma unroll 8
         for (int m = 0; m < nb; ++m) {
             const int v = *reinterpret_cast<const int *>(resid + ((int64_t)g * nb + m) * n + e);
             const int y[2] = {(int)(short)(v & 0xFFFF), v >> 16};
@@ -215,14 +274,95 @@ __global__ void k_res_join(int64_t n, int nc, int groups, int m0, int nb, const 
         }
         const long long top = (long long)(((uint64_t)hi << 32) | mid);  // signed: |L_int| < P / 2
         double v = (double)top * 4294967296.0 + (double)lo;
-        v = v * c.pscale * s[(int)((e + u) % nc)] * pow2d(-RES_T_BITS) * g0 * g1;
-        L[e + u] = (bits >> 52) == 2047 ? __longlong_as_double(0x7FF8000000000000ll) : v;  // inf or NaN moments
+        L[e + u] = v * c.pscale * s[(int)((e + u) % nc)] * pow2d(-c.tbits) * g0 * g1;
     }
 }
 
-// the largest pairwise coprime numbers below the exactness bound until their product exceeds 2^bits
-bool choose_moduli(int nc, double bits, ResConsts &c)
+// place of level l in the list's numbers and in cmax
+__host__ __device__ inline uint32_t cmax_at(int l) { return (uint32_t)((((int64_t)1 << (3 * l)) - 8) / 7); }
+
+struct ResLevels {
+    const double *M[9];
+    double *L[9];
+};
+
+// The FP64 sums of the listed targets, over the results of k_res_join.  A few targets: their offsets are split over
+// LOW_GROUPS blocks each, and the block that finishes last adds their sums in order (a thread per output took 9.6 ms for
+// 8 targets at p = 12).  Many targets take a block each, which is bound by the FP64 pipe.  Empty sources are left out.
+constexpr int LOW_THREADS = 128, LOW_CELLS = 128, LOW_GROUPS = 63;
+
+__global__ void __launch_bounds__(LOW_THREADS) k_res_low(int nc, int d, int ws, int n_il, const __grid_constant__ ResLevels lv,
+                                                         const uint32_t *__restrict__ cmax, const double *__restrict__ Top,
+                                                         const int *__restrict__ il, const uint32_t *__restrict__ list,
+                                                         const int *__restrict__ count, double *__restrict__ part,
+                                                         int *__restrict__ done)
 {
+    constexpr int Q = 256 / LOW_THREADS;  // coefficients per thread
+    __shared__ double sM[256];
+    __shared__ int last;
+    const int n = *count;
+    const int ng = n <= LOW_CELLS ? LOW_GROUPS : 1, per = (n_il + ng - 1) / ng;
+    for (int64_t it = blockIdx.x; it < (int64_t)n * ng; it += gridDim.x) {
+        const int i = (int)(it / ng), g = (int)(it - (int64_t)i * ng);
+        const uint32_t code = list[i];
+        int l = 2;
+        while (l < d && code >= cmax_at(l + 1)) ++l;
+        const int64_t cell = code - cmax_at(l);
+        double acc[Q] = {};
+        for (int o = g * per; o < n_il && o < (g + 1) * per; ++o) {
+            int slot;
+            const int64_t src = res_source(il, n_il, l - 1, ws, cell, o, slot);
+            if (cmax[cmax_at(l) + src] == 0u) continue;  // the same for the whole block
+            __syncthreads();
+            for (int k = threadIdx.x; k < nc; k += LOW_THREADS) sM[k] = lv.M[l][src * nc + k];
+            __syncthreads();
+            const double *T = Top + (size_t)slot * nc * nc;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int j = threadIdx.x + q * LOW_THREADS;
+                if (j >= nc) break;
+#pragma unroll 8
+                for (int k = 0; k < nc; ++k) acc[q] += T[(size_t)k * nc + j] * sM[k];
+            }
+        }
+        double *out = ng == 1 ? lv.L[l] + cell * nc : part + (size_t)(i * LOW_GROUPS + g) * nc;
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (threadIdx.x + q * LOW_THREADS < nc) out[threadIdx.x + q * LOW_THREADS] = acc[q];
+        if (ng == 1) continue;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(done + i, 1) == ng - 1;
+        __syncthreads();
+        if (last) {
+            __threadfence();
+            for (int j = threadIdx.x; j < nc; j += LOW_THREADS) {
+                double v = 0;
+                for (int k = 0; k < ng; ++k) v += __ldcg(part + (size_t)(i * LOW_GROUPS + k) * nc + j);
+                lv.L[l][cell * nc + j] = v;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// whether residue() takes whole numbers below 2^bits: the limbs' products fit 31 bits, and the approximate quotient
+// (three roundings of 2^-24) is off by less than 1/2
+bool limbs_fit(const ResConsts &c, int bits)
+{
+    for (int i = 0; i < c.n; ++i) {
+        const double v = ldexp(fabs((double)c.c36[i]), bits - 36) + ldexp(fabs((double)c.c18[i]), 18) + ldexp(1.0, 18);
+        if (v >= ldexp(1.0, 31) || 3.0 * v >= ldexp(0.45 * c.p[i], 24)) return false;
+    }
+    return true;
+}
+
+// the largest pairwise coprime numbers below the exactness bound until their product exceeds 2^(B + C + sum_bits), the
+// bits of the largest sum with its sign; B then takes what they have left
+bool choose_moduli(int nc, int tbits, double sum_bits, ResConsts &c)
+{
+    c.tbits = tbits;
+    const double bits = RES_M_BITS + tbits + sum_bits;
     int h = 1;
     while ((int64_t)RES_CHAIN * nc * (h + 1) * (h + 1) <= (1 << 24)) ++h;
     int top = 2 * h + 1;
@@ -272,6 +412,9 @@ bool choose_moduli(int nc, double bits, ResConsts &c)
             rem %= p;
         }
     }
+    if (!limbs_fit(c, RES_M_BITS)) return false;
+    c.mbits = RES_M_BITS;
+    while (c.mbits < RES_M_BITS_MAX && have >= c.mbits + 1 + tbits + sum_bits && limbs_fit(c, c.mbits + 1)) ++c.mbits;
     return true;
 }
 
@@ -300,6 +443,8 @@ TcKernel res_pair_kernel(int nch)
     }
 }
 
+constexpr size_t RES_CLEAR = sizeof(unsigned long long) * 9 + sizeof(int) * (1 + LOW_CELLS);  // amax and behind it
+
 bool pairs_at(const ResState *S, int l)
 {
     const int np = 1 << (l - 1);
@@ -317,8 +462,9 @@ fmm_status prepare(Plan &P, ResState *S)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return FMM_ERR_UNSUPPORTED;
-    // |L_int| < 2^56 2^56 137 (ws = 1: log2 137 = 7.10) or 277 (ws = 2: 8.12), and its sign
-    if (!choose_moduli(P.nc, RES_M_BITS + RES_T_BITS + (P.ws == 1 ? 7.2 : 8.2) + 1.0, S->c)) return FMM_ERR_UNSUPPORTED;
+    // |L_int| < 2^B 2^C 137 (ws = 1: log2 137 = 7.10) or 277 (ws = 2: 8.12), and its sign
+    S->c.keep = P.p < 3 ? 54 : P.p < 5 ? 53 : P.p < 12 ? 52 : 51;
+    if (!choose_moduli(P.nc, P.ws == 2 || P.p <= 3 ? 58 : 56, (P.ws == 1 ? 7.2 : 8.2) + 1.0, S->c)) return FMM_ERR_UNSUPPORTED;
     S->npad = (P.nc + 15) / 16 * 16;
     S->kp = (P.nc + 63) / 64 * 64;
     S->noff = noff(P.ws);
@@ -333,7 +479,14 @@ fmm_status prepare(Plan &P, ResState *S)
             if (m > 0) h_s[cim(d, m)] = sqrt(f);
         }
     FMM_CUDA_TRY(cudaMalloc(&S->s64, sizeof(double) * P.nc));
-    FMM_CUDA_TRY(cudaMalloc(&S->amax, sizeof(unsigned long long) * 9));
+    {
+        const size_t part = sizeof(double) * LOW_CELLS * LOW_GROUPS * P.nc, cells = cmax_at(P.d + 1);
+        FMM_CUDA_TRY(cudaMalloc(&S->low_part, part + RES_CLEAR + 2 * sizeof(uint32_t) * cells));  // one allocation
+        S->amax = (unsigned long long *)((char *)S->low_part + part);
+        S->low_count = (int *)(S->amax + 9);
+        S->cmax = (uint32_t *)((char *)S->amax + RES_CLEAR);
+        S->low = S->cmax + cells;
+    }
     FMM_CUDA_TRY(cudaMalloc(&S->mods, sizeof(int) * RES_MAX));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->s64, h_s.data(), sizeof(double) * P.nc, cudaMemcpyHostToDevice, P.stream));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->mods, S->c.p, sizeof(int) * RES_MAX, cudaMemcpyHostToDevice, P.stream));
@@ -428,18 +581,19 @@ fmm_status res_ensure(Plan &P)
 fmm_status res_clear_amax(Plan &P)
 {
     ResState *S = (ResState *)P.res;
-    if (S) FMM_CUDA_TRY(cudaMemsetAsync(S->amax, 0, sizeof(unsigned long long) * 9, P.stream));
+    if (S) FMM_CUDA_TRY(cudaMemsetAsync(S->amax, 0, RES_CLEAR, P.stream));
     return FMM_OK;
 }
 
-unsigned long long *res_amax(Plan &P, int l, const double **s)
+unsigned long long *res_amax(Plan &P, int l, const double **s, uint32_t **cmax)
 {
     ResState *S = (ResState *)P.res;
     *s = S ? S->s64 : nullptr;
+    *cmax = S ? S->cmax + cmax_at(l) : nullptr;
     return S ? S->amax + l : nullptr;
 }
 
-// L[l] = M2L of level l (the L2L from level l - 1 is added by launch_l2l)
+// L[l] = M2L of level l (the L2L from level l - 1 is added by launch_l2l), but for the targets that it lists
 fmm_status launch_m2l_res(Plan &P, int l)
 {
     ResState *S = (ResState *)P.res;
@@ -475,6 +629,7 @@ fmm_status launch_m2l_res(Plan &P, int l)
     a.idesc = (1u << 4) | ((uint32_t)(S->npad >> 3) << 17) | ((uint32_t)((pair ? 2 * TC_ROWS : TC_ROWS) >> 4) << 24);
     const TcKernel k = pair ? res_pair_kernel(S->npad / 16) : res_kernel(S->npad / 16);
     const size_t smem = pair ? tc_pair_smem_bytes(S->npad) : tc_smem_bytes(2, 2, S->npad, 128);
+    const ResLow low{S->cmax + cmax_at(l), P.tab.il, n_il(P.ws), l - 1, P.ws, cmax_at(l), S->low, S->low_count};
     const int64_t halo = 8 * np2 * np2 * np2 * (S->kp / 8), elems = cells * nc;
     for (int m0 = 0; m0 < n; m0 += S->batch[l]) {
         const int nb = n - m0 < S->batch[l] ? n - m0 : S->batch[l];
@@ -485,11 +640,27 @@ fmm_status launch_m2l_res(Plan &P, int l)
         a.nmods = nb;
         k<<<8u * (unsigned)a.tiles_per_class * (unsigned)a.groups * (unsigned)nb, TC_THREADS, smem, P.stream>>>(S->maps[l], a);
         FMM_LAUNCH_CHECK(P);
-        k_res_join<<<(unsigned)((elems / 2 + 255) / 256), 256, 0, P.stream>>>(
+        k_res_join<<<(unsigned)((elems / 2 + JOIN_THREADS - 1) / JOIN_THREADS), JOIN_THREADS, 0, P.stream>>>(
             elems, nc, a.groups, m0, nb, S->resid, S->frac, m0 == 0, m0 + nb == n, S->s64, S->amax + l, (double *)P.L[l],
-            S->c);
+            low, S->c);
         FMM_LAUNCH_CHECK(P);
     }
+    return FMM_OK;
+}
+
+// the listed targets of all levels
+fmm_status launch_m2l_res_low(Plan &P)
+{
+    ResState *S = (ResState *)P.res;
+    if (!S) return FMM_ERR_INTERNAL;
+    ResLevels lv = {};
+    for (int l = 2; l <= P.d; ++l) {
+        lv.M[l] = (const double *)P.M[l];
+        lv.L[l] = (double *)P.L[l];
+    }
+    k_res_low<<<4 * 152, LOW_THREADS, 0, P.stream>>>(P.nc, P.d, P.ws, n_il(P.ws), lv, S->cmax, P.tab.Top64, P.tab.il, S->low,
+                                                     S->low_count, S->low_part, S->low_count + 1);
+    FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
 
@@ -524,7 +695,7 @@ void res_free(Plan &P)
     cudaFree(S->resid);
     cudaFree(S->frac);
     cudaFree(S->s64);
-    cudaFree(S->amax);
+    cudaFree(S->low_part);  // and amax, cmax, low
     cudaFree(S->mods);
     delete S;
     P.res = nullptr;

@@ -259,20 +259,21 @@ constexpr int FOLD_SPLIT = 2;  // threads per row of A where there are few (2 x 
 // with the PB parents side by side, which one entry of A then serves in one vector load.  A lone parent's rows (PB = 1, levels
 // whose blocks leave most of the GPU idle) are read by FOLD_SPLIT threads each, whose sums are added in order: the loop
 // over a row is a chain of loads.  sx, amax (or null): the level's largest |M sx| is folded in for the gain of the
-// M2L's operands.
+// M2L's operands; cmax (FP64, with amax): that of each parent, the double's upper word.
 template <typename T, int PB, typename U>
 __global__ void k_m2m_fold(int nc, int l, const FoldEntry<T> *__restrict__ ent, const int *__restrict__ cnt,
                            const T *__restrict__ child, T *__restrict__ parent, const T *__restrict__ sx,
-                           U *__restrict__ amax)
+                           U *__restrict__ amax, uint32_t *__restrict__ cmax)
 {
     constexpr int SPLIT = PB == 1 ? FOLD_SPLIT : 1;
+    constexpr int NM = sizeof(U) == 8 ? PB : 1;  // maxima kept apart: per parent in FP64
     extern __shared__ __align__(16) unsigned char fold_smem[];
-    __shared__ U mx_sh;
+    __shared__ U mx_sh[NM];
     T *W = reinterpret_cast<T *>(fold_smem);  // [8][nc][PB], then [SPLIT - 1][nc] partial sums
     const int64_t np3 = (int64_t)1 << (3 * l), n0 = (int64_t)blockIdx.x * PB;  // PB divides 8^l
     const int width = blockDim.x / SPLIT;
     const int part = SPLIT > 1 ? threadIdx.x / width : 0, k = threadIdx.x - part * width;
-    if (threadIdx.x == 0) mx_sh = 0;
+    if (threadIdx.x < NM) mx_sh[threadIdx.x] = 0;
     if (k < nc && part == 0) {
         alignas(16) T w[8][PB];
 #pragma unroll
@@ -284,7 +285,7 @@ __global__ void k_m2m_fold(int nc, int l, const FoldEntry<T> *__restrict__ ent, 
         for (int c = 0; c < 8; ++c) put_vec<T, PB>(W + (c * nc + k) * PB, w[c]);
     }
     __syncthreads();
-    U mx = 0;
+    U mx[NM] = {};
     alignas(16) T acc[PB] = {};
     if (k < nc) {
         const int n = cnt[k];
@@ -309,18 +310,32 @@ __global__ void k_m2m_fold(int nc, int l, const FoldEntry<T> *__restrict__ ent, 
             parent[cell_index(l, p & (side - 1), (p >> l) & (side - 1), p >> (2 * l)) * nc + k] = acc[b];
             if (amax) {
                 const U v = mag_bits(acc[b] * sx[k]);
-                mx = v > mx ? v : mx;
+                mx[b % NM] = v > mx[b % NM] ? v : mx[b % NM];
             }
         }
     }
     if (amax) {
-        for (int o = 16; o > 0; o >>= 1) {
-            const U v = __shfl_xor_sync(0xffffffffu, mx, o);
-            mx = v > mx ? v : mx;
+#pragma unroll
+        for (int b = 0; b < NM; ++b) {
+            for (int o = 16; o > 0; o >>= 1) {
+                const U v = __shfl_xor_sync(0xffffffffu, mx[b], o);
+                mx[b] = v > mx[b] ? v : mx[b];
+            }
+            if ((threadIdx.x & 31) == 0 && mx[b] > 0) atomicMax(&mx_sh[b], mx[b]);
         }
-        if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(&mx_sh, mx);
         __syncthreads();
-        if (threadIdx.x == 0 && mx_sh > 0) atomicMax(amax, mx_sh);
+        if (threadIdx.x == 0) {
+            U m = mx_sh[0];
+#pragma unroll
+            for (int b = 1; b < NM; ++b) m = mx_sh[b] > m ? mx_sh[b] : m;
+            if (m > 0) atomicMax(amax, m);
+        }
+        if constexpr (sizeof(U) == 8) {
+            if (cmax && threadIdx.x < PB) {
+                const int p = (int)n0 + threadIdx.x, side = 1 << l;
+                cmax[cell_index(l, p & (side - 1), (p >> l) & (side - 1), p >> (2 * l))] = (uint32_t)(mx_sh[threadIdx.x] >> 32);
+            }
+        }
     }
 }
 
@@ -396,7 +411,7 @@ __global__ void k_l2l_fold(int nc, int l, const FoldEntry<T> *__restrict__ ent, 
 inline bool fold_wide(int64_t parents) { return parents >= 8 * 152 * FOLD_PB / 2; }
 
 template <typename T, typename U>
-fmm_status m2m_t(Plan &P, int l, const void *ent, const T *sx, U *amax)
+fmm_status m2m_t(Plan &P, int l, const void *ent, const T *sx, U *amax, uint32_t *cmax)
 {
     const int64_t n = (int64_t)1 << (3 * l);
     const int threads = (P.nc + 31) / 32 * 32;  // at most 448
@@ -405,10 +420,10 @@ fmm_status m2m_t(Plan &P, int l, const void *ent, const T *sx, U *amax)
     T *parent = (T *)P.M[l];
     if (fold_wide(n))
         k_m2m_fold<T, FOLD_PB, U><<<(unsigned)(n / FOLD_PB), threads, sizeof(T) * 8 * P.nc * FOLD_PB, P.stream>>>(
-            P.nc, l, e, P.tab.fold_cnt, child, parent, sx, amax);
+            P.nc, l, e, P.tab.fold_cnt, child, parent, sx, amax, cmax);
     else
         k_m2m_fold<T, 1, U><<<(unsigned)n, FOLD_SPLIT * threads, sizeof(T) * (7 + FOLD_SPLIT) * P.nc, P.stream>>>(
-            P.nc, l, e, P.tab.fold_cnt, child, parent, sx, amax);
+            P.nc, l, e, P.tab.fold_cnt, child, parent, sx, amax, cmax);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
@@ -489,10 +504,11 @@ fmm_status launch_m2m(Plan &P, int l)
 {
     if (P.precision == FMM_PREC_FP64) {
         const double *sx = nullptr;
-        unsigned long long *amax = res_amax(P, l, &sx);
-        return m2m_t<double, unsigned long long>(P, l, P.tab.m2m_fold64, sx, amax);
+        uint32_t *cmax = nullptr;
+        unsigned long long *amax = res_amax(P, l, &sx, &cmax);
+        return m2m_t<double, unsigned long long>(P, l, P.tab.m2m_fold64, sx, amax, cmax);
     }
-    return m2m_t<float, unsigned>(P, l, P.tab.m2m_fold32, tc_scale(P), tc_amax(P, l));
+    return m2m_t<float, unsigned>(P, l, P.tab.m2m_fold32, tc_scale(P), tc_amax(P, l), nullptr);
 }
 
 // L2L from level l - 1 into level l (added to the M2L result)
