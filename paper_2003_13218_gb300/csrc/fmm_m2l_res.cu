@@ -533,10 +533,6 @@ fmm_status prepare(Plan &P, ResState *S)
         m = S->maps[0];
         st = encode_planes(enc, &m.aS, nullptr, &m.aC, dt, S->planes, kc, S->batch[l], np2, np2, 8 * np2, S->bx[l],
                            S->by[l], S->bz[l], 128);
-        if (pairs_at(S, l)) {
-            m.bS = S->mapB2[0];
-            m.bC = S->mapB2[1];
-        }
         m.aP = m.lS = m.lP = m.aS;  // unused kernel parameters
         m.bP = m.bS;
     }
@@ -619,12 +615,18 @@ fmm_status launch_m2l_res(Plan &P, int l)
     a.ws = P.ws;
     for (int k = 0; k < S->kp / 64; ++k) a.gchunks |= 1u << (2 * k);  // one product per chunk, two chunks a stage
     a.acc_group = RES_CHAIN;
-    a.wait_ns = WAIT_LIMIT_NS;
+    a.wait_ns = P.wait_ns;
+    a.inject_stall = P.inject_stall ? 1 : 0;
     a.err = P.d_err;
     a.mods = S->mods;
     a.il = P.tab.il;
     a.resid = S->resid;
-    const bool pair = pairs_at(S, l);
+    const bool pair = P.tc_pair && pairs_at(S, l);
+    TcMaps maps = S->maps[l];
+    if (pair) {
+        maps.bS = S->mapB2[0];
+        maps.bC = S->mapB2[1];
+    }
     a.stages = pair ? tc_pair_stages(S->npad) : tc_stages(2, 2, S->npad, 128);
     a.idesc = (1u << 4) | ((uint32_t)(S->npad >> 3) << 17) | ((uint32_t)((pair ? 2 * TC_ROWS : TC_ROWS) >> 4) << 24);
     const TcKernel k = pair ? res_pair_kernel(S->npad / 16) : res_kernel(S->npad / 16);
@@ -638,7 +640,7 @@ fmm_status launch_m2l_res(Plan &P, int l)
         FMM_LAUNCH_CHECK(P);
         a.mod0 = m0;
         a.nmods = nb;
-        k<<<8u * (unsigned)a.tiles_per_class * (unsigned)a.groups * (unsigned)nb, TC_THREADS, smem, P.stream>>>(S->maps[l], a);
+        k<<<8u * (unsigned)a.tiles_per_class * (unsigned)a.groups * (unsigned)nb, TC_THREADS, smem, P.stream>>>(maps, a);
         FMM_LAUNCH_CHECK(P);
         k_res_join<<<(unsigned)((elems / 2 + JOIN_THREADS - 1) / JOIN_THREADS), JOIN_THREADS, 0, P.stream>>>(
             elems, nc, a.groups, m0, nb, S->resid, S->frac, m0 == 0, m0 + nb == n, S->s64, S->amax + l, (double *)P.L[l],
@@ -678,9 +680,8 @@ fmm_status res_share_operators(Plan &dst, const Plan &src)
     D->mapB2[0] = S->mapB2[0];
     D->mapB2[1] = S->mapB2[1];
     for (int l = 2; l <= dst.d; ++l) {
-        const bool pair = pairs_at(D, l);
-        D->maps[l].bS = D->maps[l].bP = pair ? S->mapB2[0] : S->maps[0].bS;
-        D->maps[l].bC = pair ? S->mapB2[1] : S->maps[0].bC;
+        D->maps[l].bS = D->maps[l].bP = S->maps[0].bS;
+        D->maps[l].bC = S->maps[0].bC;
     }
     return FMM_OK;
 }
