@@ -106,7 +106,11 @@ enum {
     FMM_OPT_WS = 1,        /* well-separatedness ws of App. B: 1 (default; 189-cell interaction lists,
                               27-leaf near field) or 2 (the paper's setting: 875 and 125; needs 2^depth > 5);
                               other values FMM_ERR_UNSUPPORTED (> 2) or FMM_ERR_INVALID_ARG */
-    FMM_OPT_PRECISION = 2, /* ival: FMM_PREC_FP64 (default) or FMM_PREC_MIXED */
+    FMM_OPT_PRECISION = 2, /* ival: FMM_PREC_FP64 (default) or FMM_PREC_MIXED.  The first evaluation of an FP64 plan
+                              of order <= 15 allocates and fills the operands of its tensor-core M2L (p = 12: 0.32
+                              GB at ws = 1, 1.3 GB at ws = 2, and up to 2 GB of work space in deep trees) without
+                              waiting for the stream; where the memory is short, or the stream is being captured,
+                              the M2L runs on the CUDA cores, some hundred times slower (fmm_plan_m2l_backend) */
     FMM_OPT_KAPPA = 3,     /* dval: splitting parameter kappa of Eq. 12 and Eq. 6 in 1/A;
                               <= 0 restores the default kappa = 2 / b */
     FMM_OPT_M2L_SPLIT = 4, /* ival: mixed-precision M2L operand split, FMM_SPLIT_* (default FP16X2) */

@@ -30,7 +30,6 @@
 #include <string.h>
 
 #include <new>
-#include <vector>
 
 #include "fmm_tc.cuh"
 
@@ -67,12 +66,12 @@ struct ResState {
     CUtensorMap mapB2[2];         // S, C of half operator tiles (CTA pairs)
     int batch[9];                 // moduli per launch of a level
     int bx[9], by[9], bz[9], groups[9], per_group[9];
-    double *s64 = nullptr;        // [nc] s(n,m)
+    double *s64 = nullptr;        // [nc] s(n,m); the allocation of all that follows
     unsigned long long *amax = nullptr;  // [9] bits of the largest |M^ s| per level
     uint32_t *cmax = nullptr;            // the same per cell, upper words, levels 1 .. d behind one another
     uint32_t *low = nullptr;             // targets that take the FP64 sum (numbered as in cmax)
     int *low_count = nullptr;            // behind amax: their count, then [LOW_CELLS] blocks done
-    double *low_part = nullptr;          // [LOW_CELLS][LOW_GROUPS][nc]; the allocation that amax, cmax and low share
+    int low_cells = 0;                   // targets whose offsets can be split ([LOW_GROUPS][nc] sums each, in planes)
     int *mods = nullptr;
 };
 
@@ -107,6 +106,22 @@ __device__ __forceinline__ void pow2_factors(int e, double &a, double &b)
 {
     a = pow2d(e / 2);
     b = pow2d(e - e / 2);
+}
+
+// s(n,m) = sqrt((n+m)! (n-m)!) per real coefficient, and the moduli (by a kernel: the host would have to wait for the
+// stream to stage a copy)
+__global__ void k_res_setup(int p, double *__restrict__ s, int *__restrict__ mods, const __grid_constant__ ResConsts c)
+{
+    for (int e = threadIdx.x; e < (p + 1) * (p + 1); e += blockDim.x) {
+        const int n = e / (p + 1), m = e % (p + 1);
+        if (m > n) continue;
+        double f = 1.0;
+        for (int i = 2; i <= n + m; ++i) f *= i;
+        for (int i = 2; i <= n - m; ++i) f *= i;
+        s[cre(n, m)] = sqrt(f);
+        if (m > 0) s[cim(n, m)] = sqrt(f);
+    }
+    for (int i = threadIdx.x; i < RES_MAX; i += blockDim.x) mods[i] = c.p[i];
 }
 
 // T~ of every slot -> residues times (P / p_i)^-1, [modulus][chunk][slot][j][k] with zero padding
@@ -294,14 +309,14 @@ constexpr int LOW_THREADS = 128, LOW_CELLS = 128, LOW_GROUPS = 63;
 __global__ void __launch_bounds__(LOW_THREADS) k_res_low(int nc, int d, int ws, int n_il, const __grid_constant__ ResLevels lv,
                                                          const uint32_t *__restrict__ cmax, const double *__restrict__ Top,
                                                          const int *__restrict__ il, const uint32_t *__restrict__ list,
-                                                         const int *__restrict__ count, double *__restrict__ part,
-                                                         int *__restrict__ done)
+                                                         const int *__restrict__ count, int split_max,
+                                                         double *__restrict__ part, int *__restrict__ done)
 {
     constexpr int Q = 256 / LOW_THREADS;  // coefficients per thread
     __shared__ double sM[256];
     __shared__ int last;
     const int n = *count;
-    const int ng = n <= LOW_CELLS ? LOW_GROUPS : 1, per = (n_il + ng - 1) / ng;
+    const int ng = n <= split_max ? LOW_GROUPS : 1, per = (n_il + ng - 1) / ng;
     for (int64_t it = blockIdx.x; it < (int64_t)n * ng; it += gridDim.x) {
         const int i = (int)(it / ng), g = (int)(it - (int64_t)i * ng);
         const uint32_t code = list[i];
@@ -469,27 +484,17 @@ fmm_status prepare(Plan &P, ResState *S)
     S->kp = (P.nc + 63) / 64 * 64;
     S->noff = noff(P.ws);
     const int kc = S->kp / 64, n = S->c.n;
-    std::vector<double> h_s(P.nc);
-    for (int d = 0; d <= P.p; ++d)
-        for (int m = 0; m <= d; ++m) {
-            double f = 1.0;
-            for (int i = 2; i <= d + m; ++i) f *= i;
-            for (int i = 2; i <= d - m; ++i) f *= i;
-            h_s[cre(d, m)] = sqrt(f);
-            if (m > 0) h_s[cim(d, m)] = sqrt(f);
-        }
-    FMM_CUDA_TRY(cudaMalloc(&S->s64, sizeof(double) * P.nc));
-    {
-        const size_t part = sizeof(double) * LOW_CELLS * LOW_GROUPS * P.nc, cells = cmax_at(P.d + 1);
-        FMM_CUDA_TRY(cudaMalloc(&S->low_part, part + RES_CLEAR + 2 * sizeof(uint32_t) * cells));  // one allocation
-        S->amax = (unsigned long long *)((char *)S->low_part + part);
-        S->low_count = (int *)(S->amax + 9);
-        S->cmax = (uint32_t *)((char *)S->amax + RES_CLEAR);
-        S->low = S->cmax + cells;
-    }
-    FMM_CUDA_TRY(cudaMalloc(&S->mods, sizeof(int) * RES_MAX));
-    FMM_CUDA_TRY(cudaMemcpyAsync(S->s64, h_s.data(), sizeof(double) * P.nc, cudaMemcpyHostToDevice, P.stream));
-    FMM_CUDA_TRY(cudaMemcpyAsync(S->mods, S->c.p, sizeof(int) * RES_MAX, cudaMemcpyHostToDevice, P.stream));
+    const size_t cells_all = cmax_at(P.d + 1);
+    // s64, amax and what is cleared with it, mods, cmax, low in one allocation
+    FMM_CUDA_TRY(cudaMalloc(&S->s64, sizeof(double) * P.nc + RES_CLEAR + sizeof(int) * RES_MAX +
+                                         2 * sizeof(uint32_t) * cells_all));
+    S->amax = (unsigned long long *)(S->s64 + P.nc);
+    S->low_count = (int *)(S->amax + 9);
+    S->mods = (int *)((char *)S->amax + RES_CLEAR);
+    S->cmax = (uint32_t *)(S->mods + RES_MAX);
+    S->low = S->cmax + cells_all;
+    k_res_setup<<<1, 256, 0, P.stream>>>(P.p, S->s64, S->mods, S->c);
+    FMM_LAUNCH_CHECK(P);
     S->ops_elems = (size_t)S->noff * S->npad * S->kp;
     FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_elems * n));
     k_res_ops<<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.nc, S->npad, S->kp, S->s64, S->ops, S->ops_elems, S->c);
@@ -517,6 +522,10 @@ fmm_status prepare(Plan &P, ResState *S)
         if (r > resid) resid = r;
         if (b < n && cells * P.nc > frac) frac = cells * P.nc;
     }
+    // the launch of the FP64 sums follows the last level's and takes its place in the planes (at least 16 targets)
+    const size_t low_cell = sizeof(double) * LOW_GROUPS * P.nc;
+    if (planes < 16 * low_cell) planes = 16 * low_cell;
+    S->low_cells = planes / low_cell < LOW_CELLS ? (int)(planes / low_cell) : LOW_CELLS;
     FMM_CUDA_TRY(cudaMalloc(&S->planes, planes));
     FMM_CUDA_TRY(cudaMalloc(&S->resid, resid));
     if (frac) FMM_CUDA_TRY(cudaMalloc(&S->frac, frac * 3 * sizeof(uint32_t)));
@@ -543,7 +552,6 @@ fmm_status prepare(Plan &P, ResState *S)
                                       (int)tc_smem_bytes(2, 2, S->npad, 128)));
     FMM_CUDA_TRY(cudaFuncSetAttribute((const void *)k2, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)tc_pair_smem_bytes(S->npad)));
-    FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
     return FMM_OK;
 }
 
@@ -551,7 +559,8 @@ fmm_status prepare(Plan &P, ResState *S)
 
 bool res_available(const Plan &P, int level) { return P.res != nullptr && level >= 1 && level <= P.d; }
 
-// The residue state of an FP64 plan; without the memory for it the plan keeps the CUDA-core M2L
+// The residue state of an FP64 plan; without the memory for it the plan keeps the CUDA-core M2L.  Nothing here waits for
+// the plan's stream: a call that only enqueues does so the first time as well.
 fmm_status res_ensure(Plan &P)
 {
     if (P.res || P.res_tried || P.precision != FMM_PREC_FP64 || P.p > TC_PMAX) return FMM_OK;
@@ -562,7 +571,11 @@ fmm_status res_ensure(Plan &P)
     ResState *S = new (std::nothrow) ResState();
     if (!S) return FMM_ERR_OOM;
     P.res = S;
+    // allocations of this thread leave a capture in another one alone
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    FMM_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
     const fmm_status st = prepare(P, S);
+    FMM_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
     if (st == FMM_OK) return FMM_OK;
     cudaStreamSynchronize(P.stream);
     res_free(P);
@@ -661,7 +674,7 @@ fmm_status launch_m2l_res_low(Plan &P)
         lv.L[l] = (double *)P.L[l];
     }
     k_res_low<<<4 * 152, LOW_THREADS, 0, P.stream>>>(P.nc, P.d, P.ws, n_il(P.ws), lv, S->cmax, P.tab.Top64, P.tab.il, S->low,
-                                                     S->low_count, S->low_part, S->low_count + 1);
+                                                     S->low_count, S->low_cells, (double *)S->planes, S->low_count + 1);
     FMM_LAUNCH_CHECK(P);
     return FMM_OK;
 }
@@ -695,9 +708,7 @@ void res_free(Plan &P)
     cudaFree(S->planes);
     cudaFree(S->resid);
     cudaFree(S->frac);
-    cudaFree(S->s64);
-    cudaFree(S->low_part);  // and amax, cmax, low
-    cudaFree(S->mods);
+    cudaFree(S->s64);  // and what shares its allocation
     delete S;
     P.res = nullptr;
 }
