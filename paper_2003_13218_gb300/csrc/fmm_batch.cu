@@ -78,7 +78,7 @@ fmm_status time_plan(fmm_plan h, const double *pos, const double *q, const uint8
     cudaEvent_t e0, e1;
     FMM_CUDA_TRY(cudaEventCreate(&e0));
     FMM_CUDA_TRY(cudaEventCreate(&e1));
-    fmm_status s = FMM_OK;
+    fmm_status s = res_ensure(P);  // FP64: the M2L that the boxes will run
     float best = 1e30f;
     for (int it = 0; it < 3 && s == FMM_OK; ++it) {  // one warm-up, best of two
         cudaEventRecord(e0, P.stream);
