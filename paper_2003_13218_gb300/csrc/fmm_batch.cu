@@ -610,7 +610,17 @@ fmm_status fmm_batch_create_tuned(int nbox, const double *box, const int64_t *N,
         const int i = b->order[k];
         s = make_plan(box[i], N[i], b->depth[i], porder[i], precision, b->streams[k % ns], &b->plans[i]);
     }
-    for (int i = 0; i < nbox && s == FMM_OK; ++i) s = res_ensure(b->plans[i]->P);
+    // FP64: the boxes of an order read one copy of its operators, and their planes together stay within twice a plan's
+    if (s == FMM_OK && precision == FMM_PREC_FP64) {
+        const size_t budget = nbox > 2 ? 2 * RES_PLANE_BUDGET / nbox : RES_PLANE_BUDGET;
+        for (int i = 0; i < nbox && s == FMM_OK; ++i) {
+            const Plan *src = nullptr;
+            for (int j = 0; j < i && !src; ++j)
+                if (b->plans[j]->P.p == b->plans[i]->P.p) src = &b->plans[j]->P;
+            s = res_ensure(b->plans[i]->P, src, budget);
+        }
+        if (s == FMM_OK && cudaDeviceSynchronize() != cudaSuccess) s = FMM_ERR_CUDA;  // the operators are filled
+    }
     // tile bricks of the deepest level, per depth group, by timing (before anything is recorded)
     if (s == FMM_OK && policy->tiles == 1 && precision == FMM_PREC_MIXED) s = tune_bricks(b, N, box);
     // one copy of the tensor-core operator tables per order: the boxes' tiles then read them from L2
@@ -618,7 +628,6 @@ fmm_status fmm_batch_create_tuned(int nbox, const double *box, const int64_t *N,
         for (int j = 0; j < i && s == FMM_OK; ++j)
             if (b->plans[j]->P.p == b->plans[i]->P.p) {
                 s = tc_share_operators(b->plans[i]->P, b->plans[j]->P);
-                if (s == FMM_OK) s = res_share_operators(b->plans[i]->P, b->plans[j]->P);
                 break;
             }
     // the persistent sweep over the boxes' CTA-pair levels (mixed precision)

@@ -337,15 +337,15 @@ void tc_free(Plan &P);
 // launch_m2l_res_low computes the targets that need floating-point sums
 bool res_available(const Plan &P, int level);
 // builds the state on an FP64 plan's first evaluation (a plan that is to run the mixed path never pays for it);
-// left for later while the plan's stream is being captured
-fmm_status res_ensure(Plan &P);
+// left for later while the plan's stream is being captured.  plane_budget: bytes of operand planes held at once
+constexpr size_t RES_PLANE_BUDGET = (size_t)2 << 30;
+fmm_status res_ensure(Plan &P, const Plan *src = nullptr, size_t plane_budget = RES_PLANE_BUDGET);
 // where the P2M and M2M leave a level's largest |Mhat s|, and that of each of its cells (upper word of the double), and
 // s (null without the state)
 unsigned long long *res_amax(Plan &P, int level, const double **s, uint32_t **cmax);
 fmm_status res_clear_amax(Plan &P);  // at the start of a far-field pass
 fmm_status launch_m2l_res(Plan &P, int level);
 fmm_status launch_m2l_res_low(Plan &P);
-fmm_status res_share_operators(Plan &dst, const Plan &src);
 void res_free(Plan &P);
 
 // phases of one energy + solute-solvent evaluation on device inputs (fmm_api.cu), for the batch API:

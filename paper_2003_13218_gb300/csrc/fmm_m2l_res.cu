@@ -41,7 +41,6 @@ constexpr int RES_MAX = 16;        // moduli
 constexpr int RES_CHAIN = 2;       // offsets per accumulator (G)
 constexpr int RES_M_BITS = 56, RES_M_BITS_MAX = 58;  // |M_int| < 2^B, B as the moduli allow
 constexpr int JOIN_THREADS = 256;
-constexpr size_t RES_PLANE_BUDGET = (size_t)2 << 30;  // operand planes held at once (moduli per launch)
 
 struct ResConsts {
     int n;
@@ -473,7 +472,7 @@ unsigned blocks_upto(int64_t n, int t, int64_t most)
     return (unsigned)(b < most ? b : most);
 }
 
-fmm_status prepare(Plan &P, ResState *S)
+fmm_status prepare(Plan &P, ResState *S, const ResState *src, size_t plane_budget)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return FMM_ERR_UNSUPPORTED;
@@ -496,9 +495,14 @@ fmm_status prepare(Plan &P, ResState *S)
     k_res_setup<<<1, 256, 0, P.stream>>>(P.p, S->s64, S->mods, S->c);
     FMM_LAUNCH_CHECK(P);
     S->ops_elems = (size_t)S->noff * S->npad * S->kp;
-    FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_elems * n));
-    k_res_ops<<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.nc, S->npad, S->kp, S->s64, S->ops, S->ops_elems, S->c);
-    FMM_LAUNCH_CHECK(P);
+    S->ops_borrowed = src != nullptr;
+    if (src) S->ops = src->ops;
+    else {
+        FMM_CUDA_TRY(cudaMalloc(&S->ops, sizeof(uint16_t) * S->ops_elems * n));
+        k_res_ops<<<1216, 256, 0, P.stream>>>(S->noff, P.tab.Top64, P.nc, S->npad, S->kp, S->s64, S->ops, S->ops_elems,
+                                              S->c);
+        FMM_LAUNCH_CHECK(P);
+    }
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
@@ -511,7 +515,7 @@ fmm_status prepare(Plan &P, ResState *S)
         S->by[l] = tile_dim(np, TC_ROWS / S->bx[l]);
         S->bz[l] = tile_dim(np, TC_ROWS / (S->bx[l] * S->by[l]));
         const size_t plane = 8 * np2 * np2 * np2 * S->kp * sizeof(uint16_t);
-        int b = (int)(RES_PLANE_BUDGET / plane);
+        int b = (int)(plane_budget / plane);
         b = b < 1 ? 1 : (b > n ? n : b);
         b = (n + (n + b - 1) / b - 1) / ((n + b - 1) / b);  // even launches
         S->batch[l] = b;
@@ -560,8 +564,9 @@ fmm_status prepare(Plan &P, ResState *S)
 bool res_available(const Plan &P, int level) { return P.res != nullptr && level >= 1 && level <= P.d; }
 
 // The residue state of an FP64 plan; without the memory for it the plan keeps the CUDA-core M2L.  Nothing here waits for
-// the plan's stream: a call that only enqueues does so the first time as well.
-fmm_status res_ensure(Plan &P)
+// the plan's stream: a call that only enqueues does so the first time as well.  With `src`, a plan of the same p and ws
+// that has the state, the operators are src's (which must outlive P; its stream may still be filling them).
+fmm_status res_ensure(Plan &P, const Plan *src, size_t plane_budget)
 {
     if (P.res || P.res_tried || P.precision != FMM_PREC_FP64 || P.p > TC_PMAX) return FMM_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -574,7 +579,8 @@ fmm_status res_ensure(Plan &P)
     // allocations of this thread leave a capture in another one alone
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     FMM_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
-    const fmm_status st = prepare(P, S);
+    const bool borrow = src && src->res && src->p == P.p && src->ws == P.ws;
+    const fmm_status st = prepare(P, S, borrow ? (const ResState *)src->res : nullptr, plane_budget);
     FMM_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
     if (st == FMM_OK) return FMM_OK;
     cudaStreamSynchronize(P.stream);
@@ -676,26 +682,6 @@ fmm_status launch_m2l_res_low(Plan &P)
     k_res_low<<<4 * 152, LOW_THREADS, 0, P.stream>>>(P.nc, P.d, P.ws, n_il(P.ws), lv, S->cmax, P.tab.Top64, P.tab.il, S->low,
                                                      S->low_count, S->low_cells, (double *)S->planes, S->low_count + 1);
     FMM_LAUNCH_CHECK(P);
-    return FMM_OK;
-}
-
-// dst reads src's operator residues when they are the same (p, ws); src must outlive dst
-fmm_status res_share_operators(Plan &dst, const Plan &src)
-{
-    ResState *D = (ResState *)dst.res;
-    const ResState *S = (const ResState *)src.res;
-    if (!D || !S || D == S || D->ops == S->ops || dst.p != src.p || dst.ws != src.ws) return FMM_OK;
-    FMM_CUDA_TRY(cudaDeviceSynchronize());  // nothing of dst's may still read its own table
-    if (!D->ops_borrowed) cudaFree(D->ops);
-    D->ops = S->ops;
-    D->ops_borrowed = true;
-    D->maps[0] = S->maps[0];
-    D->mapB2[0] = S->mapB2[0];
-    D->mapB2[1] = S->mapB2[1];
-    for (int l = 2; l <= dst.d; ++l) {
-        D->maps[l].bS = D->maps[l].bP = S->maps[0].bS;
-        D->maps[l].bC = S->maps[0].bC;
-    }
     return FMM_OK;
 }
 
