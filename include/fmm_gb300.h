@@ -253,9 +253,11 @@ fmm_status fmm_plan_get_timings(fmm_plan plan, fmm_timings *out);
 int64_t fmm_plan_last_launch_count(fmm_plan plan);
 
 /* Which M2L implementation the plan runs at `level` (1..depth):
- * 0 = FP64 (whole-number residue products on the tensor cores up to order 15, CUDA cores above it and where the
- * residue operands do not fit in memory), 1 = FP32 CUDA cores, 2 = tcgen05 tensor cores in 16-bit splits;
- * -1 for a NULL plan or a level out of range. */
+ * 0 = FP64 CUDA cores, 1 = FP32 CUDA cores, 2 = tcgen05 tensor cores in 16-bit splits, 3 = FP64 as whole-number
+ * residue products on the tensor cores; -1 for a NULL plan or a level out of range.  An FP64 plan of order <= 15 is
+ * at 0 until its first evaluation has built the residue operands, and stays there where they do not fit in memory.
+ * The M2L of level 1 is part of the top operator (CUDA cores, the plan's precision) in every plan: an FP64 plan
+ * reports 0 there, a mixed one what its other levels run. */
 int fmm_plan_m2l_backend(fmm_plan plan, int level);
 
 /* Release the plan and its device memory.  Accepts NULL. */

@@ -614,6 +614,7 @@ int fmm_plan_m2l_backend(fmm_plan plan, int level)
 {
     if (!plan || level < 1 || level > plan->P.d) return -1;
     if (tc_available(plan->P, level)) return 2;
+    if (level >= 2 && res_available(plan->P, level)) return 3;
     return plan->P.precision == FMM_PREC_FP64 ? 0 : 1;
 }
 

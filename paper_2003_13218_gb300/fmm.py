@@ -323,7 +323,7 @@ class FMMPlan:
 
     def m2l_backend(self, level: int) -> str:
         code = int(self._lib.fmm_plan_m2l_backend(self._h, int(level)))
-        return {0: "fp64-simt", 1: "fp32-simt", 2: "tcgen05"}.get(code, "invalid")
+        return {0: "fp64-simt", 1: "fp32-simt", 2: "tcgen05", 3: "fp64-residues"}.get(code, "invalid")
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
