@@ -14,8 +14,6 @@ using namespace fmm;
 
 namespace {
 
-size_t reduction_scratch_bytes() { return sizeof(double) * 304 * 20 * 2; }
-
 void free_buffers(Plan &P)
 {
     void *bufs[] = {P.in_pos, P.in_q,   P.out_forces, P.out_phi, P.in_sol, P.wpos,    P.key,    P.perm,   P.sleaf,
@@ -73,7 +71,7 @@ fmm_status alloc_buffers(Plan &P)
         FMM_CUDA_TRY(dalloc(&P.M[l], sizeof(double) * cells * nc));
         FMM_CUDA_TRY(dalloc(&P.L[l], sizeof(double) * cells * nc));
     }
-    FMM_CUDA_TRY(dalloc(&P.red_partial, reduction_scratch_bytes()));
+    FMM_CUDA_TRY(dalloc(&P.red_partial, sizeof(double) * reduction_scratch_doubles()));
     FMM_CUDA_TRY(dalloc(&P.red_out, sizeof(double) * 48));
     FMM_CUDA_TRY(dalloc(&P.d_err, sizeof(int) * (ERR_WORDS + P.nleaf)));
     P.cell_fill = P.d_err + ERR_WORDS;

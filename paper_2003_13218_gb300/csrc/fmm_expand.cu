@@ -25,7 +25,7 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 // ------------------------------------------------------------------ tables
 // R_n^m at the eight child-centre offsets w_c = ((c_x - 1/2)/2, ...) (in
 // units of the parent side): the M2M and L2L shift vectors.
-__global__ void k_octant_table(int p, double *__restrict__ R64, float *__restrict__ R32)
+__global__ void k_octant_table(int p, double *__restrict__ R64)
 {
     int c = threadIdx.x;
     if (c >= 8) return;
@@ -33,10 +33,7 @@ __global__ void k_octant_table(int p, double *__restrict__ R64, float *__restric
     double w[3] = {((c & 1) - 0.5) * 0.5, (((c >> 1) & 1) - 0.5) * 0.5, (((c >> 2) & 1) - 0.5) * 0.5};
     double tmp[NC_MAX];
     regular_real<double>(p, w[0], w[1], w[2], tmp);
-    for (int i = 0; i < nc; ++i) {
-        R64[c * nc + i] = tmp[i];
-        R32[c * nc + i] = (float)tmp[i];
-    }
+    for (int i = 0; i < nc; ++i) R64[c * nc + i] = tmp[i];
 }
 
 // complex I_j^k for any sign of k from the m >= 0 triangle
@@ -847,7 +844,6 @@ fmm_status build_tables(Plan &P)
     free_tables(P);
     int p = P.p, nc = P.nc;
     FMM_CUDA_TRY(cudaMalloc(&P.tab.Rw64, sizeof(double) * 8 * nc));
-    FMM_CUDA_TRY(cudaMalloc(&P.tab.Rw32, sizeof(float) * 8 * nc));
     int ntri2 = (2 * p + 1) * (2 * p + 2) / 2;
     FMM_CUDA_TRY(cudaMalloc(&P.tab.S, sizeof(double) * 2 * ntri2));
     FMM_CUDA_TRY(cudaMalloc(&P.tab.T0, sizeof(double) * nc * nc));
@@ -867,7 +863,7 @@ fmm_status build_tables(Plan &P)
         FMM_CUDA_TRY(cudaMemcpyAsync(P.tab.il, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, P.stream));
         FMM_CUDA_TRY(cudaStreamSynchronize(P.stream));
     }
-    k_octant_table<<<1, 32, 0, P.stream>>>(p, P.tab.Rw64, P.tab.Rw32);
+    k_octant_table<<<1, 32, 0, P.stream>>>(p, P.tab.Rw64);
     FMM_LAUNCH_CHECK(P);
     {
         fmm_status st = build_translation_ops(P);
@@ -906,7 +902,6 @@ fmm_status build_lattice(Plan &P)
 void free_tables(Plan &P)
 {
     cudaFree(P.tab.Rw64);
-    cudaFree(P.tab.Rw32);
     cudaFree(P.tab.S);
     cudaFree(P.tab.T0);
     cudaFree(P.tab.Top64);

@@ -84,7 +84,6 @@ __host__ __device__ inline Cx<T> cmul(Cx<T> a, Cx<T> b) { return {a.re * b.re - 
 // Level-independent tables built once per plan.
 struct Tables {
     double *Rw64 = nullptr;   // [8][NC] real R_n^m(w_c), w_c = child-centre offset / parent side (+-1/4)
-    float *Rw32 = nullptr;
     double *S = nullptr;      // [NC2] complex lattice sum S_j^k (j <= 2p, k >= 0), scaled to a unit box
     double *T0 = nullptr;     // [NC][NC] real lattice operator (input-major: T0[k * NC + j])
     double *Top64 = nullptr;  // [noff(ws)][NC][NC] real M2L operators (input-major), FP64 path
@@ -265,6 +264,7 @@ __host__ __device__ inline Cx<T> coef(const T *a, int n, int m)
 
 // ------------------------------------------------------------------ launchers
 // sort / reductions (fmm_sort.cu)
+size_t reduction_scratch_doubles();  // of red_partial
 fmm_status launch_assign_sort(Plan &P, const double *pos, const double *q, const uint8_t *sol);
 fmm_status launch_bc_moments(Plan &P, const double *q, const uint8_t *sol);
 fmm_status launch_energy_reduce(Plan &P, bool with_uv);

@@ -127,7 +127,7 @@ __global__ void k_split_halo(const float *__restrict__ M, int np, int hw, int nc
     }
 }
 
-// FP32 class-layout local expansion of level `lev` (side n = 2^lev) -> fp16
+// FP32 class-layout local expansion of level `lev` >= 1 (side n = 2^lev) -> fp16
 // split planes in natural order [part][chunk][z][y][x][k], balanced L~ = L^ / s(k) gL
 // (the A operand of the fused L2L): natural cell `cell`, lanes over the coefficients.
 __device__ __forceinline__ void split_L_cell(const float *__restrict__ L, int lev, int nc, int kp,
@@ -136,9 +136,8 @@ __device__ __forceinline__ void split_L_cell(const float *__restrict__ L, int le
 {
     const int n = 1 << lev, h = n >> 1;
     const int x = (int)(cell % n), y = (int)((cell / n) % n), z = (int)(cell / ((int64_t)n * n));
-    const int64_t src = lev == 0 ? 0
-                                 : (int64_t)((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)) * h * h * h + (x >> 1) +
-                                       (int64_t)h * ((y >> 1) + (int64_t)h * (z >> 1));
+    const int64_t src = (int64_t)((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)) * h * h * h + (x >> 1) +
+                        (int64_t)h * ((y >> 1) + (int64_t)h * (z >> 1));
     const float *row = L + src * nc;
     const int64_t ncell = (int64_t)n * n * n;
     for (int k = lane; k < kp; k += 32) {

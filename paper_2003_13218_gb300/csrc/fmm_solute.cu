@@ -64,7 +64,7 @@ struct SoluteScratch {
     cudaEvent_t ev_up = nullptr;       // full upward pass done
     cudaEvent_t ev_ready = nullptr;    // expansions ready (Phi_u on the near stream waits)
     cudaEvent_t ev_done = nullptr;     // everything on the side stream done (join)
-    bool count_pending = false, forked = false, act_done = false;
+    bool forked = false, act_done = false;
     double *Lt = nullptr;    // [9][NU_MAX][nc] the solvent's M2L sums at the active cells (FP64)
     void *Lu = nullptr;      // solute-only local expansions of every cell of levels 1..ld (class layout), T
     double *part = nullptr;  // [level][NU_MAX][act_groups][nc] partial sums of Lt
@@ -762,7 +762,6 @@ fmm_status solute_count(Plan &P)
     FMM_CUDA_TRY(cudaEventRecord(S->ev_sort, P.stream));
     FMM_CUDA_TRY(cudaMemcpyAsync(S->h_count, P.d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, P.stream));
     FMM_CUDA_TRY(cudaEventRecord(S->ev_count, P.stream));
-    S->count_pending = true;
     return FMM_OK;
 }
 
@@ -820,7 +819,7 @@ fmm_status launch_solute_pass(Plan &P, bool *done)
     if (s != FMM_OK) return s;
     // the count was copied right after the sort, or the caller knows it
     if (P.known_count < 0) FMM_CUDA_TRY(cudaEventSynchronize(S->ev_count));
-    S->count_pending = S->act_done = false;
+    S->act_done = false;
     const int n = P.known_count >= 0 ? P.known_count : *S->h_count;
     if (n > NU_MAX) return FMM_OK;  // the dense pass overwrites the (empty) result
     if (n == 0) {

@@ -68,7 +68,7 @@ struct TcArgs {
     int acc_group;          // offsets summed in one TMEM accumulator before it is drained (>= 1)
     uint64_t wait_ns;       // budget of every pipeline wait (FMM_OPT_WAIT_BUDGET_NS); the teardown keeps its own
     int inject_stall;       // test hook (single-CTA kernel): the MMA issuer first waits on a barrier nothing arrives on
-    float *L;               // output level array (L of the level, or M of the parent level)
+    float *L;               // output level array (L of the level)
     float *Lpart;           // [groups][level cells][nc] partial sums when groups > 1
     const float *post;      // fp16 split: s(j) per output coefficient, else null
     const unsigned *amax;   // fp16 split: largest |M^ s| of the A planes (gM follows from it)
@@ -225,30 +225,27 @@ __device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity)
 }
 
 // The bounded wait of a whole converged warp: every lane gets the same answer (lanes that read the clock at
-// different times must not leave a loop with warp-wide instructions in it one by one).  CLUSTER: with
-// cluster-scope acquire.  The clock is read out of line: the usual wait is one poll and one vote.
-template <bool CLUSTER>
+// different times must not leave a loop with warp-wide instructions in it one by one).  The clock is read out of
+// line: the usual wait is one poll and one vote.
 __device__ __forceinline__ bool mbar_poll_warp(uint32_t bar, uint32_t parity)
 {
-    return __all_sync(0xffffffffu, CLUSTER ? mbar_try_cluster(bar, parity) : mbar_try(bar, parity)) != 0;
+    return __all_sync(0xffffffffu, mbar_try(bar, parity)) != 0;
 }
 
-template <bool CLUSTER>
 __device__ __noinline__ bool mbar_wait_warp_slow(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                                  uint64_t limit_ns)
 {
     uint64_t t0 = global_ns();
     for (uint32_t i = 0;; ++i) {
-        if (mbar_poll_warp<CLUSTER>(bar, parity)) return true;
+        if (mbar_poll_warp(bar, parity)) return true;
         if ((i & 63) == 63 && __any_sync(0xffffffffu, *abort_flag != 0 || global_ns() - t0 > limit_ns)) return false;
     }
 }
 
-template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                                uint64_t limit_ns)
 {
-    return mbar_poll_warp<CLUSTER>(bar, parity) || mbar_wait_warp_slow<CLUSTER>(bar, parity, abort_flag, limit_ns);
+    return mbar_poll_warp(bar, parity) || mbar_wait_warp_slow(bar, parity, abort_flag, limit_ns);
 }
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2,
