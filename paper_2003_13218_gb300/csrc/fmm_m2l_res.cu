@@ -40,6 +40,7 @@ namespace {
 constexpr int RES_MAX = 16;        // moduli
 constexpr int RES_CHAIN = 2;       // offsets per accumulator (G)
 constexpr int RES_M_BITS = 56, RES_M_BITS_MAX = 58;  // |M_int| < 2^B, B as the moduli allow
+static_assert(RES_M_BITS_MAX < 63 && RES_M_BITS_MAX >= RES_M_BITS, "whole numbers of 64 bits");
 constexpr int JOIN_THREADS = 256;
 
 struct ResConsts {
@@ -65,7 +66,7 @@ struct ResState {
     CUtensorMap mapB2[2];         // S, C of half operator tiles (CTA pairs)
     int batch[9];                 // moduli per launch of a level
     int bx[9], by[9], bz[9], groups[9], per_group[9];
-    double *s64 = nullptr;        // [nc] s(n,m); the allocation of all that follows
+    double *s64 = nullptr;        // [nc] s(n,m); amax, cmax, low and mods are in its allocation
     unsigned long long *amax = nullptr;  // [9] bits of the largest |M^ s| per level
     uint32_t *cmax = nullptr;            // the same per cell, upper words, levels 1 .. d behind one another
     uint32_t *low = nullptr;             // targets that take the FP64 sum (numbered as in cmax)

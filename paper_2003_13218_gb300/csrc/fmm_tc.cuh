@@ -376,11 +376,15 @@ __device__ __forceinline__ void drain_residues(uint32_t taddr, int (&acc)[NCH * 
     }
 }
 
-// a number within about +-0.8 p that is congruent to v modulo p (|v| < 2^31; rp = 1 / p)
+// a number congruent to v modulo p, |v| < 2^31, rp = 1 / p: the quotient has three FP32 roundings, so it is within
+// p / 2 + 3 2^-24 |v| (up to p / 2 + 384)
 __device__ __forceinline__ int mod_near(int v, int p, float rp) { return v - p * __float2int_rn((float)v * rp); }
 
-// drains after which the 32-bit sums are taken modulo p: 96 x 2^24 + p stays below 2^31
+// drains after which the 32-bit sums are taken modulo p: 96 x 2^24 and what mod_near leaves (moduli below 2^11) stay
+// below 2^31; the sums that finish_residues stores fit 16 bits
 constexpr int RES_DRAINS = 96;
+static_assert((int64_t)RES_DRAINS * (1 << 24) + (1 << 10) + 384 < (int64_t)1 << 31, "sums between drains");
+static_assert((1 << 10) + 384 < 1 << 15, "stored residues");
 
 // One warp's 32 rows of residues (staged as 16-bit values, row stride srow) to out + idx(r) nc, as store_rows
 template <int NCH>
