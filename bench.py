@@ -44,13 +44,13 @@ FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 # split, fused L2L, CTA pairs) of the na_1m workload, from the ncu capture of
 # that launch summarised under profiles/, with the sha256 of the kernel's device
 # code it was taken on: the value is reported only while that code is unchanged.
-M2L_TRAFFIC = {"src": "paper_2003_13218_gb300/csrc/fmm_m2l_tc.cu",
-               "sha256": "711fa46ddc82e4c3acf198ceac77e93d844a0a4abb2a2d0c76207d4d088579b9",
+M2L_TRAFFIC = {"src": "paper_2003_13218_gb300/csrc/fmm_tc.cuh",
+               "sha256": "bd571f1e6231c7aa8d9dc6424c58f7938de53e0ce31a90ae55f85b9e93cec33b",
                "workload": "na_1m", "level": 6, "split": "fp16x2", "ws": 1, "p": 12,
-               "bytes_per_launch": 360.280320e6 + 160.011776e6}
+               "bytes_per_launch": 277.844224e6 + 155.751936e6}
 ION_LABEL = {"Na": "Na+", "Cl": "Cl-", "Mg": "Mg2+"}
 KERNEL_BEGIN = "// ------------------------------------------------------------------ the kernel"
-KERNEL_END = "// ------------------------------------------------------------------ operand preparation"
+KERNEL_END = "// ------------------------------------------------------------------ operand layout"
 
 
 def n_il(ws: int) -> int:
