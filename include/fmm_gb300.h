@@ -154,11 +154,12 @@ enum {
     FMM_OPT_WAIT_BUDGET_NS = 15,  /* ival in 1000..10^10: budget (ns) of each bounded wait in the tensor-core
                               kernels (default 2 s); a wait that runs out makes the call return FMM_ERR_TIMEOUT
                               after the kernel has waited, with its own 2 s limit, for its copies and MMAs in
-                              flight; the plan stays usable */
+                              flight; the plan stays usable.  Budgets below the default keep every level on
+                              single CTAs (FMM_OPT_M2L_PAIR) */
     FMM_OPT_INJECT_STALL = 16,    /* ival 0 / 1, a test hook for the timeout path: with 1 the single-CTA
                               tensor-core kernels first wait on a barrier that nothing arrives on, so every
                               evaluation returns FMM_ERR_TIMEOUT after the wait budget (use with
-                              FMM_OPT_M2L_PAIR = 0 and a short budget) */
+                              a short budget) */
     FMM_OPT_M2L_BRICK = 17        /* ival = l | bx << 8 | by << 16 | bz << 24: the tiles of the tensor-core M2L of
                               level l (2..depth) are bricks of bx x by x bz cells of one
                               parity class, bx by bz = 128, each dividing 2^(l-1), an even number per class.

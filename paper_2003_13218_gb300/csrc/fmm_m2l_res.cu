@@ -641,7 +641,7 @@ fmm_status launch_m2l_res(Plan &P, int l)
     a.mods = S->mods;
     a.il = P.tab.il;
     a.resid = S->resid;
-    const bool pair = P.tc_pair && pairs_at(S, l);
+    const bool pair = pairs_allowed(P) && pairs_at(S, l);
     TcMaps maps = S->maps[l];
     if (pair) {
         maps.bS = S->mapB2[0];

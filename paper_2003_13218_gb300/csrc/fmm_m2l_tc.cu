@@ -867,7 +867,7 @@ static bool m2l_args(const Plan &P, const TcState *S, int l, bool precise, int p
         a.amax_out = a.groups == 1 ? S->amaxL + l : nullptr;
         a.sx = S->s32inv;
     }
-    const bool pair = S->f16 && P.tc_pair && a.rows == TC_ROWS && a.tiles_per_class % 2 == 0;
+    const bool pair = S->f16 && pairs_allowed(P) && a.rows == TC_ROWS && a.tiles_per_class % 2 == 0;
     if (pair) {
         a.stages = tc_pair_stages(S->npad);
         a.idesc = (1u << 4) | ((uint32_t)(S->npad >> 3) << 17) | ((uint32_t)((2 * TC_ROWS) >> 4) << 24);  // M = 256
@@ -930,7 +930,7 @@ fmm_status launch_m2l_tc(Plan &P, int l, bool precise)
 int tc_sweep_first_level(const Plan &P)
 {
     const TcState *S = (const TcState *)P.tc;
-    if (!S || !S->f16 || !P.tc_pair || P.precision != FMM_PREC_MIXED) return 0;
+    if (!S || !S->f16 || !pairs_allowed(P) || P.precision != FMM_PREC_MIXED) return 0;
     for (int l = 2; l <= P.d; ++l) {
         const int np = 1 << (l - 1);
         const int tpc = (np / S->bx[l]) * (np / S->by[l]) * (np / S->bz[l]);

@@ -1441,6 +1441,11 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 
 int tile_dim(int np, int cap) { return np < cap ? np : cap; }
 
+// Whether a plan's levels may run on CTA pairs.  When a wait runs out, the pair kernel does not wait for its partner's
+// copies in flight, as the single-CTA kernel does for its own; with the default budget every copy has had two seconds
+// to land by then, a shorter one keeps to single CTAs.
+bool pairs_allowed(const Plan &P) { return P.tc_pair && P.wait_ns >= WAIT_LIMIT_NS; }
+
 // stage ring of the split (pa, pb): as many stages as the shared-memory budget allows, 2..6
 int tc_stages(int pa, int pb, int npad, int sw)
 {
