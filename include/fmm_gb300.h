@@ -89,8 +89,9 @@ typedef struct {
 } fmm_uv_terms;
 
 /* Per-stage device times of the last call, milliseconds (CUDA events on the
- * stream that runs the far field).  m2l_l2l covers M2L and L2L of levels
- * 1..l_max of the full pass; m2l_kernels the M2L launches alone; solute_pass
+ * stream that runs the far field).  lattice is the top operator (the M2L of
+ * level 1 and all above it); m2l_l2l covers M2L and L2L of levels
+ * 2..l_max of the full pass; m2l_kernels the M2L launches alone; solute_pass
  * the part of the solute-only pass of Eq. FMMcalc that runs after the full
  * pass (its prologue overlaps the full pass on a side stream; 0 when not
  * requested); m2l_top the single tensor-core M2L launch of level l_max (0 when
@@ -126,7 +127,7 @@ enum {
     FMM_OPT_OVERLAP = 9    /* ival: 1 (default) runs a call on plan-owned streams: the far field on one above
                               the default priority, the near field (P2P, which needs only the sort) on one
                               of the lowest priority filling the SMs the far field leaves idle, the sparse
-                              solute pass of Eq. FMMcalc beside the L2P; 0 runs every stage in order on the
+                              solute pass of Eq. FMMcalc beside the far field; 0 runs every stage in order on the
                               plan's stream (the per-stage times then add up) */,
     FMM_OPT_M2L_GRADE = 10 /* ival = D2 | (D1 << 8), fp16x2 tensor-core M2L only: per K chunk of input coefficients
                               (64 per chunk), by the chunk's lowest degree lambda: lambda >= D1 keeps one product
@@ -138,7 +139,7 @@ enum {
                               below the first-term precision of the low degrees.  D2, D1 in 0..20; default
                               FMM_GRADE_DEFAULT.  The fused L2L and the solute-only pass always use 3
                               products */,
-    FMM_OPT_M2L_ACC_GROUP = 11 /* ival in 1..64: tensor-core M2L offsets whose products are summed in
+    FMM_OPT_M2L_ACC_GROUP = 11 /* ival in 1..64: mixed-path tensor-core M2L offsets whose products are summed in
                               one FP32 TMEM accumulator before it is drained into registers (the fused L2L
                               always alone); longer chains drain less often but carry more of the tensor
                               core's accumulation rounding; default FMM_ACC_GROUP_DEFAULT */,

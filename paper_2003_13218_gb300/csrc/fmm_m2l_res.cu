@@ -23,7 +23,8 @@
 // Orders above 15 (more than 256 coefficients) stay on the CUDA cores.
 //
 // Measured (energy, forces and solute-solvent energy, FP64 CUDA cores -> residues): 100,000 charges at depth 5,
-// p = 12 1,290 -> 12.4 ms (M2L kernels 1,283 -> 6.0 ms, now 4.7); 2,998 charges at depth 3, p = 8 581 -> 1.6 ms.  Forces
+// p = 12 1,290 -> 12.4 ms (M2L kernels 1,283 -> 6.0 ms; now 4.7 of a call's 7.0); 2,998 charges at depth 3, p = 8 581 ->
+// 1.6 ms, now 0.51; the lists of targets that take the FP64 sum cost 5 to 40 us of these calls.  Forces
 // against the same sums in 80-bit arithmetic: 3.7e-16 relative (FP64 sums 7.2e-16) at 1,000 charges, p = 8;
 // 4.9e-16 (5.4e-16) at 2,998, p = 4; 7.4e-15 (7.5e-15, the operator tables' own rounding) at p = 12.
 #include <math.h>

@@ -462,8 +462,10 @@ namespace {
 // about 128 target charges at the mean leaf occupancy (dense leaves: short rows, more blocks); the staging
 // capacity is 1.25 times the expected particle count of a tile's rows plus 256 (a tile beyond it reads global memory;
 // twice the count plus 512 left room for one block less per SM: 10M charges 23.1 -> 22.2 ms, 100k at ws = 2 1.62 ->
-// 1.53 ms), within 96 KB of
-// shared memory.  The FP32 path keeps one thread per target: it runs beside the far field
+// 1.53 ms), within 96 KB of shared memory.  Boxes filled to half or an eighth of their volume, the near field alone: 447 ->
+// 424 and 1,320 -> 1,007 us (1M, d = 6), 428 -> 358 us (100k, ws = 2, half); but 172 -> 238 us (61k, d = 4, half) and 61
+// -> 76 us (100k, d = 5, half), where it runs beside a longer far field.  The FP32 path keeps one thread per target for
+// the same reason
 template <typename T>
 fmm_status launch_p2p_tile(Plan &P, T h, T *phi, T *field)
 {

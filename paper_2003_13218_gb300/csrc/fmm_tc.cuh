@@ -7,15 +7,16 @@
 // 2..5 drain TMEM (warp w reads TMEM lanes 32 (w mod 4) .. +31, one target row
 // per thread) and write the FP32 level array.
 //
-// The issuer's instruction stream bounds the launch, not the tensor pipe or the
-// copies: halving the copied bytes or the MMAs per stage moved the level-6
-// launch (N = 1M, p = 12) by 1-6 %, taking a quarter of the ring away by 2 %,
-// while its per-stage code took ~900 cycles against 350-700 of MMA time.
-// Issued from a single-lane branch every TMA / MMA operand is moved to uniform
-// registers first; run by the whole warp, with the chunk structure fixed at
-// compile time (NCH) and the grading unpacked once per tile, the launch went
-// 3.69 -> 2.69 ms (N = 1M, p = 12), 24.9 -> 16.1 ms (N = 10M, p = 10) and
-// 2.00 -> 1.51 ms (N = 100k, ws = 2, p = 8).  Every mbarrier wait is bounded (globaltimer); on a timeout the
+// The tensor pipe bounds the large launches: active in 91 % of a CTA's cycles
+// (level 5 of 100,000 charges, p = 12; 75 % with the last wave).  It was the
+// issuer's instruction stream: halving the copied bytes or the MMAs per stage
+// moved the level-6 launch (N = 1M, p = 12) by 1-6 %, taking a quarter of the
+// ring away by 2 %, while its per-stage code took ~900 cycles against 350-700
+// of MMA time.  Issued from a single-lane branch every TMA / MMA operand is
+// moved to uniform registers first; run by the whole warp, with the chunk
+// structure fixed at compile time (NCH) and the grading unpacked once per tile,
+// the launch went 3.69 -> 2.69 ms (N = 1M, p = 12), 24.9 -> 16.1 ms (N = 10M,
+// p = 10) and 2.00 -> 1.51 ms (N = 100k, ws = 2, p = 8).  Every mbarrier wait is bounded (globaltimer); on a timeout the
 // kernel records FMM_ERR_TIMEOUT, waits (bounded) for its copies and MMAs in
 // flight, frees TMEM and returns.
 #pragma once
