@@ -53,7 +53,7 @@ struct ResConsts {
     int inv[RES_MAX];                            // (P / p_i)^-1 mod p_i, centred
     float rp[RES_MAX];
     uint32_t w[RES_MAX][3];                      // floor(2^96 / p_i), low word first
-    double pscale;                               // P / 2^96
+    double pscale;                               // P / 2^(96 + C)
     int mbits, tbits, keep;                      // B, C, K
 };
 
@@ -97,19 +97,28 @@ __device__ __forceinline__ void limbs(long long x, int &x0, int &x1, int &x2)
     x2 = (int)(x >> 36);
 }
 
-// g of a level from the bits of its largest |M~|: |M~ 2^g| < 2^mbits for every double, -968 <= g <= 1080
-__device__ __forceinline__ int res_gain(unsigned long long bits, int mbits)
+constexpr int GAIN_MAX = 800;
+
+// g of a level from the bits of its largest |M~|: |M~ 2^g| < 2^mbits
+__device__ __forceinline__ int res_gain_raw(unsigned long long bits, int mbits)
 {
     return bits == 0ull ? 0 : mbits - 1 - ((int)(bits >> 52) - 1023);
 }
 
+// whether the whole numbers hold a level: its largest moment is finite, and 2^g and its products with the scales and
+// with P are normal doubles; else all its targets take the FP64 sum
+__device__ __forceinline__ bool res_holds(unsigned long long bits, int mbits)
+{
+    const int g = res_gain_raw(bits, mbits);
+    return (bits >> 52) != 2047 && g <= GAIN_MAX && g >= -GAIN_MAX;
+}
+
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// 2^e = a b with both factors normal (moments below 2^-967 have a gain that no double holds)
-__device__ __forceinline__ void pow2_factors(int e, double &a, double &b)
+// 2^(sign g), 1 where the level is not held
+__device__ __forceinline__ double res_gain(unsigned long long bits, int mbits, int sign)
 {
-    a = pow2d(e / 2);
-    b = pow2d(e - e / 2);
+    return res_holds(bits, mbits) ? pow2d(sign * res_gain_raw(bits, mbits)) : 1.0;
 }
 
 // s(n,m) = sqrt((n+m)! (n-m)!) per real coefficient, and the moduli (by a kernel: the host would have to wait for the
@@ -164,8 +173,7 @@ __global__ void k_res_split(const double *__restrict__ M, int np, int hw, int nc
     const int np2 = np + 2 * hw;
     const int G = kp / 8;
     const int64_t ncell = 8 * (int64_t)np2 * np2 * np2, total = ncell * G;
-    double g0, g1;
-    pow2_factors(res_gain(*amax, c.mbits), g0, g1);
+    const double g = res_gain(*amax, c.mbits, 1);
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t cell = t / G;
         const int k0 = (int)(t - cell * G) * 8;
@@ -179,7 +187,7 @@ __global__ void k_res_split(const double *__restrict__ M, int np, int hw, int nc
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int k = k0 + u;
-            const long long x = k < nc ? __double2ll_rn(row[k] * __ldg(s + k) * g0 * g1) : 0;
+            const long long x = k < nc ? __double2ll_rn(row[k] * __ldg(s + k) * g) : 0;
             limbs(x, x0[u], x1[u], x2[u]);
         }
         uint16_t *out = planes + chunk_at(cell, ncell, k0, 64);
@@ -240,7 +248,7 @@ __device__ __forceinline__ bool res_low_list(const ResLow &d, int64_t cell, uint
 // Residues y_i of nb moduli (and of the offset groups) -> the 96-bit fraction sum y_i / p_i mod 1, and on the last
 // launch of the level L^ = P (fraction) 2^-(g + C) s(j).  Two neighbouring elements per thread (their
 // residues are one 32-bit load); frac carries the sums between the launches of a level.  The last launch also lists the
-// targets whose sources are too far below the level's largest, all of them where that is inf or NaN.
+// targets whose sources are too far below the level's largest, all of them where the whole numbers do not hold that.
 __global__ void __launch_bounds__(JOIN_THREADS) k_res_join(int64_t n, int nc, int groups, int m0, int nb,
                                                            const int16_t *__restrict__ resid, uint32_t *__restrict__ frac,
                                                            bool first, bool last, const double *__restrict__ s,
@@ -254,12 +262,11 @@ __global__ void __launch_bounds__(JOIN_THREADS) k_res_join(int64_t n, int nc, in
         const int64_t e1 = e0 + 2 * JOIN_THREADS < n ? e0 + 2 * JOIN_THREADS : n;
         const uint32_t hi = (uint32_t)(bits >> 32), down = (uint32_t)(c.mbits - c.keep) << 20;
         for (int64_t cell = (e0 + nc - 1) / nc + (threadIdx.x >> 5); cell * nc < e1; cell += JOIN_THREADS / 32)
-            if ((bits >> 52) == 2047 || (hi > down && res_low_list(d, cell, hi - down, threadIdx.x & 31)))
+            if (!res_holds(bits, c.mbits) || (hi > down && res_low_list(d, cell, hi - down, threadIdx.x & 31)))
                 if ((threadIdx.x & 31) == 0) d.list[atomicAdd(d.count, 1)] = d.base + (uint32_t)cell;
     }
     if (e >= n) return;  // n is even (8 parity classes)
-    double g0, g1;
-    pow2_factors(-res_gain(bits, c.mbits), g0, g1);
+    const double f = c.pscale * res_gain(bits, c.mbits, -1);
     long long a0[2] = {0, 0}, a1[2] = {0, 0}, a2[2] = {0, 0};
     for (int g = 0; g < groups; ++g)
 #pragma unroll 8
@@ -293,7 +300,7 @@ __global__ void __launch_bounds__(JOIN_THREADS) k_res_join(int64_t n, int nc, in
         }
         const long long top = (long long)(((uint64_t)hi << 32) | mid);  // signed: |L_int| < P / 2
         double v = (double)top * 4294967296.0 + (double)lo;
-        L[e + u] = v * c.pscale * s[(int)((e + u) % nc)] * pow2d(-c.tbits) * g0 * g1;
+        L[e + u] = v * f * s[(int)((e + u) % nc)];
     }
 }
 
@@ -407,7 +414,7 @@ bool choose_moduli(int nc, int tbits, double sum_bits, ResConsts &c)
     if (have < bits) return false;
     double pscale = 1.0;
     for (int i = 0; i < c.n; ++i) pscale *= (double)c.p[i] * ldexp(1.0, -6);
-    c.pscale = ldexp(pscale, 6 * c.n - 96);
+    c.pscale = ldexp(pscale, 6 * c.n - 96 - tbits);
     for (int i = 0; i < c.n; ++i) {
         const int p = c.p[i];
         auto centred = [p](int64_t v) {
